@@ -100,9 +100,9 @@ brahms_status brahms_init_grid(brahms_ctx** out, int nx, int ny, int nt, double 
   ctx->px = (float2*)(ctx->ws + ctx->L.px);
   ctx->py = (float2*)(ctx->ws + ctx->L.py);
   ctx->pt = (float2*)(ctx->ws + ctx->L.pt);
-  ctx->twx = (float4*)(ctx->ws + ctx->L.twx);
-  ctx->twy = (float4*)(ctx->ws + ctx->L.twy);
-  ctx->twt = (float4*)(ctx->ws + ctx->L.twt);
+  ctx->twx = (float2*)(ctx->ws + ctx->L.twx);
+  ctx->twy = (float2*)(ctx->ws + ctx->L.twy);
+  ctx->twt = (float2*)(ctx->ws + ctx->L.twt);
   ctx->partial = (double*)(ctx->ws + ctx->L.partial);
   ctx->energy_dev = (double*)(ctx->ws + ctx->L.energy);
   ctx->dev_err = (int*)(ctx->ws + ctx->L.err);

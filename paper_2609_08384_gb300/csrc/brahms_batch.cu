@@ -64,8 +64,8 @@ struct ShapeT {
   static constexpr int TTPC = tiles_per_cta_t<PT, kBT>();
   static constexpr int smem_floats2() {
     const int x = xtile_smem_floats2<NXY, kBT>(2);
-    const int y = 2 * tw_table_size<PY>() + YTPC * NXY * ColTile<PY>::value;
-    const int t = 2 * tw_table_size<PT>() + TTPC * NT * ColTile<PT>::value;
+    const int y = tw_table_size<PY>() + YTPC * NXY * ColTile<PY>::value;
+    const int t = tw_table_size<PT>() + TTPC * NT * ColTile<PT>::value;
     return x > y ? (x > t ? x : t) : (y > t ? y : t);
   }
 };
@@ -83,7 +83,7 @@ struct InstDev {
   float2* state;
   const float2* ecoef;  // stage factors of every x-pass: [step + 1][6] (see stage_table)
   long long fstride;
-  const float4 *twx, *twt;  // NX = NY: one table serves x and y
+  const float2 *twx, *twt;  // NX = NY: one table serves x and y
   const float2 *px, *py, *pt;
   int nx, ny, nt, shape;
   int nz;
@@ -181,7 +181,7 @@ template <int S>
 __device__ __noinline__ void run_item(const InstDev& I, const Item& it, float4* sm4) {
   using SH = ShapeT<S>;
   constexpr int NXY = SH::NXY, NT = SH::NT;
-  float4* tw = sm4;
+  float2* tw = reinterpret_cast<float2*>(sm4);
   if (it.type == kTypeX) {
     XPassArgs p{};
     p.data = I.state;
@@ -230,7 +230,7 @@ __device__ __noinline__ void run_item(const InstDev& I, const Item& it, float4* 
     a.xtiles = (NXY + ColTile<typename SH::PT>::value - 1) / ColTile<typename SH::PT>::value;
     a.ntiles = 2LL * NXY * a.xtiles;
     a.tw = I.twt;
-    float2* xch = reinterpret_cast<float2*>(tw + tw_table_size<typename SH::PT>());
+    float2* xch = tw + tw_table_size<typename SH::PT>();
     for (int i = threadIdx.x; i < tw_table_size<typename SH::PT>(); i += kBT) tw[i] = I.twt[i];
     __syncthreads();
     for (long long c = 0; c < it.ntiles; ++c) {
@@ -241,7 +241,7 @@ __device__ __noinline__ void run_item(const InstDev& I, const Item& it, float4* 
     a.xtiles = (NXY + ColTile<typename SH::PY>::value - 1) / ColTile<typename SH::PY>::value;
     a.ntiles = 2LL * NT * a.xtiles;
     a.tw = I.twx;
-    float2* xch = reinterpret_cast<float2*>(tw + tw_table_size<typename SH::PY>());
+    float2* xch = tw + tw_table_size<typename SH::PY>();
     for (int i = threadIdx.x; i < tw_table_size<typename SH::PY>(); i += kBT) tw[i] = I.twx[i];
     __syncthreads();
     for (long long c = 0; c < it.ntiles; ++c) {
@@ -390,7 +390,7 @@ struct BatchInstHost {
   brahms_field_params fp[2];
   char* mem = nullptr;  // state + tables until the instance joins a group (then NULL)
   float2* state = nullptr;
-  float4 *twx = nullptr, *twt = nullptr;
+  float2 *twx = nullptr, *twt = nullptr;
   float2 *px = nullptr, *py = nullptr, *pt = nullptr;
   const float2* ecoef = nullptr;  // its stage factors in its group's table, [step + 1][6]
   bool have_fields = false;
@@ -407,7 +407,7 @@ struct BatchGroup {
   char* mem = nullptr;
   float2* state = nullptr;
   float2 *px = nullptr, *py = nullptr, *pt = nullptr;
-  float4 *twx = nullptr, *twy = nullptr, *twt = nullptr;
+  float2 *twx = nullptr, *twy = nullptr, *twt = nullptr;
   GroupInst* params = nullptr;
   float2* ecoef = nullptr;  // stage factors [slot][steps + 1][6]
   int ecoef_steps = 0;      // steps per slot in the table (the group's largest nz)
@@ -578,9 +578,9 @@ brahms_status layout(brahms_batch* b) {
     };
     const size_t o_state = take(sizeof(float2) * 2 * n * m), o_px = take(sizeof(float2) * 2 * m * g.nx),
                  o_py = take(sizeof(float2) * 2 * m * g.ny), o_pt = take(sizeof(float2) * 2 * m * g.nt),
-                 o_twx = take(sizeof(float4) * tw_table_size_of(g.nx)),
-                 o_twy = take(sizeof(float4) * tw_table_size_of(g.ny)),
-                 o_twt = take(sizeof(float4) * tw_table_size_of(g.nt)), o_par = take(sizeof(GroupInst) * m);
+                 o_twx = take(sizeof(float2) * tw_table_size_of(g.nx)),
+                 o_twy = take(sizeof(float2) * tw_table_size_of(g.ny)),
+                 o_twt = take(sizeof(float2) * tw_table_size_of(g.nt)), o_par = take(sizeof(GroupInst) * m);
     g.ecoef_steps = 0;
     for (int i : g.members) g.ecoef_steps = std::max(g.ecoef_steps, b->inst[i].nz);
     const size_t o_coef = take(sizeof(float2) * 6 * (size_t)(g.ecoef_steps + 1) * m);
@@ -592,9 +592,9 @@ brahms_status layout(brahms_batch* b) {
     g.px = (float2*)(g.mem + o_px);
     g.py = (float2*)(g.mem + o_py);
     g.pt = (float2*)(g.mem + o_pt);
-    g.twx = (float4*)(g.mem + o_twx);
-    g.twy = (float4*)(g.mem + o_twy);
-    g.twt = (float4*)(g.mem + o_twt);
+    g.twx = (float2*)(g.mem + o_twx);
+    g.twy = (float2*)(g.mem + o_twy);
+    g.twt = (float2*)(g.mem + o_twt);
     g.params = (GroupInst*)(g.mem + o_par);
     g.ecoef = (float2*)(g.mem + o_coef);
     if (cudaStreamCreateWithFlags(&g.stream, cudaStreamNonBlocking) != cudaSuccess ||
@@ -1004,16 +1004,16 @@ brahms_status brahms_batch_add(brahms_batch* b, int nx, int ny, int nt, double d
   I.fp[1] = fp[1];
   const size_t n = (size_t)I.npoints();
   size_t o_state = 0, o_twx = al256(sizeof(float2) * 2 * n),
-         o_twt = o_twx + al256(sizeof(float4) * tw_table_size_of(nx)),
-         o_px = o_twt + al256(sizeof(float4) * tw_table_size_of(nt)), o_py = o_px + al256(sizeof(float2) * 2 * nx),
+         o_twt = o_twx + al256(sizeof(float2) * tw_table_size_of(nx)),
+         o_px = o_twt + al256(sizeof(float2) * tw_table_size_of(nt)), o_py = o_px + al256(sizeof(float2) * 2 * nx),
          o_pt = o_py + al256(sizeof(float2) * 2 * ny), total = o_pt + al256(sizeof(float2) * 2 * nt);
   if (dev_alloc((void**)&I.mem, total) != cudaSuccess) {
     cudaGetLastError();
     return bfail(b, BRAHMS_E_OOM, "device allocation failed");
   }
   I.state = (float2*)(I.mem + o_state);
-  I.twx = (float4*)(I.mem + o_twx);
-  I.twt = (float4*)(I.mem + o_twt);
+  I.twx = (float2*)(I.mem + o_twx);
+  I.twt = (float2*)(I.mem + o_twt);
   I.px = (float2*)(I.mem + o_px);
   I.py = (float2*)(I.mem + o_py);
   I.pt = (float2*)(I.mem + o_pt);

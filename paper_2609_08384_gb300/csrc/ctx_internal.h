@@ -42,9 +42,9 @@ inline Layout make_layout(int nx, int ny, int nt, int nf) {
   L.px = take(sizeof(float2) * nx * nf);
   L.py = take(sizeof(float2) * ny * nf);
   L.pt = take(sizeof(float2) * nt * nf);
-  L.twx = take(sizeof(float4) * brahms::tw_table_size_of(nx));
-  L.twy = take(sizeof(float4) * brahms::tw_table_size_of(ny));
-  L.twt = take(sizeof(float4) * brahms::tw_table_size_of(nt));
+  L.twx = take(sizeof(float2) * brahms::tw_table_size_of(nx));
+  L.twy = take(sizeof(float2) * brahms::tw_table_size_of(ny));
+  L.twt = take(sizeof(float2) * brahms::tw_table_size_of(nt));
   L.partial = take(sizeof(double) * kRedBlocks * nf);
   L.energy = take(sizeof(double) * nf);
   L.err = take(sizeof(int));
@@ -75,7 +75,7 @@ struct brahms_ctx {
   char* ws = nullptr;
   Layout L{};
   float2 *state = nullptr, *px = nullptr, *py = nullptr, *pt = nullptr;
-  float4 *twx = nullptr, *twy = nullptr, *twt = nullptr;
+  float2 *twx = nullptr, *twy = nullptr, *twt = nullptr;
   double *partial = nullptr, *energy_dev = nullptr;
   double* energy_host = nullptr;  // pinned, nf entries + the device error word
   double* diag_dev = nullptr;     // diagnostics: power [nf][nt], spectrum [nf][nt]

@@ -3,13 +3,47 @@
 // A pencil of length N is owned by T = N/E threads; each thread keeps E
 // complex values in registers.  One Stockham pass of radix R (Govindaraju et
 // al., "High performance discrete Fourier transforms on graphics processors",
-// SC'08, autosort formulation) reads the R inputs j + r N/R of butterfly j,
-// multiplies by W_N^{r (j mod Ns) N/(Ns R)}, applies a radix-R DFT and writes
-// the results to (j/Ns) Ns R + (j mod Ns) + r Ns.  Between passes the values
-// are exchanged through shared memory; the first pass reads its inputs
-// straight from global memory and the last pass leaves the outputs in
-// registers at positions j + r N/R_last, so a kernel stores them with
-// coalesced writes and never stages the whole pencil twice.
+// SC'08, autosort formulation) combines the R sub-transforms of butterfly j,
+// multiplying number r by W_{NS R}^{r m} (NS the product of the radices of the
+// earlier passes, m = j mod NS), with a radix-R DFT, and writes the results to
+// (j/NS) NS R + m + k NS.  Between passes the values are exchanged through
+// shared memory; the first pass reads its inputs straight from global memory
+// and the last pass leaves the outputs in registers, so a kernel stores them
+// with coalesced writes and never stages the whole pencil twice.
+//
+// Centred indices.  The digits of both indices of a twiddle are taken in
+// centred form (digit d of radix R as d or d - R, in [-R/2, R/2)), so that no
+// twiddle turns by much more than a quarter of the circle.  A sub-transform of
+// r - R takes its inputs one place later than that of r, and with m' in the
+// place of m output k is number m' + k NS: the butterflies and exchanges stay
+// as they are, and only the positions of the first pass's inputs and of the
+// last pass's outputs move (pos_first, pos_last).
+//
+// Twiddles as shears.  A turn by phi is the product of three shears,
+//   x += p y,  y += s x,  x += p y,  p = -tan(phi / 2), s = sin(phi)
+// (the lifting form of a plane rotation; Buneman's tan/sin twiddles): three
+// FMAs where the product with a twiddle held as hi + lo floats took eight.
+// Each shear has determinant 1 whatever the rounding of p and s, and the same
+// three shears with the signs turned are its exact inverse.  The inverse
+// transform is built as the exact mirror of the forward one (decimation in
+// frequency against decimation in time: the same twiddles on the same values,
+// and codelets whose inner factors mirror each other), so what the rounded
+// twiddles do to a field the way back undoes, and the energy of a field that
+// passes them again and again does not drift.  (With c and s rounded to single
+// floats |c + i s| differs from 1 and it does; a pair of directions that are
+// not each other's mirror let the energy of the 3 x 256x256x512 parametric run
+// fall by 7e-9 per step.)  |phi| <= 1/4 turn, or a little more in plans of three
+// and four passes, keeps p near 1 or below.
+// Error against FP64 of 3D transforms of random fields: forward 1.51e-7 (with
+// hi + lo twiddles 1.48e-7), forward and inverse 2.11e-7 (2.10e-7); energy of
+// smooth beams over 100 z-steps: rms 1.8e-9 to 2.6e-9 per step (1.7e-9 to 5.6e-9).
+//
+// Packed arithmetic.  A complex value is an aligned register pair, and sums of
+// complex values are single add/sub.f32x2 instructions.  One FFMA2 occupies the
+// FP32 pipe as long as two FFMA but takes one issue slot, so packed sums leave
+// issue slots to the loads, address arithmetic and exchanges (measured per 16
+// FMA lanes and warp: FFMA with 4 logic operations 10.9 ns, FFMA2 with 4 logic
+// operations 8.5 ns, either alone 8.0 - 8.3 ns).
 //
 // The forward transform is unnormalised with e^{-2 pi i m n / N}; the inverse
 // uses e^{+...} and the radix order reversed, so that the inverse's first
@@ -21,8 +55,15 @@
 
 namespace brahms {
 
-__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
+__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 csub(float2 a, float2 b) {
+  float2 d;
+  asm("{\n .reg .b64 x, y, z;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %5};\n sub.rn.f32x2 z, x, y;\n"
+      " mov.b64 {%0, %1}, z;\n}"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return d;
+}
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
   return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
 }
@@ -31,51 +72,67 @@ __device__ __forceinline__ float2 cmulc(float2 a, float2 b) {
   return make_float2(fmaf(a.x, b.x, a.y * b.y), fmaf(a.y, b.x, -a.x * b.y));
 }
 __device__ __forceinline__ float2 cscale(float2 a, float s) { return make_float2(a.x * s, a.y * s); }
-// multiply by -i (forward sign) or +i (inverse sign)
-template <bool INV>
-__device__ __forceinline__ float2 rot90(float2 a) {
-  return INV ? make_float2(-a.y, a.x) : make_float2(a.y, -a.x);
+// a + t^Q b, t = -i (forward) or +i (inverse), Q taken mod 4: a quarter turn of
+// b is a choice of the components that are added or subtracted
+template <bool INV, int Q>
+__device__ __forceinline__ float2 add_turned(float2 a, float2 b) {
+  constexpr int q = ((INV ? -Q : Q) % 4 + 4) % 4;
+  if constexpr (q == 0) return cadd(a, b);
+  else if constexpr (q == 2) return csub(a, b);
+  else if constexpr (q == 1) return make_float2(a.x + b.y, a.y - b.x);
+  else return make_float2(a.x - b.y, a.y + b.x);
 }
-// Irrational codelet constants as hi + lo float pairs.  Rounded to one float
-// each, cos(pi/4), cos(pi/8) and sin(pi/8) all have |w| slightly below 1
-// (|w|^2 - 1 = -3.4e-8 for the pi/4 pair, -5.7e-8 for the pi/8 pair), and
-// because a z-step applies the same factors again and again the field energy
-// would drift by about -2e-7 per step.  Multiplying by hi and lo (one extra
-// FMA) makes each product correctly rounded, so rounding errors are unbiased.
-constexpr double kS2d = 0.70710678118654752440084436210485;   // cos(pi/4)
-constexpr double kC16d = 0.92387953251128675612818318939679;  // cos(pi/8)
-constexpr double kS16d = 0.38268343236508977172845998403040;  // sin(pi/8)
-constexpr double kS3d = 0.86602540378443864676372317075294;   // sin(pi/3)
-constexpr float kS2 = (float)kS2d, kS2lo = (float)(kS2d - (double)(float)kS2d);
-constexpr float kC16 = (float)kC16d, kC16lo = (float)(kC16d - (double)(float)kC16d);
-constexpr float kS16 = (float)kS16d, kS16lo = (float)(kS16d - (double)(float)kS16d);
-constexpr float kS3 = (float)kS3d, kS3lo = (float)(kS3d - (double)(float)kS3d);
 
-// u * c with c = hi + lo
-__device__ __forceinline__ float xmul(float u, float hi, float lo) { return fmaf(u, hi, u * lo); }
-// a * (c -/+ i s) with c = ch + cl, s = sh + sl (forward uses minus)
-template <bool INV>
-__device__ __forceinline__ float2 twx(float2 a, float ch, float cl, float sh, float sl) {
-  if (INV)
-    return make_float2(fmaf(a.x, ch, fmaf(-a.y, sh, fmaf(a.x, cl, -a.y * sl))),
-                       fmaf(a.y, ch, fmaf(a.x, sh, fmaf(a.y, cl, a.x * sl))));
-  return make_float2(fmaf(a.x, ch, fmaf(a.y, sh, fmaf(a.x, cl, a.y * sl))),
-                     fmaf(a.y, ch, fmaf(-a.x, sh, fmaf(a.y, cl, -a.x * sl))));
-}
-// a * W8^1 (forward: (1 - i)/sqrt 2; inverse: (1 + i)/sqrt 2)
-template <bool INV>
-__device__ __forceinline__ float2 w8_1(float2 a) {
-  return INV ? make_float2(xmul(a.x - a.y, kS2, kS2lo), xmul(a.x + a.y, kS2, kS2lo))
-             : make_float2(xmul(a.x + a.y, kS2, kS2lo), xmul(a.y - a.x, kS2, kS2lo));
-}
-// a * W8^3 (forward: (-1 - i)/sqrt 2; inverse: (-1 + i)/sqrt 2)
-template <bool INV>
-__device__ __forceinline__ float2 w8_3(float2 a) {
-  return INV ? make_float2(-xmul(a.x + a.y, kS2, kS2lo), xmul(a.x - a.y, kS2, kS2lo))
-             : make_float2(xmul(a.y - a.x, kS2, kS2lo), -xmul(a.x + a.y, kS2, kS2lo));
+// a turn by the three shears of (p, s) (see the header)
+__device__ __forceinline__ float2 shear_turn(float2 a, float p, float s) {
+  const float x = fmaf(p, a.y, a.x);
+  const float y = fmaf(s, x, a.y);
+  return make_float2(fmaf(p, y, x), y);
 }
 
 // ---------------------------------------------------------------- codelets
+// tan(pi k / 32) and sin(pi k / 16), k = 0..4
+__host__ __device__ constexpr double tan_pi32(int k) {
+  return k == 0 ? 0.0
+       : k == 1 ? 0.098491403357164253077197521291327
+       : k == 2 ? 0.19891236737965800691159762264468
+       : k == 3 ? 0.30334668360734239167588394694130
+                : 0.41421356237309504880168872420970;
+}
+__host__ __device__ constexpr double sin_pi16(int k) {
+  return k == 0 ? 0.0
+       : k == 1 ? 0.19509032201612826784828486847702
+       : k == 2 ? 0.38268343236508977172845998403040
+       : k == 3 ? 0.55557023301960222474283081394853
+                : 0.70710678118654752440084436210485;
+}
+// W32^E = (-/+ i)^quarter(E) W32^rest(E), rest in [-3, 4]
+__host__ __device__ constexpr int w32_quarter(int e) { return ((e + 3) / 8) % 4; }
+__host__ __device__ constexpr int w32_rest(int e) { return e - 8 * ((e + 3) / 8); }
+// a times W32^rest(E); the quarter turns are left to the additions that follow
+template <bool INV, int E>
+__device__ __forceinline__ float2 w32_shear(float2 a) {
+  constexpr int k = w32_rest(E);
+  if constexpr (k == 0) return a;
+  else {
+    constexpr int ak = k < 0 ? -k : k;
+    // forward: phi = -2 pi k / 32
+    constexpr bool pos = (k < 0) != INV;
+    if constexpr (ak == 4) {
+      // one eighth of a turn: (x -/+ y) / sqrt 2 with the factor as hi + lo.  The
+      // turn most used is kept exact: as rounded shears it is 1.9e-8 short of
+      // orthogonal, and smooth beams lost 7e-9 of their energy per z-step
+      const float2 d = pos ? make_float2(a.x - a.y, a.x + a.y) : make_float2(a.x + a.y, a.y - a.x);
+      constexpr float ch = (float)sin_pi16(4), cl = (float)(sin_pi16(4) - (double)ch);
+      return __ffma2_rn(d, make_float2(ch, ch), __fmul2_rn(d, make_float2(cl, cl)));
+    } else {
+      constexpr float p = (float)(pos ? -tan_pi32(ak) : tan_pi32(ak));
+      constexpr float s = (float)(pos ? sin_pi16(ak) : -sin_pi16(ak));
+      return shear_turn(a, p, s);
+    }
+  }
+}
+
 template <bool INV>
 __device__ __forceinline__ void dft2(float2& a, float2& b) {
   float2 t = a;
@@ -83,158 +140,139 @@ __device__ __forceinline__ void dft2(float2& a, float2& b) {
   b = csub(t, b);
 }
 
-template <bool INV>
+// four-point DFT of v0, t^Q1 v1, t^Q2 v2, t^Q3 v3 (pending quarter turns)
+template <bool INV, int Q1 = 0, int Q2 = 0, int Q3 = 0>
 __device__ __forceinline__ void dft4(float2& v0, float2& v1, float2& v2, float2& v3) {
-  float2 a = cadd(v0, v2), b = csub(v0, v2), c = cadd(v1, v3), d = rot90<INV>(csub(v1, v3));
-  v0 = cadd(a, c);
-  v2 = csub(a, c);
-  v1 = cadd(b, d);
-  v3 = csub(b, d);
+  const float2 a = add_turned<INV, Q2>(v0, v2), b = add_turned<INV, Q2 + 2>(v0, v2);
+  const float2 c = add_turned<INV, Q3 - Q1>(v1, v3), d = add_turned<INV, Q3 - Q1 + 2>(v1, v3);
+  v0 = add_turned<INV, Q1>(a, c);
+  v2 = add_turned<INV, Q1 + 2>(a, c);
+  v1 = add_turned<INV, Q1 + 1>(b, d);
+  v3 = add_turned<INV, Q1 + 3>(b, d);
 }
+
+// sin(pi/3) as hi + lo floats: in the three-point DFT it is a factor, not a
+// turn, so its rounding would change the energy of a field a little each time
+constexpr double kS3d = 0.86602540378443864676372317075294;
+constexpr float kS3 = (float)kS3d, kS3lo = (float)(kS3d - (double)(float)kS3d);
 
 template <bool INV>
 __device__ __forceinline__ void dft3(float2& v0, float2& v1, float2& v2) {
-  float2 s = cadd(v1, v2);
-  float2 t = make_float2(fmaf(-0.5f, s.x, v0.x), fmaf(-0.5f, s.y, v0.y));
+  const float2 s = cadd(v1, v2);
+  const float2 t = __ffma2_rn(s, make_float2(-0.5f, -0.5f), v0);
   const float2 d = csub(v1, v2);
-  float2 u = rot90<INV>(make_float2(xmul(d.x, kS3, kS3lo), xmul(d.y, kS3, kS3lo)));
+  const float2 u = __ffma2_rn(d, make_float2(kS3, kS3), __fmul2_rn(d, make_float2(kS3lo, kS3lo)));
   v0 = cadd(v0, s);
-  v1 = cadd(t, u);
-  v2 = csub(t, u);
+  v1 = add_turned<INV, 1>(t, u);
+  v2 = add_turned<INV, 3>(t, u);
 }
 
-// radix 8 = 2 x 4: n = 4 n1 + n2, k = k1 + 2 k2
+// Radix 8: forward n = 4 n1 + n2, k = k1 + 2 k2 as sums over n1, turns by
+// W8^{n2 k1}, four-point transforms over n2; the inverse takes the same steps
+// backwards (its input number k may carry a pending quarter turn Qk).
+template <int Q1 = 0, int Q2 = 0, int Q3 = 0, int Q4 = 0, int Q5 = 0, int Q6 = 0, int Q7 = 0>
+__device__ __forceinline__ void idft8(float2* v) {
+  static_assert(Q1 == 0, "number 1 carries no turn");
+  dft4<true, Q2, Q4, Q6>(v[0], v[2], v[4], v[6]);
+  dft4<true, Q3, Q5, Q7>(v[1], v[3], v[5], v[7]);
+  const float2 y0[4] = {v[0], v[2], v[4], v[6]};
+  const float2 y1[4] = {v[1], w32_shear<true, 4>(v[3]), v[5], w32_shear<true, 12>(v[7])};
+  v[0] = cadd(y0[0], y1[0]);
+  v[4] = csub(y0[0], y1[0]);
+  v[1] = cadd(y0[1], y1[1]);
+  v[5] = csub(y0[1], y1[1]);
+  v[2] = add_turned<true, 1>(y0[2], y1[2]);
+  v[6] = add_turned<true, 3>(y0[2], y1[2]);
+  v[3] = add_turned<true, 1>(y0[3], y1[3]);
+  v[7] = add_turned<true, 3>(y0[3], y1[3]);
+}
 template <bool INV>
 __device__ __forceinline__ void dft8(float2* v) {
-  float2 y0[4], y1[4];
+  if constexpr (INV) {
+    idft8<>(v);
+  } else {
+    float2 y0[4], y1[4];
 #pragma unroll
-  for (int n2 = 0; n2 < 4; ++n2) {
-    y0[n2] = cadd(v[n2], v[n2 + 4]);
-    y1[n2] = csub(v[n2], v[n2 + 4]);
-  }
-  y1[1] = w8_1<INV>(y1[1]);
-  y1[2] = rot90<INV>(y1[2]);
-  y1[3] = w8_3<INV>(y1[3]);
-  dft4<INV>(y0[0], y0[1], y0[2], y0[3]);
-  dft4<INV>(y1[0], y1[1], y1[2], y1[3]);
+    for (int n2 = 0; n2 < 4; ++n2) {
+      y0[n2] = cadd(v[n2], v[n2 + 4]);
+      y1[n2] = csub(v[n2], v[n2 + 4]);
+    }
+    y1[1] = w32_shear<false, 4>(y1[1]);
+    y1[3] = w32_shear<false, 12>(y1[3]);
+    dft4<false>(y0[0], y0[1], y0[2], y0[3]);
+    dft4<false, w32_quarter(4), w32_quarter(8), w32_quarter(12)>(y1[0], y1[1], y1[2], y1[3]);
 #pragma unroll
-  for (int k2 = 0; k2 < 4; ++k2) {
-    v[2 * k2] = y0[k2];
-    v[2 * k2 + 1] = y1[k2];
+    for (int k2 = 0; k2 < 4; ++k2) {
+      v[2 * k2] = y0[k2];
+      v[2 * k2 + 1] = y1[k2];
+    }
   }
 }
 
-// multiply by W16^e, e in [0, 9]
-template <bool INV, int E>
-__device__ __forceinline__ float2 w16(float2 a) {
-  if constexpr (E == 0) return a;
-  else if constexpr (E == 1) return twx<INV>(a, kC16, kC16lo, kS16, kS16lo);
-  else if constexpr (E == 2) return w8_1<INV>(a);
-  else if constexpr (E == 3) return twx<INV>(a, kS16, kS16lo, kC16, kC16lo);
-  else if constexpr (E == 4) return rot90<INV>(a);
-  else if constexpr (E == 6) return w8_3<INV>(a);
-  else if constexpr (E == 9) return twx<INV>(a, -kC16, -kC16lo, -kS16, -kS16lo);
-  else return a;
+// Radix 4 M (M = 4 or 8): n = 4 n1 + n2 (n1 < M, n2 < 4), k = k1 + M k2: M-point
+// transforms over n1, turns by W_{4M}^{n2 k1}, four-point transforms over n2
+// (radix 16 is its own mirror; radix 32's inverse runs them backwards)
+template <bool INV, int M, int K1>
+__device__ __forceinline__ void dft4m_column(float2 (&y)[4][M], float2* v) {
+  constexpr int U = 8 / M;  // W_{4M} = W32^U
+  float2 b0 = y[0][K1], b1 = w32_shear<INV, U * K1>(y[1][K1]), b2 = w32_shear<INV, 2 * U * K1>(y[2][K1]),
+         b3 = w32_shear<INV, 3 * U * K1>(y[3][K1]);
+  dft4<INV, w32_quarter(U * K1), w32_quarter(2 * U * K1), w32_quarter(3 * U * K1)>(b0, b1, b2, b3);
+  v[K1] = b0;
+  v[K1 + M] = b1;
+  v[K1 + 2 * M] = b2;
+  v[K1 + 3 * M] = b3;
+  if constexpr (K1 + 1 < M) dft4m_column<INV, M, K1 + 1>(y, v);
 }
-
-// radix 16 = 4 x 4: n = 4 n1 + n2, k = k1 + 4 k2
 template <bool INV>
 __device__ __forceinline__ void dft16(float2* v) {
   float2 y[4][4];
 #pragma unroll
   for (int n2 = 0; n2 < 4; ++n2) {
-    float2 a0 = v[n2], a1 = v[4 + n2], a2 = v[8 + n2], a3 = v[12 + n2];
-    dft4<INV>(a0, a1, a2, a3);
-    y[n2][0] = a0;
-    y[n2][1] = a1;
-    y[n2][2] = a2;
-    y[n2][3] = a3;
-  }
-  y[1][1] = w16<INV, 1>(y[1][1]);
-  y[1][2] = w16<INV, 2>(y[1][2]);
-  y[1][3] = w16<INV, 3>(y[1][3]);
-  y[2][1] = w16<INV, 2>(y[2][1]);
-  y[2][2] = w16<INV, 4>(y[2][2]);
-  y[2][3] = w16<INV, 6>(y[2][3]);
-  y[3][1] = w16<INV, 3>(y[3][1]);
-  y[3][2] = w16<INV, 6>(y[3][2]);
-  y[3][3] = w16<INV, 9>(y[3][3]);
 #pragma unroll
-  for (int k1 = 0; k1 < 4; ++k1) {
-    float2 b0 = y[0][k1], b1 = y[1][k1], b2 = y[2][k1], b3 = y[3][k1];
-    dft4<INV>(b0, b1, b2, b3);
-    v[k1] = b0;
-    v[k1 + 4] = b1;
-    v[k1 + 8] = b2;
-    v[k1 + 12] = b3;
+    for (int n1 = 0; n1 < 4; ++n1) y[n2][n1] = v[4 * n1 + n2];
+    dft4<INV>(y[n2][0], y[n2][1], y[n2][2], y[n2][3]);
   }
+  dft4m_column<INV, 4, 0>(y, v);
 }
-
-// cos(pi k / 16) for any integer k, in double (compile time): the first
-// quadrant's values, the rest by symmetry.
-__host__ __device__ constexpr double cos_pi16_q(int k) {
-  return k == 0 ? 1.0
-       : k == 1 ? 0.98078528040323044912618223613424
-       : k == 2 ? 0.92387953251128675612818318939679
-       : k == 3 ? 0.83146961230254523707878837761791
-       : k == 4 ? 0.70710678118654752440084436210485
-       : k == 5 ? 0.55557023301960222474283081394853
-       : k == 6 ? 0.38268343236508977172845998403040
-       : k == 7 ? 0.19509032201612826784828486847702
-                : 0.0;
+// row n2 of the inverse radix 32: turns by W32^{n2 k1}, eight points over k1
+template <int N2>
+__device__ __forceinline__ void idft32_row(float2 (&y)[4][8], float2* v) {
+  float2* z = y[N2];
+  z[1] = w32_shear<true, N2>(z[1]);
+  z[2] = w32_shear<true, 2 * N2>(z[2]);
+  z[3] = w32_shear<true, 3 * N2>(z[3]);
+  z[4] = w32_shear<true, 4 * N2>(z[4]);
+  z[5] = w32_shear<true, 5 * N2>(z[5]);
+  z[6] = w32_shear<true, 6 * N2>(z[6]);
+  z[7] = w32_shear<true, 7 * N2>(z[7]);
+  idft8<w32_quarter(N2), w32_quarter(2 * N2), w32_quarter(3 * N2), w32_quarter(4 * N2), w32_quarter(5 * N2),
+        w32_quarter(6 * N2), w32_quarter(7 * N2)>(z);
+#pragma unroll
+  for (int n1 = 0; n1 < 8; ++n1) v[4 * n1 + N2] = z[n1];
 }
-__host__ __device__ constexpr double cos_pi16(int k) {
-  return (k % 32 + 32) % 32 > 16 ? cos_pi16(32 - (k % 32 + 32) % 32)
-       : (k % 32 + 32) % 32 > 8  ? -cos_pi16_q(16 - (k % 32 + 32) % 32)
-                                 : cos_pi16_q((k % 32 + 32) % 32);
-}
-__host__ __device__ constexpr double sin_pi16(int k) { return cos_pi16(8 - k); }
-__host__ __device__ constexpr float hi_of(double v) { return (float)v; }
-__host__ __device__ constexpr float lo_of(double v) { return (float)(v - (double)(float)v); }
-
-// multiply by W32^e = e^{-/+ 2 pi i e / 32}: the exact cases (multiples of
-// 8) as swaps and signs, the others through W16 or as hi + lo products
-template <bool INV, int E>
-__device__ __forceinline__ float2 w32(float2 a) {
-  if constexpr (E % 2 == 0 && (E / 2 <= 4 || E / 2 == 6 || E / 2 == 9)) return w16<INV, E / 2>(a);
-  else if constexpr (E == 16) return make_float2(-a.x, -a.y);
-  else {
-    constexpr double c = cos_pi16(E), s = sin_pi16(E);
-    return twx<INV>(a, hi_of(c), lo_of(c), hi_of(s), lo_of(s));
-  }
-}
-
-// radix 32 = 8 x 4: n = 4 n1 + n2 (n1 < 8, n2 < 4), k = k1 + 8 k2; eight-point
-// transforms over n1, twiddles W32^{n2 k1}, four-point transforms over n2
 template <bool INV>
 __device__ __forceinline__ void dft32(float2* v) {
   float2 y[4][8];
+  if constexpr (INV) {
 #pragma unroll
-  for (int n2 = 0; n2 < 4; ++n2) {
+    for (int k1 = 0; k1 < 8; ++k1) {
 #pragma unroll
-    for (int n1 = 0; n1 < 8; ++n1) y[n2][n1] = v[4 * n1 + n2];
-    dft8<INV>(y[n2]);
-  }
-#define BRAHMS_W32_ROW(N2)                   \
-  y[N2][1] = w32<INV, N2 * 1>(y[N2][1]);     \
-  y[N2][2] = w32<INV, N2 * 2>(y[N2][2]);     \
-  y[N2][3] = w32<INV, N2 * 3>(y[N2][3]);     \
-  y[N2][4] = w32<INV, N2 * 4>(y[N2][4]);     \
-  y[N2][5] = w32<INV, N2 * 5>(y[N2][5]);     \
-  y[N2][6] = w32<INV, N2 * 6>(y[N2][6]);     \
-  y[N2][7] = w32<INV, N2 * 7>(y[N2][7]);
-  BRAHMS_W32_ROW(1)
-  BRAHMS_W32_ROW(2)
-  BRAHMS_W32_ROW(3)
-#undef BRAHMS_W32_ROW
+      for (int k2 = 0; k2 < 4; ++k2) y[k2][k1] = v[k1 + 8 * k2];
+      dft4<true>(y[0][k1], y[1][k1], y[2][k1], y[3][k1]);
+    }
+    idft32_row<0>(y, v);
+    idft32_row<1>(y, v);
+    idft32_row<2>(y, v);
+    idft32_row<3>(y, v);
+  } else {
 #pragma unroll
-  for (int k1 = 0; k1 < 8; ++k1) {
-    float2 b0 = y[0][k1], b1 = y[1][k1], b2 = y[2][k1], b3 = y[3][k1];
-    dft4<INV>(b0, b1, b2, b3);
-    v[k1] = b0;
-    v[k1 + 8] = b1;
-    v[k1 + 16] = b2;
-    v[k1 + 24] = b3;
+    for (int n2 = 0; n2 < 4; ++n2) {
+#pragma unroll
+      for (int n1 = 0; n1 < 8; ++n1) y[n2][n1] = v[4 * n1 + n2];
+      dft8<false>(y[n2]);
+    }
+    dft4m_column<false, 8, 0>(y, v);
   }
 }
 
@@ -305,6 +343,35 @@ __host__ __device__ constexpr int fft_ns(int p) {
   return s;
 }
 
+// Centred number of butterfly j's first-pass inputs in a direction (input r of
+// butterfly j is number centred_first(j) + r N/R0 of the pencil): the lowest
+// digit of j belongs to the last pass, the highest to pass 1.
+template <class PL, bool INV>
+__host__ __device__ __forceinline__ int centred_first(int j) {
+  int n = 0, w = 1;
+#pragma unroll
+  for (int p = PL::NP - 1; p >= 1; --p) {
+    const int R = fft_radix<PL, INV>(p);
+    const int d = j % R;
+    n += w * (d >= (R + 1) / 2 ? d - R : d);
+    j /= R;
+    w *= R;
+  }
+  return n;
+}
+// Position of input r of butterfly j in the first pass of a direction; output r
+// of butterfly j in the last pass of the other direction lies at the same place.
+template <class PL, bool INV>
+__device__ __forceinline__ int pos_first(int j, int r) {
+  constexpr int S0 = PL::N / fft_radix<PL, INV>(0);
+  const int n = centred_first<PL, INV>(j) + r * S0;
+  return r == 0 && n < 0 ? n + PL::N : n;
+}
+template <class PL, bool INV>
+__device__ __forceinline__ int pos_last(int j, int k) {
+  return pos_first<PL, !INV>(j, k);
+}
+
 // ---------------------------------------------------------------- exchange
 // Contiguous pencil (one row of x): one padding slot per 16 entries.
 struct XchRow {
@@ -334,30 +401,17 @@ struct XchColSplit {
   __device__ __forceinline__ float ld(int pos) const { return base[pos * TX + tx]; }
 };
 
-// Twiddle tables hold W = (c, s) as hi + lo float pairs, float4 (ch, sh, cl,
-// sl): a product with the table is then correctly rounded, so the FFT carries
-// no systematic modulus error from rounded twiddles.
-__device__ __forceinline__ float2 tw_mul(float2 a, float4 w) { return twx<true>(a, w.x, w.z, w.y, w.w); }
-
-// Per-pass layout: pass P >= 1 of a direction with radix R and stride NS owns
-// the R x NS block [r][m] = exp(-/+ 2 pi i r m / (NS R)) (inverse entries are
-// stored conjugated), so the threads of a warp, whose butterflies have
-// consecutive m, read consecutive entries.  Forward blocks come first.
-template <class PL, bool INV>
-__host__ __device__ constexpr int tw_dir_size() {
-  int s = 0, ns = 1;
-  for (int q = 0; q < PL::NP; ++q) {
-    const int r = INV ? PL::r(PL::NP - 1 - q) : PL::r(q);
-    if (q > 0) s += r * ns;
-    ns *= r;
-  }
-  return s;
-}
-template <class PL, bool INV>
+// Per-pass twiddle layout: forward pass P >= 1 with radix R and stride NS owns the
+// R x NS block [r][m] of the shears (p, s) of the turn by -2 pi r' m' / (NS R), r'
+// the centred r and m' the number of m with its digits centred (lowest digit:
+// pass 0), so the threads of a warp, whose butterflies have consecutive m, read
+// consecutive entries.  The inverse turns its outputs k of pass NP-1-P by the
+// same entries [k][j / NS] with the signs turned.
+template <class PL>
 __host__ __device__ constexpr int tw_pass_off(int P) {
-  int o = INV ? tw_dir_size<PL, false>() : 0, ns = 1;
+  int o = 0, ns = 1;
   for (int q = 0; q < P; ++q) {
-    const int r = INV ? PL::r(PL::NP - 1 - q) : PL::r(q);
+    const int r = PL::r(q);
     if (q > 0) o += r * ns;
     ns *= r;
   }
@@ -365,18 +419,17 @@ __host__ __device__ constexpr int tw_pass_off(int P) {
 }
 template <class PL>
 __host__ __device__ constexpr int tw_table_size() {
-  return tw_dir_size<PL, false>() + tw_dir_size<PL, true>() > 0 ? tw_dir_size<PL, false>() + tw_dir_size<PL, true>()
-                                                                  : 1;
+  return PL::NP > 1 ? tw_pass_off<PL>(PL::NP) : 1;
 }
 
 // twiddle access from shared memory or, read-only, through L1
 struct TwShared {
-  const float4* p;
-  __device__ __forceinline__ float4 operator()(int i) const { return p[i]; }
+  const float2* p;
+  __device__ __forceinline__ float2 operator()(int i) const { return p[i]; }
 };
 struct TwGlobal {
-  const float4* p;
-  __device__ __forceinline__ float4 operator()(int i) const { return __ldg(p + i); }
+  const float2* p;
+  __device__ __forceinline__ float2 operator()(int i) const { return __ldg(p + i); }
 };
 
 // Barrier used around shared-memory exchanges: the whole CTA, or only the
@@ -400,19 +453,31 @@ __device__ __forceinline__ void fft_run(float2 (&v)[PL::E], int t, const X& x, c
   constexpr int NS = fft_ns<PL, INV>(P);
   constexpr int B = E / R;
   static_assert(E % R == 0, "E must be a multiple of every radix");
-  if constexpr (NS > 1) {
+  if constexpr (!INV && P > 0) {
 #pragma unroll
     for (int b = 0; b < B; ++b) {
-      const int j = t + b * T;
-      const int m = j % NS;
+      const int m = (t + b * T) % NS;
 #pragma unroll
       for (int r = 1; r < R; ++r) {
-        v[b * R + r] = tw_mul(v[b * R + r], tw(tw_pass_off<PL, INV>(P) + r * NS + m));
+        const float2 w = tw(tw_pass_off<PL>(P) + r * NS + m);
+        v[b * R + r] = shear_turn(v[b * R + r], w.x, w.y);
       }
     }
   }
 #pragma unroll
   for (int b = 0; b < B; ++b) dft<R, INV>(&v[b * R]);
+  if constexpr (INV && P + 1 < NP) {
+    constexpr int REST = N / (NS * R);
+#pragma unroll
+    for (int b = 0; b < B; ++b) {
+      const int q = (t + b * T) / NS;
+#pragma unroll
+      for (int k = 1; k < R; ++k) {
+        const float2 w = tw(tw_pass_off<PL>(NP - 1 - P) + k * REST + q);
+        v[b * R + k] = shear_turn(v[b * R + k], -w.x, -w.y);
+      }
+    }
+  }
   if constexpr (P + 1 < NP) {
     constexpr int R2 = fft_radix<PL, INV>(P + 1);
     constexpr int B2 = E / R2;

@@ -87,36 +87,36 @@ static int plan_radices(int n, int* r) {
   }
 }
 
-// Per-pass twiddle blocks (the layout of tw_pass_off): for each direction
-// and pass P >= 1 with radix R after stride NS, entries [r][m] =
-// exp(sign 2 pi i (r m mod NS R) / (NS R)), sign -1 forward and +1 inverse,
-// evaluated in FP64 and split into hi + lo floats.
-cudaError_t upload_twiddles(float4* tw, int n, cudaStream_t s) {
+static int centred(int d, int n) { return d >= (n + 1) / 2 ? d - n : d; }
+
+// Per-pass twiddle blocks (the layout of tw_pass_off): for each pass P >= 1 with
+// radix R after stride NS, entries [r][m] = the shears (-tan(phi/2), sin(phi)) of
+// phi = -2 pi r' m' / (NS R), the digits of r and m centred, evaluated in FP64.
+cudaError_t upload_twiddles(float2* tw, int n, cudaStream_t s) {
   int rad[8];
   const int np = plan_radices(n, rad);
   if (np <= 0) return cudaErrorInvalidValue;
-  std::vector<float4> h;
-  for (int dir = 0; dir < 2; ++dir) {
-    const double sign = dir == 0 ? -1.0 : 1.0;
-    int ns = 1;
-    for (int q = 0; q < np; ++q) {
-      const int R = dir == 0 ? rad[q] : rad[np - 1 - q];
-      if (q > 0) {
-        for (int r = 0; r < R; ++r)
-          for (int mm = 0; mm < ns; ++mm) {
-            const long long k = ((long long)r * mm) % ((long long)ns * R);
-            const double ang = sign * 6.283185307179586476925286766559 * (double)k / (double)(ns * R);
-            const double c = std::cos(ang), sn = std::sin(ang);
-            const float ch = (float)c, sh = (float)sn;
-            h.push_back(make_float4(ch, sh, (float)(c - (double)ch), (float)(sn - (double)sh)));
+  std::vector<float2> h;
+  int ns = 1;
+  for (int q = 0; q < np; ++q) {
+    if (q > 0) {
+      for (int r = 0; r < rad[q]; ++r)
+        for (int m = 0; m < ns; ++m) {
+          int mc = 0, w = 1, rest = m;
+          for (int p = 0; p < q; ++p) {
+            mc += w * centred(rest % rad[p], rad[p]);
+            rest /= rad[p];
+            w *= rad[p];
           }
-      }
-      ns *= R;
+          const double phi = -6.283185307179586476925286766559 * (double)(centred(r, rad[q]) * mc) / (double)(ns * rad[q]);
+          h.push_back(make_float2((float)-std::tan(0.5 * phi), (float)std::sin(phi)));
+        }
     }
+    ns *= rad[q];
   }
-  if (h.empty()) h.push_back(make_float4(1.f, 0.f, 0.f, 0.f));
+  if (h.empty()) h.push_back(make_float2(0.f, 0.f));
   if ((int)h.size() != tw_table_size_of(n)) return cudaErrorInvalidValue;
-  cudaError_t e = cudaMemcpyAsync(tw, h.data(), sizeof(float4) * h.size(), cudaMemcpyHostToDevice, s);
+  cudaError_t e = cudaMemcpyAsync(tw, h.data(), sizeof(float2) * h.size(), cudaMemcpyHostToDevice, s);
   if (e != cudaSuccess) return e;
   return cudaStreamSynchronize(s);  // h is a local buffer
 }

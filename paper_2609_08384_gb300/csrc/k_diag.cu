@@ -70,15 +70,14 @@ __global__ void __launch_bounds__(tiles_per_cta<PL>() * tile_threads<PL>())
   constexpr int GT = T * TX;                       // threads of one tile group
   constexpr int THREADS = tiles_per_cta<PL>() * GT;
   constexpr int TPC = tiles_per_cta<PL>();
-  constexpr int R0 = fft_radix<PL, false>(0), RL = fft_radix<PL, false>(PL::NP - 1);
-  constexpr int S0 = N / R0, SL = N / RL;
+  constexpr int RL = fft_radix<PL, false>(PL::NP - 1);
   constexpr int BPT = (N + GT - 1) / GT;  // bins per thread
   extern __shared__ float4 sm4[];
   float2* xch = reinterpret_cast<float2*>(sm4);
   if constexpr (tw_in_smem<PL>()) {
-    for (int i = threadIdx.x; i < tw_table_size<PL>(); i += THREADS) sm4[i] = p.tw[i];
+    for (int i = threadIdx.x; i < tw_table_size<PL>(); i += THREADS) xch[i] = p.tw[i];
     __syncthreads();
-    xch = reinterpret_cast<float2*>(sm4 + tw_table_size<PL>());
+    xch += tw_table_size<PL>();
   }
   const int lt = threadIdx.x % GT, tl = threadIdx.x / GT;
   const int tx = lt % TX, t = lt / TX;
@@ -108,12 +107,8 @@ __global__ void __launch_bounds__(tiles_per_cta<PL>() * tile_threads<PL>())
     }
     const AxisTile<N, 2, TX> a(p, tile, tx);
     float2 v[E];
-#pragma unroll
-    for (int b = 0; b < E / R0; ++b)
-#pragma unroll
-      for (int r = 0; r < R0; ++r)
-        v[b * R0 + r] = a.act ? __ldcg(a.base + (t + b * T + r * S0) * a.stride) : make_float2(0.f, 0.f);
-    if constexpr (tw_in_smem<PL>()) fft_run<PL, false, 0, XchCol<TX>, SyncBlock, TwShared>(v, t, xc, TwShared{sm4});
+    load_pencil<PL, false>(v, a.base, a.stride, t, a.act);
+    if constexpr (tw_in_smem<PL>()) fft_run<PL, false, 0, XchCol<TX>, SyncBlock, TwShared>(v, t, xc, TwShared{reinterpret_cast<const float2*>(sm4)});
     else fft_run<PL, false, 0, XchCol<TX>, SyncBlock, TwGlobal>(v, t, xc, TwGlobal{p.tw});
     __syncthreads();  // every read of the exchange space is done
 #pragma unroll
@@ -121,7 +116,7 @@ __global__ void __launch_bounds__(tiles_per_cta<PL>() * tile_threads<PL>())
 #pragma unroll
       for (int r = 0; r < RL; ++r) {
         const float2 w = v[b * RL + r];
-        q[tx * (N + 1) + t + b * T + r * SL] = fmaf(w.x, w.x, w.y * w.y);
+        q[tx * (N + 1) + pos_last<PL, false>(t + b * T, r)] = fmaf(w.x, w.x, w.y * w.y);
       }
     __syncthreads();
 #pragma unroll

@@ -237,17 +237,9 @@ __global__ void prop_pointwise_kernel(const AxisArgs p, int nf) {
     const int x = (int)(r % p.nx);
     const int y = (int)((r / p.nx) % p.ny);
     const int t = (int)(r / plane);
-    const float2 dx = p.px[f * p.nx + x], dy = p.py[f * p.ny + y];
-    float2 dxy = cadd(cadd(dx, dy), cmul(dx, dy));
-    float2 dt = p.pt[f * p.nt + t];
-    if (p.conj_p) {
-      dxy.y = -dxy.y;
-      dt.y = -dt.y;
-    }
+    const ColumnProp g(p, p.px[f * p.nx + x], p.py[f * p.ny + y]);
     float2* q = p.data + (long long)f * p.fstride + r;
-    float2 w = *q;
-    w = make_float2(fmaf(w.x, p.scale, w.x * p.scale_lo), fmaf(w.y, p.scale, w.y * p.scale_lo));
-    *q = mul_one_plus(w, cadd(cadd(dxy, dt), cmul(dxy, dt)));
+    *q = g(*q, p.pt[f * p.nt + t]);
   }
 }
 

@@ -69,7 +69,7 @@ template <class PL>
 __host__ __device__ constexpr int tma_box_t() { return PL::N < 256 ? PL::N : 256; }
 template <class PL, int TX>
 __host__ __device__ constexpr size_t tma_smem_bytes() {
-  return 2 * (size_t)PL::N * TX * 8 + (tw_in_smem<PL>() ? (size_t)tw_table_size<PL>() * 16 : 0) + 16;
+  return 2 * (size_t)PL::N * TX * 8 + (tw_in_smem<PL>() ? (size_t)tw_table_size<PL>() * 8 : 0) + 16;
 }
 
 template <class PL, int TX>
@@ -79,14 +79,13 @@ __global__ void __launch_bounds__(PL::T * TX, PL::T * TX <= 256 ? 2 : 1)
   constexpr int BOX = tma_box_t<PL>();
   constexpr int NBOX = N / BOX;
   constexpr uint32_t TILE_BYTES = (uint32_t)(N * TX * 8);
-  constexpr int R0 = fft_radix<PL, false>(0), RL = fft_radix<PL, false>(PL::NP - 1);
-  constexpr int S0 = N / R0, SL = N / RL;
+  constexpr int R0 = fft_radix<PL, false>(0);
   extern __shared__ __align__(1024) unsigned char smraw[];
   float2* buf[2] = {reinterpret_cast<float2*>(smraw), reinterpret_cast<float2*>(smraw) + N * TX};
-  float4* tws = reinterpret_cast<float4*>(buf[1] + N * TX);
+  float2* tws = buf[1] + N * TX;
   unsigned long long* bars =
       reinterpret_cast<unsigned long long*>(reinterpret_cast<unsigned char*>(tws) +
-                                            (tw_in_smem<PL>() ? (size_t)tw_table_size<PL>() * 16 : 0));
+                                            (tw_in_smem<PL>() ? (size_t)tw_table_size<PL>() * 8 : 0));
   // TMA destinations must be 128-byte aligned
   if (smem_u32(smraw) & 127u) {
     if (threadIdx.x == 0) atomicExch(err, 2);
@@ -156,37 +155,18 @@ __global__ void __launch_bounds__(PL::T * TX, PL::T * TX <= 256 ? 2 : 1)
 #pragma unroll
     for (int bb = 0; bb < E / R0; ++bb)
 #pragma unroll
-      for (int r = 0; r < R0; ++r) v[bb * R0 + r] = xc.ld(t + bb * T + r * S0);
+      for (int r = 0; r < R0; ++r) v[bb * R0 + r] = xc.ld(pos_first<PL, false>(t + bb * T, r));
     using TWA = typename std::conditional<tw_in_smem<PL>(), TwShared, TwGlobal>::type;
     const TWA tw{tw_in_smem<PL>() ? tws : p.tw};
     fft_run<PL, false, 0, XchCol<TX>, SyncBlock, TWA>(v, t, xc, tw);
-    float2 dxy = make_float2(0.f, 0.f);
-    if (act) {
-      const float2 dx = p.px[f * p.nx + x], dy = p.py[f * p.ny + y];
-      dxy = cadd(cadd(dx, dy), cmul(dx, dy));
-    }
-    if (p.conj_p) dxy.y = -dxy.y;
-    const float2* pt = p.pt + f * p.nt;
-    const float tsign = p.conj_p ? -1.f : 1.f;
-#pragma unroll
-    for (int bb = 0; bb < E / RL; ++bb)
-#pragma unroll
-      for (int r = 0; r < RL; ++r) {
-        const int kk = t + bb * T + r * SL;
-        float2 dt = pt[kk];
-        dt.y *= tsign;
-        float2 w = v[bb * RL + r];
-        w = make_float2(fmaf(w.x, p.scale, w.x * p.scale_lo), fmaf(w.y, p.scale, w.y * p.scale_lo));
-        v[bb * RL + r] = mul_one_plus(w, cadd(cadd(dxy, dt), cmul(dxy, dt)));
-      }
+    const float2 zero = make_float2(0.f, 0.f);
+    const ColumnProp g(p, act ? p.px[f * p.nx + x] : zero, act ? p.py[f * p.ny + y] : zero);
+    apply_prop<PL>(v, g, p.pt + f * p.nt, t);
     fft_run<PL, true, 0, XchCol<TX>, SyncBlock, TWA>(v, t, xc, tw);
     if (act) {
       float2* base = p.data + (long long)f * p.fstride + (long long)y * p.nx + x;
       const long long stride = (long long)p.nx * p.ny;
-#pragma unroll
-      for (int bb = 0; bb < E / R0; ++bb)
-#pragma unroll
-        for (int r = 0; r < R0; ++r) base[(t + bb * T + r * S0) * stride] = v[bb * R0 + r];
+      store_pencil<PL, false>(v, base, stride, t);
     }
     __syncthreads();  // buffer b is free for the copy issued in the next iteration
   }
@@ -214,8 +194,7 @@ __global__ void __launch_bounds__(PL::T * 16, 2)
   constexpr int BOX = tma_box_t<PL>();
   constexpr int NBOX = N / BOX;
   constexpr uint32_t TILE_BYTES = (uint32_t)(N * TX * 8);
-  constexpr int R0 = fft_radix<PL, false>(0), RL = fft_radix<PL, false>(PL::NP - 1);
-  constexpr int S0 = N / R0, SL = N / RL;
+  constexpr int R0 = fft_radix<PL, false>(0);
   extern __shared__ __align__(1024) unsigned char smraw[];
   float2* pre = reinterpret_cast<float2*>(smraw);
   float* xre = reinterpret_cast<float*>(pre + N * TX);
@@ -270,7 +249,7 @@ __global__ void __launch_bounds__(PL::T * 16, 2)
 #pragma unroll
     for (int bb = 0; bb < E / R0; ++bb)
 #pragma unroll
-      for (int r = 0; r < R0; ++r) v[bb * R0 + r] = pre[(t + bb * T + r * S0) * TX + tx];
+      for (int r = 0; r < R0; ++r) v[bb * R0 + r] = pre[pos_first<PL, false>(t + bb * T, r) * TX + tx];
     __syncthreads();  // the buffer is free: fetch the next tile while this one is transformed
     if (threadIdx.x == 0 && k + gridDim.x < ntiles) issue(ntiles - 1 - (k + gridDim.x));
     const int xt = (int)(tile % p.xtiles);
@@ -279,33 +258,14 @@ __global__ void __launch_bounds__(PL::T * 16, 2)
     const int x = xt * TX + tx;
     const bool act = x < p.nx;
     fft_run<PL, false, 0, XchColSplit<TX>, SyncBlock, TwGlobal>(v, t, xc, tw);
-    float2 dxy = make_float2(0.f, 0.f);
-    if (act) {
-      const float2 dx = p.px[f * p.nx + x], dy = p.py[f * p.ny + y];
-      dxy = cadd(cadd(dx, dy), cmul(dx, dy));
-    }
-    if (p.conj_p) dxy.y = -dxy.y;
-    const float2* pt = p.pt + f * p.nt;
-    const float tsign = p.conj_p ? -1.f : 1.f;
-#pragma unroll
-    for (int bb = 0; bb < E / RL; ++bb)
-#pragma unroll
-      for (int r = 0; r < RL; ++r) {
-        const int kk = t + bb * T + r * SL;
-        float2 dt = pt[kk];
-        dt.y *= tsign;
-        float2 w = v[bb * RL + r];
-        w = make_float2(fmaf(w.x, p.scale, w.x * p.scale_lo), fmaf(w.y, p.scale, w.y * p.scale_lo));
-        v[bb * RL + r] = mul_one_plus(w, cadd(cadd(dxy, dt), cmul(dxy, dt)));
-      }
+    const float2 zero = make_float2(0.f, 0.f);
+    const ColumnProp g(p, act ? p.px[f * p.nx + x] : zero, act ? p.py[f * p.ny + y] : zero);
+    apply_prop<PL>(v, g, p.pt + f * p.nt, t);
     fft_run<PL, true, 0, XchColSplit<TX>, SyncBlock, TwGlobal>(v, t, xc, tw);
     if (act) {
       float2* base = p.data + (long long)f * p.fstride + (long long)y * p.nx + x;
       const long long stride = (long long)p.nx * p.ny;
-#pragma unroll
-      for (int bb = 0; bb < E / R0; ++bb)
-#pragma unroll
-        for (int r = 0; r < R0; ++r) base[(t + bb * T + r * S0) * stride] = v[bb * R0 + r];
+      store_pencil<PL, false>(v, base, stride, t);
     }
   }
   // a CTA whose last wait succeeded has no copy in flight here

@@ -28,7 +28,7 @@ struct XPassArgs {
   float2* data;        // [nf][rows][nx]
   long long fstride;   // elements between fields
   long long rows;      // ny * nt
-  const float4* tw;    // per-pass twiddle table of the x transform (hi/lo pairs)
+  const float2* tw;    // per-pass twiddle table of the x transform
   int mode;            // XMode
   double phiA, dkA;    // step whose first half is applied: Phi(z_j), dk_j
   double phiB, dkB;    // step whose second half is applied
@@ -61,7 +61,7 @@ struct AxisArgs {
   long long fstride;
   long long ntiles;
   int xtiles;
-  const float4* tw;    // twiddles of the transformed axis (hi/lo pairs)
+  const float2* tw;    // twiddles of the transformed axis
   const float2* px;    // [nf][nx] propagator factors (t-pass only)
   const float2* py;    // [nf][ny]
   const float2* pt;    // [nf][nt]
@@ -111,12 +111,13 @@ template <class PL>
 __host__ __device__ constexpr int tile_threads() { return PL::T * ColTile<PL>::value; }
 template <class PL>
 __host__ __device__ constexpr int tiles_per_cta() { return tile_threads<PL>() >= 256 ? 1 : 256 / tile_threads<PL>(); }
-// twiddle tables up to 40 KB are copied to shared memory; larger ones are read through L1
+// twiddle tables of up to 2560 entries (20 KB: lengths up to 1024) are copied to
+// shared memory; larger ones are read through L1
 template <class PL>
-__host__ __device__ constexpr bool tw_in_smem() { return tw_table_size<PL>() * 16 <= 40960; }
+__host__ __device__ constexpr bool tw_in_smem() { return tw_table_size<PL>() <= 2560; }
 template <class PL>
 __host__ __device__ constexpr int axis_smem_floats2() {
-  return (tw_in_smem<PL>() ? 2 * tw_table_size<PL>() : 0) + tiles_per_cta<PL>() * PL::N * ColTile<PL>::value;
+  return (tw_in_smem<PL>() ? tw_table_size<PL>() : 0) + tiles_per_cta<PL>() * PL::N * ColTile<PL>::value;
 }
 // The forward y-pass reads its twiddles through L1 instead of staging them in
 // shared memory per CTA: measured on the 3 x 256x256x512 state, 285 -> 253 us
@@ -126,7 +127,7 @@ template <class PL, bool INV, int AXIS>
 __host__ __device__ constexpr bool axis_tw_staged() { return tw_in_smem<PL>() && !(AXIS == 1 && !INV); }
 template <class PL, bool INV, int AXIS>
 __host__ __device__ constexpr int axis_kernel_smem_floats2() {
-  return (axis_tw_staged<PL, INV, AXIS>() ? 2 * tw_table_size<PL>() : 0) +
+  return (axis_tw_staged<PL, INV, AXIS>() ? tw_table_size<PL>() : 0) +
          tiles_per_cta<PL>() * PL::N * ColTile<PL>::value;
 }
 
@@ -260,7 +261,7 @@ __device__ __forceinline__ void xpass_tile(const XPassArgs& p, long long tile, c
   constexpr int PITCH = XchRow::pitch(NX);
   constexpr int RF0 = fft_radix<PL, false>(0);           // forward first radix
   constexpr int RFL = fft_radix<PL, false>(PL::NP - 1);  // forward last radix
-  constexpr int SF0 = NX / RF0, SFL = NX / RFL;
+  constexpr int SF0 = NX / RF0;
   using SY = typename std::conditional<xpass_warp_sync<NX>(), SyncWarp, SyncBlock>::type;
   static_assert(ROWS >= 1 && ROWS * T == THREADS, "CTA must hold whole rows");
   const TwGlobal tw{p.tw};
@@ -284,15 +285,15 @@ __device__ __forceinline__ void xpass_tile(const XPassArgs& p, long long tile, c
       for (int b = 0; b < E / RFL; ++b)
 #pragma unroll
         for (int r = 0; r < RFL; ++r)
-          v[b * RFL + r] = act ? __ldcg(src + t + b * T + r * SFL) : make_float2(0.f, 0.f);
-      // inverse's output positions t + b T + r NX/RF0 = forward first-pass positions
+          v[b * RFL + r] = act ? __ldcg(src + pos_first<PL, true>(t + b * T, r)) : make_float2(0.f, 0.f);
+      // the inverse's outputs lie at the forward first pass's positions
       fft_run<PL, true, 0, XchRow, SY, TwGlobal>(v, t, xr, tw);
     } else {
 #pragma unroll
       for (int b = 0; b < E / RF0; ++b)
 #pragma unroll
         for (int r = 0; r < RF0; ++r)
-          v[b * RF0 + r] = act ? __ldcg(src + t + b * T + r * SF0) : make_float2(0.f, 0.f);
+          v[b * RF0 + r] = act ? __ldcg(src + pos_first<PL, false>(t + b * T, r)) : make_float2(0.f, 0.f);
     }
 #pragma unroll
     for (int b = 0; b < E / RF0; ++b)
@@ -309,21 +310,24 @@ __device__ __forceinline__ void xpass_tile(const XPassArgs& p, long long tile, c
     float2 nm[4];
     if constexpr (MAP) {
 #pragma unroll
-      for (int q = 0; q < 4; ++q) nm[q] = __ldg(emap + q * nxy + t);
+      for (int q = 0; q < 4; ++q) nm[q] = __ldg(emap + q * nxy + pos_first<PL, false>(t, 0));
     }
     // two points per iteration: their RK4 chains interleave (measured on GB300:
     // OPG x-pass 549 -> 540 us, with a fan-out map 699 -> 655 us, SFG 94 -> 90 us;
     // four points per iteration, 579 us, overflow the instruction cache)
 #pragma unroll 2
     for (int e = 0; e < E; ++e) {
-      const int pos = t + (e / RF0) * T + (e % RF0) * SF0;
-      const int off = pos + (pos >> 4);  // XchRow padding
+      // the park place of a point is its butterfly's; its position on the row
+      // (of the map and of the recorded states) is pos
+      const int place = t + (e / RF0) * T + (e % RF0) * SF0;
+      const int off = place + (place >> 4);  // XchRow padding
+      const int pos = pos_first<PL, false>(t + (e / RF0) * T, e % RF0);
       float2 cm[4];
       if constexpr (MAP) {
 #pragma unroll
         for (int q = 0; q < 4; ++q) cm[q] = nm[q];
         if (e + 1 < E) {
-          const int pn = t + ((e + 1) / RF0) * T + ((e + 1) % RF0) * SF0;
+          const int pn = pos_first<PL, false>(t + ((e + 1) / RF0) * T, (e + 1) % RF0);
 #pragma unroll
           for (int q = 0; q < 4; ++q) nm[q] = __ldg(emap + q * nxy + pn);
         }
@@ -390,7 +394,7 @@ __device__ __forceinline__ void xpass_tile(const XPassArgs& p, long long tile, c
 #pragma unroll
         for (int b = 0; b < E / RF0; ++b)
 #pragma unroll
-          for (int r = 0; r < RF0; ++r) dst[t + b * T + r * SF0] = cscale(v[b * RF0 + r], sc);
+          for (int r = 0; r < RF0; ++r) dst[pos_first<PL, false>(t + b * T, r)] = cscale(v[b * RF0 + r], sc);
       }
     } else {
       fft_run<PL, false, 0, XchRow, SY, TwGlobal>(v, t, xr, tw);
@@ -398,7 +402,7 @@ __device__ __forceinline__ void xpass_tile(const XPassArgs& p, long long tile, c
 #pragma unroll
         for (int b = 0; b < E / RFL; ++b)
 #pragma unroll
-          for (int r = 0; r < RFL; ++r) dst[t + b * T + r * SFL] = v[b * RFL + r];
+          for (int r = 0; r < RFL; ++r) dst[pos_last<PL, false>(t + b * T, r)] = v[b * RFL + r];
       }
     }
     SY::sync();  // the next field's exchanges use another buffer; keep the warp together
@@ -423,14 +427,6 @@ __global__ void __launch_bounds__(xpass_threads<NX>(), xpass_min_blocks<NX, F>()
   // rows from the last tau-plane down (see the note on pass order above)
   xpass_tile<NX, F, THREADS, MAP, REC>(p, (long long)gridDim.x - 1 - blockIdx.x, coef, rowbuf);
 }
-
-// w (1 + d) for a propagator factor in delta form: the small product w d is
-// formed first and w added with one rounding.  (Folding w into the FMA chain,
-// e.g. fma(w.x, d.x, fma(-w.y, d.y, w.x)), rounds w.x - w.y d.y before the
-// second-order term w.x (cos phi - 1) arrives; for small phases that term is
-// below half an ulp and is then always lost, so |1 + d| acts as
-// 1 + phi^2 / 2 and the energy grows step after step.)
-__device__ __forceinline__ float2 mul_one_plus(float2 w, float2 d) { return cadd(w, cmul(w, d)); }
 
 // ------------------------------------------------- strided-axis passes
 // AXIS 1: pencils along y (stride nx), tiles over (f, tau, x-tile).
@@ -464,92 +460,132 @@ struct AxisTile {
   }
 };
 
+// A pencil's registers from and to memory at the positions of the first pass of
+// a direction (which are those of the other direction's last pass): input r of
+// butterfly j at n + r N/R0, n centred, input 0 wrapped when n < 0.
+template <class PL, bool INV>
+__device__ __forceinline__ void load_pencil(float2 (&v)[PL::E], const float2* base, long long stride, int t, bool act) {
+  constexpr int R0 = fft_radix<PL, INV>(0);
+#pragma unroll
+  for (int b = 0; b < PL::E / R0; ++b) {
+    const int n = centred_first<PL, INV>(t + b * PL::T);
+    const float2* q = base + n * stride;
+#pragma unroll
+    for (int r = 0; r < R0; ++r)
+      v[b * R0 + r] = act ? __ldcg(r == 0 && n < 0 ? q + PL::N * stride : q + (r * (PL::N / R0)) * stride)
+                          : make_float2(0.f, 0.f);
+  }
+}
+template <class PL, bool INV>
+__device__ __forceinline__ void store_pencil(const float2 (&v)[PL::E], float2* base, long long stride, int t) {
+  constexpr int R0 = fft_radix<PL, INV>(0);
+#pragma unroll
+  for (int b = 0; b < PL::E / R0; ++b) {
+    const int n = centred_first<PL, INV>(t + b * PL::T);
+    float2* q = base + n * stride;
+#pragma unroll
+    for (int r = 0; r < R0; ++r)
+      *(r == 0 && n < 0 ? q + PL::N * stride : q + (r * (PL::N / R0)) * stride) = v[b * R0 + r];
+  }
+}
+
 // Tiles per CTA of THREADS threads for strided pencils.
 template <class PL, int THREADS>
 __host__ __device__ constexpr int tiles_per_cta_t() { return THREADS / tile_threads<PL>(); }
 
 template <class PL, bool INV, int AXIS, int THREADS, class TW = TwShared>
 __device__ __forceinline__ void axis_tile(const AxisArgs& p, long long cta_tile, const TW& tw, float2* xch) {
-  constexpr int N = PL::N, E = PL::E, T = PL::T, TX = ColTile<PL>::value;
+  constexpr int N = PL::N, T = PL::T, TX = ColTile<PL>::value;
   constexpr int TPC = tiles_per_cta_t<PL, THREADS>();
   static_assert(TPC >= 1 && TPC * T * TX == THREADS, "CTA must hold whole tiles");
-  constexpr int R0 = fft_radix<PL, INV>(0), RL = fft_radix<PL, INV>(PL::NP - 1);
-  constexpr int S0 = N / R0, SL = N / RL;
   const int lt = threadIdx.x % (T * TX), tl = threadIdx.x / (T * TX);
   const int tx = lt % TX, t = lt / TX;
   const AxisTile<N, AXIS, TX> a(p, cta_tile * TPC + tl, tx);
   const XchCol<TX> xc{xch + tl * N * TX, tx};
-  float2 v[E];
-#pragma unroll
-  for (int b = 0; b < E / R0; ++b)
-#pragma unroll
-    for (int r = 0; r < R0; ++r)
-      v[b * R0 + r] = a.act ? __ldcg(a.base + (t + b * T + r * S0) * a.stride) : make_float2(0.f, 0.f);
+  float2 v[PL::E];
+  load_pencil<PL, INV>(v, a.base, a.stride, t, a.act);
   fft_run<PL, INV, 0, XchCol<TX>, SyncBlock, TW>(v, t, xc, tw);
-  if (a.act) {
-#pragma unroll
-    for (int b = 0; b < E / RL; ++b)
-#pragma unroll
-      for (int r = 0; r < RL; ++r) a.base[(t + b * T + r * SL) * a.stride] = v[b * RL + r];
+  if (a.act) store_pencil<PL, !INV>(v, a.base, a.stride, t);
+}
+
+// The propagator P = (1 + Dx)(1 + Dy)(1 + Dt) / (nx ny nt) of one column, the
+// factors in delta form and 1/(nx ny nt) as scale + scale_lo: a value w becomes
+//   scale w + w E(Omega),  E = scale_lo (1 + Dxy) + scale D + ... = g0 + Dt g1,
+//   1 + Dxy = (1 + Dx)(1 + Dy),  g1 = (scale + scale_lo)(1 + Dxy),
+//   g0 = scale Dxy + scale_lo (1 + Dxy).
+// The small product w E is formed first and scale w, which is exact for powers
+// of two, added with one rounding.  (Folding w into the FMA chain rounds
+// w.x - w.y E.y before the second-order term w.x (cos phi - 1) arrives; for
+// small phases that term is below half an ulp and is then always lost, so
+// |1 + E| acts as 1 + phi^2 / 2 and the energy grows step after step.)
+// conj(P) (the adjoint) turns the sign of E's imaginary part, which sits in its
+// three constants gi.
+struct ColumnProp {
+  float scale;
+  float2 g0, g1;
+  float3 gi;  // E.y = gi.x + Dt.x gi.y + Dt.y gi.z, the sign of conj(P) in it
+  __device__ __forceinline__ ColumnProp(const AxisArgs& p, float2 dx, float2 dy) {
+    const float2 dxy = cadd(cadd(dx, dy), cmul(dx, dy));
+    scale = p.scale;
+    const float ox = 1.f + dxy.x;
+    g1 = make_float2(fmaf(p.scale_lo, ox, p.scale * ox), fmaf(p.scale_lo, dxy.y, p.scale * dxy.y));
+    g0 = make_float2(fmaf(p.scale_lo, ox, p.scale * dxy.x), fmaf(p.scale_lo, dxy.y, p.scale * dxy.y));
+    const float sg = p.conj_p ? -1.f : 1.f;
+    gi = make_float3(sg * g0.y, sg * g1.y, sg * g1.x);
   }
+  __device__ __forceinline__ float2 operator()(float2 w, float2 dt) const {
+    const float ex = fmaf(dt.x, g1.x, fmaf(-dt.y, g1.y, g0.x));
+    const float ey = fmaf(dt.x, gi.y, fmaf(dt.y, gi.z, gi.x));
+    const float2 we = make_float2(fmaf(w.x, ex, -w.y * ey), fmaf(w.x, ey, w.y * ex));
+    return __ffma2_rn(w, make_float2(scale, scale), we);
+  }
+};
+
+// The propagator on a column's registers, which hold A_hat(kx, ky, Omega_k) at
+// k = pos_last; pt: the field's tau factors
+template <class PL>
+__device__ __forceinline__ void apply_prop(float2 (&v)[PL::E], const ColumnProp& g, const float2* pt, int t) {
+  constexpr int RL = fft_radix<PL, false>(PL::NP - 1);
+#pragma unroll
+  for (int b = 0; b < PL::E / RL; ++b)
+#pragma unroll
+    for (int r = 0; r < RL; ++r)
+      v[b * RL + r] = g(v[b * RL + r], pt[pos_last<PL, false>(t + b * PL::T, r)]);
+}
+
+// Resident CTAs the tau-pass asks the register allocator for.  Left to itself
+// the compiler requests a whole column of tau factors and twiddles ahead (153 to
+// 172 registers on the 512-point plan: one CTA per SM).  Measured per launch:
+// 512-point plan 555 us unbounded, 463 at two CTAs, 600 at three (spills); 128
+// points (512x512x128, two fields) 292 us unbounded, 290 at two, 232 at three;
+// 64 points (1024x256x64) 142 us at two, 127 at four.
+template <class PL>
+__host__ __device__ constexpr int tprop_min_blocks() {
+  return tiles_per_cta<PL>() * tile_threads<PL>() > 256 ? 1 : PL::E > 16 ? 2 : PL::E > 8 ? 3 : 4;
 }
 
 // Forward tau-FFT, propagator multiply, inverse tau-FFT, in one pass.
+// (Measured slower on the 512-point plan: launch bounds of two CTAs per SM, a
+// persistent loop over tiles, the twiddle staging issued after this tile's
+// loads, the field's tau factors staged in shared memory with the twiddles.)
 template <class PL, int THREADS, class TW = TwShared>
 __device__ __forceinline__ void tprop_tile(const AxisArgs& p, long long cta_tile, const TW& tw, float2* xch) {
-  constexpr int N = PL::N, E = PL::E, T = PL::T, TX = ColTile<PL>::value;
+  constexpr int N = PL::N, T = PL::T, TX = ColTile<PL>::value;
   constexpr int TPC = tiles_per_cta_t<PL, THREADS>();
   static_assert(TPC >= 1 && TPC * T * TX == THREADS, "CTA must hold whole tiles");
-  constexpr int R0 = fft_radix<PL, false>(0), RL = fft_radix<PL, false>(PL::NP - 1);
-  constexpr int S0 = N / R0, SL = N / RL;
   const int lt = threadIdx.x % (T * TX), tl = threadIdx.x / (T * TX);
   const int tx = lt % TX, t = lt / TX;
   const AxisTile<N, 2, TX> a(p, cta_tile * TPC + tl, tx);
   const XchCol<TX> xc{xch + tl * N * TX, tx};
-  float2 v[E];
-#pragma unroll
-  for (int b = 0; b < E / R0; ++b)
-#pragma unroll
-    for (int r = 0; r < R0; ++r)
-      v[b * R0 + r] = a.act ? __ldcg(a.base + (t + b * T + r * S0) * a.stride) : make_float2(0.f, 0.f);
+  float2 v[PL::E];
+  load_pencil<PL, false>(v, a.base, a.stride, t, a.act);
   fft_run<PL, false, 0, XchCol<TX>, SyncBlock, TW>(v, t, xc, tw);
-  // now v[b RL + r] = A_hat(kx, ky, Omega_k), k = t + b T + r N/RL.
-  // P = (1 + Dx)(1 + Dy)(1 + Dt) applied as w + w D with w = v/(nx ny nt).
-  // (Measured slower on the 512-point plan: w (1 + Dt)(1 + Dxy) as two
-  // delta-form products, 127 registers and 522 us against 104 and 476; the
-  // scale and conjugation as four specialised copies, 542 us; the twiddle
-  // staging issued after this tile's loads instead of before them, 520 us;
-  // a persistent loop over tiles, 542 us; the first pass's loads issued in
-  // the order the radix-32 codelet consumes them, 549 us; launch bounds of
-  // two CTAs per SM (128 registers), 531 us; the field's tau factors staged
-  // in shared memory with the twiddles, 506 us.)
-  float2 dxy = make_float2(0.f, 0.f);
-  if (a.act) {
-    const float2 dx = p.px[a.f * p.nx + a.x], dy = p.py[a.f * p.ny + a.other];
-    dxy = cadd(cadd(dx, dy), cmul(dx, dy));
-  }
-  if (p.conj_p) dxy.y = -dxy.y;
-  const float2* pt = p.pt + (a.act ? a.f * p.nt : 0);
-  const float tsign = p.conj_p ? -1.f : 1.f;
-#pragma unroll
-  for (int b = 0; b < E / RL; ++b)
-#pragma unroll
-    for (int r = 0; r < RL; ++r) {
-      const int k = t + b * T + r * SL;
-      float2 dt = pt[k];
-      dt.y *= tsign;
-      float2 w = v[b * RL + r];
-      w = make_float2(fmaf(w.x, p.scale, w.x * p.scale_lo), fmaf(w.y, p.scale, w.y * p.scale_lo));
-      v[b * RL + r] = mul_one_plus(w, cadd(cadd(dxy, dt), cmul(dxy, dt)));
-    }
+  const float2 zero = make_float2(0.f, 0.f);
+  const ColumnProp g(p, a.act ? p.px[a.f * p.nx + a.x] : zero, a.act ? p.py[a.f * p.ny + a.other] : zero);
+  apply_prop<PL>(v, g, p.pt + (a.act ? a.f * p.nt : 0), t);
   // the inverse's first pass reads exactly these positions
   fft_run<PL, true, 0, XchCol<TX>, SyncBlock, TW>(v, t, xc, tw);
-  if (a.act) {
-#pragma unroll
-    for (int b = 0; b < E / R0; ++b)
-#pragma unroll
-      for (int r = 0; r < R0; ++r) a.base[(t + b * T + r * S0) * a.stride] = v[b * R0 + r];
-  }
+  if (a.act) store_pencil<PL, false>(v, a.base, a.stride, t);
 }
 
 template <class PL, bool INV, int AXIS>
@@ -558,29 +594,29 @@ __global__ void __launch_bounds__(tiles_per_cta<PL>() * tile_threads<PL>())
   constexpr int THREADS = tiles_per_cta<PL>() * tile_threads<PL>();
   extern __shared__ float4 sm4[];
   if constexpr (axis_tw_staged<PL, INV, AXIS>()) {
-    float4* tw = sm4;
+    float2* tw = reinterpret_cast<float2*>(sm4);
     for (int i = threadIdx.x; i < tw_table_size<PL>(); i += blockDim.x) tw[i] = p.tw[i];
     __syncthreads();
     axis_tile<PL, INV, AXIS, THREADS>(p, blockIdx.x, TwShared{tw},
-                                      reinterpret_cast<float2*>(tw + tw_table_size<PL>()));
+                                      tw + tw_table_size<PL>());
   } else {
     axis_tile<PL, INV, AXIS, THREADS>(p, blockIdx.x, TwGlobal{p.tw}, reinterpret_cast<float2*>(sm4));
   }
 }
 
 template <class PL>
-__global__ void __launch_bounds__(tiles_per_cta<PL>() * tile_threads<PL>())
+__global__ void __launch_bounds__(tiles_per_cta<PL>() * tile_threads<PL>(), tprop_min_blocks<PL>())
     tpass_prop_kernel(const AxisArgs p) {
   constexpr int THREADS = tiles_per_cta<PL>() * tile_threads<PL>();
   extern __shared__ float4 sm4[];
   if constexpr (tw_in_smem<PL>()) {
-    float4* tw = sm4;
+    float2* tw = reinterpret_cast<float2*>(sm4);
     for (int i = threadIdx.x; i < tw_table_size<PL>(); i += blockDim.x) tw[i] = p.tw[i];
     __syncthreads();
     // tiles from the last down: the pass ends on the first field's low-y
     // pencils, which the y-inverse then reads first
     tprop_tile<PL, THREADS>(p, (long long)gridDim.x - 1 - blockIdx.x, TwShared{tw},
-                            reinterpret_cast<float2*>(tw + tw_table_size<PL>()));
+                            tw + tw_table_size<PL>());
   } else {
     tprop_tile<PL, THREADS>(p, blockIdx.x, TwGlobal{p.tw}, reinterpret_cast<float2*>(sm4));
   }
@@ -619,10 +655,10 @@ cudaError_t make_tau_tensor_map(void* map128, const float2* data, int nx, int ny
 cudaError_t run_tpass_prop_tma(int nt, int tx, const void* map128, const AxisArgs& a, int* err,
                                unsigned long long wait_ns, cudaStream_t s);
 
-// per-pass twiddle table of the default plan of length n (host-built, FP64
-// split into hi + lo floats), and its size in float4 entries
+// per-pass twiddle table of the default plan of length n (shears, built on the
+// host in FP64), and its size in entries
 int tw_table_size_of(int n);
-cudaError_t upload_twiddles(float4* tw, int n, cudaStream_t s);
+cudaError_t upload_twiddles(float2* tw, int n, cudaStream_t s);
 struct TableArgs {
   float2* px;
   float2* py;
@@ -709,7 +745,7 @@ struct XAdjArgs {
   const float2* xa;
   const float2* xb;
   long long fstride, rows;
-  const float4* tw;
+  const float2* tw;
   int from_k, to_k;
   double phiA, dkA, phiB, dkB, h;  // phase and mismatch at the start of each half step; h = dz/2
   float kh[3];                     // kappa_f h (1/2 on the SH equation for two fields)

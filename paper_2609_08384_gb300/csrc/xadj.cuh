@@ -50,7 +50,7 @@ __device__ __forceinline__ void xpass_adj_tile(const XAdjArgs& p, long long tile
   constexpr int PITCH = XchRow::pitch(NX);
   constexpr int RF0 = fft_radix<PL, false>(0);
   constexpr int RFL = fft_radix<PL, false>(PL::NP - 1);
-  constexpr int SF0 = NX / RF0, SFL = NX / RFL;
+  constexpr int SF0 = NX / RF0;
   using SY = typename std::conditional<xpass_warp_sync<NX>(), SyncWarp, SyncBlock>::type;
   static_assert(ROWS >= 1 && ROWS * T == THREADS, "CTA must hold whole rows");
   const TwGlobal tw{p.tw};
@@ -72,14 +72,14 @@ __device__ __forceinline__ void xpass_adj_tile(const XAdjArgs& p, long long tile
       for (int b = 0; b < E / RFL; ++b)
 #pragma unroll
         for (int r = 0; r < RFL; ++r)
-          v[b * RFL + r] = act ? __ldcg(src + t + b * T + r * SFL) : make_float2(0.f, 0.f);
+          v[b * RFL + r] = act ? __ldcg(src + pos_first<PL, true>(t + b * T, r)) : make_float2(0.f, 0.f);
       fft_run<PL, true, 0, XchRow, SY, TwGlobal>(v, t, xr, tw);
     } else {
 #pragma unroll
       for (int b = 0; b < E / RF0; ++b)
 #pragma unroll
         for (int r = 0; r < RF0; ++r)
-          v[b * RF0 + r] = act ? __ldcg(src + t + b * T + r * SF0) : make_float2(0.f, 0.f);
+          v[b * RF0 + r] = act ? __ldcg(src + pos_first<PL, false>(t + b * T, r)) : make_float2(0.f, 0.f);
     }
 #pragma unroll
     for (int b = 0; b < E / RF0; ++b)
@@ -97,7 +97,8 @@ __device__ __forceinline__ void xpass_adj_tile(const XAdjArgs& p, long long tile
     // requesting both states of the same point up front gained nothing)
     float2 na[F], nb[F], nm[4];
     {
-      const long long at0 = row * NX + t;
+      const int p0 = pos_first<PL, false>(t, 0);
+      const long long at0 = row * NX + p0;
 #pragma unroll
       for (int f = 0; f < F; ++f) {
         na[f] = p.xa ? __ldcg(p.xa + f * p.fstride + at0) : make_float2(0.f, 0.f);
@@ -105,13 +106,13 @@ __device__ __forceinline__ void xpass_adj_tile(const XAdjArgs& p, long long tile
       }
       if constexpr (MAP) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) nm[q] = __ldg(emap + q * nxy + t);
+        for (int q = 0; q < 4; ++q) nm[q] = __ldg(emap + q * nxy + p0);
       }
     }
 #pragma unroll 1
     for (int e = 0; e < E; ++e) {
-      const int pos = t + (e / RF0) * T + (e % RF0) * SF0;
-      const int off = pos + (pos >> 4);
+      const int place = t + (e / RF0) * T + (e % RF0) * SF0;  // park place (XchRow padding)
+      const int off = place + (place >> 4);
       float2 g[F], x[F], xbv[F], cm[4];
 #pragma unroll
       for (int f = 0; f < F; ++f) {
@@ -123,7 +124,7 @@ __device__ __forceinline__ void xpass_adj_tile(const XAdjArgs& p, long long tile
         for (int q = 0; q < 4; ++q) cm[q] = nm[q];
       }
       if (e + 1 < E) {
-        const int pn = t + ((e + 1) / RF0) * T + ((e + 1) % RF0) * SF0;
+        const int pn = pos_first<PL, false>(t + ((e + 1) / RF0) * T, (e + 1) % RF0);
         const long long an = row * NX + pn;
 #pragma unroll
         for (int f = 0; f < F; ++f) {
@@ -177,7 +178,7 @@ __device__ __forceinline__ void xpass_adj_tile(const XAdjArgs& p, long long tile
 #pragma unroll
         for (int b = 0; b < E / RF0; ++b)
 #pragma unroll
-          for (int r = 0; r < RF0; ++r) dst[t + b * T + r * SF0] = v[b * RF0 + r];
+          for (int r = 0; r < RF0; ++r) dst[pos_first<PL, false>(t + b * T, r)] = v[b * RF0 + r];
       }
     } else {
       fft_run<PL, false, 0, XchRow, SY, TwGlobal>(v, t, xr, tw);
@@ -185,7 +186,7 @@ __device__ __forceinline__ void xpass_adj_tile(const XAdjArgs& p, long long tile
 #pragma unroll
         for (int b = 0; b < E / RFL; ++b)
 #pragma unroll
-          for (int r = 0; r < RFL; ++r) dst[t + b * T + r * SFL] = v[b * RFL + r];
+          for (int r = 0; r < RFL; ++r) dst[pos_last<PL, false>(t + b * T, r)] = v[b * RFL + r];
       }
     }
     SY::sync();
