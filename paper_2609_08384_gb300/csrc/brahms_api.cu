@@ -336,7 +336,9 @@ brahms_status brahms_transform(brahms_ctx* ctx, int direction) {
   const brahms::AxisArgs ay = aargs(ctx, 1), at = aargs(ctx, 2, false);
   const bool inv = direction == 1;
   brahms::XPassArgs a = xargs(ctx, inv ? brahms::XM_INV : brahms::XM_FWD, 1.0);
-  a.scale = (float)(1.0 / (double)ctx->npoints());
+  const double inv_n = 1.0 / (double)ctx->npoints();
+  a.scale = (float)inv_n;
+  a.scale_lo = (float)(inv_n - (double)a.scale);
   BR_CK(launch(ctx, 0, 1, [&] { return brahms::run_xpass(ctx->nx, ctx->nf, a, ctx->stream); }));
   if (ctx->ny > 1) BR_CK(launch(ctx, 1, 1, [&] { return brahms::run_axis_fft(ctx->ny, 1, inv, ay, ctx->stream); }));
   if (ctx->nt > 1) BR_CK(launch(ctx, 2, 1, [&] { return brahms::run_axis_fft(ctx->nt, 2, inv, at, ctx->stream); }));

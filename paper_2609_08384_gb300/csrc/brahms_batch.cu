@@ -81,7 +81,7 @@ constexpr int batch_smem_floats2() {
 
 struct InstDev {
   float2* state;
-  const float2* ecoef;  // stage factors of every x-pass: [step + 1][6] (see stage_table)
+  const float2* ecoef;  // stage factors of every x-pass: [step + 1][kStageFactors] (see stage_table)
   long long fstride;
   const float2 *twx, *twt;  // NX = NY: one table serves x and y
   const float2 *px, *py, *pt;
@@ -205,9 +205,8 @@ __device__ __noinline__ void run_item(const InstDev& I, const Item& it, float4* 
       p.phiA = I.dk * ((it.step + 1) * I.dz);
       p.dkA = I.dk;
     }
-    float2* coef = reinterpret_cast<float2*>(sm4);
-    float2* rowbuf = coef + 12;
-    if (threadIdx.x < 6) coef[threadIdx.x] = I.ecoef[(it.step + 1) * 6 + threadIdx.x];
+    float2* rowbuf = reinterpret_cast<float2*>(sm4);
+    const float2* coef = I.ecoef + (it.step + 1) * kStageFactors;
     __syncthreads();
     for (long long c = 0; c < it.ntiles; ++c) {
       xpass_tile<NXY, 2, kBT>(p, it.tile + c, coef, rowbuf);
@@ -392,7 +391,7 @@ struct BatchInstHost {
   float2* state = nullptr;
   float2 *twx = nullptr, *twt = nullptr;
   float2 *px = nullptr, *py = nullptr, *pt = nullptr;
-  const float2* ecoef = nullptr;  // its stage factors in its group's table, [step + 1][6]
+  const float2* ecoef = nullptr;  // its stage factors in its group's table, [step + 1][kStageFactors]
   bool have_fields = false;
   long long npoints() const { return (long long)nx * ny * nt; }
 };
@@ -409,7 +408,7 @@ struct BatchGroup {
   float2 *px = nullptr, *py = nullptr, *pt = nullptr;
   float2 *twx = nullptr, *twy = nullptr, *twt = nullptr;
   GroupInst* params = nullptr;
-  float2* ecoef = nullptr;  // stage factors [slot][steps + 1][6]
+  float2* ecoef = nullptr;  // stage factors [slot][steps + 1][kStageFactors]
   int ecoef_steps = 0;      // steps per slot in the table (the group's largest nz)
   cudaStream_t stream = nullptr;
   cudaEvent_t done = nullptr;
@@ -505,14 +504,14 @@ int effective_nz(const brahms_batch* b, const BatchInstHost& I) {
 }
 
 // The stage factors e^{+i Phi} of every x-pass of every instance of a group,
-// [slot][step + 1][6] (step -1: the first half step), formed on the host in
+// [slot][step + 1][kStageFactors] (step -1: the first half step), formed on the host in
 // FP64 exactly as the single-instance path forms them: the same phase
 // accumulation Phi_{j+1} = Phi_j + dk dz and the same reduction
 // (fill_stage_factors), so a batched instance computes what
 // brahms_propagate computes, bit for bit.
 cudaError_t stage_table(brahms_batch* b, BatchGroup& g) {
   const int S = g.ecoef_steps + 1;
-  std::vector<float2> h((size_t)6 * S * g.members.size(), make_float2(1.f, 0.f));
+  std::vector<float2> h((size_t)kStageFactors * S * g.members.size(), make_float2(1.f, 0.f));
   for (size_t slot = 0; slot < g.members.size(); ++slot) {
     const BatchInstHost& I = b->inst[g.members[slot]];
     XPassArgs x{};
@@ -531,7 +530,7 @@ cudaError_t stage_table(brahms_batch* b, BatchGroup& g) {
         x.dkA = I.dk;
       }
       fill_stage_factors(x);
-      for (int s = 0; s < 6; ++s) h[((size_t)slot * S + (j + 1)) * 6 + s] = x.ecoef[s];
+      for (int s = 0; s < kStageFactors; ++s) h[((size_t)slot * S + (j + 1)) * kStageFactors + s] = x.ecoef[s];
     }
   }
   cudaError_t e = cudaMemcpyAsync(g.ecoef, h.data(), sizeof(float2) * h.size(), cudaMemcpyHostToDevice, b->stream);
@@ -583,7 +582,7 @@ brahms_status layout(brahms_batch* b) {
                  o_twt = take(sizeof(float2) * tw_table_size_of(g.nt)), o_par = take(sizeof(GroupInst) * m);
     g.ecoef_steps = 0;
     for (int i : g.members) g.ecoef_steps = std::max(g.ecoef_steps, b->inst[i].nz);
-    const size_t o_coef = take(sizeof(float2) * 6 * (size_t)(g.ecoef_steps + 1) * m);
+    const size_t o_coef = take(sizeof(float2) * kStageFactors * (size_t)(g.ecoef_steps + 1) * m);
     if (dev_alloc((void**)&g.mem, off) != cudaSuccess) {
       cudaGetLastError();
       return release(bfail(b, BRAHMS_E_OOM, "batch group memory"));
@@ -629,7 +628,7 @@ brahms_status layout(brahms_batch* b) {
       I.pt = g.pt + slot * 2 * g.nt;
       I.twx = g.twx;
       I.twt = g.twt;
-      I.ecoef = g.ecoef + slot * (size_t)(g.ecoef_steps + 1) * 6;
+      I.ecoef = g.ecoef + slot * (size_t)(g.ecoef_steps + 1) * kStageFactors;
       brahms_status st = build_tables_for(b, I);
       if (st != BRAHMS_OK) {
         b->groups = gs;
@@ -676,7 +675,7 @@ brahms_status prepare_grouped(brahms_batch* b) {
     BB_CK(run_axis_fft(g.ny, 1, true, z, b->stream));
     BB_CK(run_tpass_prop(g.nt, z, b->stream));
     XPassArgs x{};
-    BB_CK(run_xpass_group(g.nx, x, g.params, g.ecoef, 6, 0, 0, b->stream));
+    BB_CK(run_xpass_group(g.nx, x, g.params, g.ecoef, kStageFactors, 0, 0, b->stream));
     BB_CK(run_xpass(g.nx, 2, x, b->stream));
   }
   cudaStream_t cap = nullptr;
@@ -709,7 +708,7 @@ brahms_status prepare_grouped(brahms_batch* b) {
     // an x-pass over the first a slots (per instance where an instance's rows
     // do not fill whole CTAs)
     auto xpass = [&](int step, int a) -> cudaError_t {
-      if (whole) return run_xpass_group(g.nx, base, g.params, g.ecoef, (g.ecoef_steps + 1) * 6, step, a, s);
+      if (whole) return run_xpass_group(g.nx, base, g.params, g.ecoef, (g.ecoef_steps + 1) * kStageFactors, step, a, s);
       for (int slot = 0; slot < a; ++slot) {
         const BatchInstHost& I = b->inst[g.members[slot]];
         XPassArgs p = base;

@@ -373,13 +373,14 @@ __device__ __forceinline__ int pos_last(int j, int k) {
 }
 
 // ---------------------------------------------------------------- exchange
-// Contiguous pencil (one row of x): one padding slot per 16 entries.
+// Contiguous pencil (one row of x): one padding slot per 16 entries; rows start
+// on 16-byte boundaries.
 struct XchRow {
   static constexpr bool kSplit = false;
   float2* base;
   __device__ __forceinline__ void st(int pos, float2 v) const { base[pos + (pos >> 4)] = v; }
   __device__ __forceinline__ float2 ld(int pos) const { return base[pos + (pos >> 4)]; }
-  __host__ __device__ static constexpr int pitch(int n) { return n + n / 16 + 1; }
+  __host__ __device__ static constexpr int pitch(int n) { return (n + n / 16 + 2) / 2 * 2; }
 };
 // Strided pencils: TX neighbouring columns, column index fastest.
 template <int TX>

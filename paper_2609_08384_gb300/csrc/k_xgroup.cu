@@ -19,8 +19,7 @@ __global__ void __launch_bounds__(xpass_threads<NX>(), xpass_min_blocks<NX, 2>()
                        int stride, int step, long long tiles_per_inst) {
   constexpr int THREADS = xpass_threads<NX>();
   extern __shared__ float4 sm4[];
-  float2* coef = reinterpret_cast<float2*>(sm4);
-  float2* rowbuf = coef + 6 * 2;
+  float2* rowbuf = reinterpret_cast<float2*>(sm4);
   // tiles from the last down, as the single-instance x-pass
   const long long t = (long long)gridDim.x - 1 - blockIdx.x;
   const int i = (int)(t / tiles_per_inst);
@@ -34,9 +33,7 @@ __global__ void __launch_bounds__(xpass_threads<NX>(), xpass_min_blocks<NX, 2>()
   p.kh2[0] = g.kh2[0];
   p.kh2[1] = g.kh2[1];
   p.mode = step < 0 ? XM_NL_FIRST : (step == g.nz - 1 ? XM_NL_LAST : XM_NL_MID);
-  if (threadIdx.x < 6) coef[threadIdx.x] = ecoef[(long long)i * stride + (step + 1) * 6 + threadIdx.x];
-  __syncthreads();
-  xpass_tile<NX, 2, THREADS>(p, lt, coef, rowbuf);
+  xpass_tile<NX, 2, THREADS>(p, lt, ecoef + (long long)i * stride + (step + 1) * kStageFactors, rowbuf);
 }
 
 template <int NX>

@@ -24,6 +24,8 @@ namespace brahms {
 
 enum XMode : int { XM_FWD = 0, XM_INV = 1, XM_NL_FIRST = 2, XM_NL_MID = 3, XM_NL_LAST = 4 };
 
+constexpr int kStageFactors = 4;
+
 struct XPassArgs {
   float2* data;        // [nf][rows][nx]
   long long fstride;   // elements between fields
@@ -35,7 +37,7 @@ struct XPassArgs {
   double dz;
   float kh[3];         // kappa_f * dz/2, including the 1/2 SH factor for 2 fields
   float kh2[3];        // kh / 2 (exact)
-  float scale;         // output scale for XM_INV
+  float scale, scale_lo;  // output scale for XM_INV, hi + lo (lo = 0 for powers of two)
   // transverse mismatch map: per-(x, y) stage phase factors [4][ny][nx]
   // (B start, B quarter-step, A start, A quarter-step; see run_map_tables),
   // or NULL for a mismatch uniform across the grid
@@ -45,11 +47,11 @@ struct XPassArgs {
   // enters the B half step and of the state that enters the A half step, or NULL
   float2* rec_b;
   float2* rec_a;
-  // the six stage factors e^{+i Phi} (B half: start, 3/4, end; A half: start,
-  // 1/4, 1/2 of the step) from the phases above, written by the host
-  // dispatchers in FP64 (map-free x-passes read them instead of computing
-  // them per CTA)
-  float2 ecoef[6];
+  // the stage factors of both half steps from the phases above, written by the
+  // host dispatchers in FP64 (map-free x-passes read them instead of computing
+  // them per CTA): e^{+i Phi} at the start of the B half, e^{+i dkB dz/4}, and
+  // the same two of the A half
+  float2 ecoef[kStageFactors];
 };
 // Host: the stage factors of an x-pass from its phases (FP64 phase, reduced
 // mod 2 pi, cos and sin in FP64, rounded to float).
@@ -81,11 +83,11 @@ template <int N>
 __host__ __device__ constexpr int xpass_rows() { return xpass_threads<N>() / fft_threads<N>(); }
 template <int N>
 __host__ __device__ constexpr bool xpass_warp_sync() { return fft_threads<N>() <= 32 && 32 % fft_threads<N>() == 0; }
-// shared memory in float2 units: twiddles (N float4), NL coefficients (6 F),
-// exchange rows, and a private stash of F-1 fields per thread
+// shared memory in float2 units: a row buffer per field and row (the reverse
+// x-pass keeps its 6 F coefficients in front of them)
 template <int N>
 __host__ __device__ constexpr int xpass_smem_floats2(int nf) {
-  return 6 * nf + nf * xpass_rows<N>() * XchRow::pitch(N);
+  return nf * xpass_rows<N>() * XchRow::pitch(N);
 }
 // resident CTAs the x-pass asks the register allocator for: 6 (80 registers)
 // where six CTAs' shared memory fits in an SM and rows are at most 256 long
@@ -149,62 +151,101 @@ __device__ __forceinline__ void nl_rhs(const float2 (&a)[F], const float2* __res
   }
 }
 
-// Stage right-hand sides in the form used by the forward half steps:
-// k_f = i (kappa_f h) m_f with e = e^{+i Phi(z_stage)} and
-//   F = 3: m_p = conj(e) A_s A_i,  m_s = e A_p conj(A_i),  m_i = e A_p conj(A_s)
-//   F = 2: m_SH = conj(e) A_F^2,   m_F = e A_SH conj(A_F)
-// (five complex products per stage for three fields instead of six; the
-// factor i kappa_f h goes into the stage updates' FMAs).
-template <int F>
-__device__ __forceinline__ void nl_m(const float2 (&a)[F], float2 e, float2 (&m)[F]) {
-  if constexpr (F == 3) {
-    const float2 u = cmul(e, a[0]);
-    m[1] = cmulc(u, a[2]);
-    m[2] = cmulc(u, a[1]);
-    m[0] = cmulc(cmul(a[1], a[2]), e);
-  } else {
-    const float2 sq = make_float2(fmaf(a[1].x, a[1].x, -a[1].y * a[1].y), (a[1].x + a[1].x) * a[1].y);
-    m[0] = cmulc(sq, e);
-    m[1] = cmulc(cmul(e, a[0]), a[1]);
-  }
+// Two grid points at once: real and imaginary parts as FP32 pairs, so that the
+// arithmetic of both points is one packed instruction (see fft_core.cuh).
+struct Pair {
+  float2 re, im;
+};
+__device__ __forceinline__ float2 dup(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float2 neg(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ Pair pair_mul(Pair a, Pair b) {
+  return {__ffma2_rn(a.re, b.re, neg(__fmul2_rn(a.im, b.im))), __ffma2_rn(a.re, b.im, __fmul2_rn(a.im, b.re))};
 }
-// a + i c m for a real c
-__device__ __forceinline__ float2 add_i_scaled(float2 a, float c, float2 m) {
-  return make_float2(fmaf(-c, m.y, a.x), fmaf(c, m.x, a.y));
+// a conj(b)
+__device__ __forceinline__ Pair pair_mulc(Pair a, Pair b) {
+  return {__ffma2_rn(a.re, b.re, __fmul2_rn(a.im, b.im)), __ffma2_rn(a.im, b.re, neg(__fmul2_rn(a.re, b.im)))};
+}
+// i a conj(b)
+__device__ __forceinline__ Pair pair_imulc(Pair a, Pair b) {
+  return {__ffma2_rn(a.re, b.im, neg(__fmul2_rn(a.im, b.re))), __ffma2_rn(a.re, b.re, __fmul2_rn(a.im, b.im))};
+}
+// a + c b and a + i c b for a real c
+__device__ __forceinline__ Pair pair_axpy(Pair a, float c, Pair b) {
+  return {__ffma2_rn(dup(c), b.re, a.re), __ffma2_rn(dup(c), b.im, a.im)};
+}
+__device__ __forceinline__ Pair pair_iaxpy(Pair a, float c, Pair b) {
+  return {__ffma2_rn(dup(-c), b.im, a.re), __ffma2_rn(dup(c), b.re, a.im)};
+}
+__device__ __forceinline__ Pair pair_add(Pair a, Pair b) { return {cadd(a.re, b.re), cadd(a.im, b.im)}; }
+
+// Products of the coupling at one stage: the driving term of field 0 (A_s A_i,
+// or A_F^2), without its phase, and i times the slopes of the others, i u
+// conj(A_i), i u conj(A_s) (or i u conj(A_F)), u = e^{+i Phi} A_0.
+template <int F>
+__device__ __forceinline__ Pair nl_drive(const Pair* t) {
+  if constexpr (F == 3) return pair_mul(t[0], t[1]);
+  else return {__ffma2_rn(t[0].re, t[0].re, neg(__fmul2_rn(t[0].im, t[0].im))),
+               __fmul2_rn(cadd(t[0].re, t[0].re), t[0].im)};
+}
+template <int F>
+__device__ __forceinline__ void nl_slopes(Pair u, const Pair* t, Pair* n) {
+  if constexpr (F == 3) {
+    n[0] = pair_imulc(u, t[1]);
+    n[1] = pair_imulc(u, t[0]);
+  } else {
+    n[0] = pair_imulc(u, t[0]);
+  }
 }
 
-// Classical RK4 over one half step h (Sec. 3.1): e3 holds e^{+i Phi} at the
-// start, the midpoint and the end of the interval; kh = kappa h and
-// kh2 = kh/2 per field.  Every stage and the final combination use the same
-// kh_f, and the 1/6 weight is common to all fields: field-dependent rounding
-// of the weights would break the Manley-Rowe balance the exact scheme keeps
-// and let the total energy drift step after step.
+// Classical RK4 over one half step h (Sec. 3.1) of Eqs. CEp/CEs/CEi (fields p,
+// s, i) or of the degenerate pair (SH, F) at two points.  e0 = e^{+i Phi} at the
+// start of the half step and v = e^{+i dk h/2}, so the midpoint and end factors
+// are e0 v and e0 v^2; kh = kappa h and kh2 = kh/2 per field.
+// Field 0 enters the others' slopes only through u = e A_0, so its stage values
+// are carried as u directly, with m the driving terms of stages 1..4:
+//   u1 = e0 A_0,  w = v u1,  u2 = w + i kh2 v m1,  u3 = w + i kh2 m2,
+//   u4 = v (w + i kh m3),  A_0 += i kh/6 conj(e0) (m1 + conj(v)(2 m2 + 2 m3 + conj(v) m4)),
+// 12 operations a point fewer than applying e and conj(e) to A_0 and to the
+// driving term of every stage (116 against 128 for three fields).
+// Every stage and the final combination use the same kh_f, and the 1/6 weight is
+// common to all fields: field-dependent rounding of the weights would break the
+// Manley-Rowe balance the exact scheme keeps and let the total energy drift step
+// after step.
 template <int F>
-__device__ __forceinline__ void rk4(float2 (&a)[F], const float2* __restrict__ e3, const float* kh,
-                                    const float* kh2) {
-  float2 m[F], acc[F], t[F];
-  nl_m<F>(a, e3[0], m);
+__device__ __forceinline__ void rk4(Pair (&a)[F], Pair e0, Pair v, const float* kh, const float* kh2) {
+  constexpr int G = F - 1;
+  Pair t[G], n[G], acc[G];
+  const Pair u1 = pair_mul(e0, a[0]);
+  const Pair w = pair_mul(v, u1);
+  const Pair m1 = nl_drive<F>(a + 1);
+  nl_slopes<F>(u1, a + 1, acc);
 #pragma unroll
-  for (int f = 0; f < F; ++f) {
-    acc[f] = m[f];
-    t[f] = add_i_scaled(a[f], kh2[f], m[f]);
+  for (int g = 0; g < G; ++g) t[g] = pair_axpy(a[g + 1], kh2[g + 1], acc[g]);
+  const Pair m2 = nl_drive<F>(t);
+  nl_slopes<F>(pair_iaxpy(w, kh2[0], pair_mul(v, m1)), t, n);
+#pragma unroll
+  for (int g = 0; g < G; ++g) {
+    acc[g] = pair_axpy(acc[g], 2.f, n[g]);
+    t[g] = pair_axpy(a[g + 1], kh2[g + 1], n[g]);
   }
-  const float2 emid = e3[1];
-  nl_m<F>(t, emid, m);
+  const Pair m3 = nl_drive<F>(t);
+  nl_slopes<F>(pair_iaxpy(w, kh2[0], m2), t, n);
 #pragma unroll
-  for (int f = 0; f < F; ++f) {
-    acc[f] = make_float2(fmaf(2.f, m[f].x, acc[f].x), fmaf(2.f, m[f].y, acc[f].y));
-    t[f] = add_i_scaled(a[f], kh2[f], m[f]);
+  for (int g = 0; g < G; ++g) {
+    acc[g] = pair_axpy(acc[g], 2.f, n[g]);
+    t[g] = pair_axpy(a[g + 1], kh[g + 1], n[g]);
   }
-  nl_m<F>(t, emid, m);
+  const Pair m4 = nl_drive<F>(t);
+  nl_slopes<F>(pair_mul(v, pair_iaxpy(w, kh[0], m3)), t, n);
 #pragma unroll
-  for (int f = 0; f < F; ++f) {
-    acc[f] = make_float2(fmaf(2.f, m[f].x, acc[f].x), fmaf(2.f, m[f].y, acc[f].y));
-    t[f] = add_i_scaled(a[f], kh[f], m[f]);
+  for (int g = 0; g < G; ++g) {
+    const Pair q = pair_add(acc[g], n[g]);
+    a[g + 1] = pair_axpy(a[g + 1], kh[g + 1], {__fmul2_rn(q.re, dup(1.f / 6.f)), __fmul2_rn(q.im, dup(1.f / 6.f))});
   }
-  nl_m<F>(t, e3[2], m);
-#pragma unroll
-  for (int f = 0; f < F; ++f) a[f] = add_i_scaled(a[f], kh[f], cscale(cadd(acc[f], m[f]), 1.f / 6.f));
+  Pair m = pair_mulc(m4, v);
+  m = pair_axpy(m, 2.f, pair_add(m2, m3));
+  m = pair_mulc(pair_add(m1, pair_mulc(m, v)), e0);
+  a[0] = pair_iaxpy(a[0], kh[0], {__fmul2_rn(m.re, dup(1.f / 6.f)), __fmul2_rn(m.im, dup(1.f / 6.f))});
 }
 
 // e^{-i Phi} with Phi in FP64, reduced to [-pi, pi] before the FP32 sincos.
@@ -216,40 +257,50 @@ __device__ __forceinline__ float2 phase_minus(double phi) {
   return make_float2(c, -s);
 }
 
-// Stage phase factors e^{+i Phi}: sets 0..2 = second half of step B at
-// z_B + dz/2, z_B + 3dz/4, z_B + dz; sets 3..5 = first half of step A at z_A,
-// z_A + dz/4, z_A + dz/2.
-template <int F>
-__device__ __forceinline__ void nl_coefficients(const XPassArgs& p, float2* coef) {
-  const int s = threadIdx.x;
-  if (s < 6) {
-    double phi;
-    if (s < 3) phi = p.phiB + p.dkB * (0.5 * p.dz + 0.25 * p.dz * s);
-    else phi = p.phiA + p.dkA * (0.25 * p.dz * (s - 3));
-    const float2 em = phase_minus(phi);  // e^{-i Phi}
-    coef[s] = make_float2(em.x, -em.y);
-  }
-}
-
 // ------------------------------------------------------------------ x-pass
 // One row (y, tau) of every field per T threads; a CTA of THREADS threads
-// handles THREADS/T rows per tile.  Each field of a row has its own padded
-// row buffer in shared memory, used both as that field's FFT exchange space
-// and to park the field between the transforms: after the inverse transform
-// every thread parks its values at the positions it owns (the last pass of a
-// Stockham transform reads and writes the same positions per thread), the
-// pointwise RK4 pair then reads all F values of each owned point, and the
-// forward transform starts from the owned positions again.  No thread ever
-// reads a position another thread parked, so parking needs no barrier, and
-// the fields and the points are processed in loops rather than unrolled
-// (the points two at a time), which keeps the kernel small enough for the
-// instruction cache.  Field data
-// is read with ld.global.cg (L2), twiddles through L1.
+// handles THREADS/T rows per tile.  Each field of a row has its own row buffer
+// in shared memory, used both as that field's FFT exchange space and to park the
+// field between the transforms: after the inverse transform every thread parks
+// its values, the pointwise RK4 pair then reads all F values of each owned point,
+// and the forward transform starts from the owned points again.  No thread ever
+// reads a value another thread parked, so parking needs no barrier, and the
+// fields and the points are processed in loops rather than unrolled, which keeps
+// the kernel small enough for the instruction cache.  Two points of a thread
+// are parked together as (re, re, im, im) in 16 bytes, which is the form the
+// packed RK4 works in.  Field data is read with ld.global.cg (L2), twiddles
+// through L1.
+// points 2 q and 2 q + 1 of thread t in a row buffer
+template <class PL>
+__device__ __forceinline__ float4* park_place(float2* row, int t, int q) {
+  return reinterpret_cast<float4*>(row) + q * PL::T + t;
+}
+template <class PL>
+__device__ __forceinline__ void park(float2* row, int t, const float2 (&v)[PL::E]) {
+#pragma unroll
+  for (int q = 0; q < PL::E / 2; ++q)
+    *park_place<PL>(row, t, q) = make_float4(v[2 * q].x, v[2 * q + 1].x, v[2 * q].y, v[2 * q + 1].y);
+}
+template <class PL>
+__device__ __forceinline__ void unpark(float2* row, int t, float2 (&v)[PL::E]) {
+#pragma unroll
+  for (int q = 0; q < PL::E / 2; ++q) {
+    const float4 a = *park_place<PL>(row, t, q);
+    v[2 * q] = make_float2(a.x, a.z);
+    v[2 * q + 1] = make_float2(a.y, a.w);
+  }
+}
+// position on the row of point e of thread t between the transforms
+template <class PL>
+__device__ __forceinline__ int point_pos(int t, int e) {
+  constexpr int R0 = fft_radix<PL, false>(0);
+  return pos_first<PL, false>(t + (e / R0) * PL::T, e % R0);
+}
 template <int NX, int THREADS>
 __host__ __device__ constexpr int xtile_rows() { return THREADS / FftPlan<NX>::T; }
 template <int NX, int THREADS>
 __host__ __device__ constexpr int xtile_smem_floats2(int nf) {
-  return 6 * nf + nf * xtile_rows<NX, THREADS>() * XchRow::pitch(NX);
+  return nf * xtile_rows<NX, THREADS>() * XchRow::pitch(NX);
 }
 
 template <int NX, int F, int THREADS, bool MAP = false, bool REC = false>
@@ -261,8 +312,7 @@ __device__ __forceinline__ void xpass_tile(const XPassArgs& p, long long tile, c
   constexpr int PITCH = XchRow::pitch(NX);
   constexpr int RF0 = fft_radix<PL, false>(0);           // forward first radix
   constexpr int RFL = fft_radix<PL, false>(PL::NP - 1);  // forward last radix
-  constexpr int SF0 = NX / RF0;
-  using SY = typename std::conditional<xpass_warp_sync<NX>(), SyncWarp, SyncBlock>::type;
+    using SY = typename std::conditional<xpass_warp_sync<NX>(), SyncWarp, SyncBlock>::type;
   static_assert(ROWS >= 1 && ROWS * T == THREADS, "CTA must hold whole rows");
   const TwGlobal tw{p.tw};
 
@@ -295,106 +345,98 @@ __device__ __forceinline__ void xpass_tile(const XPassArgs& p, long long tile, c
         for (int r = 0; r < RF0; ++r)
           v[b * RF0 + r] = act ? __ldcg(src + pos_first<PL, false>(t + b * T, r)) : make_float2(0.f, 0.f);
     }
-#pragma unroll
-    for (int b = 0; b < E / RF0; ++b)
-#pragma unroll
-      for (int r = 0; r < RF0; ++r) xr.st(t + b * T + r * SF0, v[b * RF0 + r]);
+    SY::sync();  // the last exchange's reads of this row are done
+    park<PL>(xr.base, t, v);
   }
 
-  // 2. the RK4 half steps, point by point over the owned positions
+  // 2. the RK4 half steps, two points at a time over the owned points
   if (mode == XM_NL_MID || mode == XM_NL_LAST || mode == XM_NL_FIRST) {
     const long long nxy = (long long)p.ny * NX;
     const float2* emap = MAP ? p.emap + (act ? row % p.ny : 0) * NX : nullptr;
-    // MAP: the next point's stage-factor tables are requested while this point's
-    // RK4 pair runs (with a fan-out map: 656 -> 579 us per OPG launch)
-    float2 nm[4];
+    // MAP: the next points' stage-factor tables are requested while these points'
+    // RK4 pair runs
+    float2 nm[4][2];
+    Pair eB, vB, eA, vA;
     if constexpr (MAP) {
 #pragma unroll
-      for (int q = 0; q < 4; ++q) nm[q] = __ldg(emap + q * nxy + pos_first<PL, false>(t, 0));
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int u = 0; u < 2; ++u) nm[q][u] = __ldg(emap + q * nxy + point_pos<PL>(t, u));
+    } else {
+      eB = {dup(coef[0].x), dup(coef[0].y)};
+      vB = {dup(coef[1].x), dup(coef[1].y)};
+      eA = {dup(coef[2].x), dup(coef[2].y)};
+      vA = {dup(coef[3].x), dup(coef[3].y)};
     }
-    // two points per iteration: their RK4 chains interleave (measured on GB300:
-    // OPG x-pass 549 -> 540 us, with a fan-out map 699 -> 655 us, SFG 94 -> 90 us;
-    // four points per iteration, 579 us, overflow the instruction cache)
-#pragma unroll 2
-    for (int e = 0; e < E; ++e) {
-      // the park place of a point is its butterfly's; its position on the row
-      // (of the map and of the recorded states) is pos
-      const int place = t + (e / RF0) * T + (e % RF0) * SF0;
-      const int off = place + (place >> 4);  // XchRow padding
-      const int pos = pos_first<PL, false>(t + (e / RF0) * T, e % RF0);
-      float2 cm[4];
+#pragma unroll 1
+    for (int e = 0; e < E; e += 2) {
       if constexpr (MAP) {
+        const auto pair_of = [](const float2* m) { return Pair{make_float2(m[0].x, m[1].x), make_float2(m[0].y, m[1].y)}; };
+        eB = pair_of(nm[0]);
+        vB = pair_of(nm[1]);
+        eA = pair_of(nm[2]);
+        vA = pair_of(nm[3]);
+        if (e + 2 < E) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) cm[q] = nm[q];
-        if (e + 1 < E) {
-          const int pn = pos_first<PL, false>(t + ((e + 1) / RF0) * T, (e + 1) % RF0);
+          for (int q = 0; q < 4; ++q)
 #pragma unroll
-          for (int q = 0; q < 4; ++q) nm[q] = __ldg(emap + q * nxy + pn);
+            for (int u = 0; u < 2; ++u) nm[q][u] = __ldg(emap + q * nxy + point_pos<PL>(t, e + 2 + u));
         }
       }
-      float2 a[F];
+      Pair a[F];
 #pragma unroll
-      for (int f = 0; f < F; ++f) a[f] = myrow[f * ROWS * PITCH + off];
-      // MAP: e^{i Phi(x, y, z_s)} = T V^s at this point, for the B and A stages
+      for (int f = 0; f < F; ++f) {
+        const float4 w = *park_place<PL>(myrow + f * ROWS * PITCH, t, e / 2);
+        a[f] = {make_float2(w.x, w.y), make_float2(w.z, w.w)};
+      }
+      const auto record = [&](float2* rec) {
+        if (!act) return;
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          float2* d = rec + row * NX + point_pos<PL>(t, e + u);
+#pragma unroll
+          for (int f = 0; f < F; ++f)
+            d[f * p.fstride] = u == 0 ? make_float2(a[f].re.x, a[f].im.x) : make_float2(a[f].re.y, a[f].im.y);
+        }
+      };
       if (mode != XM_NL_FIRST) {
         if constexpr (REC) {
-          if (p.rec_b && act) {
-#pragma unroll
-            for (int f = 0; f < F; ++f) p.rec_b[f * p.fstride + row * NX + pos] = a[f];
-          }
+          if (p.rec_b) record(p.rec_b);
         }
-        if constexpr (MAP) {
-          float2 e3[3];
-          const float2 v = cm[1];
-          e3[0] = cm[0];
-          e3[1] = cmul(e3[0], v);
-          e3[2] = cmul(e3[1], v);
-          rk4<F>(a, e3, p.kh, p.kh2);
-        } else {
-          rk4<F>(a, coef, p.kh, p.kh2);
-        }
+        rk4<F>(a, eB, vB, p.kh, p.kh2);
       }
       if (mode != XM_NL_LAST) {
         if constexpr (REC) {
-          if (p.rec_a && act) {
-#pragma unroll
-            for (int f = 0; f < F; ++f) p.rec_a[f * p.fstride + row * NX + pos] = a[f];
-          }
+          if (p.rec_a) record(p.rec_a);
         }
-        if constexpr (MAP) {
-          float2 e3[3];
-          const float2 v = cm[3];
-          e3[0] = cm[2];
-          e3[1] = cmul(e3[0], v);
-          e3[2] = cmul(e3[1], v);
-          rk4<F>(a, e3, p.kh, p.kh2);
-        } else {
-          rk4<F>(a, coef + 3, p.kh, p.kh2);
-        }
+        rk4<F>(a, eA, vA, p.kh, p.kh2);
       }
 #pragma unroll
-      for (int f = 0; f < F; ++f) myrow[f * ROWS * PITCH + off] = a[f];
+      for (int f = 0; f < F; ++f)
+        *park_place<PL>(myrow + f * ROWS * PITCH, t, e / 2) =
+            make_float4(a[f].re.x, a[f].re.y, a[f].im.x, a[f].im.y);
     }
   }
 
   // 3. every field: unpark, forward transform (or scale), store
   const bool to_x = (mode == XM_INV || mode == XM_NL_LAST);
-  const float sc = mode == XM_INV ? p.scale : 1.f;
 #pragma unroll 1
   for (int f = 0; f < F; ++f) {
     const XchRow xr{myrow + f * ROWS * PITCH};
     float2* dst = p.data + f * p.fstride + (act ? row : 0) * NX;
     float2 v[E];
-#pragma unroll
-    for (int b = 0; b < E / RF0; ++b)
-#pragma unroll
-      for (int r = 0; r < RF0; ++r) v[b * RF0 + r] = xr.ld(t + b * T + r * SF0);
+    unpark<PL>(xr.base, t, v);
     if (to_x) {
+      if (mode == XM_INV) {
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+          v[e] = __ffma2_rn(v[e], dup(p.scale), __fmul2_rn(v[e], dup(p.scale_lo)));
+      }
       if (act) {
 #pragma unroll
         for (int b = 0; b < E / RF0; ++b)
 #pragma unroll
-          for (int r = 0; r < RF0; ++r) dst[pos_first<PL, false>(t + b * T, r)] = cscale(v[b * RF0 + r], sc);
+          for (int r = 0; r < RF0; ++r) dst[pos_first<PL, false>(t + b * T, r)] = v[b * RF0 + r];
       }
     } else {
       fft_run<PL, false, 0, XchRow, SY, TwGlobal>(v, t, xr, tw);
@@ -416,16 +458,11 @@ __global__ void __launch_bounds__(xpass_threads<NX>(), xpass_min_blocks<NX, F>()
     xpass_kernel(const XPassArgs p) {
   constexpr int THREADS = xpass_threads<NX>();
   extern __shared__ float4 sm4[];
-  float2* coef = reinterpret_cast<float2*>(sm4);
-  float2* rowbuf = coef + 6 * F;
+  float2* rowbuf = reinterpret_cast<float2*>(sm4);
   // stage factors from the launch (formed on the host in FP64: a per-CTA FP64
-  // phase reduction ahead of this barrier stalled every CTA's first warps)
-  if constexpr (!MAP) {
-    if (threadIdx.x < 6) coef[threadIdx.x] = p.ecoef[threadIdx.x];
-  }
-  __syncthreads();
+  // phase reduction stalled every CTA's first warps)
   // rows from the last tau-plane down (see the note on pass order above)
-  xpass_tile<NX, F, THREADS, MAP, REC>(p, (long long)gridDim.x - 1 - blockIdx.x, coef, rowbuf);
+  xpass_tile<NX, F, THREADS, MAP, REC>(p, (long long)gridDim.x - 1 - blockIdx.x, p.ecoef, rowbuf);
 }
 
 // ------------------------------------------------- strided-axis passes
@@ -642,7 +679,7 @@ struct GroupInst {
   int nz;
 };
 // ecoef: the instances' stage factors, instance i's for step j at
-// ecoef[i stride + (j + 1) 6 + 0..5]
+// ecoef[i stride + (j + 1) kStageFactors + 0..]
 cudaError_t run_xpass_group(int nx, const XPassArgs& base, const GroupInst* gi, const float2* ecoef, int stride,
                             int step, int ninst, cudaStream_t s);
 int xpass_rows_of(int nx);  // rows per CTA of the x-pass of length nx

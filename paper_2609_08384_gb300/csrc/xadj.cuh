@@ -233,7 +233,7 @@ template <int NX, int F, bool MAP>
 cudaError_t launch_adjoint(const XAdjArgs& a, long long* ncta, cudaStream_t s) {
   constexpr int ROWS = xpass_rows<NX>();
   constexpr int THREADS = xpass_threads<NX>();
-  const size_t smem = (size_t)xpass_smem_floats2<NX>(F) * sizeof(float2);
+  const size_t smem = (size_t)(6 * F + xpass_smem_floats2<NX>(F)) * sizeof(float2);
   static SmemOnce once;
   cudaError_t e = raise_smem_limit(xpass_adj_kernel<NX, F, MAP>, smem, once);
   if (e != cudaSuccess) return e;
