@@ -53,6 +53,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 namespace brahms {
 
 __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
@@ -391,6 +393,16 @@ struct XchCol {
   __device__ __forceinline__ void st(int pos, float2 v) const { base[pos * TX + tx] = v; }
   __device__ __forceinline__ float2 ld(int pos) const { return base[pos * TX + tx]; }
 };
+// Tiles of 8 columns: a row is 64 bytes, so the two rows of a half-warp's access
+// must differ in parity.  The writes of pass 0 go to rows R0 j + r, whose parity
+// is the same for every j: there row pos is kept at pos ^ ((pos / R0) & 1).
+struct XchCol8 {
+  static constexpr bool kSplit = false;
+  float2* base;
+  int tx;
+  __device__ __forceinline__ void st(int pos, float2 v) const { base[pos * 8 + tx] = v; }
+  __device__ __forceinline__ float2 ld(int pos) const { return base[pos * 8 + tx]; }
+};
 // The same layout for one real component at a time: the exchange runs in two
 // rounds (real parts, then imaginary parts) through half the shared memory.
 template <int TX>
@@ -512,20 +524,30 @@ __device__ __forceinline__ void fft_run(float2 (&v)[PL::E], int t, const X& x, c
       }
     } else {
       S::sync();  // earlier readers of the exchange buffer are done
+      // exchange of pass 0 in 8-column tiles: rows in turned parity (XchCol8)
+      constexpr bool kTurn = std::is_same<X, XchCol8>::value && P == 0 && R % 2 == 0;
+      constexpr int K = N / R2;
 #pragma unroll
       for (int b = 0; b < B; ++b) {
         const int j = t + b * T;
         const int m = j % NS;
         const int d = (j / NS) * NS * R + m;
 #pragma unroll
-        for (int r = 0; r < R; ++r) x.st(d + r * NS, v[b * R + r]);
+        for (int r = 0; r < R; ++r) {
+          if constexpr (kTurn) x.st(d + r + (r % 2 ? -(j & 1) : (j & 1)), v[b * R + r]);
+          else x.st(d + r * NS, v[b * R + r]);
+        }
       }
       S::sync();
 #pragma unroll
       for (int b = 0; b < B2; ++b) {
         const int j = t + b * T;
 #pragma unroll
-        for (int r = 0; r < R2; ++r) v[b * R2 + r] = x.ld(j + r * (N / R2));
+        for (int r = 0; r < R2; ++r) {
+          if constexpr (kTurn && K % R == 0 && K <= R) v[b * R2 + r] = x.ld(((r * (K / R)) % 2 ? (j ^ 1) : j) + r * K);
+          else if constexpr (kTurn) v[b * R2 + r] = x.ld((j + r * K) ^ (((j + r * K) / R) & 1));
+          else v[b * R2 + r] = x.ld(j + r * K);
+        }
       }
     }
     fft_run<PL, INV, P + 1, X, S, TW>(v, t, x, tw);

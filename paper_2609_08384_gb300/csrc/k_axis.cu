@@ -22,19 +22,41 @@ static cudaError_t launch_axis(const AxisArgs& a, cudaStream_t s) {
   return cudaPeekAtLastError();
 }
 
+// The pipelined tau-pass: one wave of persistent CTAs over tiles of its own width.
+template <class PL>
+static cudaError_t launch_tprop_pipe(const AxisArgs& a0, cudaStream_t s) {
+  constexpr int TX = tau_pipe_cols<PL>();
+  constexpr size_t smem = (size_t)tau_pipe_smem<PL>();
+  static SmemOnce once;
+  cudaError_t e = raise_smem_limit(tpass_pipe_kernel<PL>, smem, once);
+  if (e != cudaSuccess || a0.ntiles <= 0) return e;
+  AxisArgs a = a0;
+  const long long lines = a0.ntiles / a0.xtiles;  // (field, y) lines
+  a.xtiles = (a0.nx + TX - 1) / TX;
+  a.ntiles = lines * a.xtiles;
+  const long long wave = 152 * tau_pipe_ctas<PL>();
+  const long long grid = a.ntiles < wave ? a.ntiles : wave;
+  tpass_pipe_kernel<PL><<<(unsigned)grid, tau_pipe_threads<PL>(), smem, s>>>(a);
+  return cudaPeekAtLastError();
+}
+
 template <int N>
 static cudaError_t launch_tprop(const AxisArgs& a, cudaStream_t s) {
   using PL = TauPlan<N>;
-  constexpr int TPC = tiles_per_cta<PL>();
-  constexpr int THREADS = TPC * tile_threads<PL>();
-  const size_t smem = (size_t)axis_smem_floats2<PL>() * sizeof(float2);
-  static SmemOnce once;
-  cudaError_t e = raise_smem_limit(tpass_prop_kernel<PL>, smem, once);
-  if (e != cudaSuccess) return e;
-  const long long grid = (a.ntiles + TPC - 1) / TPC;
-  if (grid <= 0) return cudaSuccess;
-  tpass_prop_kernel<PL><<<(unsigned)grid, THREADS, smem, s>>>(a);
-  return cudaPeekAtLastError();
+  if constexpr (tau_pipe<PL>()) {
+    return launch_tprop_pipe<PL>(a, s);
+  } else {
+    constexpr int TPC = tiles_per_cta<PL>();
+    constexpr int THREADS = TPC * tile_threads<PL>();
+    const size_t smem = (size_t)axis_smem_floats2<PL>() * sizeof(float2);
+    static SmemOnce once;
+    cudaError_t e = raise_smem_limit(tpass_prop_kernel<PL>, smem, once);
+    if (e != cudaSuccess) return e;
+    const long long grid = (a.ntiles + TPC - 1) / TPC;
+    if (grid <= 0) return cudaSuccess;
+    tpass_prop_kernel<PL><<<(unsigned)grid, THREADS, smem, s>>>(a);
+    return cudaPeekAtLastError();
+  }
 }
 
 cudaError_t run_axis_fft(int n, int axis, bool inv, const AxisArgs& a, cudaStream_t s) {

@@ -651,6 +651,109 @@ __device__ __forceinline__ void tprop_tile(const AxisArgs& p, long long cta_tile
   if (a.act) store_pencil<PL, false>(v, a.base, a.stride, t);
 }
 
+// ------------------------------------------------- pipelined tau-pass
+// The same pass by persistent CTAs that copy their next tile (cp.async, 16
+// bytes) into one buffer while they transform the current one in the other, so
+// the wait for memory overlaps the transforms.  Tiles are 8 columns wide (rows of
+// 64 bytes) for the plans of 16 or more threads per pencil and 128/T for those of
+// 8, small enough for two buffers and several CTAs per SM, and the exchanges run
+// in the tile's own buffer.
+// Taken by the two-pass plans (one exchange per transform) and by the plan of 32
+// threads per pencil, whose 16-column tile leaves room for one CTA per SM.
+// Measured per launch, plain tau-pass against this one: 512 points (three fields
+// of 256x256) 463 -> 415 us, 256 (three of 128x128) 57 -> 49, 128 (two of 512x512)
+// 231 -> 212, 64 (two of 1024x256) 127 -> 115, 768 (two of 192x192) 388 -> 348; the
+// four-pass plans of 192 and 384 points lost 1 to 5 % (their block barriers).
+// What bounds it: latency between the phases of a tile at 12 to 16 warps per SM
+// (512 points: issue 49 %, FP32 pipe 45 %, shared memory 49 %, DRAM 48 %); plans
+// with 16 values per thread and twice the warps were slower (494 to 580 us).
+template <class PL>
+__host__ __device__ constexpr bool tau_pipe() { return PL::T >= 8 && PL::T <= 32 && (PL::NP == 2 || PL::T == 32); }
+template <class PL>
+__host__ __device__ constexpr int tau_pipe_cols() { return PL::T >= 16 ? 8 : 128 / PL::T; }
+template <class PL>
+__host__ __device__ constexpr int tau_pipe_threads() { return PL::T * tau_pipe_cols<PL>(); }
+template <class PL>
+__host__ __device__ constexpr int tau_pipe_smem() {
+  return (2 * PL::N * tau_pipe_cols<PL>() + tw_table_size<PL>()) * (int)sizeof(float2);
+}
+// Resident CTAs: as many as shared memory holds, at most 512 threads per SM (128
+// registers) where a thread's values or its tile of 8 columns need them, 768 (80)
+// for the 128-point plan, 1024 for 64 points.  (256 points: 49 us with 512
+// threads, 53 with 640, 57 with 768; 128 points: 226, 218, 212.)
+template <class PL>
+__host__ __device__ constexpr int tau_pipe_ctas() {
+  const int fit = 227 * 1024 / (tau_pipe_smem<PL>() + 1024);
+  const int most = (PL::E <= 8 ? 1024 : PL::T == 8 ? 768 : 512) / tau_pipe_threads<PL>();
+  return fit < most ? fit : most;
+}
+
+template <class PL>
+__global__ void __launch_bounds__(tau_pipe_threads<PL>(), tau_pipe_ctas<PL>())
+    tpass_pipe_kernel(const AxisArgs p) {
+  constexpr int N = PL::N, TX = tau_pipe_cols<PL>();
+  constexpr int THREADS = tau_pipe_threads<PL>();
+  constexpr int PAIRS = TX / 2, ROWS = THREADS / PAIRS;  // 16-byte pieces per row, rows per copy step
+  using X = typename std::conditional<TX == 8, XchCol8, XchCol<TX>>::type;
+  extern __shared__ float4 sm4[];
+  float2* buf = reinterpret_cast<float2*>(sm4);
+  float2* tw = buf + 2 * N * TX;
+  for (int i = threadIdx.x; i < tw_table_size<PL>(); i += THREADS) tw[i] = p.tw[i];
+  const long long plane = (long long)p.nx * p.ny;
+  const int tx = threadIdx.x % TX, t = threadIdx.x / TX;
+  // tile k counted from the last: its first column in memory and its (field, y, x)
+  struct Tile {
+    int f, y, x;
+    float2* base;
+  };
+  const auto tile_at = [&](long long k) {
+    const long long tile = p.ntiles - 1 - k;
+    Tile a;
+    a.x = (int)(tile % p.xtiles) * TX;
+    const long long rest = tile / p.xtiles;
+    a.y = (int)(rest % p.ny);
+    a.f = (int)(rest / p.ny);
+    a.base = p.data + (long long)a.f * p.fstride + (long long)a.y * p.nx + a.x;
+    return a;
+  };
+  const auto copy_tile = [&](long long k, int b) {
+    const Tile a = tile_at(k);
+    const int c = 2 * (threadIdx.x % PAIRS), row = threadIdx.x / PAIRS;
+    if (a.x + c >= p.nx) return;  // nx is even
+    const float2* src = a.base + c + row * plane;
+    const unsigned dst = (unsigned)__cvta_generic_to_shared(buf + b * N * TX + row * TX + c);
+#pragma unroll
+    for (int q = 0; q < N / ROWS; ++q)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + q * ROWS * TX * 8),
+                   "l"(src + (long long)(q * ROWS) * plane)
+                   : "memory");
+  };
+  long long k = blockIdx.x;
+  if (k < p.ntiles) copy_tile(k, 0);
+  cp_async_commit();
+  for (int b = 0; k < p.ntiles; k += gridDim.x, b ^= 1) {
+    cp_async_wait<0>();
+    __syncthreads();  // the tile is there, and the last one's buffer is free
+    if (k + gridDim.x < p.ntiles) copy_tile(k + gridDim.x, b ^ 1);
+    cp_async_commit();
+    const Tile a = tile_at(k);
+    const bool act = a.x + tx < p.nx;
+    // the column's factors, requested ahead of the forward transform
+    const float2 dx = act ? p.px[a.f * p.nx + a.x + tx] : make_float2(0.f, 0.f), dy = p.py[a.f * p.ny + a.y];
+    const X xc{buf + b * N * TX, tx};
+    constexpr int R0 = fft_radix<PL, false>(0);
+    float2 v[PL::E];
+#pragma unroll
+    for (int i = 0; i < PL::E / R0; ++i)
+#pragma unroll
+      for (int r = 0; r < R0; ++r) v[i * R0 + r] = xc.ld(pos_first<PL, false>(t + i * PL::T, r));
+    fft_run<PL, false, 0, X, SyncBlock, TwShared>(v, t, xc, TwShared{tw});
+    apply_prop<PL>(v, ColumnProp(p, dx, dy), p.pt + a.f * p.nt, t);
+    fft_run<PL, true, 0, X, SyncBlock, TwShared>(v, t, xc, TwShared{tw});
+    if (act) store_pencil<PL, false>(v, a.base + tx, plane, t);
+  }
+}
+
 template <class PL, bool INV, int AXIS>
 __global__ void __launch_bounds__(tiles_per_cta<PL>() * tile_threads<PL>())
     axis_fft_kernel(const AxisArgs p) {
