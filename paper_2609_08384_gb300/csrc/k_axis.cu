@@ -18,8 +18,7 @@ static cudaError_t launch_axis(const AxisArgs& a, cudaStream_t s) {
   if (e != cudaSuccess) return e;
   const long long grid = (a.ntiles + TPC - 1) / TPC;
   if (grid <= 0) return cudaSuccess;
-  axis_fft_kernel<PL, INV, AXIS><<<(unsigned)grid, THREADS, smem, s>>>(a);
-  return cudaPeekAtLastError();
+  return launch_chained(axis_fft_kernel<PL, INV, AXIS>, dim3((unsigned)grid), THREADS, smem, s, a);
 }
 
 // The pipelined tau-pass: one wave of persistent CTAs over tiles of its own width.
@@ -36,8 +35,7 @@ static cudaError_t launch_tprop_pipe(const AxisArgs& a0, cudaStream_t s) {
   a.ntiles = lines * a.xtiles;
   const long long wave = 152 * tau_pipe_ctas<PL>();
   const long long grid = a.ntiles < wave ? a.ntiles : wave;
-  tpass_pipe_kernel<PL><<<(unsigned)grid, tau_pipe_threads<PL>(), smem, s>>>(a);
-  return cudaPeekAtLastError();
+  return launch_chained(tpass_pipe_kernel<PL>, dim3((unsigned)grid), tau_pipe_threads<PL>(), smem, s, a);
 }
 
 template <int N>
@@ -54,8 +52,7 @@ static cudaError_t launch_tprop(const AxisArgs& a, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     const long long grid = (a.ntiles + TPC - 1) / TPC;
     if (grid <= 0) return cudaSuccess;
-    tpass_prop_kernel<PL><<<(unsigned)grid, THREADS, smem, s>>>(a);
-    return cudaPeekAtLastError();
+    return launch_chained(tpass_prop_kernel<PL>, dim3((unsigned)grid), THREADS, smem, s, a);
   }
 }
 

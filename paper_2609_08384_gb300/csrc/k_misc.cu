@@ -1,5 +1,6 @@
 // Set-up tables, the energy reduction and dtype conversions.
 #include "kernels.cuh"
+#include "launch_cfg.h"
 #include "map_seg.h"
 
 namespace brahms {
@@ -63,6 +64,7 @@ __device__ __forceinline__ float2 phase_plus(double phi) {
 }
 
 __global__ void map_tables_kernel(const MapArgs a) {
+  chain_begin();
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < a.nxy;
        i += (long long)gridDim.x * blockDim.x) {
     const double mb = a.mapB[i], ma = a.mapA[i];
@@ -83,8 +85,7 @@ __global__ void map_tables_kernel(const MapArgs a) {
 cudaError_t run_map_tables(const MapArgs& a, cudaStream_t s) {
   long long g = (a.nxy + 255) / 256;
   if (g > 152 * 8) g = 152 * 8;
-  map_tables_kernel<<<(unsigned)g, 256, 0, s>>>(a);
-  return cudaPeekAtLastError();
+  return launch_chained(map_tables_kernel, dim3((unsigned)g), 256, 0, s, a);
 }
 
 __global__ void map_phase_advance_kernel(double* mphase, const double* m, double len, long long nxy) {
@@ -102,6 +103,7 @@ cudaError_t run_map_phase_advance(double* mphase, const double* m, double len, l
 // B: the second half of step jB (starting at its midpoint), A: the first half
 // of step jA; the same four tables as map_tables_kernel.
 __global__ void map_tables_seg_kernel(const MapSegArgs a) {
+  chain_begin();
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < a.nxy;
        i += (long long)gridDim.x * blockDim.x) {
     double qb = 0.0, qa = 0.0;
@@ -122,8 +124,7 @@ cudaError_t run_map_tables_seg(const MapSegArgs& a, cudaStream_t s) {
   if (a.nseg < 1 || a.nseg > kMapSegMax) return cudaErrorInvalidValue;
   long long g = (a.nxy + 255) / 256;
   if (g > 152 * 8) g = 152 * 8;
-  map_tables_seg_kernel<<<(unsigned)g, 256, 0, s>>>(a);
-  return cudaPeekAtLastError();
+  return launch_chained(map_tables_seg_kernel, dim3((unsigned)g), 256, 0, s, a);
 }
 
 cudaError_t run_prop_tables(const TableArgs& a, cudaStream_t s) {
@@ -228,6 +229,7 @@ static int grid_for(long long n) {
 // P = (1 + Dx)(1 + Dy)(1 + Dt) / N of the tau-pass, element by element, with
 // the tau-pass's arithmetic, on the (kx, ky)-domain state.
 __global__ void prop_pointwise_kernel(const AxisArgs p, int nf) {
+  chain_begin();
   const long long plane = (long long)p.nx * p.ny;
   const long long per_field = plane * p.nt;
   const long long n = per_field * nf;
@@ -244,8 +246,8 @@ __global__ void prop_pointwise_kernel(const AxisArgs p, int nf) {
 }
 
 cudaError_t run_prop_pointwise(const AxisArgs& a, int nf, cudaStream_t s) {
-  prop_pointwise_kernel<<<grid_for((long long)a.nx * a.ny * a.nt * nf), 256, 0, s>>>(a, nf);
-  return cudaPeekAtLastError();
+  return launch_chained(prop_pointwise_kernel, dim3((unsigned)grid_for((long long)a.nx * a.ny * a.nt * nf)), 256, 0, s, a,
+                        nf);
 }
 
 cudaError_t run_c128_to_c64(const double2* in, float2* out, long long n, cudaStream_t s) {

@@ -10,10 +10,11 @@ namespace brahms {
 __global__ void __launch_bounds__(256) sens_boundary_kernel(const double* __restrict__ partial, long long ncta,
                                                             double* sensA, double* sensB) {
   __shared__ double red[8][6];
+  chain_begin();
   double v[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
   for (long long c = threadIdx.x; c < ncta; c += blockDim.x)
 #pragma unroll
-    for (int k = 0; k < 6; ++k) v[k] += partial[c * 6 + k];
+    for (int k = 0; k < 6; ++k) v[k] += __ldcg(partial + c * 6 + k);
 #pragma unroll
   for (int k = 0; k < 6; ++k) {
 #pragma unroll
@@ -79,8 +80,7 @@ long long xpass_adjoint_ctas(int nx, long long rows) {
 }
 
 cudaError_t run_sens_boundary(const double* partial, long long ncta, double* sensA, double* sensB, cudaStream_t s) {
-  sens_boundary_kernel<<<1, 256, 0, s>>>(partial, ncta, sensA, sensB);
-  return cudaPeekAtLastError();
+  return launch_chained(sens_boundary_kernel, dim3(1), 256, 0, s, partial, ncta, sensA, sensB);
 }
 
 }  // namespace brahms

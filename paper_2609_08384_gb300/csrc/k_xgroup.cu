@@ -20,6 +20,7 @@ __global__ void __launch_bounds__(xpass_threads<NX>(), xpass_min_blocks<NX, 2>()
   constexpr int THREADS = xpass_threads<NX>();
   extern __shared__ float4 sm4[];
   float2* rowbuf = reinterpret_cast<float2*>(sm4);
+  chain_begin();
   // tiles from the last down, as the single-instance x-pass
   const long long t = (long long)gridDim.x - 1 - blockIdx.x;
   const int i = (int)(t / tiles_per_inst);
@@ -49,8 +50,8 @@ static cudaError_t launch_group(const XPassArgs& base, const GroupInst* gi, cons
   const long long tiles = base.rows / ROWS;
   const long long grid = tiles * ninst;
   if (grid <= 0) return cudaSuccess;
-  xpass_group_kernel<NX><<<(unsigned)grid, THREADS, smem, s>>>(base, gi, ecoef, stride, step, tiles);
-  return cudaPeekAtLastError();
+  return launch_chained(xpass_group_kernel<NX>, dim3((unsigned)grid), THREADS, smem, s, base, gi, ecoef, stride, step,
+                        tiles);
 }
 
 cudaError_t run_xpass_group(int nx, const XPassArgs& base, const GroupInst* gi, const float2* ecoef, int stride,

@@ -27,8 +27,7 @@ static cudaError_t launch_x_variant(const XPassArgs& a0, cudaStream_t s) {
   if (e != cudaSuccess) return e;
   const long long grid = (a.rows + ROWS - 1) / ROWS;
   if (grid <= 0) return cudaSuccess;
-  xpass_kernel<NX, F, MAP><<<(unsigned)grid, THREADS, smem, s>>>(a);
-  return cudaPeekAtLastError();
+  return launch_chained(xpass_kernel<NX, F, MAP, false>, dim3((unsigned)grid), THREADS, smem, s, a);
 }
 
 template <int NX, int F>

@@ -387,7 +387,7 @@ __device__ __forceinline__ void xpass_tile(const XPassArgs& p, long long tile, c
 #pragma unroll
       for (int q = 0; q < 4; ++q)
 #pragma unroll
-        for (int u = 0; u < 2; ++u) nm[q][u] = __ldg(emap + q * nxy + point_pos<PL>(t, u));
+        for (int u = 0; u < 2; ++u) nm[q][u] = __ldcg(emap + q * nxy + point_pos<PL>(t, u));
     } else {
       eB = {dup(coef[0].x), dup(coef[0].y)};
       vB = {dup(coef[1].x), dup(coef[1].y)};
@@ -406,7 +406,7 @@ __device__ __forceinline__ void xpass_tile(const XPassArgs& p, long long tile, c
 #pragma unroll
           for (int q = 0; q < 4; ++q)
 #pragma unroll
-            for (int u = 0; u < 2; ++u) nm[q][u] = __ldg(emap + q * nxy + point_pos<PL>(t, e + 2 + u));
+            for (int u = 0; u < 2; ++u) nm[q][u] = __ldcg(emap + q * nxy + point_pos<PL>(t, e + 2 + u));
         }
       }
       Pair a[F];
@@ -485,6 +485,7 @@ __global__ void __launch_bounds__(xpass_threads<NX>(), xpass_min_blocks<NX, F>()
   constexpr int THREADS = xpass_threads<NX>();
   extern __shared__ float4 sm4[];
   float2* rowbuf = reinterpret_cast<float2*>(sm4);
+  chain_begin();
   // stage factors from the launch (formed on the host in FP64: a per-CTA FP64
   // phase reduction stalled every CTA's first warps)
   // rows from the last tau-plane down (see the note on pass order above)
@@ -729,6 +730,7 @@ __global__ void __launch_bounds__(tau_pipe_threads<PL>(), tau_pipe_ctas<PL>())
                    : "memory");
   };
   long long k = blockIdx.x;
+  chain_begin();
   if (k < p.ntiles) copy_tile(k, 0);
   cp_async_commit();
   for (int b = 0; k < p.ntiles; k += gridDim.x, b ^= 1) {
@@ -763,9 +765,11 @@ __global__ void __launch_bounds__(tiles_per_cta<PL>() * tile_threads<PL>())
     float2* tw = reinterpret_cast<float2*>(sm4);
     for (int i = threadIdx.x; i < tw_table_size<PL>(); i += blockDim.x) tw[i] = p.tw[i];
     __syncthreads();
+    chain_begin();
     axis_tile<PL, INV, AXIS, THREADS>(p, blockIdx.x, TwShared{tw},
                                       tw + tw_table_size<PL>());
   } else {
+    chain_begin();
     axis_tile<PL, INV, AXIS, THREADS>(p, blockIdx.x, TwGlobal{p.tw}, reinterpret_cast<float2*>(sm4));
   }
 }
@@ -779,11 +783,13 @@ __global__ void __launch_bounds__(tiles_per_cta<PL>() * tile_threads<PL>(), tpro
     float2* tw = reinterpret_cast<float2*>(sm4);
     for (int i = threadIdx.x; i < tw_table_size<PL>(); i += blockDim.x) tw[i] = p.tw[i];
     __syncthreads();
+    chain_begin();
     // tiles from the last down: the pass ends on the first field's low-y
     // pencils, which the y-inverse then reads first
     tprop_tile<PL, THREADS>(p, (long long)gridDim.x - 1 - blockIdx.x, TwShared{tw},
                             tw + tw_table_size<PL>());
   } else {
+    chain_begin();
     tprop_tile<PL, THREADS>(p, blockIdx.x, TwGlobal{p.tw}, reinterpret_cast<float2*>(sm4));
   }
 }

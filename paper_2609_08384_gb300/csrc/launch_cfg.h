@@ -56,4 +56,27 @@ inline cudaError_t raise_smem_limit_to(K kernel, size_t smem, SmemMax& rec) {
   return e;
 }
 
+// Launch of a kernel of the z-step's chain: the grid may start while the one
+// before it on the stream drains (programmatic dependent launch), so its launch
+// and prologue overlap the other's last CTAs.  Only for kernels that call
+// chain_begin() before they touch what earlier kernels wrote; any other kernel,
+// copy or event on the stream waits for the whole grid as ever.  Time per z-step
+// without and with it: 18.5 -> 10.3 us (2 x 32x32x64), 31.0 -> 20.8 (2 x 64x64x128),
+// 82 -> 72 (2 x 96x96x192), 57.7 -> 48.8 (2 x 1024x1024x1), 166 -> 156
+// (3 x 128x128x256), 1316 -> 1306 (3 x 256x256x512).
+template <class... P, class... A>
+inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s, A&&... args) {
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = grid;
+  c.blockDim = dim3((unsigned)threads);
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  c.attrs = &attr;
+  c.numAttrs = 1;
+  return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+}
+
 }  // namespace brahms

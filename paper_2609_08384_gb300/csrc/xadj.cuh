@@ -106,7 +106,7 @@ __device__ __forceinline__ void xpass_adj_tile(const XAdjArgs& p, long long tile
       }
       if constexpr (MAP) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) nm[q] = __ldg(emap + q * nxy + p0);
+        for (int q = 0; q < 4; ++q) nm[q] = __ldcg(emap + q * nxy + p0);
       }
     }
 #pragma unroll 1
@@ -133,7 +133,7 @@ __device__ __forceinline__ void xpass_adj_tile(const XAdjArgs& p, long long tile
         }
         if constexpr (MAP) {
 #pragma unroll
-          for (int q = 0; q < 4; ++q) nm[q] = __ldg(emap + q * nxy + pn);
+          for (int q = 0; q < 4; ++q) nm[q] = __ldcg(emap + q * nxy + pn);
         }
       }
 #pragma unroll
@@ -210,6 +210,7 @@ __global__ void __launch_bounds__(xpass_threads<NX>(), xpass_threads<NX>() <= 12
     }
   }
   __syncthreads();
+  chain_begin();
   float sens[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
   xpass_adj_tile<NX, F, THREADS, MAP>(p, blockIdx.x, cA, cB, rowbuf, sens);
   // block sums in FP64, fixed order (deterministic)
@@ -240,8 +241,7 @@ cudaError_t launch_adjoint(const XAdjArgs& a, long long* ncta, cudaStream_t s) {
   const long long grid = (a.rows + ROWS - 1) / ROWS;
   *ncta = grid;
   if (grid <= 0) return cudaSuccess;
-  xpass_adj_kernel<NX, F, MAP><<<(unsigned)grid, THREADS, smem, s>>>(a);
-  return cudaPeekAtLastError();
+  return launch_chained(xpass_adj_kernel<NX, F, MAP>, dim3((unsigned)grid), THREADS, smem, s, a);
 }
 
 

@@ -20,8 +20,7 @@ cudaError_t launch_record(const XPassArgs& a0, cudaStream_t s) {
   if (e != cudaSuccess) return e;
   const long long grid = (a.rows + ROWS - 1) / ROWS;
   if (grid <= 0) return cudaSuccess;
-  xpass_kernel<NX, F, MAP, true><<<(unsigned)grid, THREADS, smem, s>>>(a);
-  return cudaPeekAtLastError();
+  return launch_chained(xpass_kernel<NX, F, MAP, true>, dim3((unsigned)grid), THREADS, smem, s, a);
 }
 
 }  // namespace brahms
