@@ -104,7 +104,6 @@ brahms_status brahms_init_grid(brahms_ctx** out, int nx, int ny, int nt, double 
   ctx->twy = (float2*)(ctx->ws + ctx->L.twy);
   ctx->twt = (float2*)(ctx->ws + ctx->L.twt);
   ctx->partial = (double*)(ctx->ws + ctx->L.partial);
-  ctx->energy_dev = (double*)(ctx->ws + ctx->L.energy);
   ctx->dev_err = (int*)(ctx->ws + ctx->L.err);
   ctx->diag_dev = (double*)(ctx->ws + ctx->L.diag);
   ctx->ws_map = (double*)(ctx->ws + ctx->L.dkmap);
@@ -117,7 +116,7 @@ brahms_status brahms_init_grid(brahms_ctx** out, int nx, int ny, int nt, double 
   if (e == cudaSuccess) e = brahms::upload_twiddles(ctx->twx, nx, ctx->stream);
   if (e == cudaSuccess && ny > 1) e = brahms::upload_twiddles(ctx->twy, ny, ctx->stream);
   if (e == cudaSuccess && nt > 1) e = brahms::upload_twiddles(ctx->twt, nt, ctx->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(ctx->dev_err, 0, sizeof(int), ctx->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(ctx->dev_err, 0, 2 * sizeof(int), ctx->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(ctx->mphase_dev, 0, sizeof(double) * nx * ny, ctx->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
   if (e != cudaSuccess) {
@@ -158,7 +157,8 @@ brahms_status brahms_set_fields(brahms_ctx* ctx, const void* const* fields, int 
   for (int f = 0; f < ctx->nf; ++f)
     if (!fields[f]) return fail(ctx, BRAHMS_E_ARG, "a field pointer is NULL");
   std::vector<float2> stage;
-  for (int f = 0; f < ctx->nf; ++f) {
+  const bool fused = dtype == BRAHMS_C64 && on_device && kernel_can_copy(ctx, fields, false);
+  for (int f = 0; f < ctx->nf && !fused; ++f) {
     float2* dst = ctx->state + f * n;
     if (dtype == BRAHMS_C64) {
       BR_CK(cudaMemcpyAsync(dst, fields[f], sizeof(float2) * n,
@@ -182,7 +182,7 @@ brahms_status brahms_set_fields(brahms_ctx* ctx, const void* const* fields, int 
   }
   ctx->have_fields = true;
   touch(ctx);
-  brahms_status s = finish_with_check(ctx);
+  brahms_status s = finish_with_check(ctx, fused ? fields : nullptr);
   if (s == BRAHMS_E_NONFINITE) {
     ctx->have_fields = false;
     return fail(ctx, BRAHMS_E_ARG, "input fields contain non-finite values");
@@ -269,7 +269,8 @@ brahms_status brahms_get_fields(brahms_ctx* ctx, void* const* out, int dtype, in
     if (!out[f]) return fail(ctx, BRAHMS_E_ARG, "an output pointer is NULL");
   const long long n = ctx->npoints();
   std::vector<float2> stage;
-  for (int f = 0; f < ctx->nf; ++f) {
+  const bool fused = dtype == BRAHMS_C64 && on_device && kernel_can_copy(ctx, out, true);
+  for (int f = 0; f < ctx->nf && !fused; ++f) {
     const float2* src = ctx->state + f * n;
     if (dtype == BRAHMS_C64) {
       BR_CK(cudaMemcpyAsync(out[f], src, sizeof(float2) * n,
@@ -287,7 +288,7 @@ brahms_status brahms_get_fields(brahms_ctx* ctx, void* const* out, int dtype, in
       }
     }
   }
-  return finish_with_check(ctx);
+  return finish_with_check(ctx, nullptr, fused ? out : nullptr);
 }
 
 brahms_status brahms_energy(brahms_ctx* ctx, double* energy_j, double* photons) {

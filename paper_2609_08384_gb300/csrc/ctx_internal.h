@@ -26,7 +26,7 @@ constexpr int kMaxMapSegments = 4096;  // z-segments of a mismatch map
 inline size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
 
 struct Layout {
-  size_t state, px, py, pt, twx, twy, twt, partial, energy, err, diag, dkmap, usermap, mphase, emap, total;
+  size_t state, px, py, pt, twx, twy, twt, partial, err, diag, dkmap, usermap, mphase, emap, total;
 };
 
 inline Layout make_layout(int nx, int ny, int nt, int nf) {
@@ -46,8 +46,7 @@ inline Layout make_layout(int nx, int ny, int nt, int nf) {
   L.twy = take(sizeof(float2) * brahms::tw_table_size_of(ny));
   L.twt = take(sizeof(float2) * brahms::tw_table_size_of(nt));
   L.partial = take(sizeof(double) * kRedBlocks * nf);
-  L.energy = take(sizeof(double) * nf);
-  L.err = take(sizeof(int));
+  L.err = take(2 * sizeof(int));
   L.diag = take(sizeof(double) * 2 * nt * nf);
   L.dkmap = take(sizeof(double) * nx * ny);
   L.usermap = take(sizeof(double) * nx * ny);
@@ -76,7 +75,7 @@ struct brahms_ctx {
   Layout L{};
   float2 *state = nullptr, *px = nullptr, *py = nullptr, *pt = nullptr;
   float2 *twx = nullptr, *twy = nullptr, *twt = nullptr;
-  double *partial = nullptr, *energy_dev = nullptr;
+  double* partial = nullptr;
   double* energy_host = nullptr;  // pinned, nf entries + the device error word
   double* diag_dev = nullptr;     // diagnostics: power [nf][nt], spectrum [nf][nt]
   // Transverse mismatch maps, one per z-segment (nseg segments separated by
@@ -98,7 +97,7 @@ struct brahms_ctx {
   bool have_map = false;          // the x-pass takes the map path
   bool have_user_map = false;
   bool have_therm = false;        // a thermal map is installed
-  int* dev_err = nullptr;          // set by kernels whose bounded waits expired
+  int* dev_err = nullptr;          // set by kernels whose bounded waits expired; behind it the energy kernel's block count
   unsigned long long tma_wait_ns = 2000000000ULL;  // limit of each TMA tile wait (BRAHMS_OPT_TMA_WAIT_US)
   alignas(64) unsigned char tmap_state[128];  // TMA map of the state for the tau-pass
   int use_tma = 0;  // 0 plain tau-pass; 16 or 8: TMA tau-pass with tiles of that many columns
@@ -438,22 +437,56 @@ inline double dk_of_step(const brahms_ctx* c, long long j) {
   return j < (long long)c->dk_profile.size() ? c->dk_profile[(size_t)j] : c->dk;
 }
 
-// Enqueue an FP64 |A|^2 reduction per field into energy_host (pinned).
-inline brahms_status enqueue_energy(brahms_ctx* ctx) {
-  BR_CK(launch(ctx, 4, 2, [&] {
-    return brahms::run_energy(ctx->state, ctx->npoints(), ctx->nf, ctx->npoints(), ctx->partial, kRedBlocks,
-                              ctx->energy_dev, ctx->stream);
-  }));
-  BR_CK(cudaMemcpyAsync(ctx->energy_host, ctx->energy_dev, sizeof(double) * ctx->nf, cudaMemcpyDeviceToHost,
-                        ctx->stream));
+// Whether a kernel of the current device can bring the fields in from a caller's
+// buffers, or hand them out to them, as 16-byte pairs: device memory of this
+// device, aligned, apart from the workspace and, when written, from each other.
+// Otherwise the driver's copies move the fields one after another.
+inline bool kernel_can_copy(const brahms_ctx* ctx, const void* const* ptrs, bool written) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  const uintptr_t bytes = sizeof(float2) * (uintptr_t)ctx->npoints();
+  const uintptr_t ws0 = (uintptr_t)ctx->ws, ws1 = ws0 + ctx->L.total;
+  for (int f = 0; f < ctx->nf; ++f) {
+    const uintptr_t p = (uintptr_t)ptrs[f];
+    if ((p & 15) != 0 || (p < ws1 && ws0 < p + bytes)) return false;
+    for (int g = 0; written && g < f; ++g) {
+      const uintptr_t q = (uintptr_t)ptrs[g];
+      if (p < q + bytes && q < p + bytes) return false;
+    }
+    cudaPointerAttributes at{};
+    if (cudaPointerGetAttributes(&at, ptrs[f]) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    if (at.type != cudaMemoryTypeDevice || at.device != dev) return false;
+  }
+  return true;
+}
+
+// Enqueue an FP64 |A|^2 reduction per field into energy_host (pinned); from or to
+// not NULL: the fields are brought in from there, or handed out to there, on the
+// way (806 MB both ways and their check: 240 us for the copy and 125 for the check
+// as separate passes, 245 together).
+inline brahms_status enqueue_energy(brahms_ctx* ctx, const void* const* from = nullptr, void* const* to = nullptr) {
+  brahms::EnergyArgs a{};
+  for (int f = 0; f < ctx->nf; ++f) {
+    float2* field = ctx->state + f * ctx->npoints();
+    a.src[f] = from ? (const float2*)from[f] : field;
+    a.dst[f] = from ? field : to ? (float2*)to[f] : nullptr;
+  }
+  a.n = ctx->npoints();
+  a.partial = ctx->partial;
+  a.host = ctx->energy_host;
+  a.count = reinterpret_cast<unsigned int*>(ctx->dev_err) + 1;
+  a.err = ctx->dev_err;
+  BR_CK(launch(ctx, 4, 1, [&] { return brahms::run_energy(a, ctx->nf, kRedBlocks, ctx->stream); }));
   return BRAHMS_OK;
 }
 
-inline brahms_status finish_with_check(brahms_ctx* ctx) {
-  brahms_status s = enqueue_energy(ctx);
+inline brahms_status finish_with_check(brahms_ctx* ctx, const void* const* from = nullptr, void* const* to = nullptr) {
+  brahms_status s = enqueue_energy(ctx, from, to);
   if (s != BRAHMS_OK) return s;
-  int* herr = reinterpret_cast<int*>(ctx->energy_host + 3);
-  BR_CK(cudaMemcpyAsync(herr, ctx->dev_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+  const int* herr = reinterpret_cast<const int*>(ctx->energy_host + 3);
   BR_CK(cudaStreamSynchronize(ctx->stream));
   if (*herr != 0) {
     BR_CK(cudaMemsetAsync(ctx->dev_err, 0, sizeof(int), ctx->stream));

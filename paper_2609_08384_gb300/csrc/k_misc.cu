@@ -143,19 +143,29 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-__global__ void __launch_bounds__(256) energy_partial_kernel(const float2* __restrict__ data, long long n,
-                                                             long long fstride, double* partial) {
-  const float2* a = data + blockIdx.y * fstride;
+// COPY: the fields read are also written to dst, so that a field brought in or
+// handed out is read once for both.  The last block to finish adds the partial
+// sums in their fixed order and writes the sums and the device error word to
+// the pinned host words as well, so a check is one launch and no copies.
+template <bool COPY>
+__global__ void __launch_bounds__(256) energy_kernel(const EnergyArgs p) {
+  const float4* a4 = reinterpret_cast<const float4*>(p.src[blockIdx.y]);
+  float4* d4 = reinterpret_cast<float4*>(p.dst[blockIdx.y]);
   double s = 0.0;
-  // pairs (every length is even, so a field starts on a 16-byte boundary)
-  const float4* a4 = reinterpret_cast<const float4*>(a);
-  const long long n2 = n / 2;
+  // pairs (every length is even, so a field holds whole 16-byte pairs)
+  const long long n2 = p.n / 2;
   const long long stride = (long long)gridDim.x * blockDim.x;
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   // four independent pairs per round: the loads overlap, one FP64 add per eight points
   for (; i + 3 * stride < n2; i += 4 * stride) {
     const float4 v0 = __ldcg(a4 + i), v1 = __ldcg(a4 + i + stride), v2 = __ldcg(a4 + i + 2 * stride),
                  v3 = __ldcg(a4 + i + 3 * stride);
+    if constexpr (COPY) {
+      d4[i] = v0;
+      d4[i + stride] = v1;
+      d4[i + 2 * stride] = v2;
+      d4[i + 3 * stride] = v3;
+    }
     const float q0 = fmaf(v0.x, v0.x, fmaf(v0.y, v0.y, fmaf(v0.z, v0.z, v0.w * v0.w)));
     const float q1 = fmaf(v1.x, v1.x, fmaf(v1.y, v1.y, fmaf(v1.z, v1.z, v1.w * v1.w)));
     const float q2 = fmaf(v2.x, v2.x, fmaf(v2.y, v2.y, fmaf(v2.z, v2.z, v2.w * v2.w)));
@@ -164,43 +174,41 @@ __global__ void __launch_bounds__(256) energy_partial_kernel(const float2* __res
   }
   for (; i < n2; i += stride) {
     const float4 v = __ldcg(a4 + i);
+    if constexpr (COPY) d4[i] = v;
     s += (double)fmaf(v.x, v.x, fmaf(v.y, v.y, fmaf(v.z, v.z, v.w * v.w)));
   }
-  if (n & 1) {  // odd length (not produced by the supported grids): the last point
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-      const float2 v = a[n - 1];
-      s += (double)fmaf(v.x, v.x, v.y * v.y);
-    }
-  }
   __shared__ double red[8];
-  s = warp_sum(s);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double v = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.0;
+  __shared__ bool last;
+  const auto block_sum = [&](double v) {
     v = warp_sum(v);
-    if (threadIdx.x == 0) partial[blockIdx.y * gridDim.x + blockIdx.x] = v;
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    __syncthreads();
+    v = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.0;
+    return threadIdx.x < 32 ? warp_sum(v) : 0.0;
+  };
+  s = block_sum(s);
+  if (threadIdx.x == 0) {
+    p.partial[blockIdx.y * gridDim.x + blockIdx.x] = s;
+    __threadfence();
+    // wraps to zero for the next launch
+    last = atomicInc(p.count, gridDim.x * gridDim.y - 1) == gridDim.x * gridDim.y - 1;
   }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  for (int f = 0; f < (int)gridDim.y; ++f) {
+    double v = 0.0;
+    for (int k = threadIdx.x; k < (int)gridDim.x; k += blockDim.x) v += __ldcg(p.partial + f * gridDim.x + k);
+    v = block_sum(v);
+    if (threadIdx.x == 0) p.host[f] = v;
+  }
+  if (threadIdx.x == 0) *reinterpret_cast<int*>(p.host + 3) = *p.err;
 }
 
-__global__ void __launch_bounds__(256) energy_final_kernel(const double* partial, int nblocks, double* out) {
-  double s = 0.0;
-  for (int i = threadIdx.x; i < nblocks; i += blockDim.x) s += partial[blockIdx.x * nblocks + i];
-  __shared__ double red[8];
-  s = warp_sum(s);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double v = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.0;
-    v = warp_sum(v);
-    if (threadIdx.x == 0) out[blockIdx.x] = v;
-  }
-}
-
-cudaError_t run_energy(const float2* data, long long n, int nf, long long fstride, double* partial,
-                       int nblocks, double* out, cudaStream_t s) {
-  energy_partial_kernel<<<dim3(nblocks, nf), 256, 0, s>>>(data, n, fstride, partial);
-  energy_final_kernel<<<nf, 256, 0, s>>>(partial, nblocks, out);
+cudaError_t run_energy(const EnergyArgs& a, int nf, int nblocks, cudaStream_t s) {
+  if (a.dst[0]) energy_kernel<true><<<dim3(nblocks, nf), 256, 0, s>>>(a);
+  else energy_kernel<false><<<dim3(nblocks, nf), 256, 0, s>>>(a);
   return cudaPeekAtLastError();
 }
 

@@ -897,8 +897,20 @@ struct ThermalArgs {
   int* bad;       // set if a temperature is not finite
 };
 cudaError_t run_thermal_solve(const ThermalArgs& a, int* nlaunch, cudaStream_t s);
-cudaError_t run_energy(const float2* data, long long n, int nf, long long fstride, double* partial,
-                       int nblocks, double* out, cudaStream_t s);
+// Per-field sums of |A|^2 over n points (even) of src[f], 16-byte aligned, into
+// host[f] (pinned), with the device error word in host[3]; dst[f] not NULL: the
+// field is copied there too.  partial: nf x nblocks; *count is zero before the
+// first launch and after every one.
+struct EnergyArgs {
+  const float2* src[3];
+  float2* dst[3];
+  long long n;
+  double* partial;
+  double* host;
+  unsigned int* count;
+  const int* err;
+};
+cudaError_t run_energy(const EnergyArgs& a, int nf, int nblocks, cudaStream_t s);
 cudaError_t run_c128_to_c64(const double2* in, float2* out, long long n, cudaStream_t s);
 cudaError_t run_c64_to_c128(const float2* in, double2* out, long long n, cudaStream_t s);
 
