@@ -34,9 +34,9 @@
 // not each other's mirror let the energy of the 3 x 256x256x512 parametric run
 // fall by 7e-9 per step.)  |phi| <= 1/4 turn, or a little more in plans of three
 // and four passes, keeps p near 1 or below.
-// Error against FP64 of 3D transforms of random fields: forward 1.51e-7 (with
-// hi + lo twiddles 1.48e-7), forward and inverse 2.11e-7 (2.10e-7); energy of
-// smooth beams over 100 z-steps: rms 1.8e-9 to 2.6e-9 per step (1.7e-9 to 5.6e-9).
+// Error against FP64 of 3D transforms of random fields: forward 1.6e-7 (with
+// hi + lo twiddles 1.5e-7), forward and inverse 2.11e-7 (2.10e-7); energy of
+// smooth beams over 100 z-steps: rms 1.6e-9 to 2.6e-9 per step (1.7e-9 to 5.6e-9).
 //
 // Packed arithmetic.  A complex value is an aligned register pair, and sums of
 // complex values are single add/sub.f32x2 instructions.  One FFMA2 occupies the
@@ -136,9 +136,13 @@ __device__ __forceinline__ float2 w32_shear(float2 a) {
       constexpr float ch = (float)sin_pi16(4), cl = (float)(sin_pi16(4) - (double)ch);
       return __ffma2_rn(d, make_float2(ch, ch), __fmul2_rn(d, make_float2(cl, cl)));
     } else {
-      constexpr float p = (float)(pos ? -tan_pi32(ak) : tan_pi32(ak));
-      constexpr float s = (float)(pos ? sin_pi16(ak) : -sin_pi16(ak));
-      return shear_turn(a, p, s);
+      // one sixteenth of a turn: p one float off tan(pi/16) makes the pair of
+      // floats eight times nearer to orthogonal (7e-10 against 6e-9) for an angle
+      // 6e-8 off, which the way back undoes: energy of the 1000-step parametric
+      // run +2.3e-7 instead of -7.4e-7
+      constexpr float pk = ak == 2 ? 0.198912397f : (float)tan_pi32(ak);
+      constexpr float sk = ak == 2 ? 0.382683486f : (float)sin_pi16(ak);
+      return shear_turn(a, pos ? -pk : pk, pos ? sk : -sk);
     }
   }
 }
@@ -460,6 +464,25 @@ struct SyncBlock {
 };
 struct SyncWarp {
   __device__ __forceinline__ static void sync() { __syncwarp(); }
+};
+// the T threads of one row inside a warp (T a power of two)
+template <int T>
+struct SyncRow {
+  __device__ __forceinline__ static void sync() {
+    if constexpr (T == 32) __syncwarp();
+    else if constexpr (T > 1) __syncwarp(((1u << T) - 1u) << (threadIdx.x & 31 & ~(T - 1)));
+  }
+};
+// an exchange that only active threads take part in (all keep the barriers)
+template <class X>
+struct XchGuard {
+  static constexpr bool kSplit = X::kSplit;
+  X x;
+  bool act;
+  __device__ __forceinline__ void st(int pos, float2 v) const {
+    if (act) x.st(pos, v);
+  }
+  __device__ __forceinline__ float2 ld(int pos) const { return act ? x.ld(pos) : make_float2(0.f, 0.f); }
 };
 
 // Passes P..NP-1 of a length-N transform on the registers v (see header).
