@@ -214,13 +214,17 @@ brahms_status brahms_propagate(brahms_ctx* ctx, int nz, double dz) {
   double phi = ctx->phi;  // Phi(z_j) of the current step j
   long long j = ctx->step;
   const double z0 = ctx->z;
+  const bool plane = use_plane_pass(ctx);
   {
     brahms::XPassArgs a = xargs(ctx, brahms::XM_NL_FIRST, dz);
     a.phiA = phi;
     a.dkA = dk_of_step(ctx, j);
     s = enqueue_map_tables(ctx, 0.0, 0.0, z0, a.phiA, a.dkA, z0, dz);
     if (s != BRAHMS_OK) return s;
-    BR_CK(launch(ctx, 0, 1, [&] { return brahms::run_xpass(nx, nf, a, ctx->stream); }));
+    if (plane)
+      BR_CK(launch(ctx, 0, 1, [&] { return brahms::run_plane(nx, ny, nf, a, ctx->twy, ctx->stream); }));
+    else
+      BR_CK(launch(ctx, 0, 1, [&] { return brahms::run_xpass(nx, nf, a, ctx->stream); }));
   }
   // per-field streams for the y/tau/y passes only when the option asks for
   // them (off by default: a gain on 128x128x256 with three fields only)
@@ -231,7 +235,8 @@ brahms_status brahms_propagate(brahms_ctx* ctx, int nz, double dz) {
       s = enqueue_linear_split(ctx, ay, at);
       if (s != BRAHMS_OK) return s;
     } else {
-      if (ny > 1) BR_CK(launch(ctx, 1, 1, [&] { return brahms::run_axis_fft(ny, 1, false, ay, ctx->stream); }));
+      if (ny > 1 && !plane)
+        BR_CK(launch(ctx, 1, 1, [&] { return brahms::run_axis_fft(ny, 1, false, ay, ctx->stream); }));
       if (nt == 1)
         BR_CK(launch(ctx, 2, 1, [&] { return brahms::run_prop_pointwise(at, nf, ctx->stream); }));
       else if (ctx->use_tma)
@@ -241,7 +246,8 @@ brahms_status brahms_propagate(brahms_ctx* ctx, int nz, double dz) {
         }));
       else
         BR_CK(launch(ctx, 2, 1, [&] { return brahms::run_tpass_prop(nt, at, ctx->stream); }));
-      if (ny > 1) BR_CK(launch(ctx, 3, 1, [&] { return brahms::run_axis_fft(ny, 1, true, ay, ctx->stream); }));
+      if (ny > 1 && !plane)
+        BR_CK(launch(ctx, 3, 1, [&] { return brahms::run_axis_fft(ny, 1, true, ay, ctx->stream); }));
     }
     const bool last = (i == nz - 1);
     brahms::XPassArgs a = xargs(ctx, last ? brahms::XM_NL_LAST : brahms::XM_NL_MID, dz);
@@ -252,7 +258,10 @@ brahms_status brahms_propagate(brahms_ctx* ctx, int nz, double dz) {
     a.dkA = dk_of_step(ctx, j + 1);
     s = enqueue_map_tables(ctx, a.phiB, a.dkB, z0 + i * dz, a.phiA, a.dkA, z0 + (i + 1) * dz, dz);
     if (s != BRAHMS_OK) return s;
-    BR_CK(launch(ctx, 0, 1, [&] { return brahms::run_xpass(nx, nf, a, ctx->stream); }));
+    if (plane)
+      BR_CK(launch(ctx, 0, 1, [&] { return brahms::run_plane(nx, ny, nf, a, ctx->twy, ctx->stream); }));
+    else
+      BR_CK(launch(ctx, 0, 1, [&] { return brahms::run_xpass(nx, nf, a, ctx->stream); }));
   }
   ctx->phi = phi;
   ctx->step = j;

@@ -677,6 +677,8 @@ brahms_status prepare_grouped(brahms_batch* b) {
     XPassArgs x{};
     BB_CK(run_xpass_group(g.nx, x, g.params, g.ecoef, kStageFactors, 0, 0, b->stream));
     BB_CK(run_xpass(g.nx, 2, x, b->stream));
+    if (plane_supported(g.nx, g.ny))
+      BB_CK(run_plane_group(g.nx, g.ny, x, g.twy, g.params, g.ecoef, kStageFactors, 0, 0, b->stream));
   }
   cudaStream_t cap = nullptr;
   BB_CK(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
@@ -705,9 +707,13 @@ brahms_status prepare_grouped(brahms_batch* b) {
     base.tw = g.twx;
     base.scale = 1.f;
     base.ny = g.ny;
-    // an x-pass over the first a slots (per instance where an instance's rows
-    // do not fill whole CTAs)
+    // an x-pass over the first a slots (the plane pass, which takes the y-passes
+    // with it, where the plane has one; per instance where an instance's rows do
+    // not fill whole CTAs)
+    const bool plane = plane_supported(g.nx, g.ny);
     auto xpass = [&](int step, int a) -> cudaError_t {
+      if (plane)
+        return run_plane_group(g.nx, g.ny, base, g.twy, g.params, g.ecoef, (g.ecoef_steps + 1) * kStageFactors, step, a, s);
       if (whole) return run_xpass_group(g.nx, base, g.params, g.ecoef, (g.ecoef_steps + 1) * kStageFactors, step, a, s);
       for (int slot = 0; slot < a; ++slot) {
         const BatchInstHost& I = b->inst[g.members[slot]];
@@ -757,17 +763,17 @@ brahms_status prepare_grouped(brahms_batch* b) {
     at.scale = (float)inv_n;
     at.scale_lo = (float)(inv_n - (double)at.scale);
     if (e == cudaSuccess) e = xpass(-1, m);
-    nl += whole ? 1 : m;
+    nl += plane || whole ? 1 : m;
     int a = m;
     for (int j = 0; j < nz_max && e == cudaSuccess; ++j) {
       while (a > 0 && nzs[a - 1] <= j) --a;  // slots still running at step j
       ay.ntiles = 2LL * a * g.nt * ay.xtiles;
       at.ntiles = 2LL * a * g.ny * at.xtiles;
-      e = run_axis_fft(g.ny, 1, false, ay, s);
+      if (!plane) e = run_axis_fft(g.ny, 1, false, ay, s);
       if (e == cudaSuccess) e = run_tpass_prop(g.nt, at, s);
-      if (e == cudaSuccess) e = run_axis_fft(g.ny, 1, true, ay, s);
+      if (e == cudaSuccess && !plane) e = run_axis_fft(g.ny, 1, true, ay, s);
       if (e == cudaSuccess) e = xpass(j, a);
-      nl += 3 + (whole ? 1 : a);
+      nl += (plane ? 1 : 3) + (plane || whole ? 1 : a);
     }
     if (e == cudaSuccess) e = cudaEventRecord(g.done, s);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(cap, g.done, 0);

@@ -387,6 +387,12 @@ inline bool use_field_streams(const brahms_ctx* c) {
   return c->field_streams == 1 && c->ny > 1 && c->nt > 1 && !c->use_tma;
 }
 
+// The plane pass (one kernel for y-inverse, x-pass and y-forward) where the
+// plane has one; not under a map.
+inline bool use_plane_pass(const brahms_ctx* c) {
+  return brahms::plane_supported(c->nx, c->ny) && !c->have_map && !use_field_streams(c);
+}
+
 // streams and events of the per-field chains, created on first use
 inline brahms_status field_streams_ready(brahms_ctx* ctx) {
   if (ctx->ev_x) return BRAHMS_OK;

@@ -817,7 +817,16 @@ struct GroupInst {
 // ecoef[i stride + (j + 1) kStageFactors + 0..]
 cudaError_t run_xpass_group(int nx, const XPassArgs& base, const GroupInst* gi, const float2* ecoef, int stride,
                             int step, int ninst, cudaStream_t s);
+// the same pass of the grouped form on ninst instances (k_planegroup.cu)
+cudaError_t run_plane_group(int nx, int ny, const XPassArgs& base, const float2* twy, const GroupInst* gi,
+                            const float2* ecoef, int stride, int step, int ninst, cudaStream_t s);
 int xpass_rows_of(int nx);  // rows per CTA of the x-pass of length nx
+
+// plane pass (k_plane.cu): y-inverse, x-pass and y-forward of a step in one
+// kernel, for the (nx, ny) below; a.mode NL_FIRST, NL_MID or NL_LAST, no map
+bool plane_supported(int nx, int ny);
+cudaError_t run_plane(int nx, int ny, int nf, const XPassArgs& a, const float2* twy, cudaStream_t s);
+cudaError_t run_plane3(int nx, int ny, const XPassArgs& a, const float2* twy, cudaStream_t s);
 
 // misc kernels (k_misc.cu)
 // TMA tau-pass (k_tma.cu)
@@ -963,3 +972,18 @@ cudaError_t run_phase_tables(float2* px, int nx, float2* py, int ny, float2* pt,
 #define BRAHMS_FOR_EACH_SIZE(X) \
   X(2) X(4) X(8) X(16) X(32) X(64) X(128) X(256) X(512) X(1024) X(2048) X(4096) \
   X(6) X(12) X(24) X(48) X(96) X(192) X(384) X(768)
+
+// Planes with a plane-pass kernel: 24 to 64 by 8 to 64 points and 16 by 8 to 64, up
+// to 1536 points.  A larger plane keeps one CTA busy for longer than the three
+// passes take over the whole GPU: time per z-step of the plane pass with the
+// tau-pass against the four passes, two fields, 64 / 512 planes: 32x32 7.3 against
+// 10.5 us / 17.7 against 22.4, 24x64 11.0 against 13.2 / 30.6 against 34.1, 48x48
+// 14.6 against 14.4 / 48.0 against 47.0, 64x64 17.2 against 14.0 / 56.9 against 55.7,
+// 96x96 45.5 against 29.2 / 197 against 161 (three fields 32x32: 9.9 against 11.8 /
+// 26.3 against 29.1).
+#define BRAHMS_FOR_EACH_PLANE(X)                                        \
+  X(16, 8) X(16, 12) X(16, 16) X(16, 24) X(16, 32) X(16, 48) X(16, 64)  \
+  X(24, 8) X(24, 12) X(24, 16) X(24, 24) X(24, 32) X(24, 48) X(24, 64)  \
+  X(32, 8) X(32, 12) X(32, 16) X(32, 24) X(32, 32) X(32, 48)            \
+  X(48, 8) X(48, 12) X(48, 16) X(48, 24) X(48, 32)                      \
+  X(64, 8) X(64, 12) X(64, 16) X(64, 24)
