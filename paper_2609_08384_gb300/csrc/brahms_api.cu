@@ -214,7 +214,9 @@ brahms_status brahms_propagate(brahms_ctx* ctx, int nz, double dz) {
   double phi = ctx->phi;  // Phi(z_j) of the current step j
   long long j = ctx->step;
   const double z0 = ctx->z;
-  const bool plane = use_plane_pass(ctx);
+  const bool cw = nt == 1 && ny > 1;  // the linear step is one pass along y
+  const brahms::AxisArgs acw = cw ? cw_args(ctx) : brahms::AxisArgs{};
+  const bool plane = !cw && use_plane_pass(ctx);
   {
     brahms::XPassArgs a = xargs(ctx, brahms::XM_NL_FIRST, dz);
     a.phiA = phi;
@@ -235,9 +237,11 @@ brahms_status brahms_propagate(brahms_ctx* ctx, int nz, double dz) {
       s = enqueue_linear_split(ctx, ay, at);
       if (s != BRAHMS_OK) return s;
     } else {
-      if (ny > 1 && !plane)
+      if (ny > 1 && !plane && !cw)
         BR_CK(launch(ctx, 1, 1, [&] { return brahms::run_axis_fft(ny, 1, false, ay, ctx->stream); }));
-      if (nt == 1)
+      if (cw)
+        BR_CK(launch(ctx, 2, 1, [&] { return brahms::run_tpass_prop(ny, acw, ctx->stream); }));
+      else if (nt == 1)
         BR_CK(launch(ctx, 2, 1, [&] { return brahms::run_prop_pointwise(at, nf, ctx->stream); }));
       else if (ctx->use_tma)
         BR_CK(launch(ctx, 2, 1, [&] {
@@ -246,7 +250,7 @@ brahms_status brahms_propagate(brahms_ctx* ctx, int nz, double dz) {
         }));
       else
         BR_CK(launch(ctx, 2, 1, [&] { return brahms::run_tpass_prop(nt, at, ctx->stream); }));
-      if (ny > 1 && !plane)
+      if (ny > 1 && !plane && !cw)
         BR_CK(launch(ctx, 3, 1, [&] { return brahms::run_axis_fft(ny, 1, true, ay, ctx->stream); }));
     }
     const bool last = (i == nz - 1);
