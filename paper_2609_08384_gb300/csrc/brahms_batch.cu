@@ -40,6 +40,7 @@
 
 #include "alloc_hook.h"
 #include "brahms.h"
+#include "device_buffers.h"
 #include "kernels.cuh"
 
 namespace brahms {
@@ -577,9 +578,9 @@ brahms_status layout(brahms_batch* b) {
     };
     const size_t o_state = take(sizeof(float2) * 2 * n * m), o_px = take(sizeof(float2) * 2 * m * g.nx),
                  o_py = take(sizeof(float2) * 2 * m * g.ny), o_pt = take(sizeof(float2) * 2 * m * g.nt),
-                 o_twx = take(sizeof(float2) * tw_table_size_of(g.nx)),
-                 o_twy = take(sizeof(float2) * tw_table_size_of(g.ny)),
-                 o_twt = take(sizeof(float2) * tw_table_size_of(g.nt)), o_par = take(sizeof(GroupInst) * m);
+                 o_twx = take(sizeof(float2) * tw_table_size_of(g.nx, true)),
+                 o_twy = take(sizeof(float2) * tw_table_size_of(g.ny, false)),
+                 o_twt = take(sizeof(float2) * tw_table_size_of(g.nt, false)), o_par = take(sizeof(GroupInst) * m);
     g.ecoef_steps = 0;
     for (int i : g.members) g.ecoef_steps = std::max(g.ecoef_steps, b->inst[i].nz);
     const size_t o_coef = take(sizeof(float2) * kStageFactors * (size_t)(g.ecoef_steps + 1) * m);
@@ -599,9 +600,9 @@ brahms_status layout(brahms_batch* b) {
     if (cudaStreamCreateWithFlags(&g.stream, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&g.done, cudaEventDisableTiming) != cudaSuccess)
       return release(bfail(b, BRAHMS_E_CUDA, "group stream"));
-    cudaError_t e = upload_twiddles(g.twx, g.nx, b->stream);
-    if (e == cudaSuccess) e = upload_twiddles(g.twy, g.ny, b->stream);
-    if (e == cudaSuccess) e = upload_twiddles(g.twt, g.nt, b->stream);
+    cudaError_t e = upload_twiddles(g.twx, g.nx, true, b->stream);
+    if (e == cudaSuccess) e = upload_twiddles(g.twy, g.ny, false, b->stream);
+    if (e == cudaSuccess) e = upload_twiddles(g.twt, g.nt, false, b->stream);
     if (e == cudaSuccess) e = stage_table(b, g);
     if (e != cudaSuccess) return release(bfail(b, BRAHMS_E_CUDA, std::string("twiddles: ") + cudaGetErrorString(e)));
     for (size_t slot = 0; slot < m; ++slot) {
@@ -943,8 +944,8 @@ brahms_status build_tables_for(brahms_batch* b, BatchInstHost& I) {
     a.alpha[f] = I.fp[f].alpha;
   }
   BB_CK(run_prop_tables(a, b->stream));
-  BB_CK(upload_twiddles(I.twx, I.nx, b->stream));
-  BB_CK(upload_twiddles(I.twt, I.nt, b->stream));
+  BB_CK(upload_twiddles(I.twx, I.nx, true, b->stream));
+  BB_CK(upload_twiddles(I.twt, I.nt, false, b->stream));
   b->launches += 1;
   return BRAHMS_OK;
 }
@@ -1009,8 +1010,8 @@ brahms_status brahms_batch_add(brahms_batch* b, int nx, int ny, int nt, double d
   I.fp[1] = fp[1];
   const size_t n = (size_t)I.npoints();
   size_t o_state = 0, o_twx = al256(sizeof(float2) * 2 * n),
-         o_twt = o_twx + al256(sizeof(float2) * tw_table_size_of(nx)),
-         o_px = o_twt + al256(sizeof(float2) * tw_table_size_of(nt)), o_py = o_px + al256(sizeof(float2) * 2 * nx),
+         o_twt = o_twx + al256(sizeof(float2) * tw_table_size_of(nx, true)),
+         o_px = o_twt + al256(sizeof(float2) * tw_table_size_of(nt, false)), o_py = o_px + al256(sizeof(float2) * 2 * nx),
          o_pt = o_py + al256(sizeof(float2) * 2 * ny), total = o_pt + al256(sizeof(float2) * 2 * nt);
   if (dev_alloc((void**)&I.mem, total) != cudaSuccess) {
     cudaGetLastError();
@@ -1042,9 +1043,12 @@ brahms_status brahms_batch_set_fields(brahms_batch* b, int index, const void* co
   if (dtype != BRAHMS_C64) return bfail(b, BRAHMS_E_ARG, "batched fields must be complex64");
   BatchInstHost& I = b->inst[index];
   const size_t n = (size_t)I.npoints();
-  for (int f = 0; f < 2; ++f)
-    BB_CK(cudaMemcpyAsync(I.state + f * n, fields[f], sizeof(float2) * n,
-                          on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, b->stream));
+  if (on_device && kernel_can_copy(fields, 2, sizeof(float2) * n, I.state, I.state + 2 * n, false))
+    BB_CK(run_copy_pair((const float2*)fields[0], I.state, (const float2*)fields[1], I.state + n, (long long)n, b->stream));
+  else
+    for (int f = 0; f < 2; ++f)
+      BB_CK(cudaMemcpyAsync(I.state + f * n, fields[f], sizeof(float2) * n,
+                            on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, b->stream));
   if (!on_device) BB_CK(cudaStreamSynchronize(b->stream));
   if (!I.have_fields) b->dirty = true;
   I.have_fields = true;
@@ -1113,9 +1117,12 @@ brahms_status brahms_batch_get_fields(brahms_batch* b, int index, void* const* o
   if (dtype != BRAHMS_C64) return bfail(b, BRAHMS_E_ARG, "batched fields are complex64");
   BatchInstHost& I = b->inst[index];
   const size_t n = (size_t)I.npoints();
-  for (int f = 0; f < 2; ++f)
-    BB_CK(cudaMemcpyAsync(out[f], I.state + f * n, sizeof(float2) * n,
-                          on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, b->stream));
+  if (on_device && kernel_can_copy(out, 2, sizeof(float2) * n, I.state, I.state + 2 * n, true))
+    BB_CK(run_copy_pair(I.state, (float2*)out[0], I.state + n, (float2*)out[1], (long long)n, b->stream));
+  else
+    for (int f = 0; f < 2; ++f)
+      BB_CK(cudaMemcpyAsync(out[f], I.state + f * n, sizeof(float2) * n,
+                            on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, b->stream));
   return brahms_batch_sync(b);
 }
 

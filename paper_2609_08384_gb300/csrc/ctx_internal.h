@@ -11,6 +11,7 @@
 
 #include "alloc_hook.h"
 #include "brahms.h"
+#include "device_buffers.h"
 #include "kernels.cuh"
 
 namespace brahms_host {
@@ -42,9 +43,9 @@ inline Layout make_layout(int nx, int ny, int nt, int nf) {
   L.px = take(sizeof(float2) * nx * nf);
   L.py = take(sizeof(float2) * ny * nf);
   L.pt = take(sizeof(float2) * nt * nf);
-  L.twx = take(sizeof(float2) * brahms::tw_table_size_of(nx));
-  L.twy = take(sizeof(float2) * brahms::tw_table_size_of(ny));
-  L.twt = take(sizeof(float2) * brahms::tw_table_size_of(nt));
+  L.twx = take(sizeof(float2) * brahms::tw_table_size_of(nx, true));
+  L.twy = take(sizeof(float2) * brahms::tw_table_size_of(ny, false));
+  L.twt = take(sizeof(float2) * brahms::tw_table_size_of(nt, false));
   L.partial = take(sizeof(double) * kRedBlocks * nf);
   L.err = take(2 * sizeof(int));
   L.diag = take(sizeof(double) * 2 * nt * nf);
@@ -460,30 +461,9 @@ inline double dk_of_step(const brahms_ctx* c, long long j) {
   return j < (long long)c->dk_profile.size() ? c->dk_profile[(size_t)j] : c->dk;
 }
 
-// Whether a kernel of the current device can bring the fields in from a caller's
-// buffers, or hand them out to them, as 16-byte pairs: device memory of this
-// device, aligned, apart from the workspace and, when written, from each other.
-// Otherwise the driver's copies move the fields one after another.
 inline bool kernel_can_copy(const brahms_ctx* ctx, const void* const* ptrs, bool written) {
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return false;
-  const uintptr_t bytes = sizeof(float2) * (uintptr_t)ctx->npoints();
-  const uintptr_t ws0 = (uintptr_t)ctx->ws, ws1 = ws0 + ctx->L.total;
-  for (int f = 0; f < ctx->nf; ++f) {
-    const uintptr_t p = (uintptr_t)ptrs[f];
-    if ((p & 15) != 0 || (p < ws1 && ws0 < p + bytes)) return false;
-    for (int g = 0; written && g < f; ++g) {
-      const uintptr_t q = (uintptr_t)ptrs[g];
-      if (p < q + bytes && q < p + bytes) return false;
-    }
-    cudaPointerAttributes at{};
-    if (cudaPointerGetAttributes(&at, ptrs[f]) != cudaSuccess) {
-      cudaGetLastError();
-      return false;
-    }
-    if (at.type != cudaMemoryTypeDevice || at.device != dev) return false;
-  }
-  return true;
+  return brahms::kernel_can_copy(ptrs, ctx->nf, sizeof(float2) * (size_t)ctx->npoints(), ctx->ws,
+                                 ctx->ws + ctx->L.total, written);
 }
 
 // Enqueue an FP64 |A|^2 reduction per field into energy_host (pinned); from or to

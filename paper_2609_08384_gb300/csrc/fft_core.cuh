@@ -313,7 +313,7 @@ struct Plan {
   __host__ __device__ static constexpr int r(int p) { return p == 0 ? R0_ : p == 1 ? R1_ : p == 2 ? R2_ : R3_; }
 };
 
-// default plans (x- and y-passes)
+// default plans
 template <int N>
 struct FftPlan;
 template <> struct FftPlan<2> : Plan<2, 2, 1, 2> {};
@@ -340,11 +340,16 @@ template <> struct FftPlan<192> : Plan<192, 12, 4, 3, 4, 4, 4> {};
 template <> struct FftPlan<384> : Plan<384, 24, 4, 3, 8, 4, 4> {};
 template <> struct FftPlan<768> : Plan<768, 24, 4, 3, 4, 8, 8> {};
 
-// tau-pass plans (a 512-point plan with 8 values per thread and 1024-thread
-// tiles measured slower on GB300 than the default, 742 vs 709 us per OPG
-// launch; the tau pass shares the default plans and their twiddle tables)
+// Plans of the strided axes (y and tau), where they differ from the rows'.  1024
+// points as 32 x 32 (one exchange, 32 threads per pencil): tau-pass of 2 x
+// 256x256x1024 833 -> 658 us, step of 2 x 512x1024x1 25 -> 20 us; on rows it needs
+// twice the rows for the same threads (2 x 1024x128x1: 11 -> 15 us).
 template <int N>
-struct TauPlan : FftPlan<N> {};
+struct ColPlan : FftPlan<N> {};
+template <>
+struct ColPlan<1024> : Plan<1024, 32, 2, 32, 32> {};
+template <int N>
+struct TauPlan : ColPlan<N> {};
 
 template <class PL, bool INV>
 __host__ __device__ constexpr int fft_radix(int p) {

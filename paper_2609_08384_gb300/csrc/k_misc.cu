@@ -226,6 +226,15 @@ __global__ void c64_to_c128_kernel(const float2* __restrict__ in, double2* __res
   }
 }
 
+// two fields of n points (even) in one launch, 16-byte pairs
+__global__ void copy_pair_kernel(const float4* __restrict__ s0, float4* __restrict__ d0, const float4* __restrict__ s1,
+                                 float4* __restrict__ d1, long long n2) {
+  const float4* s = blockIdx.y ? s1 : s0;
+  float4* d = blockIdx.y ? d1 : d0;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n2; i += (long long)gridDim.x * blockDim.x)
+    d[i] = __ldcg(s + i);
+}
+
 static int grid_for(long long n) {
   long long g = (n + 255) / 256;
   return (int)(g > 152 * 16 ? 152 * 16 : (g < 1 ? 1 : g));
@@ -256,6 +265,13 @@ __global__ void prop_pointwise_kernel(const AxisArgs p, int nf) {
 cudaError_t run_prop_pointwise(const AxisArgs& a, int nf, cudaStream_t s) {
   return launch_chained(prop_pointwise_kernel, dim3((unsigned)grid_for((long long)a.nx * a.ny * a.nt * nf)), 256, 0, s, a,
                         nf);
+}
+
+cudaError_t run_copy_pair(const float2* s0, float2* d0, const float2* s1, float2* d1, long long n, cudaStream_t s) {
+  copy_pair_kernel<<<dim3(grid_for(n / 2), 2), 256, 0, s>>>(
+      reinterpret_cast<const float4*>(s0), reinterpret_cast<float4*>(d0), reinterpret_cast<const float4*>(s1),
+      reinterpret_cast<float4*>(d1), n / 2);
+  return cudaPeekAtLastError();
 }
 
 cudaError_t run_c128_to_c64(const double2* in, float2* out, long long n, cudaStream_t s) {

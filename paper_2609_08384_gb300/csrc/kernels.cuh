@@ -689,66 +689,76 @@ __host__ __device__ constexpr int tau_pipe_ctas() {
   return fit < most ? fit : most;
 }
 
+// tile number `tile` of a pipelined tau kernel: its (field, y, x) and its first
+// column in memory
+template <int TX>
+struct PipeTile {
+  int f, y, x;
+  float2* base;
+  __device__ __forceinline__ PipeTile(const AxisArgs& p, long long tile) {
+    x = (int)(tile % p.xtiles) * TX;
+    const long long rest = tile / p.xtiles;
+    y = (int)(rest % p.ny);
+    f = (int)(rest / p.ny);
+    base = p.data + (long long)f * p.fstride + (long long)y * p.nx + x;
+  }
+};
+// requests the thread's share of a tile, in 16-byte pieces, into [tau][column]
+template <class PL>
+__device__ __forceinline__ void pipe_copy(const AxisArgs& p, long long tile, float2* buf) {
+  constexpr int TX = tau_pipe_cols<PL>();
+  constexpr int PAIRS = TX / 2, ROWS = tau_pipe_threads<PL>() / PAIRS;  // pieces per row, rows per copy step
+  const PipeTile<TX> a(p, tile);
+  const long long plane = (long long)p.nx * p.ny;
+  const int c = 2 * (threadIdx.x % PAIRS), row = threadIdx.x / PAIRS;
+  if (a.x + c >= p.nx) return;  // nx is even
+  const float2* src = a.base + c + row * plane;
+  const unsigned dst = (unsigned)__cvta_generic_to_shared(buf + row * TX + c);
+#pragma unroll
+  for (int q = 0; q < PL::N / ROWS; ++q)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + q * ROWS * TX * 8),
+                 "l"(src + (long long)(q * ROWS) * plane)
+                 : "memory");
+}
+template <class PL>
+using PipeXch = typename std::conditional<tau_pipe_cols<PL>() == 8, XchCol8, XchCol<tau_pipe_cols<PL>()>>::type;
+// the thread's first-pass inputs of a tile that has arrived
+template <class PL>
+__device__ __forceinline__ void pipe_take(float2 (&v)[PL::E], const PipeXch<PL>& xc, int t) {
+  constexpr int R0 = fft_radix<PL, false>(0);
+#pragma unroll
+  for (int i = 0; i < PL::E / R0; ++i)
+#pragma unroll
+    for (int r = 0; r < R0; ++r) v[i * R0 + r] = xc.ld(pos_first<PL, false>(t + i * PL::T, r));
+}
+
 template <class PL>
 __global__ void __launch_bounds__(tau_pipe_threads<PL>(), tau_pipe_ctas<PL>())
     tpass_pipe_kernel(const AxisArgs p) {
-  constexpr int N = PL::N, TX = tau_pipe_cols<PL>();
-  constexpr int THREADS = tau_pipe_threads<PL>();
-  constexpr int PAIRS = TX / 2, ROWS = THREADS / PAIRS;  // 16-byte pieces per row, rows per copy step
-  using X = typename std::conditional<TX == 8, XchCol8, XchCol<TX>>::type;
+  constexpr int N = PL::N, TX = tau_pipe_cols<PL>(), THREADS = tau_pipe_threads<PL>();
+  using X = PipeXch<PL>;
   extern __shared__ float4 sm4[];
   float2* buf = reinterpret_cast<float2*>(sm4);
   float2* tw = buf + 2 * N * TX;
   for (int i = threadIdx.x; i < tw_table_size<PL>(); i += THREADS) tw[i] = p.tw[i];
   const long long plane = (long long)p.nx * p.ny;
   const int tx = threadIdx.x % TX, t = threadIdx.x / TX;
-  // tile k counted from the last: its first column in memory and its (field, y, x)
-  struct Tile {
-    int f, y, x;
-    float2* base;
-  };
-  const auto tile_at = [&](long long k) {
-    const long long tile = p.ntiles - 1 - k;
-    Tile a;
-    a.x = (int)(tile % p.xtiles) * TX;
-    const long long rest = tile / p.xtiles;
-    a.y = (int)(rest % p.ny);
-    a.f = (int)(rest / p.ny);
-    a.base = p.data + (long long)a.f * p.fstride + (long long)a.y * p.nx + a.x;
-    return a;
-  };
-  const auto copy_tile = [&](long long k, int b) {
-    const Tile a = tile_at(k);
-    const int c = 2 * (threadIdx.x % PAIRS), row = threadIdx.x / PAIRS;
-    if (a.x + c >= p.nx) return;  // nx is even
-    const float2* src = a.base + c + row * plane;
-    const unsigned dst = (unsigned)__cvta_generic_to_shared(buf + b * N * TX + row * TX + c);
-#pragma unroll
-    for (int q = 0; q < N / ROWS; ++q)
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + q * ROWS * TX * 8),
-                   "l"(src + (long long)(q * ROWS) * plane)
-                   : "memory");
-  };
-  long long k = blockIdx.x;
+  long long k = blockIdx.x;  // tiles from the last down
   chain_begin();
-  if (k < p.ntiles) copy_tile(k, 0);
+  if (k < p.ntiles) pipe_copy<PL>(p, p.ntiles - 1 - k, buf);
   cp_async_commit();
   for (int b = 0; k < p.ntiles; k += gridDim.x, b ^= 1) {
     cp_async_wait<0>();
     __syncthreads();  // the tile is there, and the last one's buffer is free
-    if (k + gridDim.x < p.ntiles) copy_tile(k + gridDim.x, b ^ 1);
+    if (k + gridDim.x < p.ntiles) pipe_copy<PL>(p, p.ntiles - 1 - (k + gridDim.x), buf + (b ^ 1) * N * TX);
     cp_async_commit();
-    const Tile a = tile_at(k);
+    const PipeTile<TX> a(p, p.ntiles - 1 - k);
     const bool act = a.x + tx < p.nx;
     // the column's factors, requested ahead of the forward transform
     const float2 dx = act ? p.px[a.f * p.nx + a.x + tx] : make_float2(0.f, 0.f), dy = p.py[a.f * p.ny + a.y];
     const X xc{buf + b * N * TX, tx};
-    constexpr int R0 = fft_radix<PL, false>(0);
     float2 v[PL::E];
-#pragma unroll
-    for (int i = 0; i < PL::E / R0; ++i)
-#pragma unroll
-      for (int r = 0; r < R0; ++r) v[i * R0 + r] = xc.ld(pos_first<PL, false>(t + i * PL::T, r));
+    pipe_take<PL>(v, xc, t);
     fft_run<PL, false, 0, X, SyncBlock, TwShared>(v, t, xc, TwShared{tw});
     apply_prop<PL>(v, ColumnProp(p, dx, dy), p.pt + a.f * p.nt, t);
     fft_run<PL, true, 0, X, SyncBlock, TwShared>(v, t, xc, TwShared{tw});
@@ -836,10 +846,10 @@ cudaError_t make_tau_tensor_map(void* map128, const float2* data, int nx, int ny
 cudaError_t run_tpass_prop_tma(int nt, int tx, const void* map128, const AxisArgs& a, int* err,
                                unsigned long long wait_ns, cudaStream_t s);
 
-// per-pass twiddle table of the default plan of length n (shears, built on the
-// host in FP64), and its size in entries
-int tw_table_size_of(int n);
-cudaError_t upload_twiddles(float2* tw, int n, cudaStream_t s);
+// per-pass twiddle table of the plan of length n on rows (x) or strided axes (y,
+// tau), built on the host in FP64, and its size in entries
+int tw_table_size_of(int n, bool rows);
+cudaError_t upload_twiddles(float2* tw, int n, bool rows, cudaStream_t s);
 struct TableArgs {
   float2* px;
   float2* py;
@@ -920,6 +930,8 @@ struct EnergyArgs {
   const int* err;
 };
 cudaError_t run_energy(const EnergyArgs& a, int nf, int nblocks, cudaStream_t s);
+// d0 = s0 and d1 = s1, n points (even) each, 16-byte aligned
+cudaError_t run_copy_pair(const float2* s0, float2* d0, const float2* s1, float2* d1, long long n, cudaStream_t s);
 cudaError_t run_c128_to_c64(const double2* in, float2* out, long long n, cudaStream_t s);
 cudaError_t run_c64_to_c128(const float2* in, double2* out, long long n, cudaStream_t s);
 

@@ -82,3 +82,24 @@ def test_non_finite_points_are_seen_wherever_they_are(where, value):
     assert e.value.status == br.BRAHMS_E_ARG
     s.set_fields([x, x, x])  # the context stays usable
     s.close()
+
+
+@pytest.mark.parametrize("shift", [0, 1])
+def test_batch_fields_at_any_alignment(shift):
+    import paper_2609_08384_gb300 as br
+    b = br.Batch()
+    shapes = [(32, 32, 64), (24, 48, 12)]
+    f = [wl.FieldParams(532e-9, 2.234), wl.FieldParams(1064e-9, 2.156)]
+    a = []
+    for i, (nx, ny, nt) in enumerate(shapes):
+        b.add(wl.Grid(nx, ny, nt, 3e-6, 3e-6, 3e-14), f, wl.D_EFF, 0.0, 1, 1e-5)
+        raw = torch.randn(2, nx * ny * nt + 2, dtype=torch.complex64, device="cuda")
+        a.append([raw[k, shift:shift + nx * ny * nt].clone() if not shift else raw[k, 1:1 + nx * ny * nt]
+                  for k in range(2)])
+        b.set_fields(i, [x.view(nt, ny, nx) for x in a[-1]])
+    for i, (nx, ny, nt) in enumerate(shapes):
+        for got, x in zip(b.get_fields(i, on_device=True), a[i]):
+            assert torch.equal(got.view(-1), x)
+        for got, x in zip(b.get_fields(i), a[i]):
+            assert np.array_equal(got.reshape(-1), x.cpu().numpy())
+    b.close()
