@@ -1,6 +1,7 @@
 // Diagnostics of the fields: the temporal power trace and the energy
 // spectrum over Omega (the Sec. 6 power formula resolved in tau or Omega).
 // Neither kernel writes the state.
+#include "float_sum.cuh"
 #include "kernels.cuh"
 #include "launch_cfg.h"
 
@@ -15,27 +16,30 @@ __device__ __forceinline__ double warp_sum_d(double v) {
 }
 
 // sum_{x,y} |A_f(x, y, tau_k)|^2 for every (k, f): one CTA per plane; two
-// points per 16-byte load, their squares summed in FP32 and accumulated in
-// FP64 (planes hold an even number of points)
+// points per 16-byte load, their squares summed in FP32 and accumulated without
+// loss (planes hold an even number of points)
 __global__ void __launch_bounds__(256) power_trace_kernel(const float2* __restrict__ data, long long plane,
                                                           int nt, long long fstride, double* out) {
   const int k = blockIdx.x, f = blockIdx.y;
   const float2* a = data + (long long)f * fstride + (long long)k * plane;
-  double s = 0.0;
+  FloatSum sum[2];
   const float4* a4 = reinterpret_cast<const float4*>(a);
   const long long n2 = plane / 2;
+  const auto pair = [](float4 v) { return fmaf(v.x, v.x, fmaf(v.y, v.y, fmaf(v.z, v.z, v.w * v.w))); };
   long long i = threadIdx.x;
-  // four loads in flight per thread; each pair's FP32 sum goes into FP64 as before
-  for (; i + 3 * (long long)blockDim.x < n2; i += 4 * (long long)blockDim.x) {
-    float4 v[4];
+  // eight loads in flight per thread
+  for (; i + 7 * (long long)blockDim.x < n2; i += 8 * (long long)blockDim.x) {
+    float4 v[8];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) v[u] = __ldcg(a4 + i + u * (long long)blockDim.x);
+    for (int u = 0; u < 8; ++u) v[u] = __ldcg(a4 + i + u * (long long)blockDim.x);
 #pragma unroll
-    for (int u = 0; u < 4; ++u) s += (double)fmaf(v[u].x, v[u].x, fmaf(v[u].y, v[u].y, fmaf(v[u].z, v[u].z, v[u].w * v[u].w)));
+    for (int u = 0; u < 8; ++u) sum[u & 1].add(pair(v[u]));
   }
-  for (; i < n2; i += blockDim.x) {
-    const float4 v = __ldcg(a4 + i);
-    s += (double)fmaf(v.x, v.x, fmaf(v.y, v.y, fmaf(v.z, v.z, v.w * v.w)));
+  for (; i < n2; i += blockDim.x) sum[0].add(pair(__ldcg(a4 + i)));
+  double s = sum[0].value() + sum[1].value();
+  if (!isfinite(s)) {  // beyond FP32's range, or fields that are not finite
+    s = 0.0;
+    for (i = threadIdx.x; i < n2; i += blockDim.x) s += (double)pair(__ldcg(a4 + i));
   }
   if ((plane & 1) && threadIdx.x == 0) {
     const float2 v = __ldcg(a + plane - 1);
@@ -62,7 +66,9 @@ __global__ void __launch_bounds__(256) power_trace_kernel(const float2* __restri
 // per-thread FP64 accumulators of its bins; a change of field and the end of
 // the range flush them with one atomicAdd per bin.  (Summing the columns in
 // FP64 made the FP64 pipe the bound: 0.94 against 0.60 ms per call with the
-// power trace on the OPG state.)
+// power trace on the 3 x 256x256x512 state.  Persistent CTAs whose next tile
+// arrives during the transform, as in the pipelined tau-pass, took 260 us against
+// 220.)
 template <class PL>
 __global__ void __launch_bounds__(tiles_per_cta<PL>() * tile_threads<PL>())
     tau_spectrum_kernel(const AxisArgs p, long long range, double* out) {

@@ -1,4 +1,5 @@
 // Set-up tables, the energy reduction and dtype conversions.
+#include "float_sum.cuh"
 #include "kernels.cuh"
 #include "launch_cfg.h"
 #include "map_seg.h"
@@ -135,8 +136,8 @@ cudaError_t run_prop_tables(const TableArgs& a, cudaStream_t s) {
 
 // ------------------------------------------------------------- energy
 // Per-field sum of |A|^2: two complex values per 16-byte load, squares
-// summed in FP32 over eight points (round-to-nearest, unbiased) and added to
-// an FP64 accumulator, so the FP64 work is one add per eight points.
+// summed in FP32 over eight points (round-to-nearest, unbiased), the groups
+// without loss (FloatSum) and the threads' sums in FP64.
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
@@ -151,31 +152,29 @@ template <bool COPY>
 __global__ void __launch_bounds__(256) energy_kernel(const EnergyArgs p) {
   const float4* a4 = reinterpret_cast<const float4*>(p.src[blockIdx.y]);
   float4* d4 = reinterpret_cast<float4*>(p.dst[blockIdx.y]);
-  double s = 0.0;
+  FloatSum sum;
   // pairs (every length is even, so a field holds whole 16-byte pairs)
   const long long n2 = p.n / 2;
   const long long stride = (long long)gridDim.x * blockDim.x;
-  long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  // four independent pairs per round: the loads overlap, one FP64 add per eight points
-  for (; i + 3 * stride < n2; i += 4 * stride) {
-    const float4 v0 = __ldcg(a4 + i), v1 = __ldcg(a4 + i + stride), v2 = __ldcg(a4 + i + 2 * stride),
-                 v3 = __ldcg(a4 + i + 3 * stride);
-    if constexpr (COPY) {
-      d4[i] = v0;
-      d4[i + stride] = v1;
-      d4[i + 2 * stride] = v2;
-      d4[i + 3 * stride] = v3;
-    }
-    const float q0 = fmaf(v0.x, v0.x, fmaf(v0.y, v0.y, fmaf(v0.z, v0.z, v0.w * v0.w)));
-    const float q1 = fmaf(v1.x, v1.x, fmaf(v1.y, v1.y, fmaf(v1.z, v1.z, v1.w * v1.w)));
-    const float q2 = fmaf(v2.x, v2.x, fmaf(v2.y, v2.y, fmaf(v2.z, v2.z, v2.w * v2.w)));
-    const float q3 = fmaf(v3.x, v3.x, fmaf(v3.y, v3.y, fmaf(v3.z, v3.z, v3.w * v3.w)));
-    s += (double)((q0 + q1) + (q2 + q3));
+  const long long i0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  long long i = i0;
+  // eight independent pairs per round, four to a sum: the loads overlap
+  const auto square = [](float4 v) { return fmaf(v.x, v.x, fmaf(v.y, v.y, fmaf(v.z, v.z, v.w * v.w))); };
+  for (; i + 7 * stride < n2; i += 8 * stride) {
+    float4 v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = __ldcg(a4 + i + u * stride);
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if constexpr (COPY) d4[i + u * stride] = v[u];
+#pragma unroll
+    for (int u = 0; u < 8; u += 4)
+      sum.add((square(v[u]) + square(v[u + 1])) + (square(v[u + 2]) + square(v[u + 3])));
   }
   for (; i < n2; i += stride) {
     const float4 v = __ldcg(a4 + i);
     if constexpr (COPY) d4[i] = v;
-    s += (double)fmaf(v.x, v.x, fmaf(v.y, v.y, fmaf(v.z, v.z, v.w * v.w)));
+    sum.add(square(v));
   }
   __shared__ double red[8];
   __shared__ bool last;
@@ -187,7 +186,12 @@ __global__ void __launch_bounds__(256) energy_kernel(const EnergyArgs p) {
     v = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.0;
     return threadIdx.x < 32 ? warp_sum(v) : 0.0;
   };
-  s = block_sum(s);
+  double own = sum.value();
+  if (!isfinite(own)) {  // beyond FP32's range, or fields that are not finite
+    own = 0.0;
+    for (long long k = i0; k < n2; k += stride) own += (double)square(__ldcg(a4 + k));
+  }
+  const double s = block_sum(own);
   if (threadIdx.x == 0) {
     p.partial[blockIdx.y * gridDim.x + blockIdx.x] = s;
     __threadfence();

@@ -103,3 +103,22 @@ def test_batch_fields_at_any_alignment(shift):
         for got, x in zip(b.get_fields(i), a[i]):
             assert np.array_equal(got.reshape(-1), x.cpu().numpy())
     b.close()
+
+
+@pytest.mark.parametrize("size", [1e-15, 1.0, 3e17])
+def test_energy_and_power_of_tiny_and_huge_fields(size):
+    """Sums of squares across FP32's range: at 3e17 a point's square fits a float
+    and the sums of a thread's points do not."""
+    shape = (96, 96, 64)
+    nx, ny, nt = shape
+    s = _solver(shape)
+    x = [size * torch.randn(nt, ny, nx, dtype=torch.complex64, device="cuda") for _ in range(3)]
+    s.set_fields(x)
+    e, _ = s.energy()
+    p, _ = s.diagnostics()
+    for f in range(3):
+        c = 0.5 * wl.C0 * wl.EPS0 * (2.15, 2.14, 2.08)[f] * 3e-6 * 3e-6
+        ref = c * x[f].to(torch.complex128).abs().square().sum((1, 2)).cpu().numpy()
+        assert np.allclose(p[f], ref, rtol=4 * 6e-8, atol=0)  # FP32 squares of pairs of points
+        assert abs(e[f] / (ref.sum() * 3e-14) - 1) < 8 * 6e-8
+    s.close()
