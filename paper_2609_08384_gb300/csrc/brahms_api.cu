@@ -113,9 +113,9 @@ brahms_status brahms_init_grid(brahms_ctx** out, int nx, int ny, int nt, double 
   ctx->mphase_dev = (double*)(ctx->ws + ctx->L.mphase);
   ctx->emap_dev = (float2*)(ctx->ws + ctx->L.emap);
   cudaError_t e = cudaSuccess;
-  if (e == cudaSuccess) e = brahms::upload_twiddles(ctx->twx, nx, true, ctx->stream);
-  if (e == cudaSuccess && ny > 1) e = brahms::upload_twiddles(ctx->twy, ny, false, ctx->stream);
-  if (e == cudaSuccess && nt > 1) e = brahms::upload_twiddles(ctx->twt, nt, false, ctx->stream);
+  if (e == cudaSuccess) e = brahms::upload_twiddles(ctx->twx, nx, 0, ctx->stream);
+  if (e == cudaSuccess && ny > 1) e = brahms::upload_twiddles(ctx->twy, ny, 1, ctx->stream);
+  if (e == cudaSuccess && nt > 1) e = brahms::upload_twiddles(ctx->twt, nt, 2, ctx->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(ctx->dev_err, 0, 2 * sizeof(int), ctx->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(ctx->mphase_dev, 0, sizeof(double) * nx * ny, ctx->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);

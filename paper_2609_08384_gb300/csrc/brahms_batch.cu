@@ -59,7 +59,7 @@ template <int S>
 struct ShapeT {
   static constexpr int NXY = kShapes[S].nxy;
   static constexpr int NT = kShapes[S].nt;
-  using PY = FftPlan<NXY>;
+  using PY = ColPlan<NXY>;
   using PT = TauPlan<NT>;
   static constexpr int YTPC = tiles_per_cta_t<PY, kBT>();
   static constexpr int TTPC = tiles_per_cta_t<PT, kBT>();
@@ -84,7 +84,7 @@ struct InstDev {
   float2* state;
   const float2* ecoef;  // stage factors of every x-pass: [step + 1][kStageFactors] (see stage_table)
   long long fstride;
-  const float2 *twx, *twt;  // NX = NY: one table serves x and y
+  const float2 *twx, *twy, *twt;
   const float2 *px, *py, *pt;
   int nx, ny, nt, shape;
   int nz;
@@ -240,9 +240,9 @@ __device__ __noinline__ void run_item(const InstDev& I, const Item& it, float4* 
   } else {
     a.xtiles = (NXY + ColTile<typename SH::PY>::value - 1) / ColTile<typename SH::PY>::value;
     a.ntiles = 2LL * NT * a.xtiles;
-    a.tw = I.twx;
+    a.tw = I.twy;
     float2* xch = tw + tw_table_size<typename SH::PY>();
-    for (int i = threadIdx.x; i < tw_table_size<typename SH::PY>(); i += kBT) tw[i] = I.twx[i];
+    for (int i = threadIdx.x; i < tw_table_size<typename SH::PY>(); i += kBT) tw[i] = I.twy[i];
     __syncthreads();
     for (long long c = 0; c < it.ntiles; ++c) {
       if (it.type == kTypeYF) axis_tile<typename SH::PY, false, 1, kBT>(a, it.tile + c, TwShared{tw}, xch);
@@ -390,7 +390,7 @@ struct BatchInstHost {
   brahms_field_params fp[2];
   char* mem = nullptr;  // state + tables until the instance joins a group (then NULL)
   float2* state = nullptr;
-  float2 *twx = nullptr, *twt = nullptr;
+  float2 *twx = nullptr, *twy = nullptr, *twt = nullptr;  // twy: once it has joined a group
   float2 *px = nullptr, *py = nullptr, *pt = nullptr;
   const float2* ecoef = nullptr;  // its stage factors in its group's table, [step + 1][kStageFactors]
   bool have_fields = false;
@@ -578,9 +578,9 @@ brahms_status layout(brahms_batch* b) {
     };
     const size_t o_state = take(sizeof(float2) * 2 * n * m), o_px = take(sizeof(float2) * 2 * m * g.nx),
                  o_py = take(sizeof(float2) * 2 * m * g.ny), o_pt = take(sizeof(float2) * 2 * m * g.nt),
-                 o_twx = take(sizeof(float2) * tw_table_size_of(g.nx, true)),
-                 o_twy = take(sizeof(float2) * tw_table_size_of(g.ny, false)),
-                 o_twt = take(sizeof(float2) * tw_table_size_of(g.nt, false)), o_par = take(sizeof(GroupInst) * m);
+                 o_twx = take(sizeof(float2) * tw_table_size_of(g.nx, 0)),
+                 o_twy = take(sizeof(float2) * tw_table_size_of(g.ny, 1)),
+                 o_twt = take(sizeof(float2) * tw_table_size_of(g.nt, 2)), o_par = take(sizeof(GroupInst) * m);
     g.ecoef_steps = 0;
     for (int i : g.members) g.ecoef_steps = std::max(g.ecoef_steps, b->inst[i].nz);
     const size_t o_coef = take(sizeof(float2) * kStageFactors * (size_t)(g.ecoef_steps + 1) * m);
@@ -600,9 +600,9 @@ brahms_status layout(brahms_batch* b) {
     if (cudaStreamCreateWithFlags(&g.stream, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&g.done, cudaEventDisableTiming) != cudaSuccess)
       return release(bfail(b, BRAHMS_E_CUDA, "group stream"));
-    cudaError_t e = upload_twiddles(g.twx, g.nx, true, b->stream);
-    if (e == cudaSuccess) e = upload_twiddles(g.twy, g.ny, false, b->stream);
-    if (e == cudaSuccess) e = upload_twiddles(g.twt, g.nt, false, b->stream);
+    cudaError_t e = upload_twiddles(g.twx, g.nx, 0, b->stream);
+    if (e == cudaSuccess) e = upload_twiddles(g.twy, g.ny, 1, b->stream);
+    if (e == cudaSuccess) e = upload_twiddles(g.twt, g.nt, 2, b->stream);
     if (e == cudaSuccess) e = stage_table(b, g);
     if (e != cudaSuccess) return release(bfail(b, BRAHMS_E_CUDA, std::string("twiddles: ") + cudaGetErrorString(e)));
     for (size_t slot = 0; slot < m; ++slot) {
@@ -628,6 +628,7 @@ brahms_status layout(brahms_batch* b) {
       I.py = g.py + slot * 2 * g.ny;
       I.pt = g.pt + slot * 2 * g.nt;
       I.twx = g.twx;
+      I.twy = g.twy;
       I.twt = g.twt;
       I.ecoef = g.ecoef + slot * (size_t)(g.ecoef_steps + 1) * kStageFactors;
       brahms_status st = build_tables_for(b, I);
@@ -833,6 +834,7 @@ brahms_status prepare_persistent(brahms_batch* b) {
     d.ecoef = I.ecoef;
     d.fstride = I.npoints();
     d.twx = I.twx;
+    d.twy = I.twy;
     d.twt = I.twt;
     d.px = I.px;
     d.py = I.py;
@@ -944,8 +946,8 @@ brahms_status build_tables_for(brahms_batch* b, BatchInstHost& I) {
     a.alpha[f] = I.fp[f].alpha;
   }
   BB_CK(run_prop_tables(a, b->stream));
-  BB_CK(upload_twiddles(I.twx, I.nx, true, b->stream));
-  BB_CK(upload_twiddles(I.twt, I.nt, false, b->stream));
+  BB_CK(upload_twiddles(I.twx, I.nx, 0, b->stream));
+  BB_CK(upload_twiddles(I.twt, I.nt, 2, b->stream));
   b->launches += 1;
   return BRAHMS_OK;
 }
@@ -1010,8 +1012,8 @@ brahms_status brahms_batch_add(brahms_batch* b, int nx, int ny, int nt, double d
   I.fp[1] = fp[1];
   const size_t n = (size_t)I.npoints();
   size_t o_state = 0, o_twx = al256(sizeof(float2) * 2 * n),
-         o_twt = o_twx + al256(sizeof(float2) * tw_table_size_of(nx, true)),
-         o_px = o_twt + al256(sizeof(float2) * tw_table_size_of(nt, false)), o_py = o_px + al256(sizeof(float2) * 2 * nx),
+         o_twt = o_twx + al256(sizeof(float2) * tw_table_size_of(nx, 0)),
+         o_px = o_twt + al256(sizeof(float2) * tw_table_size_of(nt, 2)), o_py = o_px + al256(sizeof(float2) * 2 * nx),
          o_pt = o_py + al256(sizeof(float2) * 2 * ny), total = o_pt + al256(sizeof(float2) * 2 * nt);
   if (dev_alloc((void**)&I.mem, total) != cudaSuccess) {
     cudaGetLastError();

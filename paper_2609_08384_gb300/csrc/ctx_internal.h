@@ -43,9 +43,9 @@ inline Layout make_layout(int nx, int ny, int nt, int nf) {
   L.px = take(sizeof(float2) * nx * nf);
   L.py = take(sizeof(float2) * ny * nf);
   L.pt = take(sizeof(float2) * nt * nf);
-  L.twx = take(sizeof(float2) * brahms::tw_table_size_of(nx, true));
-  L.twy = take(sizeof(float2) * brahms::tw_table_size_of(ny, false));
-  L.twt = take(sizeof(float2) * brahms::tw_table_size_of(nt, false));
+  L.twx = take(sizeof(float2) * brahms::tw_table_size_of(nx, 0));
+  L.twy = take(sizeof(float2) * brahms::tw_table_size_of(ny, 1));
+  L.twt = take(sizeof(float2) * brahms::tw_table_size_of(nt, 2));
   L.partial = take(sizeof(double) * kRedBlocks * nf);
   L.err = take(2 * sizeof(int));
   L.diag = take(sizeof(double) * 2 * nt * nf);

@@ -290,12 +290,39 @@ __device__ __forceinline__ void dft32(float2* v) {
   }
 }
 
+// Radix 3 M (M = 2, 4, 8) by the prime-factor mapping (Good 1958): with
+// n = M n1 + 3 n2 and k = M (1/M mod 3) k1 + 3 (1/3 mod M) k2, both mod 3 M, the
+// transform is M-point transforms over n2 and three-point ones over n1 with no
+// turns between them.
+template <bool INV, int M>
+__device__ __forceinline__ void dft3m(float2* v) {
+  constexpr int N = 3 * M, K1 = M * (M % 3 == 1 ? 1 : 2), K2 = 3 * (M == 2 ? 1 : 3);
+  float2 y[3][M];
+#pragma unroll
+  for (int n1 = 0; n1 < 3; ++n1) {
+#pragma unroll
+    for (int n2 = 0; n2 < M; ++n2) y[n1][n2] = v[(M * n1 + 3 * n2) % N];
+    if constexpr (M == 2) dft2<INV>(y[n1][0], y[n1][1]);
+    else if constexpr (M == 4) dft4<INV>(y[n1][0], y[n1][1], y[n1][2], y[n1][3]);
+    else dft8<INV>(y[n1]);
+  }
+#pragma unroll
+  for (int k2 = 0; k2 < M; ++k2) {
+    dft3<INV>(y[0][k2], y[1][k2], y[2][k2]);
+#pragma unroll
+    for (int k1 = 0; k1 < 3; ++k1) v[(K1 * k1 + K2 * k2) % N] = y[k1][k2];
+  }
+}
+
 template <int R, bool INV>
 __device__ __forceinline__ void dft(float2* v) {
   if constexpr (R == 2) dft2<INV>(v[0], v[1]);
   else if constexpr (R == 3) dft3<INV>(v[0], v[1], v[2]);
   else if constexpr (R == 4) dft4<INV>(v[0], v[1], v[2], v[3]);
+  else if constexpr (R == 6) dft3m<INV, 2>(v);
   else if constexpr (R == 8) dft8<INV>(v);
+  else if constexpr (R == 12) dft3m<INV, 4>(v);
+  else if constexpr (R == 24) dft3m<INV, 8>(v);
   else if constexpr (R == 16) dft16<INV>(v);
   else if constexpr (R == 32) dft32<INV>(v);
   else static_assert(R == 2, "unsupported radix");
@@ -331,25 +358,43 @@ template <> struct FftPlan<512> : Plan<512, 32, 2, 32, 16> {};
 template <> struct FftPlan<1024> : Plan<1024, 16, 3, 16, 8, 8> {};
 template <> struct FftPlan<2048> : Plan<2048, 16, 3, 16, 16, 8> {};
 template <> struct FftPlan<4096> : Plan<4096, 16, 3, 16, 16, 16> {};
-template <> struct FftPlan<6> : Plan<6, 6, 2, 3, 2> {};
-template <> struct FftPlan<12> : Plan<12, 12, 2, 3, 4> {};
-template <> struct FftPlan<24> : Plan<24, 12, 3, 3, 2, 4> {};
-template <> struct FftPlan<48> : Plan<48, 12, 3, 3, 4, 4> {};
-template <> struct FftPlan<96> : Plan<96, 12, 4, 3, 4, 4, 2> {};
-template <> struct FftPlan<192> : Plan<192, 12, 4, 3, 4, 4, 4> {};
-template <> struct FftPlan<384> : Plan<384, 24, 4, 3, 8, 4, 4> {};
-template <> struct FftPlan<768> : Plan<768, 24, 4, 3, 4, 8, 8> {};
+template <> struct FftPlan<6> : Plan<6, 6, 1, 6> {};
+template <> struct FftPlan<12> : Plan<12, 12, 1, 12> {};
+template <> struct FftPlan<24> : Plan<24, 12, 2, 12, 2> {};
+template <> struct FftPlan<48> : Plan<48, 12, 2, 12, 4> {};
+template <> struct FftPlan<96> : Plan<96, 12, 3, 12, 4, 2> {};
+template <> struct FftPlan<192> : Plan<192, 24, 2, 24, 8> {};
+template <> struct FftPlan<384> : Plan<384, 24, 3, 8, 12, 4> {};
+template <> struct FftPlan<768> : Plan<768, 24, 3, 8, 24, 4> {};
 
-// Plans of the strided axes (y and tau), where they differ from the rows'.  1024
-// points as 32 x 32 (one exchange, 32 threads per pencil): tau-pass of 2 x
-// 256x256x1024 833 -> 658 us, step of 2 x 512x1024x1 25 -> 20 us; on rows it needs
-// twice the rows for the same threads (2 x 1024x128x1: 11 -> 15 us).
+// The lengths 3 2^k take radices 6, 12 and 24, which need one exchange where 3 x 4
+// x 4 x 4 needs three: the four-pass plans were bound by shared memory (x-pass of
+// 3 x 48x192x384: 82 % of its wavefronts, FP32 pipe 47 %).  Step of 2 x 96x96x192
+// 72 -> 56 us, of 3 x 48x192x384 192 -> 148, of 2 x 192x192x768 1063 -> 850.
+//
+// Plans of y and tau where they differ from the rows'.  1024 points as 32 x 32
+// (one exchange, 32 threads per pencil): tau-pass of 2 x 256x256x1024 833 -> 658
+// us, step of 2 x 512x1024x1 25 -> 20 us; on rows it needs twice the rows for the
+// same threads (2 x 1024x128x1: 11 -> 15 us).  96 as 24 x 4: y-passes of 2 x
+// 96x96x192 14.4 + 14.6 -> 12.2 + 13.1 us, tau-pass of 3 x 96x384x96 46 -> 40 (rows
+// 26.9 against 27.3).  384 as 24 x 16: y-passes of 3 x 96x384x96 63.5 -> 61.4,
+// tau-pass of 3 x 48x192x384 53.5 -> 47.8 (rows of 2 x 384x48x192 46 against 55).
+// 192 as 8 x 24 along y: y-passes of 2 x 192x192x768 305 -> 278 us (its tau-pass
+// and rows are better as 24 x 8: 18.5 against 20.4 us on 2 x 96x96x192).
 template <int N>
 struct ColPlan : FftPlan<N> {};
+template <>
+struct ColPlan<96> : Plan<96, 24, 2, 24, 4> {};
+template <>
+struct ColPlan<192> : Plan<192, 24, 2, 8, 24> {};
+template <>
+struct ColPlan<384> : Plan<384, 48, 2, 24, 16> {};
 template <>
 struct ColPlan<1024> : Plan<1024, 32, 2, 32, 32> {};
 template <int N>
 struct TauPlan : ColPlan<N> {};
+template <>
+struct TauPlan<192> : FftPlan<192> {};
 
 template <class PL, bool INV>
 __host__ __device__ constexpr int fft_radix(int p) {

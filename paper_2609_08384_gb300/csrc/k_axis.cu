@@ -9,7 +9,7 @@ namespace brahms {
 
 template <int N, bool INV, int AXIS>
 static cudaError_t launch_axis(const AxisArgs& a, cudaStream_t s) {
-  using PL = ColPlan<N>;
+  using PL = AxisPlan<N, AXIS>;
   constexpr int TPC = tiles_per_cta<PL>();
   constexpr int THREADS = TPC * tile_threads<PL>();
   const size_t smem = (size_t)axis_kernel_smem_floats2<PL, INV, AXIS>() * sizeof(float2);
@@ -81,11 +81,13 @@ cudaError_t run_tpass_prop(int nt, const AxisArgs& a, cudaStream_t s) {
   }
 }
 
-int tw_table_size_of(int n, bool rows) {
+int tw_table_size_of(int n, int axis) {
   switch (n) {
 #define BRAHMS_W_CASE(N) \
   case N:                \
-    return rows ? tw_table_size<FftPlan<N>>() : tw_table_size<ColPlan<N>>();
+    return axis == 0   ? tw_table_size<AxisPlan<N, 0>>()  \
+           : axis == 1 ? tw_table_size<AxisPlan<N, 1>>()  \
+                       : tw_table_size<AxisPlan<N, 2>>();
     BRAHMS_FOR_EACH_SIZE(BRAHMS_W_CASE)
 #undef BRAHMS_W_CASE
     default:
@@ -98,11 +100,11 @@ static int radices(int* r) {
   for (int p = 0; p < PL::NP; ++p) r[p] = PL::r(p);
   return PL::NP;
 }
-static int plan_radices(int n, bool rows, int* r) {
+static int plan_radices(int n, int axis, int* r) {
   switch (n) {
 #define BRAHMS_R_CASE(N) \
   case N:                \
-    return rows ? radices<FftPlan<N>>(r) : radices<ColPlan<N>>(r);
+    return axis == 0 ? radices<AxisPlan<N, 0>>(r) : axis == 1 ? radices<AxisPlan<N, 1>>(r) : radices<AxisPlan<N, 2>>(r);
     BRAHMS_FOR_EACH_SIZE(BRAHMS_R_CASE)
 #undef BRAHMS_R_CASE
     default:
@@ -115,9 +117,9 @@ static int centred(int d, int n) { return d >= (n + 1) / 2 ? d - n : d; }
 // Per-pass twiddle blocks (the layout of tw_pass_off): for each pass P >= 1 with
 // radix R after stride NS, entries [r][m] = the shears (-tan(phi/2), sin(phi)) of
 // phi = -2 pi r' m' / (NS R), the digits of r and m centred, evaluated in FP64.
-cudaError_t upload_twiddles(float2* tw, int n, bool rows, cudaStream_t s) {
+cudaError_t upload_twiddles(float2* tw, int n, int axis, cudaStream_t s) {
   int rad[8];
-  const int np = plan_radices(n, rows, rad);
+  const int np = plan_radices(n, axis, rad);
   if (np <= 0) return cudaErrorInvalidValue;
   std::vector<float2> h;
   int ns = 1;
@@ -138,7 +140,7 @@ cudaError_t upload_twiddles(float2* tw, int n, bool rows, cudaStream_t s) {
     ns *= rad[q];
   }
   if (h.empty()) h.push_back(make_float2(0.f, 0.f));
-  if ((int)h.size() != tw_table_size_of(n, rows)) return cudaErrorInvalidValue;
+  if ((int)h.size() != tw_table_size_of(n, axis)) return cudaErrorInvalidValue;
   cudaError_t e = cudaMemcpyAsync(tw, h.data(), sizeof(float2) * h.size(), cudaMemcpyHostToDevice, s);
   if (e != cudaSuccess) return e;
   return cudaStreamSynchronize(s);  // h is a local buffer

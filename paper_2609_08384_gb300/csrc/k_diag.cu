@@ -157,7 +157,7 @@ cudaError_t run_power_trace(const float2* data, int nx, int ny, int nt, int nf, 
 
 template <int N>
 static cudaError_t launch_spectrum(const AxisArgs& a, double* out, cudaStream_t s) {
-  using PL = ColPlan<N>;
+  using PL = TauPlan<N>;
   constexpr int TPC = tiles_per_cta<PL>();
   constexpr int THREADS = TPC * tile_threads<PL>();
   const size_t smem = (size_t)axis_smem_floats2<PL>() * sizeof(float2);

@@ -71,6 +71,11 @@ struct AxisArgs {
   int conj_p;             // apply conj(P) (the adjoint of the linear step)
 };
 
+// plan of length N on an axis (0 x, 1 y, 2 tau)
+template <int N, int AXIS>
+using AxisPlan = typename std::conditional<AXIS == 0, FftPlan<N>,
+                                           typename std::conditional<AXIS == 1, ColPlan<N>, TauPlan<N>>::type>::type;
+
 // ------------------------------------------------------------ tile shapes
 template <int N>
 __host__ __device__ constexpr int fft_threads() { return FftPlan<N>::T; }
@@ -846,10 +851,10 @@ cudaError_t make_tau_tensor_map(void* map128, const float2* data, int nx, int ny
 cudaError_t run_tpass_prop_tma(int nt, int tx, const void* map128, const AxisArgs& a, int* err,
                                unsigned long long wait_ns, cudaStream_t s);
 
-// per-pass twiddle table of the plan of length n on rows (x) or strided axes (y,
-// tau), built on the host in FP64, and its size in entries
-int tw_table_size_of(int n, bool rows);
-cudaError_t upload_twiddles(float2* tw, int n, bool rows, cudaStream_t s);
+// per-pass twiddle table of the plan of length n on an axis (0 x, 1 y, 2 tau), built
+// on the host in FP64, and its size in entries
+int tw_table_size_of(int n, int axis);
+cudaError_t upload_twiddles(float2* tw, int n, int axis, cudaStream_t s);
 struct TableArgs {
   float2* px;
   float2* py;
