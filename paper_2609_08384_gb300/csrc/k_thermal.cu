@@ -17,9 +17,17 @@
 //                    28 (1980), with the sine transform read off the cosine
 //                    transform of the sign-alternated line), and its
 //                    synthesis undoes those steps one by one.  The FFT is an
-//                    in-place Stockham FFT in FP64 shared memory, radix 2 and
-//                    3, with one barrier between the reads and the writes of
-//                    every stage.
+//                    in-place Stockham FFT in FP64 shared memory, radix 4, 2
+//                    and 3, with one barrier between the reads and the writes of
+//                    every stage.  The axis solved last keeps its coefficients in
+//                    shared memory between analysis, division and synthesis, and
+//                    the last synthesis writes the map: three kernels, one if y
+//                    has a single point.  With the host's wait 104 us at 512 x 512,
+//                    0.32 ms at 1024 x 1024 and 4.5 ms at 4096 x 4096; as a copy,
+//                    four line kernels of radix 2, a division (FP64 sines per
+//                    point) and a map kernel 199 us, 0.54 and 7.8 ms.  Bound by the
+//                    FP64 pipe and, up to 512 points a line (3.4 lines of two
+//                    warps an SM), by latency.
 #include "kernels.cuh"
 #include "launch_cfg.h"
 
@@ -30,13 +38,28 @@ namespace {
 constexpr int kHeatX = 64;    // x-points per CTA (32 pairs)
 constexpr int kHeatLanes = 8;  // tau-lanes per CTA
 constexpr int kHeatU = 8;      // tau samples per thread and iteration
-constexpr int kSineThreads = 256;
-constexpr int kSineMaxB2 = 8;  // radix-2 butterflies per thread: m / 2 <= 8 * 256, m <= 4096
-constexpr int kSineMaxB3 = 2;  // radix-3 butterflies per thread: m / 3 <= 2 * 256
 constexpr int kSineMaxStages = 16;
+// Threads of a line, and butterflies per thread and stage of radix 2, 3 and 4.  A line
+// of 512 points has 64 radix-4 butterflies a stage, so two warps keep all their threads
+// at work.  Lines of up to 512 points have m = n / 2 <= 256, the longer ones m <= 2048.
+template <int TH, int B2, int B3, int B4>
+struct SineShape {
+  static constexpr int kThreads = TH, kB2 = B2, kB3 = B3, kB4 = B4;
+};
+using SineShort = SineShape<64, 2, 1, 1>;
+using SineLong = SineShape<256, 4, 1, 2>;
 
 struct SineArgs {
-  double* d;
+  const double* in;   // lines of the input and of the output (the same layout)
+  double* out;
+  // the Laplacian's symbol along this axis: 1 / (kappa (mu_k + mu of the
+  // other axis)), with 4 / d^2 of this axis and of the other (0 if it has length 1)
+  double kappa, c_this, c_other;
+  const double2* tw_other;
+  int n_other;
+  double dkdT;        // map output (synthesis): dkmap = dkdT T, *bad set if T is not finite
+  double* dkmap;
+  int* bad;
   const double2* tw;  // 2n entries: e^{-i pi j / n} (j < n), then e^{-i pi k / (2n)} (k < n)
   long long elem;     // stride between the entries of a line
   long long pitch;    // stride between lines
@@ -59,39 +82,72 @@ __device__ __forceinline__ double2 sine_tw(const double2* tw, int m, int e, bool
 }
 
 // unnormalised DFT of buf[0..m) in place: sign -1 (forward) or +1 (inv)
+// The radix-2 and radix-4 stages come first, so that ns is a power of two in them.
+template <class S>
 __device__ void fft64_inplace(double2* buf, const SineArgs& a, int m, bool inv) {
   int ns = 1;
-  for (int s = 0; s < a.nst; ++s) {
-    const int R = a.rad[s];
+  for (int st = 0; st < a.nst; ++st) {
+    const int R = a.rad[st];
     const int nb = m / R;
     const int step = m / (ns * R);
-    if (R == 2) {
-      double2 v[kSineMaxB2][2];
+    if (R == 4) {
+      double2 v[S::kB4][4];
 #pragma unroll
-      for (int b = 0; b < kSineMaxB2; ++b) {
-        const int j = threadIdx.x + b * kSineThreads;
+      for (int b = 0; b < S::kB4; ++b) {
+        const int j = threadIdx.x + b * S::kThreads;
         if (j < nb) {
-          const int k = j % ns;
-          v[b][0] = buf[j];
-          v[b][1] = z_mul(buf[j + nb], sine_tw(a.tw, m, k * step, inv));
+          const int e = (j & (ns - 1)) * step;
+#pragma unroll
+          for (int r = 0; r < 4; ++r) v[b][r] = buf[j + r * nb];
+          if (ns > 1) {
+#pragma unroll
+            for (int r = 1; r < 4; ++r) v[b][r] = z_mul(v[b][r], sine_tw(a.tw, m, r * e, inv));
+          }
         }
       }
       __syncthreads();
 #pragma unroll
-      for (int b = 0; b < kSineMaxB2; ++b) {
-        const int j = threadIdx.x + b * kSineThreads;
+      for (int b = 0; b < S::kB4; ++b) {
+        const int j = threadIdx.x + b * S::kThreads;
         if (j < nb) {
-          const int k = j % ns;
-          const int base = (j / ns) * ns * 2 + k;
+          const int base = 4 * j - 3 * (j & (ns - 1));
+          const double2 t0 = make_double2(v[b][0].x + v[b][2].x, v[b][0].y + v[b][2].y);
+          const double2 t1 = make_double2(v[b][0].x - v[b][2].x, v[b][0].y - v[b][2].y);
+          const double2 t2 = make_double2(v[b][1].x + v[b][3].x, v[b][1].y + v[b][3].y);
+          const double2 t3 = make_double2(v[b][1].x - v[b][3].x, v[b][1].y - v[b][3].y);
+          const double2 lo = make_double2(t1.x + t3.y, t1.y - t3.x);  // t1 - i t3
+          const double2 hi = make_double2(t1.x - t3.y, t1.y + t3.x);
+          buf[base] = make_double2(t0.x + t2.x, t0.y + t2.y);
+          buf[base + ns] = inv ? hi : lo;
+          buf[base + 2 * ns] = make_double2(t0.x - t2.x, t0.y - t2.y);
+          buf[base + 3 * ns] = inv ? lo : hi;
+        }
+      }
+    } else if (R == 2) {
+      double2 v[S::kB2][2];
+#pragma unroll
+      for (int b = 0; b < S::kB2; ++b) {
+        const int j = threadIdx.x + b * S::kThreads;
+        if (j < nb) {
+          v[b][0] = buf[j];
+          v[b][1] = z_mul(buf[j + nb], sine_tw(a.tw, m, (j & (ns - 1)) * step, inv));
+        }
+      }
+      __syncthreads();
+#pragma unroll
+      for (int b = 0; b < S::kB2; ++b) {
+        const int j = threadIdx.x + b * S::kThreads;
+        if (j < nb) {
+          const int base = 2 * j - (j & (ns - 1));
           buf[base] = make_double2(v[b][0].x + v[b][1].x, v[b][0].y + v[b][1].y);
           buf[base + ns] = make_double2(v[b][0].x - v[b][1].x, v[b][0].y - v[b][1].y);
         }
       }
     } else {
-      double2 v[kSineMaxB3][3];
+      double2 v[S::kB3][3];
 #pragma unroll
-      for (int b = 0; b < kSineMaxB3; ++b) {
-        const int j = threadIdx.x + b * kSineThreads;
+      for (int b = 0; b < S::kB3; ++b) {
+        const int j = threadIdx.x + b * S::kThreads;
         if (j < nb) {
           const int k = j % ns;
           v[b][0] = buf[j];
@@ -103,11 +159,10 @@ __device__ void fft64_inplace(double2* buf, const SineArgs& a, int m, bool inv) 
       // X1,2 = x0 - (x1 + x2) / 2 -+ i s (sqrt(3) / 2) (x1 - x2), s = +1 forward, -1 inverse
       const double h3 = inv ? -0.86602540378443864676 : 0.86602540378443864676;
 #pragma unroll
-      for (int b = 0; b < kSineMaxB3; ++b) {
-        const int j = threadIdx.x + b * kSineThreads;
+      for (int b = 0; b < S::kB3; ++b) {
+        const int j = threadIdx.x + b * S::kThreads;
         if (j < nb) {
-          const int k = j % ns;
-          const int base = (j / ns) * ns * 3 + k;
+          const int base = 3 * j - 2 * (j % ns);
           const double2 x0 = v[b][0], x1 = v[b][1], x2 = v[b][2];
           const double2 t1 = make_double2(x1.x + x2.x, x1.y + x2.y);
           const double2 t2 = make_double2(x0.x - 0.5 * t1.x, x0.y - 0.5 * t1.y);
@@ -139,69 +194,111 @@ __device__ void fft64_inplace(double2* buf, const SineArgs& a, int m, bool inv) 
 // Z_q = E_q + i O_q with E_q = (V_q + conj V_{m-q}) / 2 and
 // O_q = e^{2 pi i q / n} (V_q - conj V_{m-q}) / 2, the inverse n/2-point DFT, and
 // the unpacking.
-template <bool SYNTH>
-__global__ void __launch_bounds__(kSineThreads) sine_lines_kernel(const SineArgs a) {
-  extern __shared__ double2 zbuf[];
+// A kernel does the analysis, the synthesis, or, along the axis that is solved
+// last, both with the division by the eigenvalues between them (the coefficients
+// stay in shared memory).
+enum SineMode : int { kAnalysis = 0, kSynthesis = 1, kSolve = 2 };
+
+// analysis of the line src (entries elem apart): S_k goes to put(k - 1, S_k)
+template <class S, class Put>
+__device__ __forceinline__ void sine_analysis(const SineArgs& a, double2* zbuf, const double* src, Put put) {
   const int n = a.n, m = n / 2;
   const double2* th = a.tw + n;  // e^{-i pi k / (2n)}
-  double* p = a.d + (long long)blockIdx.x * a.pitch;
-  if (!SYNTH) {
-    // z_q = v_{2q} + i v_{2q+1}, v_i = x'_{2i} (i < m) or x'_{2n-1-2i} (i >= m)
-    for (int q = threadIdx.x; q < m; q += kSineThreads) {
-      double c[2];
+  // z_q = v_{2q} + i v_{2q+1}, v_i = x'_{2i} (i < m) or x'_{2n-1-2i} (i >= m)
+  for (int q = threadIdx.x; q < m; q += S::kThreads) {
+    double c[2];
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int i = 2 * q + h;
-        const int jj = i < m ? 2 * i : 2 * n - 1 - 2 * i;
-        const double x = p[(long long)jj * a.elem];
-        c[h] = (jj & 1) ? -x : x;
-      }
-      zbuf[q] = make_double2(c[0], c[1]);
+    for (int h = 0; h < 2; ++h) {
+      const int i = 2 * q + h;
+      const int jj = i < m ? 2 * i : 2 * n - 1 - 2 * i;
+      const double x = src[(long long)jj * a.elem];
+      c[h] = (jj & 1) ? -x : x;
     }
-  } else {
-    // Z_q from the coefficients: C_k = a[n-1-k] (k >= 1), C_0 = a[n-1]
-    for (int q = threadIdx.x; q < m; q += kSineThreads) {
-      double2 v[2];
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int k = h == 0 ? q : m - q;
-        const double ck = k == 0 ? p[(long long)(n - 1) * a.elem] : p[(long long)(n - 1 - k) * a.elem];
-        const double cn = k == 0 ? 0.0 : p[(long long)(k - 1) * a.elem];
-        const double2 w = th[k];  // V_k = conj(w_k) (C_k - i C_{n-k})
-        v[h] = make_double2(w.x * ck - w.y * cn, -w.y * ck - w.x * cn);
-      }
-      const double2 vq = v[0], vc = make_double2(v[1].x, -v[1].y);  // V_q, conj V_{m-q}
-      const double2 e = make_double2(0.5 * (vq.x + vc.x), 0.5 * (vq.y + vc.y));
-      const double2 d = make_double2(0.5 * (vq.x - vc.x), 0.5 * (vq.y - vc.y));
-      const double2 wq = a.tw[2 * q];  // e^{-2 pi i q / n}; O_q = conj(wq) d
-      const double2 o = make_double2(wq.x * d.x + wq.y * d.y, wq.x * d.y - wq.y * d.x);
-      zbuf[q] = make_double2(e.x - o.y, e.y + o.x);  // E + i O
-    }
+    zbuf[q] = make_double2(c[0], c[1]);
   }
   __syncthreads();
-  fft64_inplace(zbuf, a, m, SYNTH);
-  if (!SYNTH) {
-    for (int k = threadIdx.x; k <= m; k += kSineThreads) {
-      const double2 zk = zbuf[k % m], zr = zbuf[(m - k) % m];
-      const double2 zc = make_double2(zr.x, -zr.y);
-      const double2 e = make_double2(0.5 * (zk.x + zc.x), 0.5 * (zk.y + zc.y));
-      const double2 o = make_double2(0.5 * (zk.y - zc.y), -0.5 * (zk.x - zc.x));  // (Z_k - conj Z_{m-k}) / (2i)
-      const double2 wk = k < m ? a.tw[2 * k] : make_double2(-1.0, 0.0);        // e^{-2 pi i k / n}
-      const double2 vk = make_double2(e.x + wk.x * o.x - wk.y * o.y, e.y + wk.x * o.y + wk.y * o.x);
-      const double2 w = th[k];
-      const double ur = w.x * vk.x - w.y * vk.y, ui = w.x * vk.y + w.y * vk.x;  // w_k V_k
-      if (k < m) p[(long long)(k == 0 ? n - 1 : n - 1 - k) * a.elem] = ur;        // C_k
-      if (k >= 1) p[(long long)(k - 1) * a.elem] = -ui;                           // C_{n-k}
+  fft64_inplace<S>(zbuf, a, m, false);
+  for (int k = threadIdx.x; k <= m; k += S::kThreads) {
+    const double2 zk = zbuf[k % m], zr = zbuf[(m - k) % m];
+    const double2 zc = make_double2(zr.x, -zr.y);
+    const double2 e = make_double2(0.5 * (zk.x + zc.x), 0.5 * (zk.y + zc.y));
+    const double2 o = make_double2(0.5 * (zk.y - zc.y), -0.5 * (zk.x - zc.x));  // (Z_k - conj Z_{m-k}) / (2i)
+    const double2 wk = k < m ? a.tw[2 * k] : make_double2(-1.0, 0.0);        // e^{-2 pi i k / n}
+    const double2 vk = make_double2(e.x + wk.x * o.x - wk.y * o.y, e.y + wk.x * o.y + wk.y * o.x);
+    const double2 w = th[k];
+    const double ur = w.x * vk.x - w.y * vk.y, ui = w.x * vk.y + w.y * vk.x;  // w_k V_k
+    if (k < m) put(k == 0 ? n - 1 : n - 1 - k, ur);                            // C_k
+    if (k >= 1) put(k - 1, -ui);                                               // C_{n-k}
+  }
+}
+
+// synthesis from the coefficients get(k - 1): x_j goes to put(j, x_j)
+template <class S, class Get, class Put>
+__device__ __forceinline__ void sine_synthesis(const SineArgs& a, double2* zbuf, Get get, Put put) {
+  const int n = a.n, m = n / 2;
+  const double2* th = a.tw + n;
+  // Z_q from the coefficients: C_k = a[n-1-k] (k >= 1), C_0 = a[n-1]
+  for (int q = threadIdx.x; q < m; q += S::kThreads) {
+    double2 v[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int k = h == 0 ? q : m - q;
+      const double ck = k == 0 ? get(n - 1) : get(n - 1 - k);
+      const double cn = k == 0 ? 0.0 : get(k - 1);
+      const double2 w = th[k];  // V_k = conj(w_k) (C_k - i C_{n-k})
+      v[h] = make_double2(w.x * ck - w.y * cn, -w.y * ck - w.x * cn);
     }
+    const double2 vq = v[0], vc = make_double2(v[1].x, -v[1].y);  // V_q, conj V_{m-q}
+    const double2 e = make_double2(0.5 * (vq.x + vc.x), 0.5 * (vq.y + vc.y));
+    const double2 d = make_double2(0.5 * (vq.x - vc.x), 0.5 * (vq.y - vc.y));
+    const double2 wq = a.tw[2 * q];  // e^{-2 pi i q / n}; O_q = conj(wq) d
+    const double2 o = make_double2(wq.x * d.x + wq.y * d.y, wq.x * d.y - wq.y * d.x);
+    zbuf[q] = make_double2(e.x - o.y, e.y + o.x);  // E + i O
+  }
+  __syncthreads();
+  fft64_inplace<S>(zbuf, a, m, true);
+  const double inv_m = 1.0 / (double)m;
+  for (int j = threadIdx.x; j < n; j += S::kThreads) {
+    // x_j = (-1)^j x'_j, x'_{2i} = v_i, x'_{2i+1} = v_{n-1-i}, v_i from z_{i/2}
+    const int i = (j & 1) ? n - 1 - (j >> 1) : (j >> 1);
+    const double2 zq = zbuf[i >> 1];
+    const double v = ((i & 1) ? zq.y : zq.x) * inv_m;
+    put(j, (j & 1) ? -v : v);
+  }
+}
+
+// sin(pi (k + 1) / (2n)) from the table of e^{-i pi k / (2n)}
+__device__ __forceinline__ double half_sine(const double2* tw, int n, int k) { return k + 1 < n ? -tw[n + k + 1].y : 1.0; }
+
+template <class S, int MODE>
+__global__ void __launch_bounds__(S::kThreads) sine_lines_kernel(const SineArgs a) {
+  extern __shared__ double2 zbuf[];
+  const long long line = (long long)blockIdx.x * a.pitch;
+  const double* src = a.in + line;
+  double* dst = a.out + line;
+  const auto store = [&](int j, double v) {
+    const long long at = (long long)j * a.elem;
+    dst[at] = v;
+    if (a.dkmap) {
+      if (!isfinite(v)) atomicOr(a.bad, 1);
+      a.dkmap[line + at] = a.dkdT * v;
+    }
+  };
+  if constexpr (MODE == kAnalysis) {
+    sine_analysis<S>(a, zbuf, src, store);
+  } else if constexpr (MODE == kSynthesis) {
+    sine_synthesis<S>(a, zbuf, [&](int k) { return src[(long long)k * a.elem]; }, store);
   } else {
-    const double inv_m = 1.0 / (double)m;
-    for (int j = threadIdx.x; j < n; j += kSineThreads) {
-      // x_j = (-1)^j x'_j, x'_{2i} = v_i, x'_{2i+1} = v_{n-1-i}, v_i from z_{i/2}
-      const int i = (j & 1) ? n - 1 - (j >> 1) : (j >> 1);
-      const double2 zq = zbuf[i >> 1];
-      const double v = ((i & 1) ? zq.y : zq.x) * inv_m;
-      p[(long long)j * a.elem] = (j & 1) ? -v : v;
-    }
+    // T-hat = Q-hat / (kappa mu), mu = 4 sin^2(pi (k+1) / (2n)) / d^2 + (same of the other axis)
+    double* coef = reinterpret_cast<double*>(zbuf + a.n / 2);
+    const double so = a.c_other != 0.0 ? half_sine(a.tw_other, a.n_other, (int)blockIdx.x) : 0.0;
+    const double mu_other = a.c_other * so * so;
+    sine_analysis<S>(a, zbuf, src, [&](int k, double v) {
+      const double s = half_sine(a.tw, a.n, k);
+      coef[k] = v / (a.kappa * (a.c_this * s * s + mu_other));
+    });
+    __syncthreads();
+    sine_synthesis<S>(a, zbuf, [&](int k) { return coef[k]; }, store);
   }
 }
 
@@ -215,28 +312,6 @@ __global__ void sine_twiddles_kernel(double2* tw, int n) {
   else
     sincospi(-(double)(j - n) / (2.0 * n), &sn, &cs);
   tw[j] = make_double2(cs, sn);
-}
-
-// T-hat /= kappa mu_pq, mu_pq = 4 sin^2(pi (p+1) / (2 nx)) / dx^2 + (same in y)
-__global__ void thermal_divide_kernel(double* d, int nx, int ny, double dx, double dy, double kappa) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (long long)nx * ny) return;
-  const int p = (int)(i % nx), q = (int)(i / nx);
-  const double sx = sinpi((double)(p + 1) / (2.0 * nx));
-  double mu = 4.0 * sx * sx / (dx * dx);
-  if (ny > 1) {
-    const double sy = sinpi((double)(q + 1) / (2.0 * ny));
-    mu += 4.0 * sy * sy / (dy * dy);
-  }
-  d[i] /= kappa * mu;
-}
-
-__global__ void thermal_map_kernel(const double* __restrict__ t, long long n, double dkdT, double* dkmap, int* bad) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const double v = t[i];
-  if (!isfinite(v)) atomicOr(bad, 1);
-  dkmap[i] = dkdT * v;
 }
 
 __global__ void __launch_bounds__(kHeatX / 2 * kHeatLanes) heat_load_kernel(const HeatArgs a) {
@@ -300,46 +375,54 @@ __global__ void __launch_bounds__(kHeatX / 2 * kHeatLanes) heat_load_kernel(cons
   }
 }
 
-bool sine_plan(int n, SineArgs& a) {
-  if (n < 2 || n % 2) return false;
-  int m = n / 2, st = 0;
-  while (m % 2 == 0) {
-    if (st == kSineMaxStages) return false;
-    a.rad[st++] = 2;
-    m /= 2;
-  }
-  while (m % 3 == 0) {
-    if (st == kSineMaxStages) return false;
-    a.rad[st++] = 3;
-    m /= 3;
-  }
-  if (m != 1) return false;
-  a.nst = st;
-  a.n = n;
-  const int mm = n / 2;
-  for (int s = 0; s < st; ++s) {
-    const int nb = mm / a.rad[s];
-    const int cap = (a.rad[s] == 2 ? kSineMaxB2 : kSineMaxB3) * kSineThreads;
-    if (nb > cap) return false;
+template <class S>
+bool stages_fit(const SineArgs& a, int m) {
+  for (int st = 0; st < a.nst; ++st) {
+    const int per_thread = a.rad[st] == 4 ? S::kB4 : a.rad[st] == 2 ? S::kB2 : S::kB3;
+    if (m / a.rad[st] > per_thread * S::kThreads) return false;
   }
   return true;
 }
 
-template <bool SYNTH>
-cudaError_t sine_lines(double* d, const double2* tw, int n, long long elem, long long pitch, int lines,
-                       cudaStream_t s) {
-  SineArgs a{};
+// the lines that the short shape takes
+bool short_line(int n) { return n <= 512; }
+
+bool sine_plan(int n, SineArgs& a) {
+  if (n < 2 || n % 2) return false;
+  int m = n / 2, st = 0;
+  while (m % 2 == 0 || m % 3 == 0) {
+    if (st == kSineMaxStages) return false;
+    a.rad[st] = m % 4 == 0 ? 4 : m % 2 == 0 ? 2 : 3;
+    m /= a.rad[st++];
+  }
+  if (m != 1) return false;
+  a.nst = st;
+  a.n = n;
+  return short_line(n) ? stages_fit<SineShort>(a, n / 2) : stages_fit<SineLong>(a, n / 2);
+}
+
+template <class S, int MODE>
+cudaError_t launch_sine_lines(const SineArgs& a, int lines, cudaStream_t s) {
+  // the FFT's n/2 complex points, and the n coefficients of a solve
+  const size_t smem = sizeof(double2) * (size_t)(a.n / 2) * (MODE == kSolve ? 2 : 1);
+  static SmemMax limit;
+  cudaError_t e = raise_smem_limit_to(sine_lines_kernel<S, MODE>, std::max<size_t>(smem, 48 * 1024), limit);
+  if (e != cudaSuccess) return e;
+  sine_lines_kernel<S, MODE><<<lines, S::kThreads, smem, s>>>(a);
+  return cudaPeekAtLastError();
+}
+
+// lines of length n, elem between a line's entries and pitch between lines
+template <int MODE>
+cudaError_t sine_lines(SineArgs a, const double* in, double* out, const double2* tw, int n, long long elem,
+                       long long pitch, int lines, cudaStream_t s) {
   if (!sine_plan(n, a)) return cudaErrorInvalidValue;
-  a.d = d;
+  a.in = in;
+  a.out = out;
   a.tw = tw;
   a.elem = elem;
   a.pitch = pitch;
-  const size_t smem = sizeof(double2) * (size_t)(n / 2);
-  static SmemMax limit;
-  cudaError_t e = raise_smem_limit_to(sine_lines_kernel<SYNTH>, std::max<size_t>(smem, 48 * 1024), limit);
-  if (e != cudaSuccess) return e;
-  sine_lines_kernel<SYNTH><<<lines, kSineThreads, smem, s>>>(a);
-  return cudaPeekAtLastError();
+  return short_line(n) ? launch_sine_lines<SineShort, MODE>(a, lines, s) : launch_sine_lines<SineLong, MODE>(a, lines, s);
 }
 
 }  // namespace
@@ -375,23 +458,27 @@ cudaError_t run_map_add(double* dkmap, const double* base, long long n, cudaStre
   return cudaPeekAtLastError();
 }
 
+// The solve: analysis along x (of the load), the solve along y, synthesis along x,
+// which also writes the map; one kernel along x where y has a single point.
 cudaError_t run_thermal_solve(const ThermalArgs& a, int* nlaunch, cudaStream_t s) {
-  const long long n = (long long)a.nx * a.ny;
-  int nl = 0;
-  cudaError_t e = cudaMemcpyAsync(a.temp, a.heat, sizeof(double) * n, cudaMemcpyDeviceToDevice, s);
-  if (e == cudaSuccess) e = sine_lines<false>(a.temp, a.twx, a.nx, 1, a.nx, a.ny, s), ++nl;
-  if (e == cudaSuccess && a.ny > 1) e = sine_lines<false>(a.temp, a.twy, a.ny, a.nx, 1, a.nx, s), ++nl;
-  if (e == cudaSuccess) {
-    thermal_divide_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(a.temp, a.nx, a.ny, a.dx, a.dy, a.kappa);
-    e = cudaPeekAtLastError(), ++nl;
+  SineArgs plain{}, solve{}, map{};
+  map.dkdT = a.dkdT;
+  map.dkmap = a.dkmap;
+  map.bad = a.bad;
+  solve.kappa = a.kappa;
+  *nlaunch = a.ny > 1 ? 3 : 1;
+  if (a.ny == 1) {
+    map.kappa = a.kappa;
+    map.c_this = 4.0 / (a.dx * a.dx);
+    return sine_lines<kSolve>(map, a.heat, a.temp, a.twx, a.nx, 1, a.nx, 1, s);
   }
-  if (e == cudaSuccess && a.ny > 1) e = sine_lines<true>(a.temp, a.twy, a.ny, a.nx, 1, a.nx, s), ++nl;
-  if (e == cudaSuccess) e = sine_lines<true>(a.temp, a.twx, a.nx, 1, a.nx, a.ny, s), ++nl;
-  if (e == cudaSuccess) {
-    thermal_map_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(a.temp, n, a.dkdT, a.dkmap, a.bad);
-    e = cudaPeekAtLastError(), ++nl;
-  }
-  *nlaunch = nl;
+  solve.c_this = 4.0 / (a.dy * a.dy);
+  solve.c_other = 4.0 / (a.dx * a.dx);
+  solve.tw_other = a.twx;
+  solve.n_other = a.nx;
+  cudaError_t e = sine_lines<kAnalysis>(plain, a.heat, a.temp, a.twx, a.nx, 1, a.nx, a.ny, s);
+  if (e == cudaSuccess) e = sine_lines<kSolve>(solve, a.temp, a.temp, a.twy, a.ny, a.nx, 1, a.nx, s);
+  if (e == cudaSuccess) e = sine_lines<kSynthesis>(map, a.temp, a.temp, a.twx, a.nx, 1, a.nx, a.ny, s);
   return e;
 }
 

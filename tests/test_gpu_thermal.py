@@ -333,3 +333,33 @@ def test_thermal_status_codes():
     s.heat_set(np.ones((8, 16)))
     assert np.isfinite(s.thermal_map(1.0, 1.0)).all()
     s.close()
+
+
+@pytest.mark.parametrize("nx,ny", [(512, 1), (1024, 1), (4096, 1), (512, 1024), (1024, 16), (24, 512), (2, 128), (128, 2)])
+def test_thermal_solve_line_shapes_and_their_map(nx, ny):
+    """Lines on either side of 512 points (64 and 256 threads), one and two axes: the
+    temperature against the direct solve, and the map that the last kernel writes: a
+    propagation under it equals, bit for bit, one under dkdT T set as a map."""
+    br = _br()
+    g = wl.Grid(nx, ny, 1, 2.5e-6, 4e-6, 1e-15)
+    rng = np.random.default_rng(nx * 5 + ny)
+    q = rng.standard_normal((ny, nx)) * 1e9 + 5e8
+    want = oracle.thermal_solve(q, g.dx, g.dy, 4.6)
+    f0 = _random_fields(g, 2, rng, amp=1e6)
+    s = br.Solver(g, _fields(2), wl.D_EFF, 50.0)
+    nz, dz = 4, 50e-6
+    dkdT = 1.0 / (np.abs(want).max() * nz * dz)
+    s.heat_set(q)
+    t = s.thermal_map(4.6, dkdT)
+    assert np.abs(t - want).max() / np.abs(want).max() < SOLVE_TOL
+    s.set_fields(_dev(f0))
+    s.propagate(nz, dz)
+    under_solve = [np.asarray(a) for a in s.get_fields()]
+    s.close()
+    s = br.Solver(g, _fields(2), wl.D_EFF, 50.0)
+    s.set_dk_map(dkdT * t)
+    s.set_fields(_dev(f0))
+    s.propagate(nz, dz)
+    for a, b in zip(under_solve, s.get_fields()):
+        assert np.array_equal(a, np.asarray(b))
+    s.close()
