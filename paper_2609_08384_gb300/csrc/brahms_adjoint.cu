@@ -296,25 +296,29 @@ brahms_status brahms_adjoint_backward(brahms_ctx* ctx, double gscale, double* gr
   float2* recB = ctx->adj_seg;
   float2* recA = ctx->adj_seg + (size_t)K * nf * n;
   // reverse x-pass at boundary b (xa: A_b or NULL, xb: a2_{b-1} or NULL)
-  auto reverse_x = [&](int b, const float2* xa, const float2* xb) -> brahms_status {
+  auto reverse_x = [&](int b, const float2* xa, bool xa_is_checkpoint, const float2* xb) -> brahms_status {
     brahms::XAdjArgs r{};
     r.g = ctx->adj_g;
     r.xa = xa;
     r.xb = xb;
+    r.xa_row_order = xa_is_checkpoint ? 1 : 0;
     r.fstride = n;
     r.rows = (long long)ctx->ny * ctx->nt;
     r.tw = ctx->twx;
     r.from_k = b < nz ? 1 : 0;
     r.to_k = b > 0 ? 1 : 0;
-    r.h = 0.5 * dz;
-    for (int f = 0; f < nf; ++f) r.kh[f] = base.kh[f];
+    r.dz = dz;
+    for (int f = 0; f < nf; ++f) {
+      r.kh[f] = base.kh[f];
+      r.kh2[f] = base.kh2[f];
+    }
     if (xa) {
       r.phiA = ctx->adj_phis[b];
       r.dkA = dk_at(b);
     }
     if (xb) {
       r.dkB = dk_at(b - 1);
-      r.phiB = ctx->adj_phis[b - 1] + r.dkB * 0.5 * dz;
+      r.phiB = ctx->adj_phis[b - 1];
     }
     r.partial = ctx->adj_part;
     r.ny = ctx->ny;
@@ -349,7 +353,7 @@ brahms_status brahms_adjoint_backward(brahms_ctx* ctx, double gscale, double* gr
                                  : (b == j1 ? ctx->adj_ckpt + (size_t)(seg + 1) * nf * n
                                             : recA + (size_t)(b - j0) * nf * n);
       const float2* xb = recB + (size_t)(b - 1 - j0) * nf * n;
-      brahms_status s2 = reverse_x(b, xa, xb);
+      brahms_status s2 = reverse_x(b, xa, b == j1, xb);
       if (s2 != BRAHMS_OK) return s2;
       s2 = linear_yty(ctx, ctx->adj_g, true);
       if (s2 != BRAHMS_OK) return s2;
@@ -357,7 +361,7 @@ brahms_status brahms_adjoint_backward(brahms_ctx* ctx, double gscale, double* gr
   }
   // boundary 0: the reverse of step 0's A half step, back to real space
   {
-    brahms_status s2 = reverse_x(0, ctx->adj_ckpt, nullptr);
+    brahms_status s2 = reverse_x(0, ctx->adj_ckpt, true, nullptr);
     if (s2 != BRAHMS_OK) return s2;
   }
   // mismatch gradient from the stage sensitivities

@@ -44,7 +44,8 @@ struct XPassArgs {
   const float2* emap;
   int ny;
   // recording (adjoint recomputation): real-space copies of the state that
-  // enters the B half step and of the state that enters the A half step, or NULL
+  // enters the B half step and of the state that enters the A half step, or NULL;
+  // each row in place order (park_place), as the reverse x-pass reads it
   float2* rec_b;
   float2* rec_a;
   // the stage factors of both half steps from the phases above, written by the
@@ -139,23 +140,6 @@ __host__ __device__ constexpr int axis_kernel_smem_floats2() {
 }
 
 // -------------------------------------------------------- nonlinear step
-// Right-hand sides of Eqs. CEp/CEs/CEi (3 fields p, s, i) or of the
-// degenerate SHG pair (SH, F), already multiplied by the step h, with
-//   c[f] = i kappa_f h e^{-/+ i Phi(z)}  (minus for field 0);
-// the adjoint's stage recomputation uses this form.
-template <int F>
-__device__ __forceinline__ void nl_rhs(const float2 (&a)[F], const float2* __restrict__ c,
-                                       float2 (&k)[F]) {
-  if constexpr (F == 3) {
-    k[0] = cmul(c[0], cmul(a[1], a[2]));
-    k[1] = cmul(c[1], cmulc(a[0], a[2]));
-    k[2] = cmul(c[2], cmulc(a[0], a[1]));
-  } else {
-    k[0] = cmul(c[0], cmul(a[1], a[1]));
-    k[1] = cmul(c[1], cmulc(a[0], a[1]));
-  }
-}
-
 // Two grid points at once: real and imaginary parts as FP32 pairs, so that the
 // arithmetic of both points is one packed instruction (see fft_core.cuh).
 struct Pair {
@@ -423,12 +407,9 @@ __device__ __forceinline__ void xpass_tile(const XPassArgs& p, long long tile, c
       const auto record = [&](float2* rec) {
         if (!act) return;
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-          float2* d = rec + row * NX + point_pos<PL>(t, e + u);
-#pragma unroll
-          for (int f = 0; f < F; ++f)
-            d[f * p.fstride] = u == 0 ? make_float2(a[f].re.x, a[f].im.x) : make_float2(a[f].re.y, a[f].im.y);
-        }
+        for (int f = 0; f < F; ++f)
+          *park_place<PL>(rec + f * p.fstride + row * NX, t, e / 2) =
+              make_float4(a[f].re.x, a[f].re.y, a[f].im.x, a[f].im.y);
       };
       if (mode != XM_NL_FIRST) {
         if constexpr (REC) {
@@ -954,21 +935,21 @@ struct XAdjArgs {
   float2* g;
   const float2* xa;
   const float2* xb;
+  int xa_row_order;    // xa lies in row order (a checkpoint), not as recorded
   long long fstride, rows;
   const float2* tw;
   int from_k, to_k;
-  double phiA, dkA, phiB, dkB, h;  // phase and mismatch at the start of each half step; h = dz/2
+  double phiA, dkA, phiB, dkB, dz;  // phase at the start and mismatch of the steps b (A) and b - 1 (B), as in XPassArgs
   float kh[3];                     // kappa_f h (1/2 on the SH equation for two fields)
+  float kh2[3];                    // kh / 2 (exact)
   double* partial;
   // transverse mismatch map: the per-(x, y) stage phase factors of this
   // boundary's B and A half steps [4][ny][nx] (as in XPassArgs), or NULL
   const float2* emap;
   int ny;
-  // map-free: the coefficient sets i kappa_f h e^{-/+ i Phi} at the start,
-  // middle and end of the A half step (cset[0]) and of the B half step
-  // (cset[1]), [stage][field], written by the host dispatcher in FP64 from
-  // the phases above (the stage factors the forward x-pass uses)
-  float2 cset[2][9];
+  // map-free: the stage factors as in XPassArgs, written by the host dispatcher in
+  // FP64 from the phases above
+  float2 ecoef[kStageFactors];
 };
 cudaError_t run_xpass_adjoint(int nx, int nf, const XAdjArgs& a, long long* ncta, cudaStream_t s);
 cudaError_t run_xpass_adjoint_map(int nx, int nf, const XAdjArgs& a, long long* ncta, cudaStream_t s);

@@ -1,126 +1,140 @@
-// Reverse mode of the RK4 half step (Sec. 3.1) at one grid point, shared by
-// the stand-alone VJP kernel and the fused adjoint x-pass.
+// Reverse mode of the RK4 half step (Sec. 3.1) at two grid points, the nonlinear
+// part of the reverse x-pass.
 //
 // Complex gradients follow G_z = dJ/dRe z + i dJ/dIm z.  For y = f(x):
 //   G_x = sum_y [ conj(G_y) dy/dconj(x) + G_y conj(dy/dx) ].
-// The stages are recomputed in registers from the state at the start of the
-// half step; the mismatch phase sensitivity at a stage is
+// The stages are recomputed in registers from the state at the start of the half
+// step, in the form of rk4 (kernels.cuh): field 0 as u = e^{i Phi} A_0 of the
+// stage, m the driving term of field 0 and n the slopes of the others, so that no
+// product of a stage carries a phase or a coupling.  The sensitivity to a stage's
+// phase is
 //   dJ/dPhi = sum_f Re( conj(G_k_f) dk_f/dPhi ),  dk_0/dPhi = -i k_0,
-//   dk_f/dPhi = +i k_f (f >= 1).
+//   dk_f/dPhi = +i k_f (f >= 1),
+// which is Im(conj(G_m) m) - sum_f Im(conj(G_n_f) n_f); the second sum equals
+// Im(conj(G_u) u), G_u the gradient that the stage's slopes give u, and the first
+// Im(conj(X) t) of the part X of a field's gradient that comes from m (half of it
+// for two fields), so that neither m nor n is kept.
 #pragma once
 
 #include "kernels.cuh"
 
 namespace brahms {
 
-__device__ __forceinline__ float2 cconj(float2 a) { return make_float2(a.x, -a.y); }
 // Im(conj(a) b)
 __device__ __forceinline__ float im_cb(float2 a, float2 b) { return a.x * b.y - a.y * b.x; }
+// acc + Im(conj(a) b)
+__device__ __forceinline__ float2 add_im_cb(float2 acc, Pair a, Pair b) {
+  return __ffma2_rn(a.re, b.im, __ffma2_rn(neg(a.im), b.re, acc));
+}
+// c g and -i c g for a real c; a - i c g
+__device__ __forceinline__ Pair pair_scale(float c, Pair g) { return {__fmul2_rn(dup(c), g.re), __fmul2_rn(dup(c), g.im)}; }
+__device__ __forceinline__ Pair pair_niscale(float c, Pair g) {
+  return {__fmul2_rn(dup(c), g.im), __fmul2_rn(dup(-c), g.re)};
+}
+__device__ __forceinline__ Pair pair_niaxpy(Pair a, float c, Pair g) {
+  return {__ffma2_rn(dup(c), g.im, a.re), __ffma2_rn(dup(-c), g.re, a.im)};
+}
+// acc + i a conj(b)
+__device__ __forceinline__ Pair pair_add_imulc(Pair acc, Pair a, Pair b) {
+  return {__ffma2_rn(a.re, b.im, __ffma2_rn(neg(a.im), b.re, acc.re)),
+          __ffma2_rn(a.re, b.re, __ffma2_rn(a.im, b.im, acc.im))};
+}
+// -i a b, and acc - i a b
+__device__ __forceinline__ Pair pair_nimul(Pair a, Pair b) {
+  return {__ffma2_rn(a.re, b.im, __fmul2_rn(a.im, b.re)), __ffma2_rn(a.im, b.im, neg(__fmul2_rn(a.re, b.re)))};
+}
+__device__ __forceinline__ Pair pair_add_nimul(Pair acc, Pair a, Pair b) {
+  return {__ffma2_rn(a.re, b.im, __ffma2_rn(a.im, b.re, acc.re)),
+          __ffma2_rn(a.im, b.im, __ffma2_rn(neg(a.re), b.re, acc.im))};
+}
 
-// gu += adjoint of k = f(u) (coefficients c) applied to gk
+// Reverse of one stage's products at (u, t): from the gradients gm of the driving
+// term (twice it for two fields) and gn of the slopes to those of u and t; s gains
+// the sensitivity to the stage's phase.
 template <int F>
-__device__ __forceinline__ void rhs_vjp(const float2* __restrict__ c, const float2 (&u)[F], const float2 (&gk)[F],
-                                        float2 (&gu)[F]) {
+__device__ __forceinline__ void nl_vjp(Pair u, const Pair* t, Pair gm, const Pair* gn, Pair& gu, Pair* gt, float2& s) {
+  const Pair x = pair_mulc(gm, t[F - 2]);  // what field 1's driving term takes from gm
   if constexpr (F == 3) {
-    gu[0] = cadd(gu[0], cadd(cmul(gk[1], cmul(cconj(c[1]), u[2])), cmul(gk[2], cmul(cconj(c[2]), u[1]))));
-    gu[1] = cadd(gu[1], cadd(cmul(gk[0], cmul(cconj(c[0]), cconj(u[2]))), cmul(cconj(gk[2]), cmul(c[2], u[0]))));
-    gu[2] = cadd(gu[2], cadd(cmul(gk[0], cmul(cconj(c[0]), cconj(u[1]))), cmul(cconj(gk[1]), cmul(c[1], u[0]))));
+    gu = pair_add_nimul(pair_nimul(t[1], gn[0]), t[0], gn[1]);
+    s = add_im_cb(s, x, t[0]);
+    gt[0] = pair_add_imulc(x, u, gn[1]);
+    gt[1] = pair_add_imulc(pair_mulc(gm, t[0]), u, gn[0]);
   } else {
-    gu[0] = cadd(gu[0], cmul(gk[1], cmul(cconj(c[1]), u[1])));
-    const float2 t = cmul(gk[0], cmul(cconj(c[0]), cconj(u[1])));
-    gu[1] = cadd(gu[1], cadd(cadd(t, t), cmul(cconj(gk[1]), cmul(c[1], u[0]))));
+    gu = pair_nimul(t[0], gn[0]);
+    s = __ffma2_rn(dup(0.5f), add_im_cb(make_float2(0.f, 0.f), x, t[0]), s);
+    gt[0] = pair_add_imulc(x, u, gn[0]);
   }
+  s = add_im_cb(s, {neg(gu.re), neg(gu.im)}, u);
 }
 
-// sum_f Re(conj(gk_f) dk_f/dPhi)
+// One RK4 half step in reverse at two points: x is the forward state at the start
+// of the half step, e0, v, kh and kh2 as in rk4; g enters as the gradient with
+// respect to the end state and leaves as the gradient with respect to x.  s[0],
+// s[1], s[2] gain the sensitivities to the stage phases at the start, the midpoint
+// (both middle stages) and the end.  The gradients of the stages' u are kept in the
+// stage's own frame; v and e0 take them from one to the next.
 template <int F>
-__device__ __forceinline__ float phase_sens(const float2 (&gk)[F], const float2 (&k)[F]) {
-  float s = im_cb(gk[0], k[0]);  // Re(conj(g)(-i k)) = Im(conj(g) k)
+__device__ __forceinline__ void rk4_vjp(const Pair (&x)[F], Pair (&g)[F], Pair e0, Pair v, const float* kh,
+                                        const float* kh2, float2* s) {
+  constexpr int G = F - 1;
+  const Pair* t1 = x + 1;
+  Pair t2[G], t3[G], t4[G], n[G];
+  const Pair u1 = pair_mul(e0, x[0]);
+  const Pair w = pair_mul(v, u1);
+  nl_slopes<F>(u1, t1, n);
 #pragma unroll
-  for (int f = 1; f < F; ++f) s -= im_cb(gk[f], k[f]);
-  return s;
-}
+  for (int f = 0; f < G; ++f) t2[f] = pair_axpy(t1[f], kh2[f + 1], n[f]);
+  const Pair u2 = pair_iaxpy(w, kh2[0], pair_mul(v, nl_drive<F>(t1)));
+  nl_slopes<F>(u2, t2, n);
+#pragma unroll
+  for (int f = 0; f < G; ++f) t3[f] = pair_axpy(t1[f], kh2[f + 1], n[f]);
+  const Pair u3 = pair_iaxpy(w, kh2[0], nl_drive<F>(t2));
+  nl_slopes<F>(u3, t3, n);
+#pragma unroll
+  for (int f = 0; f < G; ++f) t4[f] = pair_axpy(t1[f], kh[f + 1], n[f]);
+  const Pair u4 = pair_mul(v, pair_iaxpy(w, kh[0], nl_drive<F>(t3)));
 
-// One RK4 half step in reverse at a point: x is the forward state at the
-// start of the half step, c the coefficient sets i kappa h e^{-/+ i Phi} at
-// the start, middle and end ([3][F]); g enters as the gradient with respect
-// to the end state and leaves as the gradient with respect to x.  s0, s1, s2
-// gain the sensitivities to the stage phases at the start, the midpoint
-// (both middle stages) and the end.
-template <int F>
-__device__ __forceinline__ void rk4_vjp_point(const float2 (&x)[F], float2 (&g)[F], const float2* __restrict__ c,
-                                              float& s0, float& s1, float& s2) {
-  float2 u2[F], u3[F], u4[F], k1[F], k2[F], k3[F], k4[F];
-  nl_rhs<F>(x, c, k1);
+  // direct shares of the end state: 1/6 of its gradient to stages 1 and 4, 1/3 to 2
+  // and 3; the driving term's in the frame of the stage's u
+  const float kd = F == 2 ? 2.f * kh[0] : kh[0], kd2 = F == 2 ? kh[0] : kh2[0];
+  const Pair p1 = pair_mul(e0, g[0]), p2 = pair_mul(v, p1);
+  const Pair d23 = pair_niscale(kd * (1.f / 3.f), p2);
+  Pair dn[G], gn[G], gt[G], gu;
 #pragma unroll
-  for (int f = 0; f < F; ++f) u2[f] = make_float2(fmaf(0.5f, k1[f].x, x[f].x), fmaf(0.5f, k1[f].y, x[f].y));
-  nl_rhs<F>(u2, c + F, k2);
-#pragma unroll
-  for (int f = 0; f < F; ++f) u3[f] = make_float2(fmaf(0.5f, k2[f].x, x[f].x), fmaf(0.5f, k2[f].y, x[f].y));
-  nl_rhs<F>(u3, c + F, k3);
-#pragma unroll
-  for (int f = 0; f < F; ++f) u4[f] = cadd(x[f], k3[f]);
-  nl_rhs<F>(u4, c + 2 * F, k4);
-  // y = x + (k1 + 2 k2 + 2 k3 + k4)/6
-  float2 gx[F], g1[F], g2[F], g3[F], g4[F], gu[F];
-#pragma unroll
-  for (int f = 0; f < F; ++f) {
-    gx[f] = g[f];
-    g1[f] = cscale(g[f], 1.f / 6.f);
-    g2[f] = cscale(g[f], 1.f / 3.f);
-    g3[f] = g2[f];
-    g4[f] = g1[f];
-    gu[f] = make_float2(0.f, 0.f);
+  for (int f = 0; f < G; ++f) {
+    dn[f] = pair_scale(kh[f + 1] * (1.f / 3.f), g[f + 1]);
+    gn[f] = pair_scale(0.5f, dn[f]);
   }
-  // stage 4: u4 = x + k3
-  rhs_vjp<F>(c + 2 * F, u4, g4, gu);
-  s2 += phase_sens<F>(g4, k4);
+  // stage 4: u4 = v (w + i kh m3), t4 = A + kh n3
+  nl_vjp<F>(u4, t4, pair_niscale(kd * (1.f / 6.f), pair_mul(v, p2)), gn, gu, gt, s[2]);
+  Pair gw = pair_mulc(gu, v);
 #pragma unroll
-  for (int f = 0; f < F; ++f) {
-    gx[f] = cadd(gx[f], gu[f]);
-    g3[f] = cadd(g3[f], gu[f]);
-    gu[f] = make_float2(0.f, 0.f);
+  for (int f = 0; f < G; ++f) {
+    g[f + 1] = pair_add(g[f + 1], gt[f]);
+    gn[f] = pair_axpy(dn[f], kh[f + 1], gt[f]);
   }
-  // stage 3: u3 = x + k2/2
-  rhs_vjp<F>(c + F, u3, g3, gu);
-  s1 += phase_sens<F>(g3, k3);
+  // stage 3: u3 = w + i kh/2 m2, t3 = A + kh/2 n2
+  nl_vjp<F>(u3, t3, pair_niaxpy(d23, kd, gw), gn, gu, gt, s[1]);
+  gw = pair_add(gw, gu);
 #pragma unroll
-  for (int f = 0; f < F; ++f) {
-    gx[f] = cadd(gx[f], gu[f]);
-    g2[f] = make_float2(fmaf(0.5f, gu[f].x, g2[f].x), fmaf(0.5f, gu[f].y, g2[f].y));
-    gu[f] = make_float2(0.f, 0.f);
+  for (int f = 0; f < G; ++f) {
+    g[f + 1] = pair_add(g[f + 1], gt[f]);
+    gn[f] = pair_axpy(dn[f], kh2[f + 1], gt[f]);
   }
-  // stage 2: u2 = x + k1/2
-  rhs_vjp<F>(c + F, u2, g2, gu);
-  s1 += phase_sens<F>(g2, k2);
+  // stage 2: u2 = w + i kh/2 v m1, t2 = A + kh/2 n1
+  nl_vjp<F>(u2, t2, pair_niaxpy(d23, kd2, gu), gn, gu, gt, s[1]);
+  const Pair r = pair_mulc(gu, v);
 #pragma unroll
-  for (int f = 0; f < F; ++f) {
-    gx[f] = cadd(gx[f], gu[f]);
-    g1[f] = make_float2(fmaf(0.5f, gu[f].x, g1[f].x), fmaf(0.5f, gu[f].y, g1[f].y));
-    gu[f] = make_float2(0.f, 0.f);
+  for (int f = 0; f < G; ++f) {
+    g[f + 1] = pair_add(g[f + 1], gt[f]);
+    gn[f] = pair_axpy(pair_scale(0.5f, dn[f]), kh2[f + 1], gt[f]);
   }
-  // stage 1: u1 = x
-  rhs_vjp<F>(c, x, g1, gu);
-  s0 += phase_sens<F>(g1, k1);
+  // stage 1: u1 = e0 A_0, w = v u1
+  nl_vjp<F>(u1, t1, pair_niaxpy(pair_niscale(kd * (1.f / 6.f), p1), kd2, r), gn, gu, gt, s[0]);
 #pragma unroll
-  for (int f = 0; f < F; ++f) g[f] = cadd(gx[f], gu[f]);
-}
-
-// Coefficient sets c = i kappa_f h e^{-/+ i Phi} (minus for field 0) at the
-// start, middle and end of a half step from phase phi_a with mismatch dk
-// (thread s < 3 writes set s).
-template <int F>
-__device__ __forceinline__ void vjp_coef_sets(double phi_a, double dk, double h, const float* kh, float2* c) {
-  const int s = threadIdx.x;
-  if (s < 3) {
-    const double phi = phi_a + dk * (0.5 * h * s);
-    const float2 em = phase_minus(phi);
-#pragma unroll
-    for (int f = 0; f < F; ++f) {
-      const float k = kh[f];
-      c[s * F + f] = f == 0 ? make_float2(-em.y * k, em.x * k) : make_float2(em.y * k, em.x * k);
-    }
-  }
+  for (int f = 0; f < G; ++f) g[f + 1] = pair_add(g[f + 1], gt[f]);
+  gu = pair_add(pair_add(gu, r), pair_mulc(gw, v));
+  g[0] = pair_add(g[0], pair_mulc(gu, e0));
 }
 
 }  // namespace brahms

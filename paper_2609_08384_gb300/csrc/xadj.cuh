@@ -6,7 +6,7 @@
 // A_b and through N_A of step b.  In reverse the same boundary takes the
 // adjoint through the inverse x-FFT, the reverse of N_A at A_b, the reverse
 // of N_B at a2 and the forward x-FFT -- the structure of the forward x-pass
-// with each RK4 replaced by its vector-Jacobian product (rk4_vjp_point).
+// with each RK4 replaced by its vector-Jacobian product (rk4_vjp).
 // Between two such passes the adjoint of the linear step, IDFT3(conj(P)
 // DFT3), runs as the usual y-forward, tau-propagator (conjugated) and
 // y-inverse passes.
@@ -24,25 +24,25 @@
 
 namespace brahms {
 
-// i kappa_f h e^{-/+ i Phi} at the start, middle and end of a half step from
-// the point's start factor e0 = e^{i Phi_0} and quarter-step factor v
-template <int F>
-__device__ __forceinline__ void map_coef_sets(float2 e0, float2 v, const float* kh, float2 (&c)[3 * F]) {
-  float2 e = e0;
-#pragma unroll
-  for (int s = 0; s < 3; ++s) {
-#pragma unroll
-    for (int f = 0; f < F; ++f) {
-      const float k = kh[f];
-      c[s * F + f] = f == 0 ? make_float2(e.y * k, e.x * k) : make_float2(-e.y * k, e.x * k);
-    }
-    if (s < 2) e = cmul(e, v);
-  }
+// points 2 q and 2 q + 1 of thread t from a row in place order (as recorded) or in
+// row order
+template <class PL>
+__device__ __forceinline__ float4 load_points(const float2* row, bool row_order, int t, int q) {
+  if (!row_order) return __ldcg(reinterpret_cast<const float4*>(row) + q * PL::T + t);
+  const float2 a = __ldcg(row + point_pos<PL>(t, 2 * q)), b = __ldcg(row + point_pos<PL>(t, 2 * q + 1));
+  return make_float4(a.x, b.x, a.y, b.y);
 }
 
+// The tile of the forward x-pass (kernels.cuh: rows by asynchronous copies, parked
+// two points together), with the two RK4 half steps in reverse, on two points at a
+// time.  The recorded states come in place order, one 16-byte load a field and two
+// points.  Backward of the 2 x 128x128x256 state over 36 steps 10.65 -> 10.13 ms (so
+// about 14 of 75 us of this pass), 3 x 128x128x256 over 25 steps 11.58 -> 10.79, under
+// a map 11.87 -> 11.51 and 12.59 -> 11.74.  What bounds it: the FP32 pipe (184
+// operations a point, half step and pair of fields) beside 48 B a point and field of
+// memory traffic against the forward pass's 16.
 template <int NX, int F, int THREADS, bool MAP>
-__device__ __forceinline__ void xpass_adj_tile(const XAdjArgs& p, long long tile, const float2* cA, const float2* cB,
-                                               float2* rowbuf, float (&sens)[6]) {
+__device__ __forceinline__ void xpass_adj_tile(const XAdjArgs& p, long long tile, float2* rowbuf, float (&sens)[6]) {
   using PL = FftPlan<NX>;
   constexpr int E = PL::E;
   constexpr int T = PL::T;
@@ -50,7 +50,6 @@ __device__ __forceinline__ void xpass_adj_tile(const XAdjArgs& p, long long tile
   constexpr int PITCH = XchRow::pitch(NX);
   constexpr int RF0 = fft_radix<PL, false>(0);
   constexpr int RFL = fft_radix<PL, false>(PL::NP - 1);
-  constexpr int SF0 = NX / RF0;
   using SY = typename std::conditional<xpass_warp_sync<NX>(), SyncWarp, SyncBlock>::type;
   static_assert(ROWS >= 1 && ROWS * T == THREADS, "CTA must hold whole rows");
   const TwGlobal tw{p.tw};
@@ -62,105 +61,95 @@ __device__ __forceinline__ void xpass_adj_tile(const XAdjArgs& p, long long tile
   float2* myrow = rowbuf + rl * PITCH;
 
   // 1. every field: load, inverse transform (from k-space), park
+#pragma unroll
+  for (int f = 0; f < F; ++f) {
+    if (act) copy_row<PL>(myrow + f * ROWS * PITCH, p.g + f * p.fstride + row * NX, t);
+    cp_async_commit();
+  }
 #pragma unroll 1
   for (int f = 0; f < F; ++f) {
     const XchRow xr{myrow + f * ROWS * PITCH};
-    const float2* src = p.g + f * p.fstride + (act ? row : 0) * NX;
+    if (f == F - 1) cp_async_wait<0>();
+    else if (f == F - 2) cp_async_wait<1>();
+    else cp_async_wait<2>();
+    SY::sync();
     float2 v[E];
     if (p.from_k) {
 #pragma unroll
       for (int b = 0; b < E / RFL; ++b)
 #pragma unroll
-        for (int r = 0; r < RFL; ++r)
-          v[b * RFL + r] = act ? __ldcg(src + pos_first<PL, true>(t + b * T, r)) : make_float2(0.f, 0.f);
+        for (int r = 0; r < RFL; ++r) v[b * RFL + r] = xr.base[pos_first<PL, true>(t + b * T, r)];
       fft_run<PL, true, 0, XchRow, SY, TwGlobal>(v, t, xr, tw);
     } else {
 #pragma unroll
       for (int b = 0; b < E / RF0; ++b)
 #pragma unroll
-        for (int r = 0; r < RF0; ++r)
-          v[b * RF0 + r] = act ? __ldcg(src + pos_first<PL, false>(t + b * T, r)) : make_float2(0.f, 0.f);
+        for (int r = 0; r < RF0; ++r) v[b * RF0 + r] = xr.base[pos_first<PL, false>(t + b * T, r)];
     }
-#pragma unroll
-    for (int b = 0; b < E / RF0; ++b)
-#pragma unroll
-      for (int r = 0; r < RF0; ++r) xr.st(t + b * T + r * SF0, v[b * RF0 + r]);
+    SY::sync();  // the row's last reads are done
+    park<PL>(xr.base, t, v);
   }
 
-  // 2. reverse of N_A (at xa), then of N_B (at xb), point by point
+  // 2. reverse of N_A (at xa), then of N_B (at xb), two points at a time; the states
+  // (and under a map the stage-factor tables) of the next points are requested
+  // while these are reversed
   if (act) {
     const long long nxy = (long long)p.ny * NX;
     const float2* emap = MAP ? p.emap + (row % p.ny) * NX : nullptr;
-    // the recorded states (and under a map the stage-factor tables) of the next
-    // point are requested while this one is reversed (measured on the adjoint
-    // workload: backward 152 -> 143 ms, under a fan-out map 168 -> 153 ms;
-    // requesting both states of the same point up front gained nothing)
-    float2 na[F], nb[F], nm[4];
-    {
-      const int p0 = pos_first<PL, false>(t, 0);
-      const long long at0 = row * NX + p0;
+    float4 na[F], nb[F];
+    float2 nm[4][2];
+    const float4 none = make_float4(0.f, 0.f, 0.f, 0.f);
+    const auto request = [&](int q) {
 #pragma unroll
       for (int f = 0; f < F; ++f) {
-        na[f] = p.xa ? __ldcg(p.xa + f * p.fstride + at0) : make_float2(0.f, 0.f);
-        nb[f] = p.xb ? __ldcg(p.xb + f * p.fstride + at0) : make_float2(0.f, 0.f);
+        const long long at = f * p.fstride + row * NX;
+        na[f] = p.xa ? load_points<PL>(p.xa + at, p.xa_row_order, t, q) : none;
+        nb[f] = p.xb ? load_points<PL>(p.xb + at, false, t, q) : none;
       }
       if constexpr (MAP) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) nm[q] = __ldcg(emap + q * nxy + p0);
+        for (int m = 0; m < 4; ++m)
+#pragma unroll
+          for (int u = 0; u < 2; ++u) nm[m][u] = __ldcg(emap + m * nxy + point_pos<PL>(t, 2 * q + u));
       }
+    };
+    Pair eB, vB, eA, vA;
+    if constexpr (!MAP) {
+      eB = {dup(p.ecoef[0].x), dup(p.ecoef[0].y)};
+      vB = {dup(p.ecoef[1].x), dup(p.ecoef[1].y)};
+      eA = {dup(p.ecoef[2].x), dup(p.ecoef[2].y)};
+      vA = {dup(p.ecoef[3].x), dup(p.ecoef[3].y)};
     }
+    float2 s[6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) s[k] = make_float2(0.f, 0.f);
+    request(0);
 #pragma unroll 1
-    for (int e = 0; e < E; ++e) {
-      const int place = t + (e / RF0) * T + (e % RF0) * SF0;  // park place (XchRow padding)
-      const int off = place + (place >> 4);
-      float2 g[F], x[F], xbv[F], cm[4];
+    for (int q = 0; q < E / 2; ++q) {
+      Pair g[F], x[F], xbv[F];
 #pragma unroll
       for (int f = 0; f < F; ++f) {
-        x[f] = na[f];
-        xbv[f] = nb[f];
+        const float4 w = *park_place<PL>(myrow + f * ROWS * PITCH, t, q);
+        g[f] = {make_float2(w.x, w.y), make_float2(w.z, w.w)};
+        x[f] = {make_float2(na[f].x, na[f].y), make_float2(na[f].z, na[f].w)};
+        xbv[f] = {make_float2(nb[f].x, nb[f].y), make_float2(nb[f].z, nb[f].w)};
       }
       if constexpr (MAP) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) cm[q] = nm[q];
+        const auto pair_of = [](const float2* m) { return Pair{make_float2(m[0].x, m[1].x), make_float2(m[0].y, m[1].y)}; };
+        eB = pair_of(nm[0]);
+        vB = pair_of(nm[1]);
+        eA = pair_of(nm[2]);
+        vA = pair_of(nm[3]);
       }
-      if (e + 1 < E) {
-        const int pn = pos_first<PL, false>(t + ((e + 1) / RF0) * T, (e + 1) % RF0);
-        const long long an = row * NX + pn;
+      if (q + 1 < E / 2) request(q + 1);
+      if (p.xa) rk4_vjp<F>(x, g, eA, vA, p.kh, p.kh2, s);
+      if (p.xb) rk4_vjp<F>(xbv, g, eB, vB, p.kh, p.kh2, s + 3);
 #pragma unroll
-        for (int f = 0; f < F; ++f) {
-          if (p.xa) na[f] = __ldcg(p.xa + f * p.fstride + an);
-          if (p.xb) nb[f] = __ldcg(p.xb + f * p.fstride + an);
-        }
-        if constexpr (MAP) {
-#pragma unroll
-          for (int q = 0; q < 4; ++q) nm[q] = __ldcg(emap + q * nxy + pn);
-        }
-      }
-#pragma unroll
-      for (int f = 0; f < F; ++f) g[f] = myrow[f * ROWS * PITCH + off];
-      if (p.xa) {
-        if constexpr (MAP) {
-          float2 c[3 * F];
-          map_coef_sets<F>(cm[2], cm[3], p.kh, c);
-          rk4_vjp_point<F>(x, g, c, sens[0], sens[1], sens[2]);
-        } else {
-          rk4_vjp_point<F>(x, g, cA, sens[0], sens[1], sens[2]);
-        }
-      }
-      if (p.xb) {
-#pragma unroll
-        for (int f = 0; f < F; ++f) x[f] = xbv[f];
-        if constexpr (MAP) {
-          float2 c[3 * F];
-          map_coef_sets<F>(cm[0], cm[1], p.kh, c);
-          rk4_vjp_point<F>(x, g, c, sens[3], sens[4], sens[5]);
-        } else {
-          rk4_vjp_point<F>(x, g, cB, sens[3], sens[4], sens[5]);
-        }
-      }
-#pragma unroll
-      for (int f = 0; f < F; ++f) myrow[f * ROWS * PITCH + off] = g[f];
+      for (int f = 0; f < F; ++f)
+        *park_place<PL>(myrow + f * ROWS * PITCH, t, q) = make_float4(g[f].re.x, g[f].re.y, g[f].im.x, g[f].im.y);
     }
+#pragma unroll
+    for (int k = 0; k < 6; ++k) sens[k] = s[k].x + s[k].y;
   }
 
   // 3. every field: unpark, forward transform (or leave in real space), store
@@ -169,10 +158,7 @@ __device__ __forceinline__ void xpass_adj_tile(const XAdjArgs& p, long long tile
     const XchRow xr{myrow + f * ROWS * PITCH};
     float2* dst = p.g + f * p.fstride + (act ? row : 0) * NX;
     float2 v[E];
-#pragma unroll
-    for (int b = 0; b < E / RF0; ++b)
-#pragma unroll
-      for (int r = 0; r < RF0; ++r) v[b * RF0 + r] = xr.ld(t + b * T + r * SF0);
+    unpark<PL>(xr.base, t, v);
     if (!p.to_k) {
       if (act) {
 #pragma unroll
@@ -193,26 +179,19 @@ __device__ __forceinline__ void xpass_adj_tile(const XAdjArgs& p, long long tile
   }
 }
 
+// Four CTAs (128 registers) hold two fields without spills; three fields and the
+// tables of a map need three (168).
 template <int NX, int F, bool MAP>
-__global__ void __launch_bounds__(xpass_threads<NX>(), xpass_threads<NX>() <= 128 ? 4 : 1)
+__global__ void __launch_bounds__(xpass_threads<NX>(), xpass_threads<NX>() > 128 ? 1 : F == 3 || MAP ? 3 : 4)
     xpass_adj_kernel(const XAdjArgs p) {
   constexpr int THREADS = xpass_threads<NX>();
   extern __shared__ float4 sm4[];
-  float2* cA = reinterpret_cast<float2*>(sm4);  // [3][F]
-  float2* cB = cA + 3 * F;                      // [3][F]
-  float2* rowbuf = cA + 6 * F;
+  float2* rowbuf = reinterpret_cast<float2*>(sm4);
   __shared__ double red[THREADS / 32][6];
-  if constexpr (!MAP) {
-    // coefficient sets from the launch (formed on the host in FP64)
-    if (threadIdx.x < 3 * F) {
-      cA[threadIdx.x] = p.cset[0][threadIdx.x];
-      cB[threadIdx.x] = p.cset[1][threadIdx.x];
-    }
-  }
-  __syncthreads();
   chain_begin();
   float sens[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  xpass_adj_tile<NX, F, THREADS, MAP>(p, blockIdx.x, cA, cB, rowbuf, sens);
+  // rows from the last tau-plane down, as the forward x-pass
+  xpass_adj_tile<NX, F, THREADS, MAP>(p, (long long)gridDim.x - 1 - blockIdx.x, rowbuf, sens);
   // block sums in FP64, fixed order (deterministic)
 #pragma unroll
   for (int k = 0; k < 6; ++k) {
@@ -234,7 +213,7 @@ template <int NX, int F, bool MAP>
 cudaError_t launch_adjoint(const XAdjArgs& a, long long* ncta, cudaStream_t s) {
   constexpr int ROWS = xpass_rows<NX>();
   constexpr int THREADS = xpass_threads<NX>();
-  const size_t smem = (size_t)(6 * F + xpass_smem_floats2<NX>(F)) * sizeof(float2);
+  const size_t smem = (size_t)xpass_smem_floats2<NX>(F) * sizeof(float2);
   static SmemOnce once;
   cudaError_t e = raise_smem_limit(xpass_adj_kernel<NX, F, MAP>, smem, once);
   if (e != cudaSuccess) return e;

@@ -292,3 +292,34 @@ def test_gradient_under_map_changing_along_z_matches_oracle(three):
     # the z-resolution is felt: the gradient under the first segment's map alone is far off
     _, _, gdk1 = oracle.adjoint_gradient(prob, ins128, nz, dz, dk, w, phi=phi, phi_field=pf, dk_map=maps[0])
     assert rel_l2(gdk1, gdk_r) > 20 * GRAD_TOL
+
+
+@pytest.mark.parametrize("nx,nf,mapped", [(2, 2, False), (6, 3, False), (16, 2, True), (24, 2, False), (48, 3, True),
+                                          (96, 2, False), (192, 3, False), (256, 2, True), (384, 2, False),
+                                          (512, 3, False), (768, 3, True), (1024, 2, False), (4096, 3, False)])
+def test_reverse_x_pass_of_every_kind_of_row(nx, nf, mapped):
+    """The gradient on short y and tau axes against the oracle's: a segment's
+    boundary reads a checkpoint, the others the recorded states; 36 rows (4 of 4096 points) leave the
+    last CTA of the rows of up to 256 points partly filled."""
+    rng = np.random.default_rng(nx + nf)
+    g = wl.Grid(nx, 6 if nx <= 1024 else 2, 6 if nx <= 1024 else 2, 6 * wl.UM, 6 * wl.UM, 30 * wl.FS)
+    if nf == 2:
+        fields = [wl.FieldParams(wl.LAM_SH, wl.N_SH, rho=1e-3), wl.FieldParams(wl.LAM_F, wl.N_F, alpha=15.0)]
+    else:
+        fields = [wl.FieldParams(wl.LAM_P, wl.N_P, rho=2e-3), wl.FieldParams(wl.LAM_S, wl.N_S, alpha=15.0),
+                  wl.FieldParams(wl.LAM_I, wl.N_I)]
+    shape = (g.nt, g.ny, g.nx)
+    ins = [(4e7 * (rng.standard_normal(shape) + 1j * rng.standard_normal(shape))).astype(np.complex64)
+           for _ in range(nf)]
+    nz, dz = 5, 25 * wl.UM
+    dk = rng.normal(300.0, 200.0, nz)
+    phi = rng.normal(0, 0.2, g.nt)
+    w = np.array([1e-15, 5e-16, 0.0][:nf])
+    m = rng.normal(0.0, 2e3, (g.ny, g.nx)) if mapped else None
+    J, gphi, gdk = _gpu_grad(g, fields, ins, phi, dk, nz, dz, w, interval=2, dk_map=m)
+    prob = oracle.make_problem(g, fields, wl.D_EFF)
+    Jr, gphi_r, gdk_r = oracle.adjoint_gradient(prob, [a.astype(np.complex128) for a in ins], nz, dz, dk, w,
+                                                phi=phi, phi_field=1, dk_map=m)
+    assert abs(J / Jr - 1) < 1e-4
+    assert rel_l2(gphi, gphi_r) < GRAD_TOL
+    assert rel_l2(gdk, gdk_r) < GRAD_TOL
