@@ -213,9 +213,10 @@ brahms_status brahms_get_z(const brahms_ctx* ctx, double* z, double* phi);
  * launch, enable = k > 1 every k-th launch of each kernel kind (the events
  * cost about 2 us of device time each); enable == 0 stops.  With
  * ms/launches non-NULL the accumulated device time [ms] and count of the
- * timed launches of each kernel kind (0 x-pass, 1 y-pass forward, 2 tau-pass,
- * 3 y-pass inverse, 4 other) are written to the first nkinds entries; this
- * waits for the stream. */
+ * timed launches of each kernel kind (0 x-pass, or the plane pass that does the
+ * y-inverse, x-pass and y-forward on small planes; 1 y-pass forward; 2 tau-pass, or
+ * the linear step of a grid with nt = 1; 3 y-pass inverse; 4 other) are written to
+ * the first nkinds entries; this waits for the stream. */
 brahms_status brahms_timing(brahms_ctx* ctx, int enable, double* ms, long long* launches, int nkinds);
 
 /* Implementation options; every setting computes identical numbers.
@@ -224,10 +225,11 @@ brahms_status brahms_timing(brahms_ctx* ctx, int enable, double* ms, long long* 
  * each field's y-forward starting after the previous field's, so that
  * DRAM-bound and compute-bound passes of different fields overlap; the
  * x-pass, which couples the fields, waits for all of them on the context
- * stream.  0 (the default) runs every pass on the context stream.  Measured
- * on GB300: 5 % faster per step on 128x128x256 with three fields, slower on
- * two-field and small grids.  Per-kernel timing with field streams measures
- * kernels that may share the GPU.
+ * stream.  0 (the default) runs every pass on the context stream, each launch
+ * overlapping the end of the one before it.  Measured on GB300: slower on
+ * every grid since then (time per step, off and on: 3 x 128x128x256 156 and
+ * 163 us, 2 x 32x32x64 7.4 and 20.6).  Per-kernel timing with field streams
+ * measures kernels that may share the GPU.
  * BRAHMS_OPT_TMA_TAU: value 16 or 8 makes the
  * tau-pass of brahms_propagate a persistent kernel that stages tiles of that
  * many x columns through shared memory with double-buffered TMA copies; 1
@@ -235,9 +237,10 @@ brahms_status brahms_timing(brahms_ctx* ctx, int enable, double* ms, long long* 
  * next 16-column tile with a TMA copy while it transforms the current one
  * (its FFT exchanges go through half the shared memory, one real component
  * at a time).  Both need nt in {256, 512} and nx >= 16, else E_SIZE; both
- * compute the plain tau-pass's numbers and measured slower on GB300.  0 (the
- * default) keeps the plain tau-pass (and turns the field streams off while
- * set).
+ * compute the default tau-pass's numbers and measured slower on GB300 (step of
+ * 3 x 256x256x512: 1324 us with 8, 1494 with 16, 1380 with 1, 1306 by default).
+ * 0 (the default) keeps the library's own choice of tau-pass.  Any other value
+ * turns the field streams off while set.
  * BRAHMS_OPT_TMA_WAIT_US: the limit, in microseconds (0 .. 2000000, default
  * 2000000 = 2 s), of each wait of the TMA tau-pass for a tile's copy; 0
  * gives up at the first check that finds the copy unfinished.  When a

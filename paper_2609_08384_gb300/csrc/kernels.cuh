@@ -1,7 +1,7 @@
 // Kernels of one split-step z-step (Sec. 3.1, Eq. expon) on the layout
 // fields[f][tau][y][x] (x fastest), complex64.
 //
-// A z-step is four HBM passes per field:
+// A z-step is four passes over memory per field:
 //   x-pass  inverse x-FFT, the second RK4 half step of step j, the first RK4
 //           half step of step j+1, forward x-FFT (all fields of a row at once,
 //           the nonlinear coupling is pointwise across fields)
@@ -9,6 +9,9 @@
 //   t-pass  forward tau-FFT, multiply by the linear propagator
 //           P = Px(kx) Py(ky) Pt(Omega) / (NX NY NT), inverse tau-FFT
 //   y-pass  inverse y-FFT
+// On planes of up to 1536 points the y-inverse, x-pass and y-forward are one
+// kernel (plane.cuh), and on cw grids (nt = 1) the linear step is one pass along y
+// (the tau-pass's kernel on the axes x, tau, y).
 // Between calls the state is in real space; the first and the last step of
 // a call peel the x-pass (NL_FIRST / NL_LAST).
 #pragma once
@@ -113,8 +116,6 @@ template <class PL>
 struct ColTile {
   static constexpr int value = col_tile_n(PL::N);
 };
-// (A plan may override its tile width; 8-column tiles for the 512-point tau
-// propagator measured slower than 16 on GB300, 575 vs 546 us per OPG launch.)
 template <class PL>
 __host__ __device__ constexpr int tile_threads() { return PL::T * ColTile<PL>::value; }
 template <class PL>
@@ -129,8 +130,8 @@ __host__ __device__ constexpr int axis_smem_floats2() {
 }
 // The forward y-pass reads its twiddles through L1 instead of staging them in
 // shared memory per CTA: measured on the 3 x 256x256x512 state, 285 -> 253 us
-// per launch (the inverse y-pass, 259 -> 266, and the tau propagator,
-// 477 -> 485, measured the other way and keep the staging).
+// per launch (the inverse y-pass, 259 -> 266, measured the other way and keeps the
+// staging; now 231 and 237, 7.0 and 6.8 TB/s).
 template <class PL, bool INV, int AXIS>
 __host__ __device__ constexpr bool axis_tw_staged() { return tw_in_smem<PL>() && !(AXIS == 1 && !INV); }
 template <class PL, bool INV, int AXIS>
@@ -489,7 +490,7 @@ __global__ void __launch_bounds__(xpass_threads<NX>(), xpass_min_blocks<NX, F>()
 // 1000-step call; a tau-major y order (every field of a plane together)
 // made the y-passes 20 us slower and the step 1622 ms.  The tau-propagator
 // also walks its tiles from the last down (tau 476 -> 473, y-inverse
-// 258 -> 257 us).
+// 258 -> 257 us).  (The step now takes 1307 us on that state.)
 template <int N, int AXIS, int TX>
 struct AxisTile {
   float2* base;  // element (x, pencil index 0)
@@ -645,12 +646,13 @@ __device__ __forceinline__ void tprop_tile(const AxisArgs& p, long long cta_tile
 // 64 bytes) for the plans of 16 or more threads per pencil and 128/T for those of
 // 8, small enough for two buffers and several CTAs per SM, and the exchanges run
 // in the tile's own buffer.
-// Taken by the two-pass plans (one exchange per transform) and by the plan of 32
+// Taken by the two-pass plans (one exchange per transform) and by the plans of 32
 // threads per pencil, whose 16-column tile leaves room for one CTA per SM.
 // Measured per launch, plain tau-pass against this one: 512 points (three fields
 // of 256x256) 463 -> 415 us, 256 (three of 128x128) 57 -> 49, 128 (two of 512x512)
-// 231 -> 212, 64 (two of 1024x256) 127 -> 115, 768 (two of 192x192) 388 -> 348; the
-// four-pass plans of 192 and 384 points lost 1 to 5 % (their block barriers).
+// 231 -> 212, 64 (two of 1024x256) 127 -> 115, 768 (two of 192x192, then in four
+// passes) 388 -> 348.  Plans of three or four passes and fewer threads lost 1 to 5 %
+// (192 and 384 points in four passes, their block barriers).
 // What bounds it: latency between the phases of a tile at 12 to 16 warps per SM
 // (512 points: issue 49 %, FP32 pipe 45 %, shared memory 49 %, DRAM 48 %); plans
 // with 16 values per thread and twice the warps were slower (494 to 580 us).
