@@ -84,27 +84,30 @@ using AxisPlan = typename std::conditional<AXIS == 0, FftPlan<N>,
 template <int N>
 __host__ __device__ constexpr int fft_threads() { return FftPlan<N>::T; }
 
-// x-pass CTA: 128 threads (or one row when a row needs more); rows whose
-// threads lie inside one warp synchronise their exchanges with __syncwarp.
+// x-pass CTA: 128 threads, or one row when a row needs 64 threads or more (its block
+// barriers then wait for one row alone: x-pass of 2 x 1024x256x64 197 -> 188 us with
+// one row of 64 threads instead of two, 3 x 1024x64x64 82.6 -> 79.0, step of 2 x
+// 1024x1024x1 31.9 -> 30.9); rows whose threads lie inside one warp synchronise
+// their exchanges with __syncwarp.
 template <int N>
-__host__ __device__ constexpr int xpass_threads() { return fft_threads<N>() >= 128 ? fft_threads<N>() : 128; }
+__host__ __device__ constexpr int xpass_threads() { return fft_threads<N>() >= 64 ? fft_threads<N>() : 128; }
 template <int N>
 __host__ __device__ constexpr int xpass_rows() { return xpass_threads<N>() / fft_threads<N>(); }
 template <int N>
 __host__ __device__ constexpr bool xpass_warp_sync() { return fft_threads<N>() <= 32 && 32 % fft_threads<N>() == 0; }
-// shared memory in float2 units: a row buffer per field and row (the reverse
-// x-pass keeps its 6 F coefficients in front of them)
+// shared memory in float2 units: a row buffer per field and row
 template <int N>
 __host__ __device__ constexpr int xpass_smem_floats2(int nf) {
   return nf * xpass_rows<N>() * XchRow::pitch(N);
 }
 // resident CTAs the x-pass asks the register allocator for: 6 (80 registers)
 // where six CTAs' shared memory fits in an SM and rows are at most 256 long
-// (no spills there); otherwise 4 (128 registers)
+// (no spills there); otherwise 4, or 8 of 64 threads (128 registers)
 template <int N, int F>
 __host__ __device__ constexpr int xpass_min_blocks() {
   return xpass_threads<N>() > 128                                                          ? 1
          : (N <= 256 && 6 * (xpass_smem_floats2<N>(F) * 8 + 1024) <= 228 * 1024) ? 6
+         : xpass_threads<N>() == 64                                              ? 8
                                                                                           : 4;
 }
 

@@ -179,10 +179,10 @@ __device__ __forceinline__ void xpass_adj_tile(const XAdjArgs& p, long long tile
   }
 }
 
-// Four CTAs (128 registers) hold two fields without spills; three fields and the
-// tables of a map need three (168).
+// Four CTAs of 128 threads (128 registers) hold two fields without spills; three
+// fields and the tables of a map need three (168).
 template <int NX, int F, bool MAP>
-__global__ void __launch_bounds__(xpass_threads<NX>(), xpass_threads<NX>() > 128 ? 1 : F == 3 || MAP ? 3 : 4)
+__global__ void __launch_bounds__(xpass_threads<NX>(), xpass_threads<NX>() > 128 ? 1 : (F == 3 || MAP ? 3 : 4) * 128 / xpass_threads<NX>())
     xpass_adj_kernel(const XAdjArgs p) {
   constexpr int THREADS = xpass_threads<NX>();
   extern __shared__ float4 sm4[];
