@@ -115,7 +115,8 @@ brahms_status brahms_init_grid(brahms_ctx** out, int nx, int ny, int nt, double 
   cudaError_t e = cudaSuccess;
   if (e == cudaSuccess) e = brahms::upload_twiddles(ctx->twx, nx, 0, ctx->stream);
   if (e == cudaSuccess && ny > 1) e = brahms::upload_twiddles(ctx->twy, ny, 1, ctx->stream);
-  if (e == cudaSuccess && nt > 1) e = brahms::upload_twiddles(ctx->twt, nt, 2, ctx->stream);
+  const int nlast = tau_pass_length(ny, nt);
+  if (e == cudaSuccess && nlast > 1) e = brahms::upload_twiddles(ctx->twt, nlast, 2, ctx->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(ctx->dev_err, 0, 2 * sizeof(int), ctx->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(ctx->mphase_dev, 0, sizeof(double) * nx * ny, ctx->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);

@@ -26,6 +26,9 @@ constexpr int kMaxMapSegments = 4096;  // z-segments of a mismatch map
 
 inline size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
 
+// length of the transforms of the tau-pass's kernels: tau, or y on a grid with nt = 1
+inline int tau_pass_length(int ny, int nt) { return nt > 1 ? nt : ny; }
+
 struct Layout {
   size_t state, px, py, pt, twx, twy, twt, partial, err, diag, dkmap, usermap, mphase, emap, total;
 };
@@ -45,7 +48,7 @@ inline Layout make_layout(int nx, int ny, int nt, int nf) {
   L.pt = take(sizeof(float2) * nt * nf);
   L.twx = take(sizeof(float2) * brahms::tw_table_size_of(nx, 0));
   L.twy = take(sizeof(float2) * brahms::tw_table_size_of(ny, 1));
-  L.twt = take(sizeof(float2) * brahms::tw_table_size_of(nt, 2));
+  L.twt = take(sizeof(float2) * brahms::tw_table_size_of(tau_pass_length(ny, nt), 2));
   L.partial = take(sizeof(double) * kRedBlocks * nf);
   L.err = take(2 * sizeof(int));
   L.diag = take(sizeof(double) * 2 * nt * nf);
@@ -382,7 +385,8 @@ inline brahms::AxisArgs aargs(brahms_ctx* c, int axis, bool tau_prop = true) {
 
 // The linear step of a grid without a tau axis (nt = 1, ny > 1) as one pass along
 // y: forward y transform, propagator, inverse y transform, which is the tau-pass
-// on the grid read as nx x 1 x ny, the roles of the y and tau factors exchanged.
+// on the grid read as nx x 1 x ny, the roles of the y and tau factors exchanged;
+// twt holds the twiddles of ny in the tau-pass's plan there.
 // (1024x1024, two fields: y-forward, pointwise multiply and y-inverse took 43 us
 // of a step of 49; one pass 17.)
 inline brahms::AxisArgs cw_args(brahms_ctx* c) {
@@ -392,15 +396,16 @@ inline brahms::AxisArgs cw_args(brahms_ctx* c) {
   const int tx = brahms::tau_col_tile_of(c->ny);
   a.xtiles = (c->nx + tx - 1) / tx;
   a.ntiles = (long long)c->nf * a.xtiles;
+  a.tw = c->twt;
   a.py = c->pt;
   a.pt = c->py;
   return a;
 }
 
 // Per-field streams for the y-forward, tau-propagator and y-inverse of a
-// step, when the option asks for them (measured on GB300: 5 % faster on
-// 128x128x256 with three fields, 2-28 % slower on two-field and small grids,
-// within 3 % either way on larger ones).
+// step, when the option asks for them (measured on GB300, step without and with:
+// 3 x 128x128x256 156 and 163 us, 2 x 32x32x64 7.4 and 20.6, 3 x 256x256x256 627 and
+// 629).
 inline bool use_field_streams(const brahms_ctx* c) {
   return c->field_streams == 1 && c->ny > 1 && c->nt > 1 && !c->use_tma;
 }

@@ -60,3 +60,10 @@ def test_linear_step_matches_fp64(shape, nf):
     for x, r in zip(got, _reference(g, fields, a, dz, nz)):
         assert np.linalg.norm(x - r) / np.linalg.norm(r) < tol
     s.close()
+
+
+@pytest.mark.parametrize("ny", [2, 4, 6, 8, 12, 16, 24, 32, 48, 64, 96, 128, 192, 256, 384, 512, 768, 1024, 2048, 4096])
+def test_cw_linear_step_of_every_y_length(ny):
+    """nt = 1: the linear step is one pass along y, whose kernel and twiddle table
+    are the tau-pass's."""
+    test_linear_step_matches_fp64((24, ny, 1), 3)
