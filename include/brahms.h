@@ -84,7 +84,9 @@ brahms_status brahms_init_grid(brahms_ctx** out, int nx, int ny, int nt, double 
  * complex values of dtype BRAHMS_C64 (float pairs) or BRAHMS_C128 (double
  * pairs), on the device if on_device != 0 else in host memory.  Resets z and
  * Phi to zero.  Host copies are complete when the call returns; device copies
- * are ordered on the context stream.  Non-finite host input gives E_ARG. */
+ * are ordered on the context stream.  Non-finite host input gives E_ARG; device
+ * memory that ends before a field's last point gives E_CUDA, with the fields of
+ * before left as they are. */
 brahms_status brahms_set_fields(brahms_ctx* ctx, const void* const* fields, int dtype, int on_device);
 
 /* Piecewise mismatch profile: step j (counted from the last set_fields) uses

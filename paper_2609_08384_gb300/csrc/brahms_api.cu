@@ -158,7 +158,9 @@ brahms_status brahms_set_fields(brahms_ctx* ctx, const void* const* fields, int 
   for (int f = 0; f < ctx->nf; ++f)
     if (!fields[f]) return fail(ctx, BRAHMS_E_ARG, "a field pointer is NULL");
   std::vector<float2> stage;
-  const bool fused = dtype == BRAHMS_C64 && on_device && kernel_can_copy(ctx, fields, false);
+  const brahms::Route route = on_device ? device_route(ctx, fields, dtype, false) : brahms::Route::kDriver;
+  if (route == brahms::Route::kRefuse) return fail(ctx, BRAHMS_E_CUDA, "a field's device memory ends before its last point");
+  const bool fused = dtype == BRAHMS_C64 && route == brahms::Route::kKernel;
   for (int f = 0; f < ctx->nf && !fused; ++f) {
     float2* dst = ctx->state + f * n;
     if (dtype == BRAHMS_C64) {
@@ -283,7 +285,9 @@ brahms_status brahms_get_fields(brahms_ctx* ctx, void* const* out, int dtype, in
     if (!out[f]) return fail(ctx, BRAHMS_E_ARG, "an output pointer is NULL");
   const long long n = ctx->npoints();
   std::vector<float2> stage;
-  const bool fused = dtype == BRAHMS_C64 && on_device && kernel_can_copy(ctx, out, true);
+  const brahms::Route route = on_device ? device_route(ctx, out, dtype, true) : brahms::Route::kDriver;
+  if (route == brahms::Route::kRefuse) return fail(ctx, BRAHMS_E_CUDA, "an output's device memory ends before its last point");
+  const bool fused = dtype == BRAHMS_C64 && route == brahms::Route::kKernel;
   for (int f = 0; f < ctx->nf && !fused; ++f) {
     const float2* src = ctx->state + f * n;
     if (dtype == BRAHMS_C64) {

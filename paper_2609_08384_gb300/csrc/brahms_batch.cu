@@ -1045,7 +1045,9 @@ brahms_status brahms_batch_set_fields(brahms_batch* b, int index, const void* co
   if (dtype != BRAHMS_C64) return bfail(b, BRAHMS_E_ARG, "batched fields must be complex64");
   BatchInstHost& I = b->inst[index];
   const size_t n = (size_t)I.npoints();
-  if (on_device && kernel_can_copy(fields, 2, sizeof(float2) * n, I.state, I.state + 2 * n, false))
+  const Route route = on_device ? device_route(fields, 2, sizeof(float2) * n, I.state, I.state + 2 * n, false) : Route::kDriver;
+  if (route == Route::kRefuse) return bfail(b, BRAHMS_E_CUDA, "a field's device memory ends before its last point");
+  if (route == Route::kKernel)
     BB_CK(run_copy_pair((const float2*)fields[0], I.state, (const float2*)fields[1], I.state + n, (long long)n, b->stream));
   else
     for (int f = 0; f < 2; ++f)
@@ -1119,7 +1121,9 @@ brahms_status brahms_batch_get_fields(brahms_batch* b, int index, void* const* o
   if (dtype != BRAHMS_C64) return bfail(b, BRAHMS_E_ARG, "batched fields are complex64");
   BatchInstHost& I = b->inst[index];
   const size_t n = (size_t)I.npoints();
-  if (on_device && kernel_can_copy(out, 2, sizeof(float2) * n, I.state, I.state + 2 * n, true))
+  const Route route = on_device ? device_route(out, 2, sizeof(float2) * n, I.state, I.state + 2 * n, true) : Route::kDriver;
+  if (route == Route::kRefuse) return bfail(b, BRAHMS_E_CUDA, "an output's device memory ends before its last point");
+  if (route == Route::kKernel)
     BB_CK(run_copy_pair(I.state, (float2*)out[0], I.state + n, (float2*)out[1], (long long)n, b->stream));
   else
     for (int f = 0; f < 2; ++f)

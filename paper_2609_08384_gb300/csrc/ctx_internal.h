@@ -466,9 +466,9 @@ inline double dk_of_step(const brahms_ctx* c, long long j) {
   return j < (long long)c->dk_profile.size() ? c->dk_profile[(size_t)j] : c->dk;
 }
 
-inline bool kernel_can_copy(const brahms_ctx* ctx, const void* const* ptrs, bool written) {
-  return brahms::kernel_can_copy(ptrs, ctx->nf, sizeof(float2) * (size_t)ctx->npoints(), ctx->ws,
-                                 ctx->ws + ctx->L.total, written);
+inline brahms::Route device_route(const brahms_ctx* ctx, const void* const* ptrs, int dtype, bool written) {
+  const size_t point = dtype == BRAHMS_C64 ? sizeof(float2) : sizeof(double2);
+  return brahms::device_route(ptrs, ctx->nf, point * (size_t)ctx->npoints(), ctx->ws, ctx->ws + ctx->L.total, written);
 }
 
 // Enqueue an FP64 |A|^2 reduction per field into energy_host (pinned); from or to
