@@ -9,6 +9,7 @@ CPU fallback.
 from __future__ import annotations
 
 import ctypes
+import math
 import os
 import threading
 from typing import Optional, Sequence
@@ -429,20 +430,27 @@ class Batch:
         return idx.value
 
     def set_fields(self, index, fields):
-        """fields: two contiguous complex64 torch tensors (cuda) or numpy arrays."""
+        """fields: two contiguous complex64 torch tensors (cuda) or numpy arrays of
+        at least nt * ny * nx values."""
         import torch
 
+        index = int(index)
+        points = math.prod(self.shapes[index]) if 0 <= index < len(self.shapes) else 0
         ptrs, dev = [], None
         for a in fields:
             if isinstance(a, torch.Tensor):
                 assert a.dtype == torch.complex64 and a.is_contiguous()
+                if a.numel() < points:
+                    raise ValueError(f"a field holds {a.numel()} of the grid's {points} points")
                 ptrs.append(a.data_ptr())
                 dev = a.is_cuda
             else:
                 a = np.ascontiguousarray(a, dtype=np.complex64)
+                if a.size < points:
+                    raise ValueError(f"a field holds {a.size} of the grid's {points} points")
                 ptrs.append(a.ctypes.data)
                 dev = False
-        self._chk(load().brahms_batch_set_fields(self.h, int(index), _ptr_array(ptrs), BRAHMS_C64, int(bool(dev))))
+        self._chk(load().brahms_batch_set_fields(self.h, index, _ptr_array(ptrs), BRAHMS_C64, int(bool(dev))))
 
     def set_granularity(self, shape, gx, gy, gt):
         self._chk(load().brahms_batch_set_granularity(self.h, shape, gx, gy, gt))
