@@ -262,7 +262,7 @@ __global__ void prop_pointwise_kernel(const AxisArgs p, int nf) {
     const int t = (int)(r / plane);
     const ColumnProp g(p, p.px[f * p.nx + x], p.py[f * p.ny + y]);
     float2* q = p.data + (long long)f * p.fstride + r;
-    *q = g(*q, p.pt[f * p.nt + t]);
+    *q = g(p.scale_lo == 0.f ? *q : ColumnProp::scaled(p, *q), p.pt[f * p.nt + t]);
   }
 }
 

@@ -158,6 +158,7 @@ __global__ void __launch_bounds__(PL::T * TX, PL::T * TX <= 256 ? 2 : 1)
       for (int r = 0; r < R0; ++r) v[bb * R0 + r] = xc.ld(pos_first<PL, false>(t + bb * T, r));
     using TWA = typename std::conditional<tw_in_smem<PL>(), TwShared, TwGlobal>::type;
     const TWA tw{tw_in_smem<PL>() ? tws : p.tw};
+    scale_column<PL>(v, p);
     fft_run<PL, false, 0, XchCol<TX>, SyncBlock, TWA>(v, t, xc, tw);
     const float2 zero = make_float2(0.f, 0.f);
     const ColumnProp g(p, act ? p.px[f * p.nx + x] : zero, act ? p.py[f * p.ny + y] : zero);
@@ -257,6 +258,7 @@ __global__ void __launch_bounds__(PL::T * 16, 2)
     const int y = (int)(rest % p.ny), f = (int)(rest / p.ny);
     const int x = xt * TX + tx;
     const bool act = x < p.nx;
+    scale_column<PL>(v, p);
     fft_run<PL, false, 0, XchColSplit<TX>, SyncBlock, TwGlobal>(v, t, xc, tw);
     const float2 zero = make_float2(0.f, 0.f);
     const ColumnProp g(p, act ? p.px[f * p.nx + x] : zero, act ? p.py[f * p.ny + y] : zero);

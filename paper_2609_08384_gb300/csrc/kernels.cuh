@@ -563,40 +563,60 @@ __device__ __forceinline__ void axis_tile(const AxisArgs& p, long long cta_tile,
 }
 
 // The propagator P = (1 + Dx)(1 + Dy)(1 + Dt) / (nx ny nt) of one column, the
-// factors in delta form and 1/(nx ny nt) as scale + scale_lo: a value w becomes
-//   scale w + w E(Omega),  E = scale_lo (1 + Dxy) + scale D + ... = g0 + Dt g1,
-//   1 + Dxy = (1 + Dx)(1 + Dy),  g1 = (scale + scale_lo)(1 + Dxy),
-//   g0 = scale Dxy + scale_lo (1 + Dxy).
-// The small product w E is formed first and scale w, which is exact for powers
-// of two, added with one rounding.  (Folding w into the FMA chain rounds
-// w.x - w.y E.y before the second-order term w.x (cos phi - 1) arrives; for
-// small phases that term is below half an ulp and is then always lost, so
-// |1 + E| acts as 1 + phi^2 / 2 and the energy grows step after step.)
+// factors in delta form.  1/(nx ny nt) = scale + scale_lo is applied to a value w
+// itself where it is no power of two; where it is one, it sits in the constants,
+// exactly (c = scale; c = 1 where it has been applied):
+//   c w + w E(Omega),  E = g0 + Dt g1,  1 + Dxy = (1 + Dx)(1 + Dy),
+//   g0 = c Dxy,  g1 = c (1 + Dxy).
+// (With any scale folded into g0 and g1 their rounding came on top of Dxy's, the
+// same one in every step: the parametric run of 48x256x128 points ended 12 % further
+// from FP64, and a mode of P = -1 on a grid of 3 2^k points gained 1.2e-7 of its
+// energy per step.)
+// The small product w E is formed first and c w, which is exact, added with one
+// rounding.  (Folding w into the FMA chain rounds w.x - w.y E.y before the
+// second-order term w.x (cos phi - 1) arrives; for small phases that term is below
+// half an ulp and is then always lost, so |1 + E| acts as 1 + phi^2 / 2 and the
+// energy grows step after step.)
 // conj(P) (the adjoint) turns the sign of E's imaginary part, which sits in its
 // three constants gi.
 struct ColumnProp {
-  float scale;
+  float c;
   float2 g0, g1;
   float3 gi;  // E.y = gi.x + Dt.x gi.y + Dt.y gi.z, the sign of conj(P) in it
   __device__ __forceinline__ ColumnProp(const AxisArgs& p, float2 dx, float2 dy) {
     const float2 dxy = cadd(cadd(dx, dy), cmul(dx, dy));
-    scale = p.scale;
-    const float ox = 1.f + dxy.x;
-    g1 = make_float2(fmaf(p.scale_lo, ox, p.scale * ox), fmaf(p.scale_lo, dxy.y, p.scale * dxy.y));
-    g0 = make_float2(fmaf(p.scale_lo, ox, p.scale * dxy.x), fmaf(p.scale_lo, dxy.y, p.scale * dxy.y));
+    c = p.scale_lo == 0.f ? p.scale : 1.f;
+    g0 = cscale(dxy, c);
+    g1 = make_float2(c * (1.f + dxy.x), g0.y);
     const float sg = p.conj_p ? -1.f : 1.f;
     gi = make_float3(sg * g0.y, sg * g1.y, sg * g1.x);
   }
+  // w times scale + scale_lo
+  __device__ __forceinline__ static float2 scaled(const AxisArgs& p, float2 w) {
+    return __ffma2_rn(w, make_float2(p.scale, p.scale), __fmul2_rn(w, make_float2(p.scale_lo, p.scale_lo)));
+  }
+  // w has been scaled where scale_lo != 0
   __device__ __forceinline__ float2 operator()(float2 w, float2 dt) const {
     const float ex = fmaf(dt.x, g1.x, fmaf(-dt.y, g1.y, g0.x));
     const float ey = fmaf(dt.x, gi.y, fmaf(dt.y, gi.z, gi.x));
     const float2 we = make_float2(fmaf(w.x, ex, -w.y * ey), fmaf(w.x, ey, w.y * ex));
-    return __ffma2_rn(w, make_float2(scale, scale), we);
+    return __ffma2_rn(w, make_float2(c, c), we);
   }
 };
 
+// 1/(nx ny nt) on a column's registers where it is no power of two; before the forward
+// transform, where the branch splits no block of the propagator's loads (step on grids
+// of 2^k points 1 % longer than without it; behind the transform 2 to 8 %: 128 x 256 x
+// 128 points 103.0 and 105.8 us, 2048 along tau 131.5, 133.0 and 139.8)
+template <class PL>
+__device__ __forceinline__ void scale_column(float2 (&v)[PL::E], const AxisArgs& p) {
+  if (p.scale_lo != 0.f) {
+#pragma unroll
+    for (int e = 0; e < PL::E; ++e) v[e] = ColumnProp::scaled(p, v[e]);
+  }
+}
 // The propagator on a column's registers, which hold A_hat(kx, ky, Omega_k) at
-// k = pos_last; pt: the field's tau factors
+// k = pos_last, scaled by scale_column; pt: the field's tau factors
 template <class PL>
 __device__ __forceinline__ void apply_prop(float2 (&v)[PL::E], const ColumnProp& g, const float2* pt, int t) {
   constexpr int RL = fft_radix<PL, false>(PL::NP - 1);
@@ -633,6 +653,7 @@ __device__ __forceinline__ void tprop_tile(const AxisArgs& p, long long cta_tile
   const XchCol<TX> xc{xch + tl * N * TX, tx};
   float2 v[PL::E];
   load_pencil<PL, false>(v, a.base, a.stride, t, a.act);
+  scale_column<PL>(v, p);
   fft_run<PL, false, 0, XchCol<TX>, SyncBlock, TW>(v, t, xc, tw);
   const float2 zero = make_float2(0.f, 0.f);
   const ColumnProp g(p, a.act ? p.px[a.f * p.nx + a.x] : zero, a.act ? p.py[a.f * p.ny + a.other] : zero);
@@ -750,6 +771,7 @@ __global__ void __launch_bounds__(tau_pipe_threads<PL>(), tau_pipe_ctas<PL>())
     const X xc{buf + b * N * TX, tx};
     float2 v[PL::E];
     pipe_take<PL>(v, xc, t);
+    scale_column<PL>(v, p);
     fft_run<PL, false, 0, X, SyncBlock, TwShared>(v, t, xc, TwShared{tw});
     apply_prop<PL>(v, ColumnProp(p, dx, dy), p.pt + a.f * p.nt, t);
     fft_run<PL, true, 0, X, SyncBlock, TwShared>(v, t, xc, TwShared{tw});
