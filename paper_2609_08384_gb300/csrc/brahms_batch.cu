@@ -234,7 +234,7 @@ __device__ __noinline__ void run_item(const InstDev& I, const Item& it, float4* 
     for (int i = threadIdx.x; i < tw_table_size<typename SH::PT>(); i += kBT) tw[i] = I.twt[i];
     __syncthreads();
     for (long long c = 0; c < it.ntiles; ++c) {
-      tprop_tile<typename SH::PT, kBT>(a, it.tile + c, TwShared{tw}, xch);
+      tprop_tile<typename SH::PT, (NXY & (NXY - 1)) != 0 || (NT & (NT - 1)) != 0, kBT>(a, it.tile + c, TwShared{tw}, xch);
       __syncthreads();
     }
   } else {
@@ -673,6 +673,9 @@ brahms_status prepare_grouped(brahms_batch* b) {
     z.ny = g.ny;
     z.nt = g.nt;
     z.xtiles = 1;
+    const double inv_n = 1.0 / ((double)g.nx * g.ny * g.nt);  // picks the tau-pass's instance
+    z.scale = (float)inv_n;
+    z.scale_lo = (float)(inv_n - (double)z.scale);
     BB_CK(run_axis_fft(g.ny, 1, false, z, b->stream));
     BB_CK(run_axis_fft(g.ny, 1, true, z, b->stream));
     BB_CK(run_tpass_prop(g.nt, z, b->stream));

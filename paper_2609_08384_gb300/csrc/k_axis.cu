@@ -22,12 +22,12 @@ static cudaError_t launch_axis(const AxisArgs& a, cudaStream_t s) {
 }
 
 // The pipelined tau-pass: one wave of persistent CTAs over tiles of its own width.
-template <class PL>
+template <class PL, bool SCALED>
 static cudaError_t launch_tprop_pipe(const AxisArgs& a0, cudaStream_t s) {
   constexpr int TX = tau_pipe_cols<PL>();
   constexpr size_t smem = (size_t)tau_pipe_smem<PL>();
   static SmemOnce once;
-  cudaError_t e = raise_smem_limit(tpass_pipe_kernel<PL>, smem, once);
+  cudaError_t e = raise_smem_limit(tpass_pipe_kernel<PL, SCALED>, smem, once);
   if (e != cudaSuccess || a0.ntiles <= 0) return e;
   AxisArgs a = a0;
   const long long lines = a0.ntiles / a0.xtiles;  // (field, y) lines
@@ -35,24 +35,24 @@ static cudaError_t launch_tprop_pipe(const AxisArgs& a0, cudaStream_t s) {
   a.ntiles = lines * a.xtiles;
   const long long wave = 152 * tau_pipe_ctas<PL>();
   const long long grid = a.ntiles < wave ? a.ntiles : wave;
-  return launch_chained(tpass_pipe_kernel<PL>, dim3((unsigned)grid), tau_pipe_threads<PL>(), smem, s, a);
+  return launch_chained(tpass_pipe_kernel<PL, SCALED>, dim3((unsigned)grid), tau_pipe_threads<PL>(), smem, s, a);
 }
 
-template <int N>
+template <int N, bool SCALED>
 static cudaError_t launch_tprop(const AxisArgs& a, cudaStream_t s) {
   using PL = TauPlan<N>;
   if constexpr (tau_pipe<PL>()) {
-    return launch_tprop_pipe<PL>(a, s);
+    return launch_tprop_pipe<PL, SCALED>(a, s);
   } else {
     constexpr int TPC = tiles_per_cta<PL>();
     constexpr int THREADS = TPC * tile_threads<PL>();
     const size_t smem = (size_t)axis_smem_floats2<PL>() * sizeof(float2);
     static SmemOnce once;
-    cudaError_t e = raise_smem_limit(tpass_prop_kernel<PL>, smem, once);
+    cudaError_t e = raise_smem_limit(tpass_prop_kernel<PL, SCALED>, smem, once);
     if (e != cudaSuccess) return e;
     const long long grid = (a.ntiles + TPC - 1) / TPC;
     if (grid <= 0) return cudaSuccess;
-    return launch_chained(tpass_prop_kernel<PL>, dim3((unsigned)grid), THREADS, smem, s, a);
+    return launch_chained(tpass_prop_kernel<PL, SCALED>, dim3((unsigned)grid), THREADS, smem, s, a);
   }
 }
 
@@ -71,9 +71,11 @@ cudaError_t run_axis_fft(int n, int axis, bool inv, const AxisArgs& a, cudaStrea
 
 cudaError_t run_tpass_prop(int nt, const AxisArgs& a, cudaStream_t s) {
   switch (nt) {
-#define BRAHMS_T_CASE(N) \
-  case N:                \
-    return launch_tprop<N>(a, s);
+#define BRAHMS_T_CASE(N)                                       \
+  case N:                                                      \
+    if constexpr ((N & (N - 1)) == 0)                          \
+      if (a.scale_lo == 0.f) return launch_tprop<N, false>(a, s); \
+    return launch_tprop<N, true>(a, s);
     BRAHMS_FOR_EACH_SIZE(BRAHMS_T_CASE)
 #undef BRAHMS_T_CASE
     default:

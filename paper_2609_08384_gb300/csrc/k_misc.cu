@@ -260,9 +260,9 @@ __global__ void prop_pointwise_kernel(const AxisArgs p, int nf) {
     const int x = (int)(r % p.nx);
     const int y = (int)((r / p.nx) % p.ny);
     const int t = (int)(r / plane);
-    const ColumnProp g(p, p.px[f * p.nx + x], p.py[f * p.ny + y]);
+    const float2 dx = p.px[f * p.nx + x], dy = p.py[f * p.ny + y], dt = p.pt[f * p.nt + t];
     float2* q = p.data + (long long)f * p.fstride + r;
-    *q = g(p.scale_lo == 0.f ? *q : ColumnProp::scaled(p, *q), p.pt[f * p.nt + t]);
+    *q = p.scale_lo == 0.f ? ColumnProp<false>(p, dx, dy)(p, *q, dt) : ColumnProp<true>(p, dx, dy)(p, *q, dt);
   }
 }
 

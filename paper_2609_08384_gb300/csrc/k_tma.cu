@@ -158,11 +158,11 @@ __global__ void __launch_bounds__(PL::T * TX, PL::T * TX <= 256 ? 2 : 1)
       for (int r = 0; r < R0; ++r) v[bb * R0 + r] = xc.ld(pos_first<PL, false>(t + bb * T, r));
     using TWA = typename std::conditional<tw_in_smem<PL>(), TwShared, TwGlobal>::type;
     const TWA tw{tw_in_smem<PL>() ? tws : p.tw};
-    scale_column<PL>(v, p);
     fft_run<PL, false, 0, XchCol<TX>, SyncBlock, TWA>(v, t, xc, tw);
     const float2 zero = make_float2(0.f, 0.f);
-    const ColumnProp g(p, act ? p.px[f * p.nx + x] : zero, act ? p.py[f * p.ny + y] : zero);
-    apply_prop<PL>(v, g, p.pt + f * p.nt, t);
+    const float2 dx = act ? p.px[f * p.nx + x] : zero, dy = act ? p.py[f * p.ny + y] : zero;
+    if (p.scale_lo == 0.f) apply_prop<PL>(v, p, ColumnProp<false>(p, dx, dy), p.pt + f * p.nt, t);
+    else apply_prop<PL>(v, p, ColumnProp<true>(p, dx, dy), p.pt + f * p.nt, t);
     fft_run<PL, true, 0, XchCol<TX>, SyncBlock, TWA>(v, t, xc, tw);
     if (act) {
       float2* base = p.data + (long long)f * p.fstride + (long long)y * p.nx + x;
@@ -258,11 +258,11 @@ __global__ void __launch_bounds__(PL::T * 16, 2)
     const int y = (int)(rest % p.ny), f = (int)(rest / p.ny);
     const int x = xt * TX + tx;
     const bool act = x < p.nx;
-    scale_column<PL>(v, p);
     fft_run<PL, false, 0, XchColSplit<TX>, SyncBlock, TwGlobal>(v, t, xc, tw);
     const float2 zero = make_float2(0.f, 0.f);
-    const ColumnProp g(p, act ? p.px[f * p.nx + x] : zero, act ? p.py[f * p.ny + y] : zero);
-    apply_prop<PL>(v, g, p.pt + f * p.nt, t);
+    const float2 dx = act ? p.px[f * p.nx + x] : zero, dy = act ? p.py[f * p.ny + y] : zero;
+    if (p.scale_lo == 0.f) apply_prop<PL>(v, p, ColumnProp<false>(p, dx, dy), p.pt + f * p.nt, t);
+    else apply_prop<PL>(v, p, ColumnProp<true>(p, dx, dy), p.pt + f * p.nt, t);
     fft_run<PL, true, 0, XchColSplit<TX>, SyncBlock, TwGlobal>(v, t, xc, tw);
     if (act) {
       float2* base = p.data + (long long)f * p.fstride + (long long)y * p.nx + x;

@@ -570,8 +570,7 @@ __device__ __forceinline__ void axis_tile(const AxisArgs& p, long long cta_tile,
 //   g0 = c Dxy,  g1 = c (1 + Dxy).
 // (With any scale folded into g0 and g1 their rounding came on top of Dxy's, the
 // same one in every step: the parametric run of 48x256x128 points ended 12 % further
-// from FP64, and a mode of P = -1 on a grid of 3 2^k points gained 1.2e-7 of its
-// energy per step.)
+// from FP64, and noise on a grid of 3 2^k points gained 6e-8 of its energy per step.)
 // The small product w E is formed first and c w, which is exact, added with one
 // rounding.  (Folding w into the FMA chain rounds w.x - w.y E.y before the
 // second-order term w.x (cos phi - 1) arrives; for small phases that term is below
@@ -579,24 +578,22 @@ __device__ __forceinline__ void axis_tile(const AxisArgs& p, long long cta_tile,
 // energy grows step after step.)
 // conj(P) (the adjoint) turns the sign of E's imaginary part, which sits in its
 // three constants gi.
+template <bool SCALED>  // the values are scaled first
 struct ColumnProp {
   float c;
   float2 g0, g1;
   float3 gi;  // E.y = gi.x + Dt.x gi.y + Dt.y gi.z, the sign of conj(P) in it
   __device__ __forceinline__ ColumnProp(const AxisArgs& p, float2 dx, float2 dy) {
     const float2 dxy = cadd(cadd(dx, dy), cmul(dx, dy));
-    c = p.scale_lo == 0.f ? p.scale : 1.f;
+    c = SCALED ? 1.f : p.scale;
     g0 = cscale(dxy, c);
     g1 = make_float2(c * (1.f + dxy.x), g0.y);
     const float sg = p.conj_p ? -1.f : 1.f;
     gi = make_float3(sg * g0.y, sg * g1.y, sg * g1.x);
   }
-  // w times scale + scale_lo
-  __device__ __forceinline__ static float2 scaled(const AxisArgs& p, float2 w) {
-    return __ffma2_rn(w, make_float2(p.scale, p.scale), __fmul2_rn(w, make_float2(p.scale_lo, p.scale_lo)));
-  }
-  // w has been scaled where scale_lo != 0
-  __device__ __forceinline__ float2 operator()(float2 w, float2 dt) const {
+  __device__ __forceinline__ float2 operator()(const AxisArgs& p, float2 w, float2 dt) const {
+    if constexpr (SCALED)
+      w = __ffma2_rn(w, make_float2(p.scale, p.scale), __fmul2_rn(w, make_float2(p.scale_lo, p.scale_lo)));
     const float ex = fmaf(dt.x, g1.x, fmaf(-dt.y, g1.y, g0.x));
     const float ey = fmaf(dt.x, gi.y, fmaf(dt.y, gi.z, gi.x));
     const float2 we = make_float2(fmaf(w.x, ex, -w.y * ey), fmaf(w.x, ey, w.y * ex));
@@ -604,27 +601,21 @@ struct ColumnProp {
   }
 };
 
-// 1/(nx ny nt) on a column's registers where it is no power of two; before the forward
-// transform, where the branch splits no block of the propagator's loads (step on grids
-// of 2^k points 1 % longer than without it; behind the transform 2 to 8 %: 128 x 256 x
-// 128 points 103.0 and 105.8 us, 2048 along tau 131.5, 133.0 and 139.8)
-template <class PL>
-__device__ __forceinline__ void scale_column(float2 (&v)[PL::E], const AxisArgs& p) {
-  if (p.scale_lo != 0.f) {
-#pragma unroll
-    for (int e = 0; e < PL::E; ++e) v[e] = ColumnProp::scaled(p, v[e]);
-  }
-}
 // The propagator on a column's registers, which hold A_hat(kx, ky, Omega_k) at
-// k = pos_last, scaled by scale_column; pt: the field's tau factors
-template <class PL>
-__device__ __forceinline__ void apply_prop(float2 (&v)[PL::E], const ColumnProp& g, const float2* pt, int t) {
+// k = pos_last; pt: the field's tau factors.  (The kernels are instantiated for both
+// kinds of grid where the plan has 2^k points: a branch here cost grids of 2^k points
+// 2 to 8 % of their step, one before the forward transform 1 %, and there the rounding
+// of the scaled values weighs more: 2 x 96x96x192 over 50 steps 1.52e-6 from FP64
+// against 1.36e-6.)
+template <class PL, bool SCALED>
+__device__ __forceinline__ void apply_prop(float2 (&v)[PL::E], const AxisArgs& p, const ColumnProp<SCALED>& g,
+                                           const float2* pt, int t) {
   constexpr int RL = fft_radix<PL, false>(PL::NP - 1);
 #pragma unroll
   for (int b = 0; b < PL::E / RL; ++b)
 #pragma unroll
     for (int r = 0; r < RL; ++r)
-      v[b * RL + r] = g(v[b * RL + r], pt[pos_last<PL, false>(t + b * PL::T, r)]);
+      v[b * RL + r] = g(p, v[b * RL + r], pt[pos_last<PL, false>(t + b * PL::T, r)]);
 }
 
 // Resident CTAs the tau-pass asks the register allocator for.  Left to itself
@@ -642,7 +633,7 @@ __host__ __device__ constexpr int tprop_min_blocks() {
 // (Measured slower on the 512-point plan: launch bounds of two CTAs per SM, a
 // persistent loop over tiles, the twiddle staging issued after this tile's
 // loads, the field's tau factors staged in shared memory with the twiddles.)
-template <class PL, int THREADS, class TW = TwShared>
+template <class PL, bool SCALED, int THREADS, class TW = TwShared>
 __device__ __forceinline__ void tprop_tile(const AxisArgs& p, long long cta_tile, const TW& tw, float2* xch) {
   constexpr int N = PL::N, T = PL::T, TX = ColTile<PL>::value;
   constexpr int TPC = tiles_per_cta_t<PL, THREADS>();
@@ -653,11 +644,10 @@ __device__ __forceinline__ void tprop_tile(const AxisArgs& p, long long cta_tile
   const XchCol<TX> xc{xch + tl * N * TX, tx};
   float2 v[PL::E];
   load_pencil<PL, false>(v, a.base, a.stride, t, a.act);
-  scale_column<PL>(v, p);
   fft_run<PL, false, 0, XchCol<TX>, SyncBlock, TW>(v, t, xc, tw);
   const float2 zero = make_float2(0.f, 0.f);
-  const ColumnProp g(p, a.act ? p.px[a.f * p.nx + a.x] : zero, a.act ? p.py[a.f * p.ny + a.other] : zero);
-  apply_prop<PL>(v, g, p.pt + (a.act ? a.f * p.nt : 0), t);
+  const ColumnProp<SCALED> g(p, a.act ? p.px[a.f * p.nx + a.x] : zero, a.act ? p.py[a.f * p.ny + a.other] : zero);
+  apply_prop<PL>(v, p, g, p.pt + (a.act ? a.f * p.nt : 0), t);
   // the inverse's first pass reads exactly these positions
   fft_run<PL, true, 0, XchCol<TX>, SyncBlock, TW>(v, t, xc, tw);
   if (a.act) store_pencil<PL, false>(v, a.base, a.stride, t);
@@ -744,7 +734,7 @@ __device__ __forceinline__ void pipe_take(float2 (&v)[PL::E], const PipeXch<PL>&
     for (int r = 0; r < R0; ++r) v[i * R0 + r] = xc.ld(pos_first<PL, false>(t + i * PL::T, r));
 }
 
-template <class PL>
+template <class PL, bool SCALED>
 __global__ void __launch_bounds__(tau_pipe_threads<PL>(), tau_pipe_ctas<PL>())
     tpass_pipe_kernel(const AxisArgs p) {
   constexpr int N = PL::N, TX = tau_pipe_cols<PL>(), THREADS = tau_pipe_threads<PL>();
@@ -771,9 +761,8 @@ __global__ void __launch_bounds__(tau_pipe_threads<PL>(), tau_pipe_ctas<PL>())
     const X xc{buf + b * N * TX, tx};
     float2 v[PL::E];
     pipe_take<PL>(v, xc, t);
-    scale_column<PL>(v, p);
-    fft_run<PL, false, 0, X, SyncBlock, TwShared>(v, t, xc, TwShared{tw});
-    apply_prop<PL>(v, ColumnProp(p, dx, dy), p.pt + a.f * p.nt, t);
+      fft_run<PL, false, 0, X, SyncBlock, TwShared>(v, t, xc, TwShared{tw});
+    apply_prop<PL>(v, p, ColumnProp<SCALED>(p, dx, dy), p.pt + a.f * p.nt, t);
     fft_run<PL, true, 0, X, SyncBlock, TwShared>(v, t, xc, TwShared{tw});
     if (act) store_pencil<PL, false>(v, a.base + tx, plane, t);
   }
@@ -797,7 +786,7 @@ __global__ void __launch_bounds__(tiles_per_cta<PL>() * tile_threads<PL>())
   }
 }
 
-template <class PL>
+template <class PL, bool SCALED>
 __global__ void __launch_bounds__(tiles_per_cta<PL>() * tile_threads<PL>(), tprop_min_blocks<PL>())
     tpass_prop_kernel(const AxisArgs p) {
   constexpr int THREADS = tiles_per_cta<PL>() * tile_threads<PL>();
@@ -809,11 +798,11 @@ __global__ void __launch_bounds__(tiles_per_cta<PL>() * tile_threads<PL>(), tpro
     chain_begin();
     // tiles from the last down: the pass ends on the first field's low-y
     // pencils, which the y-inverse then reads first
-    tprop_tile<PL, THREADS>(p, (long long)gridDim.x - 1 - blockIdx.x, TwShared{tw},
+    tprop_tile<PL, SCALED, THREADS>(p, (long long)gridDim.x - 1 - blockIdx.x, TwShared{tw},
                             tw + tw_table_size<PL>());
   } else {
     chain_begin();
-    tprop_tile<PL, THREADS>(p, blockIdx.x, TwGlobal{p.tw}, reinterpret_cast<float2*>(sm4));
+    tprop_tile<PL, SCALED, THREADS>(p, blockIdx.x, TwGlobal{p.tw}, reinterpret_cast<float2*>(sm4));
   }
 }
 
