@@ -32,9 +32,9 @@ brahms_status linear_yty(brahms_ctx* ctx, float2* data, bool adjoint) {
   at.data = data;
   at.conj_p = adjoint ? 1 : 0;
   if (use_field_streams(ctx)) return enqueue_linear_split(ctx, ay, at);
-  BR_CK(launch(ctx, 1, 1, [&] { return brahms::run_axis_fft(ctx->ny, 1, false, ay, ctx->stream); }));
+  BR_CK(launch(ctx, 1, 1, [&] { return brahms::run_ypass(ctx->ny, false, ay, ctx->stream); }));
   BR_CK(launch(ctx, 2, 1, [&] { return brahms::run_tpass_prop(ctx->nt, at, ctx->stream); }));
-  BR_CK(launch(ctx, 3, 1, [&] { return brahms::run_axis_fft(ctx->ny, 1, true, ay, ctx->stream); }));
+  BR_CK(launch(ctx, 3, 1, [&] { return brahms::run_ypass(ctx->ny, true, ay, ctx->stream); }));
   return BRAHMS_OK;
 }
 

@@ -103,6 +103,9 @@ brahms_status brahms_init_grid(brahms_ctx** out, int nx, int ny, int nt, double 
   ctx->twx = (float2*)(ctx->ws + ctx->L.twx);
   ctx->twy = (float2*)(ctx->ws + ctx->L.twy);
   ctx->twt = (float2*)(ctx->ws + ctx->L.twt);
+  ctx->twpx = (float4*)(ctx->ws + ctx->L.twpx);
+  ctx->twpy = (float4*)(ctx->ws + ctx->L.twpy);
+  ctx->twpt = (float4*)(ctx->ws + ctx->L.twpt);
   ctx->partial = (double*)(ctx->ws + ctx->L.partial);
   ctx->dev_err = (int*)(ctx->ws + ctx->L.err);
   ctx->diag_dev = (double*)(ctx->ws + ctx->L.diag);
@@ -117,6 +120,9 @@ brahms_status brahms_init_grid(brahms_ctx** out, int nx, int ny, int nt, double 
   if (e == cudaSuccess && ny > 1) e = brahms::upload_twiddles(ctx->twy, ny, 1, ctx->stream);
   const int nlast = tau_pass_length(ny, nt);
   if (e == cudaSuccess && nlast > 1) e = brahms::upload_twiddles(ctx->twt, nlast, 2, ctx->stream);
+  if (e == cudaSuccess) e = brahms::upload_twiddles(ctx->twpx, nx, 0, ctx->stream);
+  if (e == cudaSuccess && ny > 1) e = brahms::upload_twiddles(ctx->twpy, ny, 1, ctx->stream);
+  if (e == cudaSuccess && nt > 1) e = brahms::upload_twiddles(ctx->twpt, nt, 2, ctx->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(ctx->dev_err, 0, 2 * sizeof(int), ctx->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(ctx->mphase_dev, 0, sizeof(double) * nx * ny, ctx->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
@@ -241,7 +247,7 @@ brahms_status brahms_propagate(brahms_ctx* ctx, int nz, double dz) {
       if (s != BRAHMS_OK) return s;
     } else {
       if (ny > 1 && !plane && !cw)
-        BR_CK(launch(ctx, 1, 1, [&] { return brahms::run_axis_fft(ny, 1, false, ay, ctx->stream); }));
+        BR_CK(launch(ctx, 1, 1, [&] { return brahms::run_ypass(ny, false, ay, ctx->stream); }));
       if (cw)
         BR_CK(launch(ctx, 2, 1, [&] { return brahms::run_tpass_prop(ny, acw, ctx->stream); }));
       else if (nt == 1)
@@ -254,7 +260,7 @@ brahms_status brahms_propagate(brahms_ctx* ctx, int nz, double dz) {
       else
         BR_CK(launch(ctx, 2, 1, [&] { return brahms::run_tpass_prop(nt, at, ctx->stream); }));
       if (ny > 1 && !plane && !cw)
-        BR_CK(launch(ctx, 3, 1, [&] { return brahms::run_axis_fft(ny, 1, true, ay, ctx->stream); }));
+        BR_CK(launch(ctx, 3, 1, [&] { return brahms::run_ypass(ny, true, ay, ctx->stream); }));
     }
     const bool last = (i == nz - 1);
     brahms::XPassArgs a = xargs(ctx, last ? brahms::XM_NL_LAST : brahms::XM_NL_MID, dz);
@@ -354,11 +360,14 @@ brahms_status brahms_transform(brahms_ctx* ctx, int direction) {
   touch(ctx);
   const brahms::AxisArgs ay = aargs(ctx, 1), at = aargs(ctx, 2, false);
   const bool inv = direction == 1;
-  brahms::XPassArgs a = xargs(ctx, inv ? brahms::XM_INV : brahms::XM_FWD, 1.0);
+  brahms::XLineArgs a{};
+  a.data = ctx->state;
+  a.rows = (long long)ctx->nf * ctx->ny * ctx->nt;
+  a.twp = ctx->twpx;
   const double inv_n = 1.0 / (double)ctx->npoints();
   a.scale = (float)inv_n;
   a.scale_lo = (float)(inv_n - (double)a.scale);
-  BR_CK(launch(ctx, 0, 1, [&] { return brahms::run_xpass(ctx->nx, ctx->nf, a, ctx->stream); }));
+  BR_CK(launch(ctx, 0, 1, [&] { return brahms::run_xline_fft(ctx->nx, inv, a, ctx->stream); }));
   if (ctx->ny > 1) BR_CK(launch(ctx, 1, 1, [&] { return brahms::run_axis_fft(ctx->ny, 1, inv, ay, ctx->stream); }));
   if (ctx->nt > 1) BR_CK(launch(ctx, 2, 1, [&] { return brahms::run_axis_fft(ctx->nt, 2, inv, at, ctx->stream); }));
   BR_CK(cudaStreamSynchronize(ctx->stream));

@@ -194,7 +194,6 @@ __device__ __noinline__ void run_item(const InstDev& I, const Item& it, float4* 
       p.kh[f] = I.kh[f];
       p.kh2[f] = I.kh2[f];
     }
-    p.scale = 1.f;
     if (it.step < 0) {
       p.mode = XM_NL_FIRST;
       p.phiA = 0.0;
@@ -676,8 +675,8 @@ brahms_status prepare_grouped(brahms_batch* b) {
     const double inv_n = 1.0 / ((double)g.nx * g.ny * g.nt);  // picks the tau-pass's instance
     z.scale = (float)inv_n;
     z.scale_lo = (float)(inv_n - (double)z.scale);
-    BB_CK(run_axis_fft(g.ny, 1, false, z, b->stream));
-    BB_CK(run_axis_fft(g.ny, 1, true, z, b->stream));
+    BB_CK(run_ypass(g.ny, false, z, b->stream));
+    BB_CK(run_ypass(g.ny, true, z, b->stream));
     BB_CK(run_tpass_prop(g.nt, z, b->stream));
     XPassArgs x{};
     BB_CK(run_xpass_group(g.nx, x, g.params, g.ecoef, kStageFactors, 0, 0, b->stream));
@@ -710,7 +709,6 @@ brahms_status prepare_grouped(brahms_batch* b) {
     base.fstride = n;
     base.rows = (long long)g.ny * g.nt;
     base.tw = g.twx;
-    base.scale = 1.f;
     base.ny = g.ny;
     // an x-pass over the first a slots (the plane pass, which takes the y-passes
     // with it, where the plane has one; per instance where an instance's rows do
@@ -774,9 +772,9 @@ brahms_status prepare_grouped(brahms_batch* b) {
       while (a > 0 && nzs[a - 1] <= j) --a;  // slots still running at step j
       ay.ntiles = 2LL * a * g.nt * ay.xtiles;
       at.ntiles = 2LL * a * g.ny * at.xtiles;
-      if (!plane) e = run_axis_fft(g.ny, 1, false, ay, s);
+      if (!plane) e = run_ypass(g.ny, false, ay, s);
       if (e == cudaSuccess) e = run_tpass_prop(g.nt, at, s);
-      if (e == cudaSuccess && !plane) e = run_axis_fft(g.ny, 1, true, ay, s);
+      if (e == cudaSuccess && !plane) e = run_ypass(g.ny, true, ay, s);
       if (e == cudaSuccess) e = xpass(j, a);
       nl += (plane ? 1 : 3) + (plane || whole ? 1 : a);
     }

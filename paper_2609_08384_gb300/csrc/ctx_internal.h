@@ -30,7 +30,7 @@ inline size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
 inline int tau_pass_length(int ny, int nt) { return nt > 1 ? nt : ny; }
 
 struct Layout {
-  size_t state, px, py, pt, twx, twy, twt, partial, err, diag, dkmap, usermap, mphase, emap, total;
+  size_t state, px, py, pt, twx, twy, twt, twpx, twpy, twpt, partial, err, diag, dkmap, usermap, mphase, emap, total;
 };
 
 inline Layout make_layout(int nx, int ny, int nt, int nf) {
@@ -49,6 +49,9 @@ inline Layout make_layout(int nx, int ny, int nt, int nf) {
   L.twx = take(sizeof(float2) * brahms::tw_table_size_of(nx, 0));
   L.twy = take(sizeof(float2) * brahms::tw_table_size_of(ny, 1));
   L.twt = take(sizeof(float2) * brahms::tw_table_size_of(tau_pass_length(ny, nt), 2));
+  L.twpx = take(sizeof(float4) * brahms::tw_table_size_of(nx, 0));
+  L.twpy = take(sizeof(float4) * brahms::tw_table_size_of(ny, 1));
+  L.twpt = take(sizeof(float4) * brahms::tw_table_size_of(nt, 2));
   L.partial = take(sizeof(double) * kRedBlocks * nf);
   L.err = take(2 * sizeof(int));
   L.diag = take(sizeof(double) * 2 * nt * nf);
@@ -79,6 +82,7 @@ struct brahms_ctx {
   Layout L{};
   float2 *state = nullptr, *px = nullptr, *py = nullptr, *pt = nullptr;
   float2 *twx = nullptr, *twy = nullptr, *twt = nullptr;
+  float4 *twpx = nullptr, *twpy = nullptr, *twpt = nullptr;  // as products
   double* partial = nullptr;
   double* energy_host = nullptr;  // pinned, nf entries + the device error word
   double* diag_dev = nullptr;     // diagnostics: power [nf][nt], spectrum [nf][nt]
@@ -282,7 +286,6 @@ inline brahms::XPassArgs xargs(brahms_ctx* c, int mode, double dz) {
     a.kh[f] = (float)(k * 0.5 * dz);
     a.kh2[f] = 0.5f * a.kh[f];
   }
-  a.scale = 1.f;
   a.ny = c->ny;
   a.emap = c->have_map ? c->emap_dev : nullptr;
   return a;
@@ -374,6 +377,7 @@ inline brahms::AxisArgs aargs(brahms_ctx* c, int axis, bool tau_prop = true) {
   a.xtiles = (c->nx + tx - 1) / tx;
   a.ntiles = (long long)c->nf * (axis == 1 ? c->nt : c->ny) * a.xtiles;
   a.tw = axis == 1 ? c->twy : c->twt;
+  a.twp = axis == 1 ? c->twpy : c->twpt;
   a.px = c->px;
   a.py = c->py;
   a.pt = c->pt;
@@ -452,10 +456,10 @@ inline brahms_status enqueue_linear_split(brahms_ctx* ctx, const brahms::AxisArg
     const brahms::AxisArgs ayf = field_args(ctx, ay, f), atf = field_args(ctx, at, f);
     BR_CK(cudaStreamWaitEvent(st, ctx->ev_x, 0));
     if (f > 0) BR_CK(cudaStreamWaitEvent(st, ctx->ev_y[f - 1], 0));
-    BR_CK(launch_on(ctx, st, 1, 1, [&] { return brahms::run_axis_fft(ctx->ny, 1, false, ayf, st); }));
+    BR_CK(launch_on(ctx, st, 1, 1, [&] { return brahms::run_ypass(ctx->ny, false, ayf, st); }));
     BR_CK(cudaEventRecord(ctx->ev_y[f], st));
     BR_CK(launch_on(ctx, st, 2, 1, [&] { return brahms::run_tpass_prop(ctx->nt, atf, st); }));
-    BR_CK(launch_on(ctx, st, 3, 1, [&] { return brahms::run_axis_fft(ctx->ny, 1, true, ayf, st); }));
+    BR_CK(launch_on(ctx, st, 3, 1, [&] { return brahms::run_ypass(ctx->ny, true, ayf, st); }));
     BR_CK(cudaEventRecord(ctx->ev_done[f], st));
   }
   for (int f = 0; f < ctx->nf; ++f) BR_CK(cudaStreamWaitEvent(ctx->stream, ctx->ev_done[f], 0));

@@ -100,8 +100,21 @@ __device__ __forceinline__ float2 shear_turn(float2 a, float p, float s) {
   return make_float2(fmaf(p, y, x), y);
 }
 
+// A turn by a table entry, and the turn back: by the shears of w, or by the product
+// with (cos + i sin) as hi + lo floats, w = (cos hi, sin hi, cos lo, sin lo), which
+// single transforms take (TwProduct)
+__device__ __forceinline__ float2 turn(float2 a, float2 w) { return shear_turn(a, w.x, w.y); }
+__device__ __forceinline__ float2 turn_back(float2 a, float2 w) { return shear_turn(a, -w.x, -w.y); }
+__device__ __forceinline__ float2 turn(float2 a, float4 w) {
+  return make_float2(fmaf(w.x, a.x, fmaf(-w.y, a.y, fmaf(w.z, a.x, -w.w * a.y))),
+                     fmaf(w.x, a.y, fmaf(w.y, a.x, fmaf(w.z, a.y, w.w * a.x))));
+}
+__device__ __forceinline__ float2 turn_back(float2 a, float4 w) {
+  return turn(a, make_float4(w.x, -w.y, w.z, -w.w));
+}
+
 // ---------------------------------------------------------------- codelets
-// tan(pi k / 32) and sin(pi k / 16), k = 0..4
+// tan(pi k / 32), sin(pi k / 16) and cos(pi k / 16), k = 0..4
 __host__ __device__ constexpr double tan_pi32(int k) {
   return k == 0 ? 0.0
        : k == 1 ? 0.098491403357164253077197521291327
@@ -116,12 +129,20 @@ __host__ __device__ constexpr double sin_pi16(int k) {
        : k == 3 ? 0.55557023301960222474283081394853
                 : 0.70710678118654752440084436210485;
 }
+__host__ __device__ constexpr double cos_pi16(int k) {
+  return k == 0 ? 1.0
+       : k == 1 ? 0.98078528040323044912618223613424
+       : k == 2 ? 0.92387953251128675612818318939679
+       : k == 3 ? 0.83146961230254523707878837761791
+                : 0.70710678118654752440084436210485;
+}
 // W32^E = (-/+ i)^quarter(E) W32^rest(E), rest in [-3, 4]
 __host__ __device__ constexpr int w32_quarter(int e) { return ((e + 3) / 8) % 4; }
 __host__ __device__ constexpr int w32_rest(int e) { return e - 8 * ((e + 3) / 8); }
-// a times W32^rest(E); the quarter turns are left to the additions that follow
-template <bool INV, int E>
-__device__ __forceinline__ float2 w32_shear(float2 a) {
+// a times W32^rest(E); the quarter turns are left to the additions that follow.
+// PROD: the product with hi + lo floats, for single transforms
+template <bool INV, int E, bool PROD>
+__device__ __forceinline__ float2 w32_turn(float2 a) {
   constexpr int k = w32_rest(E);
   if constexpr (k == 0) return a;
   else {
@@ -135,11 +156,16 @@ __device__ __forceinline__ float2 w32_shear(float2 a) {
       const float2 d = pos ? make_float2(a.x - a.y, a.x + a.y) : make_float2(a.x + a.y, a.y - a.x);
       constexpr float ch = (float)sin_pi16(4), cl = (float)(sin_pi16(4) - (double)ch);
       return __ffma2_rn(d, make_float2(ch, ch), __fmul2_rn(d, make_float2(cl, cl)));
+    } else if constexpr (PROD) {
+      constexpr double c = cos_pi16(ak), sn = pos ? sin_pi16(ak) : -sin_pi16(ak);
+      constexpr float ch = (float)c, sh = (float)sn;
+      return turn(a, make_float4(ch, sh, (float)(c - (double)ch), (float)(sn - (double)sh)));
     } else {
       // one sixteenth of a turn: p one float off tan(pi/16) makes the pair of
       // floats eight times nearer to orthogonal (7e-10 against 6e-9) for an angle
       // 6e-8 off, which the way back undoes: energy of the 1000-step parametric
-      // run +2.3e-7 instead of -7.4e-7
+      // run +2.3e-7 instead of -7.4e-7 (a single transform shows it: 8 % more error
+      // at 256 and 512 points)
       constexpr float pk = ak == 2 ? 0.198912397f : (float)tan_pi32(ak);
       constexpr float sk = ak == 2 ? 0.382683486f : (float)sin_pi16(ak);
       return shear_turn(a, pos ? -pk : pk, pos ? sk : -sk);
@@ -184,13 +210,13 @@ __device__ __forceinline__ void dft3(float2& v0, float2& v1, float2& v2) {
 // Radix 8: forward n = 4 n1 + n2, k = k1 + 2 k2 as sums over n1, turns by
 // W8^{n2 k1}, four-point transforms over n2; the inverse takes the same steps
 // backwards (its input number k may carry a pending quarter turn Qk).
-template <int Q1 = 0, int Q2 = 0, int Q3 = 0, int Q4 = 0, int Q5 = 0, int Q6 = 0, int Q7 = 0>
+template <bool PROD, int Q1 = 0, int Q2 = 0, int Q3 = 0, int Q4 = 0, int Q5 = 0, int Q6 = 0, int Q7 = 0>
 __device__ __forceinline__ void idft8(float2* v) {
   static_assert(Q1 == 0, "number 1 carries no turn");
   dft4<true, Q2, Q4, Q6>(v[0], v[2], v[4], v[6]);
   dft4<true, Q3, Q5, Q7>(v[1], v[3], v[5], v[7]);
   const float2 y0[4] = {v[0], v[2], v[4], v[6]};
-  const float2 y1[4] = {v[1], w32_shear<true, 4>(v[3]), v[5], w32_shear<true, 12>(v[7])};
+  const float2 y1[4] = {v[1], w32_turn<true, 4, PROD>(v[3]), v[5], w32_turn<true, 12, PROD>(v[7])};
   v[0] = cadd(y0[0], y1[0]);
   v[4] = csub(y0[0], y1[0]);
   v[1] = cadd(y0[1], y1[1]);
@@ -200,10 +226,10 @@ __device__ __forceinline__ void idft8(float2* v) {
   v[3] = add_turned<true, 1>(y0[3], y1[3]);
   v[7] = add_turned<true, 3>(y0[3], y1[3]);
 }
-template <bool INV>
+template <bool INV, bool PROD>
 __device__ __forceinline__ void dft8(float2* v) {
   if constexpr (INV) {
-    idft8<>(v);
+    idft8<PROD>(v);
   } else {
     float2 y0[4], y1[4];
 #pragma unroll
@@ -211,8 +237,8 @@ __device__ __forceinline__ void dft8(float2* v) {
       y0[n2] = cadd(v[n2], v[n2 + 4]);
       y1[n2] = csub(v[n2], v[n2 + 4]);
     }
-    y1[1] = w32_shear<false, 4>(y1[1]);
-    y1[3] = w32_shear<false, 12>(y1[3]);
+    y1[1] = w32_turn<false, 4, PROD>(y1[1]);
+    y1[3] = w32_turn<false, 12, PROD>(y1[3]);
     dft4<false>(y0[0], y0[1], y0[2], y0[3]);
     dft4<false, w32_quarter(4), w32_quarter(8), w32_quarter(12)>(y1[0], y1[1], y1[2], y1[3]);
 #pragma unroll
@@ -226,19 +252,19 @@ __device__ __forceinline__ void dft8(float2* v) {
 // Radix 4 M (M = 4 or 8): n = 4 n1 + n2 (n1 < M, n2 < 4), k = k1 + M k2: M-point
 // transforms over n1, turns by W_{4M}^{n2 k1}, four-point transforms over n2
 // (radix 16 is its own mirror; radix 32's inverse runs them backwards)
-template <bool INV, int M, int K1>
+template <bool INV, int M, int K1, bool PROD>
 __device__ __forceinline__ void dft4m_column(float2 (&y)[4][M], float2* v) {
   constexpr int U = 8 / M;  // W_{4M} = W32^U
-  float2 b0 = y[0][K1], b1 = w32_shear<INV, U * K1>(y[1][K1]), b2 = w32_shear<INV, 2 * U * K1>(y[2][K1]),
-         b3 = w32_shear<INV, 3 * U * K1>(y[3][K1]);
+  float2 b0 = y[0][K1], b1 = w32_turn<INV, U * K1, PROD>(y[1][K1]), b2 = w32_turn<INV, 2 * U * K1, PROD>(y[2][K1]),
+         b3 = w32_turn<INV, 3 * U * K1, PROD>(y[3][K1]);
   dft4<INV, w32_quarter(U * K1), w32_quarter(2 * U * K1), w32_quarter(3 * U * K1)>(b0, b1, b2, b3);
   v[K1] = b0;
   v[K1 + M] = b1;
   v[K1 + 2 * M] = b2;
   v[K1 + 3 * M] = b3;
-  if constexpr (K1 + 1 < M) dft4m_column<INV, M, K1 + 1>(y, v);
+  if constexpr (K1 + 1 < M) dft4m_column<INV, M, K1 + 1, PROD>(y, v);
 }
-template <bool INV>
+template <bool INV, bool PROD>
 __device__ __forceinline__ void dft16(float2* v) {
   float2 y[4][4];
 #pragma unroll
@@ -247,25 +273,25 @@ __device__ __forceinline__ void dft16(float2* v) {
     for (int n1 = 0; n1 < 4; ++n1) y[n2][n1] = v[4 * n1 + n2];
     dft4<INV>(y[n2][0], y[n2][1], y[n2][2], y[n2][3]);
   }
-  dft4m_column<INV, 4, 0>(y, v);
+  dft4m_column<INV, 4, 0, PROD>(y, v);
 }
 // row n2 of the inverse radix 32: turns by W32^{n2 k1}, eight points over k1
-template <int N2>
+template <int N2, bool PROD>
 __device__ __forceinline__ void idft32_row(float2 (&y)[4][8], float2* v) {
   float2* z = y[N2];
-  z[1] = w32_shear<true, N2>(z[1]);
-  z[2] = w32_shear<true, 2 * N2>(z[2]);
-  z[3] = w32_shear<true, 3 * N2>(z[3]);
-  z[4] = w32_shear<true, 4 * N2>(z[4]);
-  z[5] = w32_shear<true, 5 * N2>(z[5]);
-  z[6] = w32_shear<true, 6 * N2>(z[6]);
-  z[7] = w32_shear<true, 7 * N2>(z[7]);
-  idft8<w32_quarter(N2), w32_quarter(2 * N2), w32_quarter(3 * N2), w32_quarter(4 * N2), w32_quarter(5 * N2),
+  z[1] = w32_turn<true, N2, PROD>(z[1]);
+  z[2] = w32_turn<true, 2 * N2, PROD>(z[2]);
+  z[3] = w32_turn<true, 3 * N2, PROD>(z[3]);
+  z[4] = w32_turn<true, 4 * N2, PROD>(z[4]);
+  z[5] = w32_turn<true, 5 * N2, PROD>(z[5]);
+  z[6] = w32_turn<true, 6 * N2, PROD>(z[6]);
+  z[7] = w32_turn<true, 7 * N2, PROD>(z[7]);
+  idft8<PROD, w32_quarter(N2), w32_quarter(2 * N2), w32_quarter(3 * N2), w32_quarter(4 * N2), w32_quarter(5 * N2),
         w32_quarter(6 * N2), w32_quarter(7 * N2)>(z);
 #pragma unroll
   for (int n1 = 0; n1 < 8; ++n1) v[4 * n1 + N2] = z[n1];
 }
-template <bool INV>
+template <bool INV, bool PROD>
 __device__ __forceinline__ void dft32(float2* v) {
   float2 y[4][8];
   if constexpr (INV) {
@@ -275,18 +301,18 @@ __device__ __forceinline__ void dft32(float2* v) {
       for (int k2 = 0; k2 < 4; ++k2) y[k2][k1] = v[k1 + 8 * k2];
       dft4<true>(y[0][k1], y[1][k1], y[2][k1], y[3][k1]);
     }
-    idft32_row<0>(y, v);
-    idft32_row<1>(y, v);
-    idft32_row<2>(y, v);
-    idft32_row<3>(y, v);
+    idft32_row<0, PROD>(y, v);
+    idft32_row<1, PROD>(y, v);
+    idft32_row<2, PROD>(y, v);
+    idft32_row<3, PROD>(y, v);
   } else {
 #pragma unroll
     for (int n2 = 0; n2 < 4; ++n2) {
 #pragma unroll
       for (int n1 = 0; n1 < 8; ++n1) y[n2][n1] = v[4 * n1 + n2];
-      dft8<false>(y[n2]);
+      dft8<false, PROD>(y[n2]);
     }
-    dft4m_column<false, 8, 0>(y, v);
+    dft4m_column<false, 8, 0, PROD>(y, v);
   }
 }
 
@@ -294,7 +320,7 @@ __device__ __forceinline__ void dft32(float2* v) {
 // n = M n1 + 3 n2 and k = M (1/M mod 3) k1 + 3 (1/3 mod M) k2, both mod 3 M, the
 // transform is M-point transforms over n2 and three-point ones over n1 with no
 // turns between them.
-template <bool INV, int M>
+template <bool INV, int M, bool PROD>
 __device__ __forceinline__ void dft3m(float2* v) {
   constexpr int N = 3 * M, K1 = M * (M % 3 == 1 ? 1 : 2), K2 = 3 * (M == 2 ? 1 : 3);
   float2 y[3][M];
@@ -304,7 +330,7 @@ __device__ __forceinline__ void dft3m(float2* v) {
     for (int n2 = 0; n2 < M; ++n2) y[n1][n2] = v[(M * n1 + 3 * n2) % N];
     if constexpr (M == 2) dft2<INV>(y[n1][0], y[n1][1]);
     else if constexpr (M == 4) dft4<INV>(y[n1][0], y[n1][1], y[n1][2], y[n1][3]);
-    else dft8<INV>(y[n1]);
+    else dft8<INV, PROD>(y[n1]);
   }
 #pragma unroll
   for (int k2 = 0; k2 < M; ++k2) {
@@ -314,17 +340,17 @@ __device__ __forceinline__ void dft3m(float2* v) {
   }
 }
 
-template <int R, bool INV>
+template <int R, bool INV, bool PROD = false>
 __device__ __forceinline__ void dft(float2* v) {
   if constexpr (R == 2) dft2<INV>(v[0], v[1]);
   else if constexpr (R == 3) dft3<INV>(v[0], v[1], v[2]);
   else if constexpr (R == 4) dft4<INV>(v[0], v[1], v[2], v[3]);
-  else if constexpr (R == 6) dft3m<INV, 2>(v);
-  else if constexpr (R == 8) dft8<INV>(v);
-  else if constexpr (R == 12) dft3m<INV, 4>(v);
-  else if constexpr (R == 24) dft3m<INV, 8>(v);
-  else if constexpr (R == 16) dft16<INV>(v);
-  else if constexpr (R == 32) dft32<INV>(v);
+  else if constexpr (R == 6) dft3m<INV, 2, PROD>(v);
+  else if constexpr (R == 8) dft8<INV, PROD>(v);
+  else if constexpr (R == 12) dft3m<INV, 4, PROD>(v);
+  else if constexpr (R == 24) dft3m<INV, 8, PROD>(v);
+  else if constexpr (R == 16) dft16<INV, PROD>(v);
+  else if constexpr (R == 32) dft32<INV, PROD>(v);
   else static_assert(R == 2, "unsupported radix");
 }
 
@@ -499,12 +525,26 @@ __host__ __device__ constexpr int tw_table_size() {
 
 // twiddle access from shared memory or, read-only, through L1
 struct TwShared {
+  static constexpr bool kProduct = false;
   const float2* p;
   __device__ __forceinline__ float2 operator()(int i) const { return p[i]; }
 };
 struct TwGlobal {
+  static constexpr bool kProduct = false;
   const float2* p;
   __device__ __forceinline__ float2 operator()(int i) const { return __ldg(p + i); }
+};
+// the same turns as products with hi + lo floats (codelets too), for transforms that
+// nothing undoes: the spectrum, single transforms, the spectral-phase gradient
+struct TwProduct {
+  static constexpr bool kProduct = true;
+  const float4* p;
+  __device__ __forceinline__ float4 operator()(int i) const { return __ldg(p + i); }
+};
+struct TwProductShared {
+  static constexpr bool kProduct = true;
+  const float4* p;
+  __device__ __forceinline__ float4 operator()(int i) const { return p[i]; }
 };
 
 // Barrier used around shared-memory exchanges: the whole CTA, or only the
@@ -553,13 +593,12 @@ __device__ __forceinline__ void fft_run(float2 (&v)[PL::E], int t, const X& x, c
       const int m = (t + b * T) % NS;
 #pragma unroll
       for (int r = 1; r < R; ++r) {
-        const float2 w = tw(tw_pass_off<PL>(P) + r * NS + m);
-        v[b * R + r] = shear_turn(v[b * R + r], w.x, w.y);
+        v[b * R + r] = turn(v[b * R + r], tw(tw_pass_off<PL>(P) + r * NS + m));
       }
     }
   }
 #pragma unroll
-  for (int b = 0; b < B; ++b) dft<R, INV>(&v[b * R]);
+  for (int b = 0; b < B; ++b) dft<R, INV, TW::kProduct>(&v[b * R]);
   if constexpr (INV && P + 1 < NP) {
     constexpr int REST = N / (NS * R);
 #pragma unroll
@@ -567,8 +606,7 @@ __device__ __forceinline__ void fft_run(float2 (&v)[PL::E], int t, const X& x, c
       const int q = (t + b * T) / NS;
 #pragma unroll
       for (int k = 1; k < R; ++k) {
-        const float2 w = tw(tw_pass_off<PL>(NP - 1 - P) + k * REST + q);
-        v[b * R + k] = shear_turn(v[b * R + k], -w.x, -w.y);
+        v[b * R + k] = turn_back(v[b * R + k], tw(tw_pass_off<PL>(NP - 1 - P) + k * REST + q));
       }
     }
   }

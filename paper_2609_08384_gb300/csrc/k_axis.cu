@@ -7,18 +7,18 @@
 
 namespace brahms {
 
-template <int N, bool INV, int AXIS>
-static cudaError_t launch_axis(const AxisArgs& a, cudaStream_t s) {
-  using PL = AxisPlan<N, AXIS>;
+template <int N, bool INV>
+static cudaError_t launch_ypass(const AxisArgs& a, cudaStream_t s) {
+  using PL = AxisPlan<N, 1>;
   constexpr int TPC = tiles_per_cta<PL>();
   constexpr int THREADS = TPC * tile_threads<PL>();
-  const size_t smem = (size_t)axis_kernel_smem_floats2<PL, INV, AXIS>() * sizeof(float2);
+  const size_t smem = (size_t)ypass_smem_floats2<PL, INV>() * sizeof(float2);
   static SmemOnce once;
-  cudaError_t e = raise_smem_limit(axis_fft_kernel<PL, INV, AXIS>, smem, once);
+  cudaError_t e = raise_smem_limit(ypass_kernel<PL, INV>, smem, once);
   if (e != cudaSuccess) return e;
   const long long grid = (a.ntiles + TPC - 1) / TPC;
   if (grid <= 0) return cudaSuccess;
-  return launch_chained(axis_fft_kernel<PL, INV, AXIS>, dim3((unsigned)grid), THREADS, smem, s, a);
+  return launch_chained(ypass_kernel<PL, INV>, dim3((unsigned)grid), THREADS, smem, s, a);
 }
 
 // The pipelined tau-pass: one wave of persistent CTAs over tiles of its own width.
@@ -56,12 +56,11 @@ static cudaError_t launch_tprop(const AxisArgs& a, cudaStream_t s) {
   }
 }
 
-cudaError_t run_axis_fft(int n, int axis, bool inv, const AxisArgs& a, cudaStream_t s) {
-  switch (n) {
-#define BRAHMS_A_CASE(N)                                                        \
-  case N:                                                                       \
-    if (axis == 1) return inv ? launch_axis<N, true, 1>(a, s) : launch_axis<N, false, 1>(a, s); \
-    return inv ? launch_axis<N, true, 2>(a, s) : launch_axis<N, false, 2>(a, s);
+cudaError_t run_ypass(int ny, bool inv, const AxisArgs& a, cudaStream_t s) {
+  switch (ny) {
+#define BRAHMS_A_CASE(N) \
+  case N:                \
+    return inv ? launch_ypass<N, true>(a, s) : launch_ypass<N, false>(a, s);
     BRAHMS_FOR_EACH_SIZE(BRAHMS_A_CASE)
 #undef BRAHMS_A_CASE
     default:
@@ -116,14 +115,23 @@ static int plan_radices(int n, int axis, int* r) {
 
 static int centred(int d, int n) { return d >= (n + 1) / 2 ? d - n : d; }
 
+static float2 entry(double phi, const float2*) { return make_float2((float)-std::tan(0.5 * phi), (float)std::sin(phi)); }
+static float4 entry(double phi, const float4*) {
+  const double c = std::cos(phi), sn = std::sin(phi);
+  const float ch = (float)c, sh = (float)sn;
+  return make_float4(ch, sh, (float)(c - (double)ch), (float)(sn - (double)sh));
+}
+
 // Per-pass twiddle blocks (the layout of tw_pass_off): for each pass P >= 1 with
 // radix R after stride NS, entries [r][m] = the shears (-tan(phi/2), sin(phi)) of
-// phi = -2 pi r' m' / (NS R), the digits of r and m centred, evaluated in FP64.
-cudaError_t upload_twiddles(float2* tw, int n, int axis, cudaStream_t s) {
+// phi = -2 pi r' m' / (NS R), or its cosine and sine as hi + lo, the digits of r and m
+// centred, evaluated in FP64.
+template <class T>
+static cudaError_t upload(T* tw, int n, int axis, cudaStream_t s) {
   int rad[8];
   const int np = plan_radices(n, axis, rad);
   if (np <= 0) return cudaErrorInvalidValue;
-  std::vector<float2> h;
+  std::vector<T> h;
   int ns = 1;
   for (int q = 0; q < np; ++q) {
     if (q > 0) {
@@ -135,18 +143,19 @@ cudaError_t upload_twiddles(float2* tw, int n, int axis, cudaStream_t s) {
             rest /= rad[p];
             w *= rad[p];
           }
-          const double phi = -6.283185307179586476925286766559 * (double)(centred(r, rad[q]) * mc) / (double)(ns * rad[q]);
-          h.push_back(make_float2((float)-std::tan(0.5 * phi), (float)std::sin(phi)));
+          h.push_back(entry(-6.283185307179586476925286766559 * (double)(centred(r, rad[q]) * mc) / (double)(ns * rad[q]), tw));
         }
     }
     ns *= rad[q];
   }
-  if (h.empty()) h.push_back(make_float2(0.f, 0.f));
+  if (h.empty()) h.push_back(entry(0.0, tw));
   if ((int)h.size() != tw_table_size_of(n, axis)) return cudaErrorInvalidValue;
-  cudaError_t e = cudaMemcpyAsync(tw, h.data(), sizeof(float2) * h.size(), cudaMemcpyHostToDevice, s);
+  cudaError_t e = cudaMemcpyAsync(tw, h.data(), sizeof(T) * h.size(), cudaMemcpyHostToDevice, s);
   if (e != cudaSuccess) return e;
   return cudaStreamSynchronize(s);  // h is a local buffer
 }
+cudaError_t upload_twiddles(float2* tw, int n, int axis, cudaStream_t s) { return upload(tw, n, axis, s); }
+cudaError_t upload_twiddles(float4* tw, int n, int axis, cudaStream_t s) { return upload(tw, n, axis, s); }
 
 int tau_col_tile_of(int n) {
   switch (n) {

@@ -69,22 +69,26 @@ __global__ void __launch_bounds__(256) power_trace_kernel(const float2* __restri
 // power trace on the 3 x 256x256x512 state.  Persistent CTAs whose next tile
 // arrives during the transform, as in the pipelined tau-pass, took 260 us against
 // 220.)
+// (Turns as products, see TwProduct; tables of up to 20 KB in shared memory.)
+template <class PL>
+__host__ __device__ constexpr bool spectrum_tw_staged() { return tw_table_size<PL>() <= 1280; }
 template <class PL>
 __global__ void __launch_bounds__(tiles_per_cta<PL>() * tile_threads<PL>())
     tau_spectrum_kernel(const AxisArgs p, long long range, double* out) {
   constexpr int N = PL::N, E = PL::E, T = PL::T, TX = ColTile<PL>::value;
   constexpr int GT = T * TX;                       // threads of one tile group
-  constexpr int THREADS = tiles_per_cta<PL>() * GT;
   constexpr int TPC = tiles_per_cta<PL>();
   constexpr int RL = fft_radix<PL, false>(PL::NP - 1);
   constexpr int BPT = (N + GT - 1) / GT;  // bins per thread
   extern __shared__ float4 sm4[];
   float2* xch = reinterpret_cast<float2*>(sm4);
-  if constexpr (tw_in_smem<PL>()) {
-    for (int i = threadIdx.x; i < tw_table_size<PL>(); i += THREADS) xch[i] = p.tw[i];
+  if constexpr (spectrum_tw_staged<PL>()) {
+    for (int i = threadIdx.x; i < tw_table_size<PL>(); i += blockDim.x) sm4[i] = p.twp[i];
     __syncthreads();
-    xch += tw_table_size<PL>();
+    xch = reinterpret_cast<float2*>(sm4 + tw_table_size<PL>());
   }
+  using TW = typename std::conditional<spectrum_tw_staged<PL>(), TwProductShared, TwProduct>::type;
+  const TW tw{spectrum_tw_staged<PL>() ? sm4 : p.twp};
   const int lt = threadIdx.x % GT, tl = threadIdx.x / GT;
   const int tx = lt % TX, t = lt / TX;
   const XchCol<TX> xc{xch + tl * N * TX, tx};
@@ -114,8 +118,7 @@ __global__ void __launch_bounds__(tiles_per_cta<PL>() * tile_threads<PL>())
     const AxisTile<N, 2, TX> a(p, tile, tx);
     float2 v[E];
     load_pencil<PL, false>(v, a.base, a.stride, t, a.act);
-    if constexpr (tw_in_smem<PL>()) fft_run<PL, false, 0, XchCol<TX>, SyncBlock, TwShared>(v, t, xc, TwShared{reinterpret_cast<const float2*>(sm4)});
-    else fft_run<PL, false, 0, XchCol<TX>, SyncBlock, TwGlobal>(v, t, xc, TwGlobal{p.tw});
+    fft_run<PL, false, 0, XchCol<TX>, SyncBlock, TW>(v, t, xc, tw);
     __syncthreads();  // every read of the exchange space is done
 #pragma unroll
     for (int b = 0; b < E / RL; ++b)
@@ -160,7 +163,7 @@ static cudaError_t launch_spectrum(const AxisArgs& a, double* out, cudaStream_t 
   using PL = TauPlan<N>;
   constexpr int TPC = tiles_per_cta<PL>();
   constexpr int THREADS = TPC * tile_threads<PL>();
-  const size_t smem = (size_t)axis_smem_floats2<PL>() * sizeof(float2);
+  const size_t smem = (size_t)((spectrum_tw_staged<PL>() ? 2 * tw_table_size<PL>() : 0) + TPC * PL::N * ColTile<PL>::value) * sizeof(float2);
   static SmemOnce once;
   cudaError_t e = raise_smem_limit(tau_spectrum_kernel<PL>, smem, once);
   if (e != cudaSuccess) return e;

@@ -25,7 +25,7 @@
 
 namespace brahms {
 
-enum XMode : int { XM_FWD = 0, XM_INV = 1, XM_NL_FIRST = 2, XM_NL_MID = 3, XM_NL_LAST = 4 };
+enum XMode : int { XM_NL_FIRST = 2, XM_NL_MID = 3, XM_NL_LAST = 4 };
 
 constexpr int kStageFactors = 4;
 
@@ -40,7 +40,6 @@ struct XPassArgs {
   double dz;
   float kh[3];         // kappa_f * dz/2, including the 1/2 SH factor for 2 fields
   float kh2[3];        // kh / 2 (exact)
-  float scale, scale_lo;  // output scale for XM_INV, hi + lo (lo = 0 for powers of two)
   // transverse mismatch map: per-(x, y) stage phase factors [4][ny][nx]
   // (B start, B quarter-step, A start, A quarter-step; see run_map_tables),
   // or NULL for a mismatch uniform across the grid
@@ -68,6 +67,7 @@ struct AxisArgs {
   long long ntiles;
   int xtiles;
   const float2* tw;    // twiddles of the transformed axis
+  const float4* twp;   // the same as products (single transforms, the spectrum)
   const float2* px;    // [nf][nx] propagator factors (t-pass only)
   const float2* py;    // [nf][ny]
   const float2* pt;    // [nf][nt]
@@ -135,11 +135,11 @@ __host__ __device__ constexpr int axis_smem_floats2() {
 // shared memory per CTA: measured on the 3 x 256x256x512 state, 285 -> 253 us
 // per launch (the inverse y-pass, 259 -> 266, measured the other way and keeps the
 // staging; now 231 and 237, 7.0 and 6.8 TB/s).
-template <class PL, bool INV, int AXIS>
-__host__ __device__ constexpr bool axis_tw_staged() { return tw_in_smem<PL>() && !(AXIS == 1 && !INV); }
-template <class PL, bool INV, int AXIS>
-__host__ __device__ constexpr int axis_kernel_smem_floats2() {
-  return (axis_tw_staged<PL, INV, AXIS>() ? tw_table_size<PL>() : 0) +
+template <class PL, bool INV>
+__host__ __device__ constexpr bool axis_tw_staged() { return tw_in_smem<PL>() && INV; }
+template <class PL, bool INV>
+__host__ __device__ constexpr int ypass_smem_floats2() {
+  return (axis_tw_staged<PL, INV>() ? tw_table_size<PL>() : 0) +
          tiles_per_cta<PL>() * PL::N * ColTile<PL>::value;
 }
 
@@ -334,7 +334,7 @@ __device__ __forceinline__ void xpass_tile(const XPassArgs& p, long long tile, c
   const bool act = row < p.rows;
   float2* myrow = rowbuf + rl * PITCH;  // field f at myrow + f ROWS PITCH
   const int mode = p.mode;
-  const bool from_k = (mode == XM_INV || mode == XM_NL_MID || mode == XM_NL_LAST);
+  const bool from_k = mode != XM_NL_FIRST;
 
   // 1. every field's row lands in its buffer by asynchronous copies, all requested
   // up front; then field by field inverse transform (from k-space) and park
@@ -369,7 +369,7 @@ __device__ __forceinline__ void xpass_tile(const XPassArgs& p, long long tile, c
   }
 
   // 2. the RK4 half steps, two points at a time over the owned points
-  if (mode == XM_NL_MID || mode == XM_NL_LAST || mode == XM_NL_FIRST) {
+  {
     const long long nxy = (long long)p.ny * NX;
     const float2* emap = MAP ? p.emap + (act ? row % p.ny : 0) * NX : nullptr;
     // MAP: the next points' stage-factor tables are requested while these points'
@@ -434,20 +434,14 @@ __device__ __forceinline__ void xpass_tile(const XPassArgs& p, long long tile, c
     }
   }
 
-  // 3. every field: unpark, forward transform (or scale), store
-  const bool to_x = (mode == XM_INV || mode == XM_NL_LAST);
+  // 3. every field: unpark, forward transform (but on the last x-pass of a call), store
 #pragma unroll 1
   for (int f = 0; f < F; ++f) {
     const XchRow xr{myrow + f * ROWS * PITCH};
     float2* dst = p.data + f * p.fstride + (act ? row : 0) * NX;
     float2 v[E];
     unpark<PL>(xr.base, t, v);
-    if (to_x) {
-      if (mode == XM_INV) {
-#pragma unroll
-        for (int e = 0; e < E; ++e)
-          v[e] = __ffma2_rn(v[e], dup(p.scale), __fmul2_rn(v[e], dup(p.scale_lo)));
-      }
+    if (mode == XM_NL_LAST) {
       if (act) {
 #pragma unroll
         for (int b = 0; b < E / RF0; ++b)
@@ -768,21 +762,21 @@ __global__ void __launch_bounds__(tau_pipe_threads<PL>(), tau_pipe_ctas<PL>())
   }
 }
 
-template <class PL, bool INV, int AXIS>
+// y-pass of a z-step
+template <class PL, bool INV>
 __global__ void __launch_bounds__(tiles_per_cta<PL>() * tile_threads<PL>())
-    axis_fft_kernel(const AxisArgs p) {
+    ypass_kernel(const AxisArgs p) {
   constexpr int THREADS = tiles_per_cta<PL>() * tile_threads<PL>();
   extern __shared__ float4 sm4[];
-  if constexpr (axis_tw_staged<PL, INV, AXIS>()) {
+  if constexpr (axis_tw_staged<PL, INV>()) {
     float2* tw = reinterpret_cast<float2*>(sm4);
     for (int i = threadIdx.x; i < tw_table_size<PL>(); i += blockDim.x) tw[i] = p.tw[i];
     __syncthreads();
     chain_begin();
-    axis_tile<PL, INV, AXIS, THREADS>(p, blockIdx.x, TwShared{tw},
-                                      tw + tw_table_size<PL>());
+    axis_tile<PL, INV, 1, THREADS>(p, blockIdx.x, TwShared{tw}, tw + tw_table_size<PL>());
   } else {
     chain_begin();
-    axis_tile<PL, INV, AXIS, THREADS>(p, blockIdx.x, TwGlobal{p.tw}, reinterpret_cast<float2*>(sm4));
+    axis_tile<PL, INV, 1, THREADS>(p, blockIdx.x, TwGlobal{p.tw}, reinterpret_cast<float2*>(sm4));
   }
 }
 
@@ -809,7 +803,7 @@ __global__ void __launch_bounds__(tiles_per_cta<PL>() * tile_threads<PL>(), tpro
 // ------------------------------------------------------------ dispatchers
 // Each returns cudaErrorInvalidValue for an unsupported length.
 cudaError_t run_xpass(int nx, int nf, const XPassArgs& a, cudaStream_t s);
-cudaError_t run_axis_fft(int n, int axis, bool inv, const AxisArgs& a, cudaStream_t s);
+cudaError_t run_ypass(int ny, bool inv, const AxisArgs& a, cudaStream_t s);
 cudaError_t run_tpass_prop(int nt, const AxisArgs& a, cudaStream_t s);
 bool size_supported(int n);
 int col_tile_of(int n);      // columns per tile of the y/tau FFT kernels
@@ -840,6 +834,18 @@ bool plane_supported(int nx, int ny);
 cudaError_t run_plane(int nx, int ny, int nf, const XPassArgs& a, const float2* twy, cudaStream_t s);
 cudaError_t run_plane3(int nx, int ny, const XPassArgs& a, const float2* twy, cudaStream_t s);
 
+// single transforms (k_single.cu), the turns as products (TwProduct): rows of x (rows:
+// of all fields, one behind another; the output times scale + scale_lo) and, with
+// a.twp, the y axis or the tau axis
+struct XLineArgs {
+  float2* data;
+  long long rows;
+  const float4* twp;
+  float scale, scale_lo;
+};
+cudaError_t run_xline_fft(int nx, bool inv, const XLineArgs& a, cudaStream_t s);
+cudaError_t run_axis_fft(int n, int axis, bool inv, const AxisArgs& a, cudaStream_t s);
+
 // misc kernels (k_misc.cu)
 // TMA tau-pass (k_tma.cu)
 bool tma_tau_supported(int nx, int nt);
@@ -852,6 +858,8 @@ cudaError_t run_tpass_prop_tma(int nt, int tx, const void* map128, const AxisArg
 // on the host in FP64, and its size in entries
 int tw_table_size_of(int n, int axis);
 cudaError_t upload_twiddles(float2* tw, int n, int axis, cudaStream_t s);
+// the same turns as products, cos and sin as hi + lo floats
+cudaError_t upload_twiddles(float4* tw, int n, int axis, cudaStream_t s);
 struct TableArgs {
   float2* px;
   float2* py;
