@@ -6,7 +6,7 @@
 namespace brahms {
 
 template <int NX, int NY>
-__global__ void __launch_bounds__(kPlaneThreads, 2)
+__global__ void __launch_bounds__(kPlaneThreads, plane_min_blocks<NX>())
     plane_group_kernel(const XPassArgs base, const float2* twy, const GroupInst* __restrict__ gi,
                        const float2* __restrict__ ecoef, int stride, int step, int planes) {
   extern __shared__ float4 sm4[];

@@ -8,9 +8,9 @@ namespace brahms {
 
 void fill_stage_factors(XPassArgs& a) {
   const double two_pi = 6.283185307179586476925286766559;
-  const double phi[kStageFactors] = {a.phiB + a.dkB * (0.5 * a.dz), a.dkB * (0.25 * a.dz), a.phiA, a.dkA * (0.25 * a.dz)};
   for (int s = 0; s < kStageFactors; ++s) {
-    const double r = phi[s] - two_pi * std::rint(phi[s] / two_pi);
+    const double phi = s < 3 ? a.phiB + a.dkB * (0.5 * a.dz + 0.25 * a.dz * s) : a.phiA + a.dkA * (0.25 * a.dz * (s - 3));
+    const double r = phi - two_pi * std::rint(phi / two_pi);
     a.ecoef[s] = make_float2((float)std::cos(r), (float)std::sin(r));
   }
 }

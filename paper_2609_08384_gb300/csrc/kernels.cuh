@@ -27,7 +27,7 @@ namespace brahms {
 
 enum XMode : int { XM_NL_FIRST = 2, XM_NL_MID = 3, XM_NL_LAST = 4 };
 
-constexpr int kStageFactors = 4;
+constexpr int kStageFactors = 6;  // of an x-pass: the start, middle and end of both half steps
 
 struct XPassArgs {
   float2* data;        // [nf][rows][nx]
@@ -52,8 +52,8 @@ struct XPassArgs {
   float2* rec_a;
   // the stage factors of both half steps from the phases above, written by the
   // host dispatchers in FP64 (map-free x-passes read them instead of computing
-  // them per CTA): e^{+i Phi} at the start of the B half, e^{+i dkB dz/4}, and
-  // the same two of the A half
+  // them per CTA): e^{+i Phi} at the start, middle and end of the B half and of the A
+  // half
   float2 ecoef[kStageFactors];
 };
 // Host: the stage factors of an x-pass from its phases (FP64 phase, reduced
@@ -190,32 +190,45 @@ __device__ __forceinline__ void nl_slopes(Pair u, const Pair* t, Pair* n) {
   }
 }
 
+// Stage factors of a half step of length h: e0, em, e1 = e^{+i Phi} at its start,
+// middle and end, and v = e^{+i dk h/2}.  Uniform over the grid, all three come from the
+// host, formed in FP64, and v from them; under a map a point has e0 and v (MAP), and em
+// and e1 are e0 v and e0 v^2.
+template <bool MAP>
+struct Stages {
+  Pair e0, em, e1, v;
+};
+__device__ __forceinline__ Pair pair_dup(float2 c) { return {dup(c.x), dup(c.y)}; }
+__device__ __forceinline__ Stages<false> stages_of(const float2* coef) {
+  const Pair e0 = pair_dup(coef[0]), em = pair_dup(coef[1]);
+  return {e0, em, pair_dup(coef[2]), pair_mulc(em, e0)};
+}
+
 // Classical RK4 over one half step h (Sec. 3.1) of Eqs. CEp/CEs/CEi (fields p,
-// s, i) or of the degenerate pair (SH, F) at two points.  e0 = e^{+i Phi} at the
-// start of the half step and v = e^{+i dk h/2}, so the midpoint and end factors
-// are e0 v and e0 v^2; kh = kappa h and kh2 = kh/2 per field.
+// s, i) or of the degenerate pair (SH, F) at two points; kh = kappa h and kh2 = kh/2
+// per field.
 // Field 0 enters the others' slopes only through u = e A_0, so its stage values
 // are carried as u directly, with m the driving terms of stages 1..4:
-//   u1 = e0 A_0,  w = v u1,  u2 = w + i kh2 v m1,  u3 = w + i kh2 m2,
-//   u4 = v (w + i kh m3),  A_0 += i kh/6 conj(e0) (m1 + conj(v)(2 m2 + 2 m3 + conj(v) m4)),
-// 12 operations a point fewer than applying e and conj(e) to A_0 and to the
-// driving term of every stage (116 against 128 for three fields).
+//   u1 = e0 A_0,  w = em A_0,  u2 = w + i kh2 v m1,  u3 = w + i kh2 m2,
+//   u4 = e1 A_0 + i kh v m3,  A_0 += i kh/6 (conj(e0) m1 + conj(em) 2 (m2 + m3) + conj(e1) m4),
+// 128 operations a point for three fields; under a map w = v u1, u4 = v (w + i kh m3)
+// and the sum nested in v, 124, where forming em and e1 of every point would take 8 more.
 // Every stage and the final combination use the same kh_f, and the 1/6 weight is
 // common to all fields: field-dependent rounding of the weights would break the
 // Manley-Rowe balance the exact scheme keeps and let the total energy drift step
 // after step.
-template <int F>
-__device__ __forceinline__ void rk4(Pair (&a)[F], Pair e0, Pair v, const float* kh, const float* kh2) {
+template <int F, bool MAP>
+__device__ __forceinline__ void rk4(Pair (&a)[F], const Stages<MAP>& c, const float* kh, const float* kh2) {
   constexpr int G = F - 1;
   Pair t[G], n[G], acc[G];
-  const Pair u1 = pair_mul(e0, a[0]);
-  const Pair w = pair_mul(v, u1);
+  const Pair u1 = pair_mul(c.e0, a[0]);
+  const Pair w = MAP ? pair_mul(c.v, u1) : pair_mul(c.em, a[0]);
   const Pair m1 = nl_drive<F>(a + 1);
   nl_slopes<F>(u1, a + 1, acc);
 #pragma unroll
   for (int g = 0; g < G; ++g) t[g] = pair_axpy(a[g + 1], kh2[g + 1], acc[g]);
   const Pair m2 = nl_drive<F>(t);
-  nl_slopes<F>(pair_iaxpy(w, kh2[0], pair_mul(v, m1)), t, n);
+  nl_slopes<F>(pair_iaxpy(w, kh2[0], pair_mul(c.v, m1)), t, n);
 #pragma unroll
   for (int g = 0; g < G; ++g) {
     acc[g] = pair_axpy(acc[g], 2.f, n[g]);
@@ -229,15 +242,20 @@ __device__ __forceinline__ void rk4(Pair (&a)[F], Pair e0, Pair v, const float* 
     t[g] = pair_axpy(a[g + 1], kh[g + 1], n[g]);
   }
   const Pair m4 = nl_drive<F>(t);
-  nl_slopes<F>(pair_mul(v, pair_iaxpy(w, kh[0], m3)), t, n);
+  nl_slopes<F>(MAP ? pair_mul(c.v, pair_iaxpy(w, kh[0], m3)) : pair_iaxpy(pair_mul(c.e1, a[0]), kh[0], pair_mul(c.v, m3)), t, n);
 #pragma unroll
   for (int g = 0; g < G; ++g) {
     const Pair q = pair_add(acc[g], n[g]);
     a[g + 1] = pair_axpy(a[g + 1], kh[g + 1], {__fmul2_rn(q.re, dup(1.f / 6.f)), __fmul2_rn(q.im, dup(1.f / 6.f))});
   }
-  Pair m = pair_mulc(m4, v);
-  m = pair_axpy(m, 2.f, pair_add(m2, m3));
-  m = pair_mulc(pair_add(m1, pair_mulc(m, v)), e0);
+  Pair m;
+  if constexpr (MAP) {
+    m = pair_axpy(pair_mulc(m4, c.v), 2.f, pair_add(m2, m3));
+    m = pair_mulc(pair_add(m1, pair_mulc(m, c.v)), c.e0);
+  } else {
+    m = pair_axpy(pair_mulc(m1, c.e0), 2.f, pair_mulc(pair_add(m2, m3), c.em));
+    m = pair_add(m, pair_mulc(m4, c.e1));
+  }
   a[0] = pair_iaxpy(a[0], kh[0], {__fmul2_rn(m.re, dup(1.f / 6.f)), __fmul2_rn(m.im, dup(1.f / 6.f))});
 }
 
@@ -375,26 +393,24 @@ __device__ __forceinline__ void xpass_tile(const XPassArgs& p, long long tile, c
     // MAP: the next points' stage-factor tables are requested while these points'
     // RK4 pair runs
     float2 nm[4][2];
-    Pair eB, vB, eA, vA;
+    Stages<MAP> B, A;
     if constexpr (MAP) {
 #pragma unroll
       for (int q = 0; q < 4; ++q)
 #pragma unroll
         for (int u = 0; u < 2; ++u) nm[q][u] = __ldcg(emap + q * nxy + point_pos<PL>(t, u));
     } else {
-      eB = {dup(coef[0].x), dup(coef[0].y)};
-      vB = {dup(coef[1].x), dup(coef[1].y)};
-      eA = {dup(coef[2].x), dup(coef[2].y)};
-      vA = {dup(coef[3].x), dup(coef[3].y)};
+      B = stages_of(coef);
+      A = stages_of(coef + 3);
     }
 #pragma unroll 1
     for (int e = 0; e < E; e += 2) {
       if constexpr (MAP) {
         const auto pair_of = [](const float2* m) { return Pair{make_float2(m[0].x, m[1].x), make_float2(m[0].y, m[1].y)}; };
-        eB = pair_of(nm[0]);
-        vB = pair_of(nm[1]);
-        eA = pair_of(nm[2]);
-        vA = pair_of(nm[3]);
+        B.e0 = pair_of(nm[0]);
+        B.v = pair_of(nm[1]);
+        A.e0 = pair_of(nm[2]);
+        A.v = pair_of(nm[3]);
         if (e + 2 < E) {
 #pragma unroll
           for (int q = 0; q < 4; ++q)
@@ -419,13 +435,13 @@ __device__ __forceinline__ void xpass_tile(const XPassArgs& p, long long tile, c
         if constexpr (REC) {
           if (p.rec_b) record(p.rec_b);
         }
-        rk4<F>(a, eB, vB, p.kh, p.kh2);
+        rk4<F>(a, B, p.kh, p.kh2);
       }
       if (mode != XM_NL_LAST) {
         if constexpr (REC) {
           if (p.rec_a) record(p.rec_a);
         }
-        rk4<F>(a, eA, vA, p.kh, p.kh2);
+        rk4<F>(a, A, p.kh, p.kh2);
       }
 #pragma unroll
       for (int f = 0; f < F; ++f)

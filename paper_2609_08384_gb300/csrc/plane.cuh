@@ -17,6 +17,12 @@ namespace brahms {
 
 constexpr int kPlaneThreads = 256;
 
+// Resident CTAs asked for: two (every plane fits), four (64 registers) where a row is
+// one thread's, as the compiler took by itself with fewer stage factors (62 registers;
+// at 66 a step of 3 x 16x16x512 takes 17.6 us instead of 13.5).
+template <int NX>
+__host__ __device__ constexpr int plane_min_blocks() { return FftPlan<NX>::T == 1 ? 4 : 2; }
+
 // one column of a plane buffer whose rows are PITCH apart
 template <int PITCH>
 struct XchPlane {
@@ -93,8 +99,7 @@ __device__ __forceinline__ void plane_tile(const XPassArgs& p, float2* data, con
     __syncthreads();
   }
   const int t = threadIdx.x % T;
-  const Pair eB = {dup(coef[0].x), dup(coef[0].y)}, vB = {dup(coef[1].x), dup(coef[1].y)};
-  const Pair eA = {dup(coef[2].x), dup(coef[2].y)}, vA = {dup(coef[3].x), dup(coef[3].y)};
+  const Stages<false> B = stages_of(coef), A = stages_of(coef + 3);
 #pragma unroll 1
   for (int y0 = 0; y0 < NY; y0 += ROWS) {
     const int y = y0 + threadIdx.x / T;
@@ -129,8 +134,8 @@ __device__ __forceinline__ void plane_tile(const XPassArgs& p, float2* data, con
         const float4 w = *park_place<PL>(row + f * NY * PITCH, t, q);
         a[f] = {make_float2(w.x, w.y), make_float2(w.z, w.w)};
       }
-      if (mode != XM_NL_FIRST) rk4<F>(a, eB, vB, p.kh, p.kh2);
-      if (mode != XM_NL_LAST) rk4<F>(a, eA, vA, p.kh, p.kh2);
+      if (mode != XM_NL_FIRST) rk4<F>(a, B, p.kh, p.kh2);
+      if (mode != XM_NL_LAST) rk4<F>(a, A, p.kh, p.kh2);
 #pragma unroll
       for (int f = 0; f < F; ++f)
         *park_place<PL>(row + f * NY * PITCH, t, q) = make_float4(a[f].re.x, a[f].re.y, a[f].im.x, a[f].im.y);
@@ -164,7 +169,7 @@ __device__ __forceinline__ void plane_tile(const XPassArgs& p, float2* data, con
 }
 
 template <int NX, int NY, int F>
-__global__ void __launch_bounds__(kPlaneThreads, 2) plane_kernel(const XPassArgs p, const float2* twy) {
+__global__ void __launch_bounds__(kPlaneThreads, plane_min_blocks<NX>()) plane_kernel(const XPassArgs p, const float2* twy) {
   extern __shared__ float4 sm4[];
   chain_begin();
   plane_tile<NX, NY, F>(p, p.data + (long long)blockIdx.x * NX * NY, p.ecoef, twy, reinterpret_cast<float2*>(sm4));

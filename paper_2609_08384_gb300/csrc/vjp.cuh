@@ -68,19 +68,20 @@ __device__ __forceinline__ void nl_vjp(Pair u, const Pair* t, Pair gm, const Pai
 }
 
 // One RK4 half step in reverse at two points: x is the forward state at the start
-// of the half step, e0, v, kh and kh2 as in rk4; g enters as the gradient with
-// respect to the end state and leaves as the gradient with respect to x.  s[0],
-// s[1], s[2] gain the sensitivities to the stage phases at the start, the midpoint
-// (both middle stages) and the end.  The gradients of the stages' u are kept in the
-// stage's own frame; v and e0 take them from one to the next.
-template <int F>
-__device__ __forceinline__ void rk4_vjp(const Pair (&x)[F], Pair (&g)[F], Pair e0, Pair v, const float* kh,
+// of the half step, c, kh and kh2 as in rk4; g enters as the gradient with respect
+// to the end state and leaves as the gradient with respect to x.  s[0], s[1], s[2]
+// gain the sensitivities to the stage phases at the start, the midpoint (both middle
+// stages) and the end.  The gradients of the stages' u are kept in the stage's own
+// frame; the stage factors take them to x, v from one stage to the next.
+template <int F, bool MAP>
+__device__ __forceinline__ void rk4_vjp(const Pair (&x)[F], Pair (&g)[F], const Stages<MAP>& c, const float* kh,
                                         const float* kh2, float2* s) {
   constexpr int G = F - 1;
+  const Pair v = c.v;
   const Pair* t1 = x + 1;
   Pair t2[G], t3[G], t4[G], n[G];
-  const Pair u1 = pair_mul(e0, x[0]);
-  const Pair w = pair_mul(v, u1);
+  const Pair u1 = pair_mul(c.e0, x[0]);
+  const Pair w = MAP ? pair_mul(v, u1) : pair_mul(c.em, x[0]);
   nl_slopes<F>(u1, t1, n);
 #pragma unroll
   for (int f = 0; f < G; ++f) t2[f] = pair_axpy(t1[f], kh2[f + 1], n[f]);
@@ -92,12 +93,15 @@ __device__ __forceinline__ void rk4_vjp(const Pair (&x)[F], Pair (&g)[F], Pair e
   nl_slopes<F>(u3, t3, n);
 #pragma unroll
   for (int f = 0; f < G; ++f) t4[f] = pair_axpy(t1[f], kh[f + 1], n[f]);
-  const Pair u4 = pair_mul(v, pair_iaxpy(w, kh[0], nl_drive<F>(t3)));
+  const Pair u4 = MAP ? pair_mul(v, pair_iaxpy(w, kh[0], nl_drive<F>(t3)))
+                      : pair_iaxpy(pair_mul(c.e1, x[0]), kh[0], pair_mul(v, nl_drive<F>(t3)));
 
   // direct shares of the end state: 1/6 of its gradient to stages 1 and 4, 1/3 to 2
   // and 3; the driving term's in the frame of the stage's u
   const float kd = F == 2 ? 2.f * kh[0] : kh[0], kd2 = F == 2 ? kh[0] : kh2[0];
-  const Pair p1 = pair_mul(e0, g[0]), p2 = pair_mul(v, p1);
+  const Pair p1 = pair_mul(c.e0, g[0]);
+  const Pair p2 = MAP ? pair_mul(v, p1) : pair_mul(c.em, g[0]);
+  const Pair p4 = MAP ? pair_mul(v, p2) : pair_mul(c.e1, g[0]);
   const Pair d23 = pair_niscale(kd * (1.f / 3.f), p2);
   Pair dn[G], gn[G], gt[G], gu;
 #pragma unroll
@@ -105,9 +109,10 @@ __device__ __forceinline__ void rk4_vjp(const Pair (&x)[F], Pair (&g)[F], Pair e
     dn[f] = pair_scale(kh[f + 1] * (1.f / 3.f), g[f + 1]);
     gn[f] = pair_scale(0.5f, dn[f]);
   }
-  // stage 4: u4 = v (w + i kh m3), t4 = A + kh n3
-  nl_vjp<F>(u4, t4, pair_niscale(kd * (1.f / 6.f), pair_mul(v, p2)), gn, gu, gt, s[2]);
-  Pair gw = pair_mulc(gu, v);
+  // stage 4: u4 = e1 A_0 + i kh v m3, t4 = A + kh n3
+  nl_vjp<F>(u4, t4, pair_niscale(kd * (1.f / 6.f), p4), gn, gu, gt, s[2]);
+  Pair gw = pair_mulc(gu, v);  // MAP: the gradient of w
+  if constexpr (!MAP) g[0] = pair_add(g[0], pair_mulc(gu, c.e1));
 #pragma unroll
   for (int f = 0; f < G; ++f) {
     g[f + 1] = pair_add(g[f + 1], gt[f]);
@@ -115,7 +120,7 @@ __device__ __forceinline__ void rk4_vjp(const Pair (&x)[F], Pair (&g)[F], Pair e
   }
   // stage 3: u3 = w + i kh/2 m2, t3 = A + kh/2 n2
   nl_vjp<F>(u3, t3, pair_niaxpy(d23, kd, gw), gn, gu, gt, s[1]);
-  gw = pair_add(gw, gu);
+  gw = MAP ? pair_add(gw, gu) : gu;
 #pragma unroll
   for (int f = 0; f < G; ++f) {
     g[f + 1] = pair_add(g[f + 1], gt[f]);
@@ -124,17 +129,18 @@ __device__ __forceinline__ void rk4_vjp(const Pair (&x)[F], Pair (&g)[F], Pair e
   // stage 2: u2 = w + i kh/2 v m1, t2 = A + kh/2 n1
   nl_vjp<F>(u2, t2, pair_niaxpy(d23, kd2, gu), gn, gu, gt, s[1]);
   const Pair r = pair_mulc(gu, v);
+  if constexpr (!MAP) g[0] = pair_add(g[0], pair_mulc(pair_add(gw, gu), c.em));
 #pragma unroll
   for (int f = 0; f < G; ++f) {
     g[f + 1] = pair_add(g[f + 1], gt[f]);
     gn[f] = pair_axpy(pair_scale(0.5f, dn[f]), kh2[f + 1], gt[f]);
   }
-  // stage 1: u1 = e0 A_0, w = v u1
+  // stage 1: u1 = e0 A_0
   nl_vjp<F>(u1, t1, pair_niaxpy(pair_niscale(kd * (1.f / 6.f), p1), kd2, r), gn, gu, gt, s[0]);
 #pragma unroll
   for (int f = 0; f < G; ++f) g[f + 1] = pair_add(g[f + 1], gt[f]);
-  gu = pair_add(pair_add(gu, r), pair_mulc(gw, v));
-  g[0] = pair_add(g[0], pair_mulc(gu, e0));
+  if constexpr (MAP) gu = pair_add(pair_add(gu, r), pair_mulc(gw, v));
+  g[0] = pair_add(g[0], pair_mulc(gu, c.e0));
 }
 
 }  // namespace brahms

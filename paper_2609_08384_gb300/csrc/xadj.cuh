@@ -113,12 +113,10 @@ __device__ __forceinline__ void xpass_adj_tile(const XAdjArgs& p, long long tile
           for (int u = 0; u < 2; ++u) nm[m][u] = __ldcg(emap + m * nxy + point_pos<PL>(t, 2 * q + u));
       }
     };
-    Pair eB, vB, eA, vA;
+    Stages<MAP> B, A;
     if constexpr (!MAP) {
-      eB = {dup(p.ecoef[0].x), dup(p.ecoef[0].y)};
-      vB = {dup(p.ecoef[1].x), dup(p.ecoef[1].y)};
-      eA = {dup(p.ecoef[2].x), dup(p.ecoef[2].y)};
-      vA = {dup(p.ecoef[3].x), dup(p.ecoef[3].y)};
+      B = stages_of(p.ecoef);
+      A = stages_of(p.ecoef + 3);
     }
     float2 s[6];
 #pragma unroll
@@ -136,14 +134,14 @@ __device__ __forceinline__ void xpass_adj_tile(const XAdjArgs& p, long long tile
       }
       if constexpr (MAP) {
         const auto pair_of = [](const float2* m) { return Pair{make_float2(m[0].x, m[1].x), make_float2(m[0].y, m[1].y)}; };
-        eB = pair_of(nm[0]);
-        vB = pair_of(nm[1]);
-        eA = pair_of(nm[2]);
-        vA = pair_of(nm[3]);
+        B.e0 = pair_of(nm[0]);
+        B.v = pair_of(nm[1]);
+        A.e0 = pair_of(nm[2]);
+        A.v = pair_of(nm[3]);
       }
       if (q + 1 < E / 2) request(q + 1);
-      if (p.xa) rk4_vjp<F>(x, g, eA, vA, p.kh, p.kh2, s);
-      if (p.xb) rk4_vjp<F>(xbv, g, eB, vB, p.kh, p.kh2, s + 3);
+      if (p.xa) rk4_vjp<F>(x, g, A, p.kh, p.kh2, s);
+      if (p.xb) rk4_vjp<F>(xbv, g, B, p.kh, p.kh2, s + 3);
 #pragma unroll
       for (int f = 0; f < F; ++f)
         *park_place<PL>(myrow + f * ROWS * PITCH, t, q) = make_float4(g[f].re.x, g[f].re.y, g[f].im.x, g[f].im.y);
