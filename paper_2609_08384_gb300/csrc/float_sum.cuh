@@ -1,11 +1,12 @@
-// Running sum of floats without loss: the rounding error of every addition
-// (Knuth's two-sum) is kept in a second float, so hi + lo carries about 2^-45 of
-// the sum through thousands of terms.  FP64 additions are scarce on this GPU
-// (about two lanes per SM and cycle): a convert and an add per pair of points made
-// the FP64 pipe the bound of the power trace (230 us on 805 MB, 143 this way).
+// Sum of a few floats in two: the rounding error of every addition (Knuth's two-sum)
+// is added up in lo, so hi + lo carries n terms to n^2 2^-50.  For short sums that go on
+// into an FP64 accumulator: over 16384 equal terms lo itself rounds, and the sum came
+// out 2^-25 off.  FP64 operations are scarce on this GPU (about two lanes per SM and
+// cycle): a convert and an add per pair of points made the FP64 pipe the bound of the
+// power trace: 149 us on the 403 MB of 3 x 512x512x64, with two of each per eight pairs
+// 101 (with one two-float sum per thread 96).
 // A sum beyond FP32's range comes out infinite or undefined; callers then add the
-// terms again in FP64.  (Moving large sums to FP64 inside add() cost every
-// addition its predicated FP64 instructions: 440 us.)
+// terms one by one in FP64.
 #pragma once
 
 #include <cuda_runtime.h>

@@ -16,13 +16,13 @@ __device__ __forceinline__ double warp_sum_d(double v) {
 }
 
 // sum_{x,y} |A_f(x, y, tau_k)|^2 for every (k, f): one CTA per plane; two
-// points per 16-byte load, their squares summed in FP32 and accumulated without
-// loss (planes hold an even number of points)
+// points per 16-byte load, their squares summed in FP32, eight pairs in two floats
+// and those in FP64 (planes hold an even number of points)
 __global__ void __launch_bounds__(256) power_trace_kernel(const float2* __restrict__ data, long long plane,
                                                           int nt, long long fstride, double* out) {
   const int k = blockIdx.x, f = blockIdx.y;
   const float2* a = data + (long long)f * fstride + (long long)k * plane;
-  FloatSum sum[2];
+  double s = 0.0;
   const float4* a4 = reinterpret_cast<const float4*>(a);
   const long long n2 = plane / 2;
   const auto pair = [](float4 v) { return fmaf(v.x, v.x, fmaf(v.y, v.y, fmaf(v.z, v.z, v.w * v.w))); };
@@ -32,11 +32,12 @@ __global__ void __launch_bounds__(256) power_trace_kernel(const float2* __restri
     float4 v[8];
 #pragma unroll
     for (int u = 0; u < 8; ++u) v[u] = __ldcg(a4 + i + u * (long long)blockDim.x);
+    FloatSum sum;
 #pragma unroll
-    for (int u = 0; u < 8; ++u) sum[u & 1].add(pair(v[u]));
+    for (int u = 0; u < 8; ++u) sum.add(pair(v[u]));
+    s += sum.value();
   }
-  for (; i < n2; i += blockDim.x) sum[0].add(pair(__ldcg(a4 + i)));
-  double s = sum[0].value() + sum[1].value();
+  for (; i < n2; i += blockDim.x) s += (double)pair(__ldcg(a4 + i));
   if (!isfinite(s)) {  // beyond FP32's range, or fields that are not finite
     s = 0.0;
     for (i = threadIdx.x; i < n2; i += blockDim.x) s += (double)pair(__ldcg(a4 + i));
