@@ -37,11 +37,16 @@ __host__ __device__ constexpr int plane_smem(int nf) {
   return nf * NY * XchRow::pitch(NX) * (int)sizeof(float2);
 }
 
+// The plan of the columns: the y axis's own, whose twiddle table the launch is given
+// (another plan of the same length would read its entries in another order).
+template <int NY>
+using PlaneColumnPlan = AxisPlan<NY, 1>;
+
 // Columns of all fields: from global memory (or the buffer) through one
 // transform along y into the buffer (or global memory).
 template <int NX, int NY, int F, bool INV>
 __device__ __forceinline__ void plane_columns(float2* buf, float2* data, long long fstride, const float2* twy) {
-  using PL = FftPlan<NY>;
+  using PL = PlaneColumnPlan<NY>;
   constexpr int PITCH = XchRow::pitch(NX);
   constexpr int COLS = kPlaneThreads / PL::T;  // columns at a time
   constexpr int R0 = fft_radix<PL, INV>(0), RL = fft_radix<PL, INV>(PL::NP - 1);
