@@ -14,7 +14,7 @@
 namespace brahms {
 
 template <int NX>
-__global__ void __launch_bounds__(xpass_threads<NX>(), xpass_min_blocks<NX, 2>())
+__global__ void __launch_bounds__(xpass_threads<NX>(), xpass_min_blocks<NX, 2, false>())
     xpass_group_kernel(const XPassArgs base, const GroupInst* __restrict__ gi, const float2* __restrict__ ecoef,
                        int stride, int step, long long tiles_per_inst) {
   constexpr int THREADS = xpass_threads<NX>();

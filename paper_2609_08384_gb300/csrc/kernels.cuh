@@ -101,14 +101,17 @@ __host__ __device__ constexpr int xpass_smem_floats2(int nf) {
   return nf * xpass_rows<N>() * XchRow::pitch(N);
 }
 // resident CTAs the x-pass asks the register allocator for: 6 (80 registers)
-// where six CTAs' shared memory fits in an SM and rows are at most 256 long
-// (no spills there); otherwise 4, or 8 of 64 threads (128 registers)
-template <int N, int F>
+// where six CTAs' shared memory fits in an SM and rows are at most 256 long, 5 there for
+// three fields under a map (at 80 registers rows of 4, 6, 8, 32 and 64 points spill:
+// step of 3 x 8, 32 and 64 points along x 155.2, 199.4 and 171.6 us with 6, 150.9, 193.6
+// and 168.5 with 5; the other lengths alike); otherwise 4, or 8 of 64 threads (128
+// registers)
+template <int N, int F, bool MAP>
 __host__ __device__ constexpr int xpass_min_blocks() {
-  return xpass_threads<N>() > 128                                                          ? 1
-         : (N <= 256 && 6 * (xpass_smem_floats2<N>(F) * 8 + 1024) <= 228 * 1024) ? 6
+  return xpass_threads<N>() > 128                                                ? 1
+         : (N <= 256 && 6 * (xpass_smem_floats2<N>(F) * 8 + 1024) <= 228 * 1024) ? (MAP && F == 3 ? 5 : 6)
          : xpass_threads<N>() == 64                                              ? 8
-                                                                                          : 4;
+                                                                                 : 4;
 }
 
 // Strided pencils: tiles of TX neighbouring columns (128-byte rows up to
@@ -480,7 +483,7 @@ __device__ __forceinline__ void xpass_tile(const XPassArgs& p, long long tile, c
 // MAP: per-point stage phases from a transverse mismatch map (p.emap);
 // REC: record the half steps' input states (p.rec_b, p.rec_a)
 template <int NX, int F, bool MAP, bool REC = false>
-__global__ void __launch_bounds__(xpass_threads<NX>(), xpass_min_blocks<NX, F>())
+__global__ void __launch_bounds__(xpass_threads<NX>(), xpass_min_blocks<NX, F, MAP>())
     xpass_kernel(const XPassArgs p) {
   constexpr int THREADS = xpass_threads<NX>();
   extern __shared__ float4 sm4[];
@@ -628,21 +631,18 @@ __device__ __forceinline__ void apply_prop(float2 (&v)[PL::E], const AxisArgs& p
       v[b * RL + r] = g(p, v[b * RL + r], pt[pos_last<PL, false>(t + b * PL::T, r)]);
 }
 
-// Resident CTAs the tau-pass asks the register allocator for.  Left to itself
-// the compiler requests a whole column of tau factors and twiddles ahead (153 to
-// 172 registers on the 512-point plan: one CTA per SM).  Measured per launch:
-// 512-point plan 555 us unbounded, 463 at two CTAs, 600 at three (spills); 128
-// points (512x512x128, two fields) 292 us unbounded, 290 at two, 232 at three;
-// 64 points (1024x256x64) 142 us at two, 127 at four.
+// Resident CTAs of 256 threads that the plain tau-pass asks the register allocator for;
+// larger CTAs (2048 and 4096 points, 1024 threads) have 64 registers a thread anyway.
+// What takes it are the plans that the pipelined one below leaves: measured per step
+// with 1, 2, 3 and 4, lengths of up to 48 points lie within 2 % of each other, 32 points
+// gain 1.5 % from 4 (63.3 us against 64.3 on 2 x 128x512x32) and 96 points lose 10 % to
+// it (2 x 256x96x1: 10.7 us with 1 and 2, 11.1 with 3, 11.9 with 4).
 template <class PL>
 __host__ __device__ constexpr int tprop_min_blocks() {
   return tiles_per_cta<PL>() * tile_threads<PL>() > 256 ? 1 : PL::E > 16 ? 2 : PL::E > 8 ? 3 : 4;
 }
 
 // Forward tau-FFT, propagator multiply, inverse tau-FFT, in one pass.
-// (Measured slower on the 512-point plan: launch bounds of two CTAs per SM, a
-// persistent loop over tiles, the twiddle staging issued after this tile's
-// loads, the field's tau factors staged in shared memory with the twiddles.)
 template <class PL, bool SCALED, int THREADS, class TW = TwShared>
 __device__ __forceinline__ void tprop_tile(const AxisArgs& p, long long cta_tile, const TW& tw, float2* xch) {
   constexpr int N = PL::N, T = PL::T, TX = ColTile<PL>::value;

@@ -177,10 +177,17 @@ __device__ __forceinline__ void xpass_adj_tile(const XAdjArgs& p, long long tile
   }
 }
 
-// Four CTAs of 128 threads (128 registers) hold two fields without spills; three
-// fields and the tables of a map need three (168).
+// Resident CTAs of 128 threads: four (128 registers) hold two fields without spills,
+// three fields or the tables of a map need three (168), both together two (at 168 they
+// spill at 18 of 20 lengths: forward and backward over 16 steps with three CTAs and two
+// 3.69 and 3.53 ms on rows of 512 points, 3.05 and 2.94 of 192, 3.61 and 3.58 of 128;
+// rows of 64 points 3.49 and 3.55).
 template <int NX, int F, bool MAP>
-__global__ void __launch_bounds__(xpass_threads<NX>(), xpass_threads<NX>() > 128 ? 1 : (F == 3 || MAP ? 3 : 4) * 128 / xpass_threads<NX>())
+__host__ __device__ constexpr int xadj_min_blocks() {
+  return xpass_threads<NX>() > 128 ? 1 : (F == 3 && MAP ? 2 : F == 3 || MAP ? 3 : 4) * 128 / xpass_threads<NX>();
+}
+template <int NX, int F, bool MAP>
+__global__ void __launch_bounds__(xpass_threads<NX>(), xadj_min_blocks<NX, F, MAP>())
     xpass_adj_kernel(const XAdjArgs p) {
   constexpr int THREADS = xpass_threads<NX>();
   extern __shared__ float4 sm4[];
