@@ -576,22 +576,21 @@ __device__ __forceinline__ void axis_tile(const AxisArgs& p, long long cta_tile,
 }
 
 // The propagator P = (1 + Dx)(1 + Dy)(1 + Dt) / (nx ny nt) of one column, the
-// factors in delta form.  1/(nx ny nt) = scale + scale_lo is applied to a value w
-// itself where it is no power of two; where it is one, it sits in the constants,
-// exactly (c = scale; c = 1 where it has been applied):
-//   c w + w E(Omega),  E = g0 + Dt g1,  1 + Dxy = (1 + Dx)(1 + Dy),
-//   g0 = c Dxy,  g1 = c (1 + Dxy).
-// (With any scale folded into g0 and g1 their rounding came on top of Dxy's, the
-// same one in every step: the parametric run of 48x256x128 points ended 12 % further
-// from FP64, and noise on a grid of 3 2^k points gained 6e-8 of its energy per step.)
-// The small product w E is formed first and c w, which is exact, added with one
-// rounding.  (Folding w into the FMA chain rounds w.x - w.y E.y before the
+// factors in delta form.  With 1 + Dxy = (1 + Dx)(1 + Dy) a value w becomes
+//   c w + w E(Omega),  E = g0 + Dt g1,  g0 = c Dxy,  g1 = c (1 + Dxy),
+// c = 1/(nx ny nt) = scale where that is a power of two.  Where it is not (SCALED), c = 1
+// and the result is scaled: scale w + (scale w E + scale_lo (w + w E)).  (With such a scale in g0
+// and g1 their rounding came on top of Dxy's, the same one in every step: the parametric
+// run of 48x256x128 points ended 12 % further from FP64, and noise on a grid of 3 2^k
+// points gained 6e-8 of its energy per step.  Scaling w before the product rounds w once
+// more: 3 x 48x32x48 over 88 steps 1.62e-6 from FP64 instead of 1.58e-6.)
+// The small product w E is formed first and c w added with one rounding.  (Folding w into the FMA chain rounds w.x - w.y E.y before the
 // second-order term w.x (cos phi - 1) arrives; for small phases that term is below
 // half an ulp and is then always lost, so |1 + E| acts as 1 + phi^2 / 2 and the
 // energy grows step after step.)
 // conj(P) (the adjoint) turns the sign of E's imaginary part, which sits in its
 // three constants gi.
-template <bool SCALED>  // the values are scaled first
+template <bool SCALED>
 struct ColumnProp {
   float c;
   float2 g0, g1;
@@ -605,21 +604,19 @@ struct ColumnProp {
     gi = make_float3(sg * g0.y, sg * g1.y, sg * g1.x);
   }
   __device__ __forceinline__ float2 operator()(const AxisArgs& p, float2 w, float2 dt) const {
-    if constexpr (SCALED)
-      w = __ffma2_rn(w, make_float2(p.scale, p.scale), __fmul2_rn(w, make_float2(p.scale_lo, p.scale_lo)));
     const float ex = fmaf(dt.x, g1.x, fmaf(-dt.y, g1.y, g0.x));
     const float ey = fmaf(dt.x, gi.y, fmaf(dt.y, gi.z, gi.x));
     const float2 we = make_float2(fmaf(w.x, ex, -w.y * ey), fmaf(w.x, ey, w.y * ex));
-    return __ffma2_rn(w, make_float2(c, c), we);
+    if constexpr (SCALED)
+      return __ffma2_rn(w, dup(p.scale), __ffma2_rn(we, dup(p.scale), __fmul2_rn(cadd(w, we), dup(p.scale_lo))));
+    else return __ffma2_rn(w, dup(c), we);
   }
 };
 
 // The propagator on a column's registers, which hold A_hat(kx, ky, Omega_k) at
 // k = pos_last; pt: the field's tau factors.  (The kernels are instantiated for both
 // kinds of grid where the plan has 2^k points: a branch here cost grids of 2^k points
-// 2 to 8 % of their step, one before the forward transform 1 %, and there the rounding
-// of the scaled values weighs more: 2 x 96x96x192 over 50 steps 1.52e-6 from FP64
-// against 1.36e-6.)
+// 2 to 8 % of their step.)
 template <class PL, bool SCALED>
 __device__ __forceinline__ void apply_prop(float2 (&v)[PL::E], const AxisArgs& p, const ColumnProp<SCALED>& g,
                                            const float2* pt, int t) {
