@@ -178,13 +178,16 @@ __device__ __forceinline__ void xpass_adj_tile(const XAdjArgs& p, long long tile
 }
 
 // Resident CTAs of 128 threads: four (128 registers) hold two fields without spills,
-// three fields or the tables of a map need three (168), both together two (at 168 they
-// spill at 18 of 20 lengths: forward and backward over 16 steps with three CTAs and two
-// 3.69 and 3.53 ms on rows of 512 points, 3.05 and 2.94 of 192, 3.61 and 3.58 of 128;
-// rows of 64 points 3.49 and 3.55).
+// three fields or the tables of a map need three (168).  Both together spill there (at 18
+// of 20 lengths) and take two CTAs where a thread has more than 16 points: mean of the
+// recording and the reverse x-pass with three and two, 3 x 512x128x128 276 and 245 us,
+// 3 x 192x128x256 214 and 191; with up to 16 the warps weigh more, 3 x 256x128x256 206
+// and 222, 3 x 128x128x256 112 and 125.
 template <int NX, int F, bool MAP>
 __host__ __device__ constexpr int xadj_min_blocks() {
-  return xpass_threads<NX>() > 128 ? 1 : (F == 3 && MAP ? 2 : F == 3 || MAP ? 3 : 4) * 128 / xpass_threads<NX>();
+  return xpass_threads<NX>() > 128
+             ? 1
+             : (F == 3 && MAP && FftPlan<NX>::E > 16 ? 2 : F == 3 || MAP ? 3 : 4) * 128 / xpass_threads<NX>();
 }
 template <int NX, int F, bool MAP>
 __global__ void __launch_bounds__(xpass_threads<NX>(), xadj_min_blocks<NX, F, MAP>())
