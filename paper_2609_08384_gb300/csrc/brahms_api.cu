@@ -115,14 +115,19 @@ brahms_status brahms_init_grid(brahms_ctx** out, int nx, int ny, int nt, double 
   ctx->umaps_dev = ctx->ws_umap;
   ctx->mphase_dev = (double*)(ctx->ws + ctx->L.mphase);
   ctx->emap_dev = (float2*)(ctx->ws + ctx->L.emap);
-  cudaError_t e = cudaSuccess;
-  if (e == cudaSuccess) e = brahms::upload_twiddles(ctx->twx, nx, 0, ctx->stream);
-  if (e == cudaSuccess && ny > 1) e = brahms::upload_twiddles(ctx->twy, ny, 1, ctx->stream);
+  // the six twiddle tables, which lie one behind another, in one copy
+  std::vector<char> tables(ctx->L.partial - ctx->L.twx);
+  const auto place = [&](size_t at) { return tables.data() + (at - ctx->L.twx); };
   const int nlast = tau_pass_length(ny, nt);
-  if (e == cudaSuccess && nlast > 1) e = brahms::upload_twiddles(ctx->twt, nlast, 2, ctx->stream);
-  if (e == cudaSuccess) e = brahms::upload_twiddles(ctx->twpx, nx, 0, ctx->stream);
-  if (e == cudaSuccess && ny > 1) e = brahms::upload_twiddles(ctx->twpy, ny, 1, ctx->stream);
-  if (e == cudaSuccess && nt > 1) e = brahms::upload_twiddles(ctx->twpt, nt, 2, ctx->stream);
+  bool filled = brahms::fill_twiddles((float2*)place(ctx->L.twx), nx, 0) &&
+                brahms::fill_twiddles((float4*)place(ctx->L.twpx), nx, 0);
+  if (ny > 1)
+    filled = filled && brahms::fill_twiddles((float2*)place(ctx->L.twy), ny, 1) &&
+             brahms::fill_twiddles((float4*)place(ctx->L.twpy), ny, 1);
+  if (nlast > 1) filled = filled && brahms::fill_twiddles((float2*)place(ctx->L.twt), nlast, 2);
+  if (nt > 1) filled = filled && brahms::fill_twiddles((float4*)place(ctx->L.twpt), nt, 2);
+  cudaError_t e = filled ? cudaMemcpyAsync(ctx->ws + ctx->L.twx, tables.data(), tables.size(), cudaMemcpyHostToDevice, ctx->stream)
+                         : cudaErrorInvalidValue;
   if (e == cudaSuccess) e = cudaMemsetAsync(ctx->dev_err, 0, 2 * sizeof(int), ctx->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(ctx->mphase_dev, 0, sizeof(double) * nx * ny, ctx->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);

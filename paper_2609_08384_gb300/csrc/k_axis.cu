@@ -127,11 +127,11 @@ static float4 entry(double phi, const float4*) {
 // phi = -2 pi r' m' / (NS R), or its cosine and sine as hi + lo, the digits of r and m
 // centred, evaluated in FP64.
 template <class T>
-static cudaError_t upload(T* tw, int n, int axis, cudaStream_t s) {
+static bool fill(T* h, int n, int axis) {
   int rad[8];
   const int np = plan_radices(n, axis, rad);
-  if (np <= 0) return cudaErrorInvalidValue;
-  std::vector<T> h;
+  if (np <= 0) return false;
+  h[0] = entry(0.0, h);  // a plan of one pass has no turns
   int ns = 1;
   for (int q = 0; q < np; ++q) {
     if (q > 0) {
@@ -143,19 +143,23 @@ static cudaError_t upload(T* tw, int n, int axis, cudaStream_t s) {
             rest /= rad[p];
             w *= rad[p];
           }
-          h.push_back(entry(-6.283185307179586476925286766559 * (double)(centred(r, rad[q]) * mc) / (double)(ns * rad[q]), tw));
+          *h = entry(-6.283185307179586476925286766559 * (double)(centred(r, rad[q]) * mc) / (double)(ns * rad[q]), h);
+          ++h;
         }
     }
     ns *= rad[q];
   }
-  if (h.empty()) h.push_back(entry(0.0, tw));
-  if ((int)h.size() != tw_table_size_of(n, axis)) return cudaErrorInvalidValue;
-  cudaError_t e = cudaMemcpyAsync(tw, h.data(), sizeof(T) * h.size(), cudaMemcpyHostToDevice, s);
+  return true;
+}
+bool fill_twiddles(float2* h, int n, int axis) { return fill(h, n, axis); }
+bool fill_twiddles(float4* h, int n, int axis) { return fill(h, n, axis); }
+cudaError_t upload_twiddles(float2* tw, int n, int axis, cudaStream_t s) {
+  std::vector<float2> h((size_t)tw_table_size_of(n, axis));
+  if (h.empty() || !fill_twiddles(h.data(), n, axis)) return cudaErrorInvalidValue;
+  const cudaError_t e = cudaMemcpyAsync(tw, h.data(), sizeof(float2) * h.size(), cudaMemcpyHostToDevice, s);
   if (e != cudaSuccess) return e;
   return cudaStreamSynchronize(s);  // h is a local buffer
 }
-cudaError_t upload_twiddles(float2* tw, int n, int axis, cudaStream_t s) { return upload(tw, n, axis, s); }
-cudaError_t upload_twiddles(float4* tw, int n, int axis, cudaStream_t s) { return upload(tw, n, axis, s); }
 
 int tau_col_tile_of(int n) {
   switch (n) {

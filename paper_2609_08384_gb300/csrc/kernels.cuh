@@ -867,12 +867,13 @@ cudaError_t make_tau_tensor_map(void* map128, const float2* data, int nx, int ny
 cudaError_t run_tpass_prop_tma(int nt, int tx, const void* map128, const AxisArgs& a, int* err,
                                unsigned long long wait_ns, cudaStream_t s);
 
-// per-pass twiddle table of the plan of length n on an axis (0 x, 1 y, 2 tau), built
-// on the host in FP64, and its size in entries
+// per-pass twiddle table of the plan of length n on an axis (0 x, 1 y, 2 tau), built on
+// the host in FP64, and its size in entries: the turns as shears, or as products (cosine
+// and sine as hi + lo floats); fill_twiddles is false for an unsupported length
 int tw_table_size_of(int n, int axis);
+bool fill_twiddles(float2* host, int n, int axis);
+bool fill_twiddles(float4* host, int n, int axis);
 cudaError_t upload_twiddles(float2* tw, int n, int axis, cudaStream_t s);
-// the same turns as products, cos and sin as hi + lo floats
-cudaError_t upload_twiddles(float4* tw, int n, int axis, cudaStream_t s);
 struct TableArgs {
   float2* px;
   float2* py;
