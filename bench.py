@@ -751,8 +751,9 @@ def run_ours(args):
                          "design_bytes_per_point_field_step": DESIGN_BYTES,
                          "design_GB_per_s": DESIGN_BYTES * value / 1e9,
                          "design_frac_of_peak": DESIGN_BYTES * value / 1e9 / peak,
-                         "note": "design bytes: what the pass structure reads and writes by construction "
-                                 "(the ncu DRAM counters of every pass equal them, profiles/); not a measured rate"},
+                         "note": "design bytes: what the pass structure reads and writes by construction; not a "
+                                 "measured rate (profiles/dram_traffic.json: the passes' ncu DRAM counters, of "
+                                 "these kernels where roofline.traffic is not null)"},
             "forms": forms}
     print(json.dumps(line), flush=True)
     return 0

@@ -68,8 +68,8 @@ brahms_status brahms_workspace_size(int nx, int ny, int nt, int nfields, size_t*
 
 /* Create a context.  nx, ny, nt: grid lengths, each one of 2,4,...,4096 or
  * 3*2^k for 6 <= 3*2^k <= 768; ny and nt may also be 1 (a 1D transverse
- * grid, or a cw field with no tau extent: its linear step is the (kx, ky)
- * multiply alone); else E_SIZE.  dx, dy [m], dt [s]: spacings > 0.
+ * grid, or a cw field with no tau extent: its linear step is one pass along y,
+ * or with ny = 1 too the multiply by the propagator alone); else E_SIZE.  dx, dy [m], dt [s]: spacings > 0.
  * nfields: 2 (SH, F) or 3 (p, s, i); fp: nfields coefficient records.
  * d_eff [m/V]; dk [1/m]: constant mismatch Delta k = k_p - k_s - k_i (Eq. mismatch).
  * workspace: device memory of at least brahms_workspace_size() bytes, 256-byte
@@ -229,8 +229,8 @@ brahms_status brahms_timing(brahms_ctx* ctx, int enable, double* ms, long long* 
  * x-pass, which couples the fields, waits for all of them on the context
  * stream.  0 (the default) runs every pass on the context stream, each launch
  * overlapping the end of the one before it.  Measured on GB300: slower on
- * every grid since then (time per step, off and on: 3 x 128x128x256 156 and
- * 163 us, 2 x 32x32x64 7.4 and 20.6).  Per-kernel timing with field streams
+ * every grid since then (time per step, off and on: 3 x 128x128x256 158 and
+ * 165 us, 2 x 32x32x64 7.2 and 20.6).  Per-kernel timing with field streams
  * measures kernels that may share the GPU.
  * BRAHMS_OPT_TMA_TAU: value 16 or 8 makes the
  * tau-pass of brahms_propagate a persistent kernel that stages tiles of that
@@ -240,7 +240,7 @@ brahms_status brahms_timing(brahms_ctx* ctx, int enable, double* ms, long long* 
  * (its FFT exchanges go through half the shared memory, one real component
  * at a time).  Both need nt in {256, 512} and nx >= 16, else E_SIZE; both
  * compute the default tau-pass's numbers and measured slower on GB300 (step of
- * 3 x 256x256x512: 1324 us with 8, 1494 with 16, 1380 with 1, 1306 by default).
+ * 3 x 256x256x512: 1335 us with 8, 1495 with 16, 1363 with 1, 1310 by default).
  * 0 (the default) keeps the library's own choice of tau-pass.  Any other value
  * turns the field streams off while set.
  * BRAHMS_OPT_TMA_WAIT_US: the limit, in microseconds (0 .. 2000000, default

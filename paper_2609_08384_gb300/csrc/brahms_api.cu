@@ -242,8 +242,8 @@ brahms_status brahms_propagate(brahms_ctx* ctx, int nz, double dz) {
     else
       BR_CK(launch(ctx, 0, 1, [&] { return brahms::run_xpass(nx, nf, a, ctx->stream); }));
   }
-  // per-field streams for the y/tau/y passes only when the option asks for
-  // them (off by default: a gain on 128x128x256 with three fields only)
+  // per-field streams for the y/tau/y passes only when the option asks for them
+  // (off by default: slower on every grid measured)
   const bool split = use_field_streams(ctx);
   for (int i = 0; i < nz; ++i, ++j) {
     const double dkj = dk_of_step(ctx, j);

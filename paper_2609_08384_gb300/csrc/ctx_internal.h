@@ -392,7 +392,7 @@ inline brahms::AxisArgs aargs(brahms_ctx* c, int axis, bool tau_prop = true) {
 // on the grid read as nx x 1 x ny, the roles of the y and tau factors exchanged;
 // twt holds the twiddles of ny in the tau-pass's plan there.
 // (1024x1024, two fields: y-forward, pointwise multiply and y-inverse took 43 us
-// of a step of 49; one pass 17.)
+// of a step of 49; one pass 18.5 of 31.)
 inline brahms::AxisArgs cw_args(brahms_ctx* c) {
   brahms::AxisArgs a = aargs(c, 1);
   a.ny = 1;
@@ -408,8 +408,8 @@ inline brahms::AxisArgs cw_args(brahms_ctx* c) {
 
 // Per-field streams for the y-forward, tau-propagator and y-inverse of a
 // step, when the option asks for them (measured on GB300, step without and with:
-// 3 x 128x128x256 156 and 163 us, 2 x 32x32x64 7.4 and 20.6, 3 x 256x256x256 627 and
-// 629).
+// 3 x 128x128x256 158 and 165 us, 2 x 32x32x64 7.2 and 20.6, 3 x 256x256x256 634 and
+// 638).
 inline bool use_field_streams(const brahms_ctx* c) {
   return c->field_streams == 1 && c->ny > 1 && c->nt > 1 && !c->use_tma;
 }

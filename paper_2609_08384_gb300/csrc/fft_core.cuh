@@ -33,10 +33,11 @@
 // floats |c + i s| differs from 1 and it does; a pair of directions that are
 // not each other's mirror let the energy of the 3 x 256x256x512 parametric run
 // fall by 7e-9 per step.)  |phi| <= 1/4 turn, or a little more in plans of three
-// and four passes, keeps p near 1 or below.
-// Error against FP64 of 3D transforms of random fields: forward 1.6e-7 (with
-// hi + lo twiddles 1.5e-7), forward and inverse 2.11e-7 (2.10e-7); energy of
-// smooth beams over 100 z-steps: rms 1.6e-9 to 2.6e-9 per step (1.7e-9 to 5.6e-9).
+// passes, keeps p near 1 or below.
+// Error against FP64 of 3D transforms of random fields by shears: forward 1.6e-7 (by
+// products with hi + lo twiddles 1.5e-7), forward and inverse 2.11e-7 (2.10e-7); energy
+// of smooth beams over 100 z-steps: rms 1.6e-9 to 2.6e-9 per step (1.7e-9 to 5.6e-9).
+// Transforms that nothing takes back turn by products (TwProduct, k_single.cu).
 //
 // Packed arithmetic.  A complex value is an aligned register pair, and sums of
 // complex values are single add/sub.f32x2 instructions.  One FFMA2 occupies the
@@ -76,10 +77,6 @@ __device__ __forceinline__ float2 csub(float2 a, float2 b) {
 }
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
   return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
-}
-// a * conj(b)
-__device__ __forceinline__ float2 cmulc(float2 a, float2 b) {
-  return make_float2(fmaf(a.x, b.x, a.y * b.y), fmaf(a.y, b.x, -a.x * b.y));
 }
 __device__ __forceinline__ float2 cscale(float2 a, float s) { return make_float2(a.x * s, a.y * s); }
 // a + t^Q b, t = -i (forward) or +i (inverse), Q taken mod 4: a quarter turn of
@@ -394,9 +391,9 @@ template <> struct FftPlan<384> : Plan<384, 24, 3, 8, 12, 4> {};
 template <> struct FftPlan<768> : Plan<768, 24, 3, 8, 24, 4> {};
 
 // The lengths 3 2^k take radices 6, 12 and 24, which need one exchange where 3 x 4
-// x 4 x 4 needs three: the four-pass plans were bound by shared memory (x-pass of
+// x 4 x 4 needs three: those four-pass plans were bound by shared memory (x-pass of
 // 3 x 48x192x384: 82 % of its wavefronts, FP32 pipe 47 %).  Step of 2 x 96x96x192
-// 72 -> 56 us, of 3 x 48x192x384 192 -> 148, of 2 x 192x192x768 1063 -> 850.
+// 72 -> 55 us, of 3 x 48x192x384 192 -> 147, of 2 x 192x192x768 1063 -> 875.
 //
 // Plans of y and tau where they differ from the rows'.  1024 points as 32 x 32
 // (one exchange, 32 threads per pencil): tau-pass of 2 x 256x256x1024 833 -> 658

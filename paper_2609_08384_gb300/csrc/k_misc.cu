@@ -253,8 +253,8 @@ static int grid_for(long long n) {
 }
 
 // ------------------------------------------------ pointwise linear step
-// The linear step of a grid without a tau extent (nt = 1, a cw field, or
-// any grid whose tau-transform is the identity): the multiply
+// The linear step of a single row (ny = nt = 1: neither a y nor a tau transform): the
+// multiply
 // P = (1 + Dx)(1 + Dy)(1 + Dt) / N of the tau-pass, element by element, with
 // the tau-pass's arithmetic, on the (kx, ky)-domain state.
 __global__ void prop_pointwise_kernel(const AxisArgs p, int nf) {

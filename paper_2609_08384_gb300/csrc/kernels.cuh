@@ -9,9 +9,9 @@
 //   t-pass  forward tau-FFT, multiply by the linear propagator
 //           P = Px(kx) Py(ky) Pt(Omega) / (NX NY NT), inverse tau-FFT
 //   y-pass  inverse y-FFT
-// On planes of up to 1536 points the y-inverse, x-pass and y-forward are one
-// kernel (plane.cuh), and on cw grids (nt = 1) the linear step is one pass along y
-// (the tau-pass's kernel on the axes x, tau, y).
+// On the small planes of BRAHMS_FOR_EACH_PLANE the y-inverse, x-pass and y-forward
+// are one kernel (plane.cuh), and on cw grids (nt = 1, ny > 1) the linear step is one
+// pass along y (the tau-pass's kernel on the axes x, tau, y).
 // Between calls the state is in real space; the first and the last step of
 // a call peel the x-pass (NL_FIRST / NL_LAST).
 #pragma once
@@ -286,9 +286,10 @@ __device__ __forceinline__ float2 phase_minus(double phi) {
 // asynchronous copies straight into the row buffers, so a field's row arrives
 // while the one before it is transformed and no registers wait for it (108 ->
 // 92 registers for three fields of 256; 482 -> 421 us per launch on
-// 3 x 256x256x512, 350 -> 326 on 2 x 512x512x128).  What bounds it now: the FP32
-// pipe, 123 operations a point and field of which 316 us at its peak rate on
-// that state.  Twiddles are read through L1.
+// 3 x 256x256x512, 350 -> 326 on 2 x 512x512x128; 423 and 333 now).  What bounds it:
+// the FP32 pipe, 131 operations a point and field (46 of the two transforms of 256
+// points, 85 of the RK4 half steps), 337 us at its measured rate on that state.
+// Twiddles are read through L1.
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() {
@@ -345,7 +346,7 @@ __device__ __forceinline__ void xpass_tile(const XPassArgs& p, long long tile, c
   constexpr int PITCH = XchRow::pitch(NX);
   constexpr int RF0 = fft_radix<PL, false>(0);           // forward first radix
   constexpr int RFL = fft_radix<PL, false>(PL::NP - 1);  // forward last radix
-    using SY = typename std::conditional<xpass_warp_sync<NX>(), SyncWarp, SyncBlock>::type;
+  using SY = typename std::conditional<xpass_warp_sync<NX>(), SyncWarp, SyncBlock>::type;
   static_assert(ROWS >= 1 && ROWS * T == THREADS, "CTA must hold whole rows");
   const TwGlobal tw{p.tw};
 
@@ -506,7 +507,7 @@ __global__ void __launch_bounds__(xpass_threads<NX>(), xpass_min_blocks<NX, F, M
 // 1000-step call; a tau-major y order (every field of a plane together)
 // made the y-passes 20 us slower and the step 1622 ms.  The tau-propagator
 // also walks its tiles from the last down (tau 476 -> 473, y-inverse
-// 258 -> 257 us).  (The step now takes 1307 us on that state.)
+// 258 -> 257 us).  (The step now takes 1310 us on that state.)
 template <int N, int AXIS, int TX>
 struct AxisTile {
   float2* base;  // element (x, pencil index 0)
@@ -672,10 +673,10 @@ __device__ __forceinline__ void tprop_tile(const AxisArgs& p, long long cta_tile
 // Measured per launch, plain tau-pass against this one: 512 points (three fields
 // of 256x256) 463 -> 415 us, 256 (three of 128x128) 57 -> 49, 128 (two of 512x512)
 // 231 -> 212, 64 (two of 1024x256) 127 -> 115, 768 (two of 192x192, then in four
-// passes) 388 -> 348.  Plans of three or four passes and fewer threads lost 1 to 5 %
-// (192 and 384 points in four passes, their block barriers).
+// passes) 388 -> 348.  (Plans of four passes, replaced since, lost 1 to 5 % on 192 and
+// 384 points to their block barriers.)
 // What bounds it: latency between the phases of a tile at 12 to 16 warps per SM
-// (512 points: issue 49 %, FP32 pipe 45 %, shared memory 49 %, DRAM 48 %); plans
+// (512 points: issue 47 %, FP32 pipe 43 %, shared memory 47 %, DRAM 47 %); plans
 // with 16 values per thread and twice the warps were slower (494 to 580 us).
 template <class PL>
 __host__ __device__ constexpr bool tau_pipe() { return PL::T >= 8 && PL::T <= 32 && (PL::NP == 2 || PL::T == 32); }
@@ -907,7 +908,7 @@ struct MapArgs {
 cudaError_t run_map_tables(const MapArgs& a, cudaStream_t s);
 // P += m * len at every point (a map replaced between propagations)
 cudaError_t run_map_phase_advance(double* mphase, const double* m, double len, long long nxy, cudaStream_t s);
-// the linear step's multiply element by element (grids with nt = 1)
+// the linear step's multiply element by element (grids with ny = nt = 1)
 cudaError_t run_prop_pointwise(const AxisArgs& a, int nf, cudaStream_t s);
 // diagnostics (k_diag.cu): out[f nt + k] = sum_{x,y} |A_f(tau_k)|^2, and
 // out[f nt + m] += sum_{x,y} |DFT_tau A_f|^2 (m) (out zeroed by the caller;
@@ -1009,14 +1010,20 @@ cudaError_t run_phase_tables(float2* px, int nx, float2* py, int ny, float2* pt,
   X(2) X(4) X(8) X(16) X(32) X(64) X(128) X(256) X(512) X(1024) X(2048) X(4096) \
   X(6) X(12) X(24) X(48) X(96) X(192) X(384) X(768)
 
-// Planes with a plane-pass kernel: 24 to 64 by 8 to 64 points and 16 by 8 to 64, up
-// to 1536 points.  A larger plane keeps one CTA busy for longer than the three
-// passes take over the whole GPU: time per z-step of the plane pass with the
-// tau-pass against the four passes, two fields, 64 / 512 planes: 32x32 7.3 against
-// 10.5 us / 17.7 against 22.4, 24x64 11.0 against 13.2 / 30.6 against 34.1, 48x48
-// 14.6 against 14.4 / 48.0 against 47.0, 64x64 17.2 against 14.0 / 56.9 against 55.7,
-// 96x96 45.5 against 29.2 / 197 against 161 (three fields 32x32: 9.9 against 11.8 /
-// 26.3 against 29.1).
+// Planes with a plane-pass kernel: rows of 16 to 64 points and columns of 8 to 64, up to
+// 1536 points.  (On other planes of up to 1536 points, with rows of up to 12 points or of
+// 96 and more or columns of up to 6, it has not been tried; they take the four passes.)
+// A larger plane keeps one CTA busy for longer than the three passes take over the
+// whole GPU.
+// Time per z-step of the plane pass with the tau-pass against the four passes, 64 / 512
+// planes: two fields 16x16 7.0 against 13.6 us / 12.3 against 17.7, 32x32 7.4 against
+// 10.5 / 17.8 against 22.6, 24x64 10.6 against 12.8 / 29.0 against 32.4; three fields
+// 32x32 10.1 against 12.0 / 26.7 against 29.5, 24x64 13.8 against 15.6 / 39.0 against
+// 43.9, 48x32 13.1 against 14.2 / 40.2 against 41.2, 64x24 12.6 against 12.7 / 40.9
+// against 40.4.  Where it loses, by up to 5 %, are 512 planes and more: 24x24 with two
+// fields (21.3 against 20.6), 32x8, 48x8 and 48x24 with three (15.8 against 15.2).  Past
+// 1536 points, two fields: 48x48 14.6 against 14.4 / 48.0 against 47.0, 64x64 17.2
+// against 14.0 / 56.9 against 55.7, 96x96 45.5 against 29.2 / 197 against 161.
 #define BRAHMS_FOR_EACH_PLANE(X)                                        \
   X(16, 8) X(16, 12) X(16, 16) X(16, 24) X(16, 32) X(16, 48) X(16, 64)  \
   X(24, 8) X(24, 12) X(24, 16) X(24, 24) X(24, 32) X(24, 48) X(24, 64)  \

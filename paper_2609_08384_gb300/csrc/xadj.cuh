@@ -12,8 +12,7 @@
 // y-inverse passes.
 //
 // MAP: under a transverse mismatch map every point has its own stage phases,
-// T V^s (s = 0, 1, 2) from the same tables as the forward x-pass; the
-// coefficient sets are formed per point instead of once per CTA.  The
+// T V^s (s = 0, 1, 2), from the same tables as the forward x-pass.  The
 // sensitivities to the stage phases keep their meaning: the map term of
 // Phi(x, y, z) does not depend on the per-step mismatch.  Instantiated by
 // k_xadj.cu (map-free) and k_xadj_map.cu.
@@ -38,9 +37,10 @@ __device__ __forceinline__ float4 load_points(const float2* row, bool row_order,
 // time.  The recorded states come in place order, one 16-byte load a field and two
 // points.  Backward of the 2 x 128x128x256 state over 36 steps 10.65 -> 10.13 ms (so
 // about 14 of 75 us of this pass), 3 x 128x128x256 over 25 steps 11.58 -> 10.79, under
-// a map 11.87 -> 11.51 and 12.59 -> 11.74.  What bounds it: the FP32 pipe (184
-// operations a point, half step and pair of fields) beside 48 B a point and field of
-// memory traffic against the forward pass's 16.
+// a map 11.87 -> 11.51 and 12.59 -> 11.74; with all stage factors from FP64 10.28, 10.96,
+// 11.59 and 11.83.  What bounds it: the FP32 pipe (196 operations a point and half step
+// of two fields) beside 48 B a point and field of memory traffic against the forward
+// pass's 16.
 template <int NX, int F, int THREADS, bool MAP>
 __device__ __forceinline__ void xpass_adj_tile(const XAdjArgs& p, long long tile, float2* rowbuf, float (&sens)[6]) {
   using PL = FftPlan<NX>;
