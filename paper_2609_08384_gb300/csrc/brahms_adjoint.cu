@@ -183,8 +183,9 @@ brahms_status brahms_adjoint_forward(brahms_ctx* ctx, const void* const* fields,
     float2* px = ctx->adj_tab;
     float2* py = px + ctx->nx;
     float2* pt = py + ctx->ny;
+    const brahms::Norm norm = brahms::norm_of((double)ctx->nt);
     BR_CK(launch(ctx, 4, 1, [&] {
-      return brahms::run_phase_tables(px, ctx->nx, py, ctx->ny, pt, ctx->nt, ctx->adj_phi_dev, +1, ctx->stream);
+      return brahms::run_phase_tables(px, ctx->nx, py, ctx->ny, pt, ctx->nt, ctx->adj_phi_dev, +1, norm.rest, ctx->stream);
     }));
     brahms::AxisArgs at = aargs(ctx, 2);
     at.data = ctx->state + phi_field * n;
@@ -192,9 +193,8 @@ brahms_status brahms_adjoint_forward(brahms_ctx* ctx, const void* const* fields,
     at.px = px;
     at.py = py;
     at.pt = pt;
-    const double inv = 1.0 / (double)ctx->nt;
-    at.scale = (float)inv;
-    at.scale_lo = (float)(inv - (double)at.scale);
+    at.scale = norm.scale;
+    at.scaled = norm.rest != 0.0;
     BR_CK(launch(ctx, 2, 1, [&] { return brahms::run_tpass_prop(ctx->nt, at, ctx->stream); }));
   }
   // bookkeeping for the reverse sweep (Phi_j exactly as brahms_propagate accumulates it)

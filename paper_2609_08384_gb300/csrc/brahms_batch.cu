@@ -90,7 +90,7 @@ struct InstDev {
   int nz;
   double dz, dk;
   float kh[2], kh2[2];
-  float scale, scale_lo;
+  float scale;  // 1/(nx ny nt) as a float
   int n_x, n_y, n_t;      // items per pass type
   int g_x, g_y, g_t;      // CTA tiles per item (tile granularity)
   long long ct_x, ct_y, ct_t;  // CTA tiles per pass type
@@ -224,7 +224,6 @@ __device__ __noinline__ void run_item(const InstDev& I, const Item& it, float4* 
   a.py = I.py;
   a.pt = I.pt;
   a.scale = I.scale;
-  a.scale_lo = I.scale_lo;
   if (it.type == kTypeT) {
     a.xtiles = (NXY + ColTile<typename SH::PT>::value - 1) / ColTile<typename SH::PT>::value;
     a.ntiles = 2LL * NXY * a.xtiles;
@@ -672,9 +671,7 @@ brahms_status prepare_grouped(brahms_batch* b) {
     z.ny = g.ny;
     z.nt = g.nt;
     z.xtiles = 1;
-    const double inv_n = 1.0 / ((double)g.nx * g.ny * g.nt);  // picks the tau-pass's instance
-    z.scale = (float)inv_n;
-    z.scale_lo = (float)(inv_n - (double)z.scale);
+    z.scaled = norm_of((double)g.nx * g.ny * g.nt).rest != 0.0;  // picks the tau-pass's instance
     BB_CK(run_ypass(g.ny, false, z, b->stream));
     BB_CK(run_ypass(g.ny, true, z, b->stream));
     BB_CK(run_tpass_prop(g.nt, z, b->stream));
@@ -762,9 +759,9 @@ brahms_status prepare_grouped(brahms_batch* b) {
     at.px = g.px;
     at.py = g.py;
     at.pt = g.pt;
-    const double inv_n = 1.0 / (double)n;
-    at.scale = (float)inv_n;
-    at.scale_lo = (float)(inv_n - (double)at.scale);
+    const Norm norm = norm_of((double)n);
+    at.scale = norm.scale;
+    at.scaled = norm.rest != 0.0;
     if (e == cudaSuccess) e = xpass(-1, m);
     nl += plane || whole ? 1 : m;
     int a = m;
@@ -853,9 +850,7 @@ brahms_status prepare_persistent(brahms_batch* b) {
       d.kh[f] = (float)(k * 0.5 * I.dz);
       d.kh2[f] = 0.5f * d.kh[f];
     }
-    const double inv_n = 1.0 / (double)I.npoints();
-    d.scale = (float)inv_n;
-    d.scale_lo = (float)(inv_n - (double)d.scale);
+    d.scale = norm_of((double)I.npoints()).scale;
     const int rows = xtile_rows_of(I.shape);
     d.ct_x = ((long long)I.ny * I.nt + rows - 1) / rows;
     const long long ytiles = 2LL * I.nt * ((I.nx + col_tile_of(I.ny) - 1) / col_tile_of(I.ny));
@@ -938,6 +933,7 @@ brahms_status build_tables_for(brahms_batch* b, BatchInstHost& I) {
   a.dy = I.dy;
   a.dt = I.dt;
   a.dz = I.dz;
+  a.rest = norm_of((double)I.npoints()).rest;
   for (int f = 0; f < 2; ++f) {
     a.k[f] = kTwoPi * I.fp[f].n / I.fp[f].lambda;
     a.rho[f] = I.fp[f].rho;

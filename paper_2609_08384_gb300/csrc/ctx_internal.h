@@ -259,6 +259,7 @@ inline brahms_status build_tables(brahms_ctx* ctx, double dz) {
   a.dy = ctx->dy;
   a.dt = ctx->dt;
   a.dz = dz;
+  a.rest = brahms::norm_of((double)ctx->npoints()).rest;
   for (int f = 0; f < ctx->nf; ++f) {
     a.k[f] = kTwoPi * ctx->fp[f].n / ctx->fp[f].lambda;
     a.rho[f] = ctx->fp[f].rho;
@@ -381,9 +382,9 @@ inline brahms::AxisArgs aargs(brahms_ctx* c, int axis, bool tau_prop = true) {
   a.px = c->px;
   a.py = c->py;
   a.pt = c->pt;
-  const double inv_n = 1.0 / (double)c->npoints();
-  a.scale = (float)inv_n;
-  a.scale_lo = (float)(inv_n - (double)a.scale);
+  const brahms::Norm norm = brahms::norm_of((double)c->npoints());
+  a.scale = norm.scale;
+  a.scaled = norm.rest != 0.0;
   return a;
 }
 

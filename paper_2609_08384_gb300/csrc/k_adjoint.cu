@@ -51,7 +51,7 @@ cudaError_t run_phase_grad(const float2* gh, const float2* ah, long long plane, 
 // Spectral-phase propagator tables in delta form: px = py = 0 (identity),
 // pt[m] = e^{i sign phi[(m + nt/2) mod nt]} - 1 for the centred phase vector.
 __global__ void phase_tables_kernel(float2* px, int nx, float2* py, int ny, float2* pt, int nt, const double* phi,
-                                    int sign) {
+                                    int sign, double rest) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < nx) px[i] = make_float2(0.f, 0.f);
   if (i < ny) py[i] = make_float2(0.f, 0.f);
@@ -59,15 +59,15 @@ __global__ void phase_tables_kernel(float2* px, int nx, float2* py, int ny, floa
     const double r = sign * phi[(i + nt / 2) % nt];
     const double two_pi = 6.283185307179586476925286766559;
     const double rr = r - two_pi * rint(r / two_pi);
-    const float sh = sinf((float)(0.5 * rr));
-    pt[i] = make_float2(-2.f * sh * sh, sinf((float)rr));
+    const double sh = sin(0.5 * rr), amp = 1.0 + rest;  // as delta_phase (k_misc.cu)
+    pt[i] = make_float2((float)(rest - 2.0 * amp * sh * sh), (float)(amp * sin(rr)));
   }
 }
 
 cudaError_t run_phase_tables(float2* px, int nx, float2* py, int ny, float2* pt, int nt, const double* phi, int sign,
-                             cudaStream_t s) {
+                             double rest, cudaStream_t s) {
   const int n = nx > ny ? (nx > nt ? nx : nt) : (ny > nt ? ny : nt);
-  phase_tables_kernel<<<(n + 255) / 256, 256, 0, s>>>(px, nx, py, ny, pt, nt, phi, sign);
+  phase_tables_kernel<<<(n + 255) / 256, 256, 0, s>>>(px, nx, py, ny, pt, nt, phi, sign, rest);
   return cudaPeekAtLastError();
 }
 

@@ -73,7 +73,7 @@ cudaError_t run_tpass_prop(int nt, const AxisArgs& a, cudaStream_t s) {
 #define BRAHMS_T_CASE(N)                                       \
   case N:                                                      \
     if constexpr ((N & (N - 1)) == 0)                          \
-      if (a.scale_lo == 0.f) return launch_tprop<N, false>(a, s); \
+      if (!a.scaled) return launch_tprop<N, false>(a, s); \
     return launch_tprop<N, true>(a, s);
     BRAHMS_FOR_EACH_SIZE(BRAHMS_T_CASE)
 #undef BRAHMS_T_CASE

@@ -11,20 +11,17 @@ __device__ __forceinline__ double ang_freq(int m, int n, double d) {
   return 6.283185307179586476925286766559 * (double)mm / ((double)n * d);
 }
 
-// amp * exp(i phi) - 1 ("delta form").  The phase argument is formed and
-// reduced to [-pi, pi] in FP64, then evaluated with FP32 sines:
+// amp * exp(i phi) - 1 ("delta form"), formed in FP64 and rounded once:
 //   amp cos(phi) - 1 = (amp - 1) - 2 amp sin^2(phi/2),   amp sin(phi).
 // Stored this way, a factor with a small phase keeps |1 + D| = amp to FP32
 // relative precision of the small part, so repeated application does not
-// bias the field energy.
+// bias the field energy.  (amp - 1 can be as small as the rest of a norm: a sine
+// rounded to a float first would swallow it, always.)
 __device__ __forceinline__ float2 delta_phase(double phi, double amp_m1) {
   const double two_pi = 6.283185307179586476925286766559;
   const double r = phi - two_pi * rint(phi / two_pi);
-  const float sh = sinf((float)(0.5 * r));
-  const float s = sinf((float)r);
-  const float am1 = (float)amp_m1;
-  const float amp = (float)(1.0 + amp_m1);
-  return make_float2(fmaf(-2.f * amp * sh, sh, am1), amp * s);
+  const double sh = sin(0.5 * r), amp = 1.0 + amp_m1;
+  return make_float2((float)(amp_m1 - 2.0 * amp * sh * sh), (float)(amp * sin(r)));
 }
 
 // Separable factors of the linear propagator over dz (Eqs. dispOp, diffOp,
@@ -39,6 +36,7 @@ __global__ void prop_tables_kernel(const TableArgs a) {
   if (i >= per * a.nf) return;
   const int f = i / per;
   int m = i % per;
+  const bool cw = a.nt == 1 && a.ny > 1;
   if (m < a.nx) {
     const double kx = ang_freq(m, a.nx, a.dx);
     const double ph = -a.dz * (kx * kx / (2.0 * a.k[f]) + tan(a.rho[f]) * kx);
@@ -48,13 +46,14 @@ __global__ void prop_tables_kernel(const TableArgs a) {
   m -= a.nx;
   if (m < a.ny) {
     const double ky = ang_freq(m, a.ny, a.dy);
-    a.py[f * a.ny + m] = delta_phase(-a.dz * ky * ky / (2.0 * a.k[f]), 0.0);
+    a.py[f * a.ny + m] = delta_phase(-a.dz * ky * ky / (2.0 * a.k[f]), cw ? a.rest : 0.0);
     return;
   }
   m -= a.ny;
   const double om = ang_freq(m, a.nt, a.dt);
   const double ph = a.dz * (-a.delta[f] * om + 0.5 * a.k2[f] * om * om - a.k3[f] / 6.0 * om * om * om);
-  a.pt[f * a.nt + m] = delta_phase(ph, expm1(-0.5 * a.alpha[f] * a.dz));
+  const double loss = expm1(-0.5 * a.alpha[f] * a.dz), rest = cw ? 0.0 : a.rest;
+  a.pt[f * a.nt + m] = delta_phase(ph, loss + rest + loss * rest);
 }
 
 // ---------------------------------------------- mismatch-map tables
@@ -270,7 +269,7 @@ __global__ void prop_pointwise_kernel(const AxisArgs p, int nf) {
     const int t = (int)(r / plane);
     const float2 dx = p.px[f * p.nx + x], dy = p.py[f * p.ny + y], dt = p.pt[f * p.nt + t];
     float2* q = p.data + (long long)f * p.fstride + r;
-    *q = p.scale_lo == 0.f ? ColumnProp<false>(p, dx, dy)(p, *q, dt) : ColumnProp<true>(p, dx, dy)(p, *q, dt);
+    *q = !p.scaled ? ColumnProp<false>(p, dx, dy)(p, *q, dt) : ColumnProp<true>(p, dx, dy)(p, *q, dt);
   }
 }
 

@@ -161,7 +161,7 @@ __global__ void __launch_bounds__(PL::T * TX, PL::T * TX <= 256 ? 2 : 1)
     fft_run<PL, false, 0, XchCol<TX>, SyncBlock, TWA>(v, t, xc, tw);
     const float2 zero = make_float2(0.f, 0.f);
     const float2 dx = act ? p.px[f * p.nx + x] : zero, dy = act ? p.py[f * p.ny + y] : zero;
-    if (p.scale_lo == 0.f) apply_prop<PL>(v, p, ColumnProp<false>(p, dx, dy), p.pt + f * p.nt, t);
+    if (!p.scaled) apply_prop<PL>(v, p, ColumnProp<false>(p, dx, dy), p.pt + f * p.nt, t);
     else apply_prop<PL>(v, p, ColumnProp<true>(p, dx, dy), p.pt + f * p.nt, t);
     fft_run<PL, true, 0, XchCol<TX>, SyncBlock, TWA>(v, t, xc, tw);
     if (act) {
@@ -261,7 +261,7 @@ __global__ void __launch_bounds__(PL::T * 16, 2)
     fft_run<PL, false, 0, XchColSplit<TX>, SyncBlock, TwGlobal>(v, t, xc, tw);
     const float2 zero = make_float2(0.f, 0.f);
     const float2 dx = act ? p.px[f * p.nx + x] : zero, dy = act ? p.py[f * p.ny + y] : zero;
-    if (p.scale_lo == 0.f) apply_prop<PL>(v, p, ColumnProp<false>(p, dx, dy), p.pt + f * p.nt, t);
+    if (!p.scaled) apply_prop<PL>(v, p, ColumnProp<false>(p, dx, dy), p.pt + f * p.nt, t);
     else apply_prop<PL>(v, p, ColumnProp<true>(p, dx, dy), p.pt + f * p.nt, t);
     fft_run<PL, true, 0, XchColSplit<TX>, SyncBlock, TwGlobal>(v, t, xc, tw);
     if (act) {

@@ -71,7 +71,8 @@ struct AxisArgs {
   const float2* px;    // [nf][nx] propagator factors (t-pass only)
   const float2* py;    // [nf][ny]
   const float2* pt;    // [nf][nt]
-  float scale, scale_lo;  // 1/(nx ny nt) = scale + scale_lo (lo = 0 for powers of two)
+  float scale;            // 1/(nx ny nt) as a float
+  int scaled;             // it is no power of two: see ColumnProp
   int conj_p;             // apply conj(P) (the adjoint of the linear step)
 };
 
@@ -580,11 +581,13 @@ __device__ __forceinline__ void axis_tile(const AxisArgs& p, long long cta_tile,
 // factors in delta form.  With 1 + Dxy = (1 + Dx)(1 + Dy) a value w becomes
 //   c w + w E(Omega),  E = g0 + Dt g1,  g0 = c Dxy,  g1 = c (1 + Dxy),
 // c = 1/(nx ny nt) = scale where that is a power of two.  Where it is not (SCALED), c = 1
-// and the result is scaled: scale w + (scale w E + scale_lo (w + w E)).  (With such a scale in g0
-// and g1 their rounding came on top of Dxy's, the same one in every step: the parametric
-// run of 48x256x128 points ended 12 % further from FP64, and noise on a grid of 3 2^k
-// points gained 6e-8 of its energy per step.  Scaling w before the product rounds w once
-// more: 3 x 48x32x48 over 88 steps 1.62e-6 from FP64 instead of 1.58e-6.)
+// and the result is scaled, scale w + scale w E, and the transformed axis's table carries
+// what the float is short of 1/(nx ny nt), a factor 1 + rest of its entries, which are
+// rounded once either way.  (With such a scale in g0 and g1 their rounding came on top of
+// Dxy's, the same one in every step: the parametric run of 48x256x128 points ended 12 %
+// further from FP64, and noise on a grid of 3 2^k points gained 6e-8 of its energy per
+// step.  Scaling w by hi + lo floats before the product rounds w once more; after it they
+// take two more operations a value, 450 instead of 406 us on 2 x 512x256x384.)
 // The small product w E is formed first and c w added with one rounding.  (Folding w into the FMA chain rounds w.x - w.y E.y before the
 // second-order term w.x (cos phi - 1) arrives; for small phases that term is below
 // half an ulp and is then always lost, so |1 + E| acts as 1 + phi^2 / 2 and the
@@ -609,7 +612,7 @@ struct ColumnProp {
     const float ey = fmaf(dt.x, gi.y, fmaf(dt.y, gi.z, gi.x));
     const float2 we = make_float2(fmaf(w.x, ex, -w.y * ey), fmaf(w.x, ey, w.y * ex));
     if constexpr (SCALED)
-      return __ffma2_rn(w, dup(p.scale), __ffma2_rn(we, dup(p.scale), __fmul2_rn(cadd(w, we), dup(p.scale_lo))));
+      return __ffma2_rn(w, dup(p.scale), __fmul2_rn(we, dup(p.scale)));
     else return __ffma2_rn(w, dup(c), we);
   }
 };
@@ -875,6 +878,17 @@ int tw_table_size_of(int n, int axis);
 bool fill_twiddles(float2* host, int n, int axis);
 bool fill_twiddles(float4* host, int n, int axis);
 cudaError_t upload_twiddles(float2* tw, int n, int axis, cudaStream_t s);
+// 1/n = scale (1 + rest); rest = 0 for a power of two
+struct Norm {
+  float scale;
+  double rest;
+};
+inline Norm norm_of(double n) {
+  const float scale = (float)(1.0 / n);
+  return {scale, 1.0 / n / (double)scale - 1.0};
+}
+// rest (of 1/(nx ny nt)) goes into pt, or into py on a cw grid (nt = 1, ny > 1), whose
+// linear step transforms y
 struct TableArgs {
   float2* px;
   float2* py;
@@ -882,6 +896,7 @@ struct TableArgs {
   int nx, ny, nt, nf;
   double dx, dy, dt, dz;
   double k[3], rho[3], delta[3], k2[3], k3[3], alpha[3];
+  double rest;
 };
 cudaError_t run_prop_tables(const TableArgs& a, cudaStream_t s);
 // Stage phase factors of one x-pass under a transverse mismatch map m(x, y):
@@ -1001,7 +1016,7 @@ cudaError_t run_scale_fields(const float2* a, float2* g, long long n, int nf, lo
                              cudaStream_t st);
 cudaError_t run_phase_grad(const float2* gh, const float2* ah, long long plane, int nt, double* acc, cudaStream_t s);
 cudaError_t run_phase_tables(float2* px, int nx, float2* py, int ny, float2* pt, int nt, const double* phi, int sign,
-                             cudaStream_t s);
+                             double rest, cudaStream_t s);
 
 }  // namespace brahms
 
